@@ -140,6 +140,8 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int32_t* __restr
   // this CTA's slice of the vocabulary
   const int chunk = (V + nblk - 1) / nblk;
   const int v_lo = rank * chunk, v_hi = min(V, v_lo + chunk);
+  pdl_wait();          // everything below may belong to earlier kernels
+  pdl_trigger();
   for (int e = tid; e < N + 2; e += kAcceptThreads) parent_child_off[e] = t.child_off[(size_t)b * (N + 2) + e];
   for (int e = tid; e < N; e += kAcceptThreads) {
     child_list[e] = t.child_list[(size_t)b * N + e];
@@ -250,11 +252,8 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int32_t* __restr
 }  // namespace
 
 cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptView& a, int lmax, int32_t* accepted,
-                          int32_t* len, int32_t* next_token, int32_t* final_node, cudaStream_t st) {
+                          int32_t* len, int32_t* next_token, int32_t* final_node, int sms, cudaStream_t st) {
   static int cache[64] = {};
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   int cluster = max_cluster_ctas(accept_kernel, kAcceptThreads, cache);
   if (cluster > kAcceptCluster && B * cluster > sms) cluster = kAcceptCluster;   // many sequences: smaller clusters
   while (cluster > 1 && a.V < cluster * kAcceptThreads) cluster >>= 1;           // small vocabularies

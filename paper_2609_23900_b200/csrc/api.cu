@@ -25,11 +25,14 @@ int cuda_fail(lumo_ctx* ctx, cudaError_t e, const char* what) {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 struct DeviceGuard {
-  int prev = -1;
+  int prev = -1;       // device to go back to; -1: nothing was changed
   bool ok = true;
   explicit DeviceGuard(int dev) {
-    if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; return; }
-    if (prev != dev && cudaSetDevice(dev) != cudaSuccess) ok = false;
+    int cur = -1;
+    if (cudaGetDevice(&cur) != cudaSuccess) { ok = false; return; }
+    if (cur == dev) return;
+    prev = cur;
+    if (cudaSetDevice(dev) != cudaSuccess) ok = false;
   }
   ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
@@ -66,26 +69,28 @@ int prepare(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_args* laye
     return fail(ctx, LUMO_ERR_ARG, "n_snap must be in [1, 256] in snapshot list mode");
   for (int l = 0; l < n_layers; ++l) {
     const lumo_gdn_args& a = layers[l];
-    const std::string at = " (layer " + std::to_string(l) + ")";
+    auto bad = [&](int code, const char* msg) { return fail(ctx, code, msg + (" (layer " + std::to_string(l) + ")")); };
     if (a.Hk != a0.Hk || a.Hv != a0.Hv || a.d != a0.d || a.in_dtype != a0.in_dtype ||
         a.gate_dtype != a0.gate_dtype || a.out_dtype != a0.out_dtype || a.scale != a0.scale ||
         a.qk_l2norm != a0.qk_l2norm || a.l2_eps != a0.l2_eps || a.n_state_rows != a0.n_state_rows ||
         a.snapshot_mode != a0.snapshot_mode || a.n_snap != a0.n_snap || (a.x == nullptr) != (a0.x == nullptr) ||
         a.gate_mode != a0.gate_mode)
-      return fail(ctx, LUMO_ERR_ARG, "all layers must share shape, dtypes and options" + at);
+      return bad(LUMO_ERR_ARG, "all layers must share shape, dtypes and options");
     if (!a.q || !a.k || !a.v || !a.alpha || !a.beta || !a.state || !a.state_row)
-      return fail(ctx, LUMO_ERR_ARG, "q, k, v, alpha, beta, state and state_row are required" + at);
+      return bad(LUMO_ERR_ARG, "q, k, v, alpha, beta, state and state_row are required");
     if (a.gate_mode == 1 && (!a.a_log || !a.dt_bias))
-      return fail(ctx, LUMO_ERR_ARG, "raw gates need a_log and dt_bias" + at);
-    if (for_verify && !a.out) return fail(ctx, LUMO_ERR_ARG, "out is required" + at);
+      return bad(LUMO_ERR_ARG, "raw gates need a_log and dt_bias");
+    if (for_verify && !a.out) return bad(LUMO_ERR_ARG, "out is required");
     if (a.x && (!a.conv_w || !a.conv_hist))
-      return fail(ctx, LUMO_ERR_ARG, "x needs conv_w and conv_hist" + at);
-    if (for_verify && a.snapshot_mode != 0 && !a.snap_out) return fail(ctx, LUMO_ERR_ARG, "snap_out is required" + at);
-    if (for_verify && a.snapshot_mode == 1 && !a.snap_nodes) return fail(ctx, LUMO_ERR_ARG, "snap_nodes is required" + at);
+      return bad(LUMO_ERR_ARG, "x needs conv_w and conv_hist");
+    if (for_verify && a.snapshot_mode != 0 && !a.snap_out) return bad(LUMO_ERR_ARG, "snap_out is required");
+    if (for_verify && a.snapshot_mode == 1 && !a.snap_nodes) return bad(LUMO_ERR_ARG, "snap_nodes is required");
+    uintptr_t bits = 0;                               // null pointers are aligned
     for (const void* p : {(const void*)a.q, (const void*)a.k, (const void*)a.v, a.x, a.conv_w, a.conv_b,
                           (const void*)a.conv_hist, (const void*)a.state, (const void*)a.out,
                           (const void*)a.snap_out})
-      if (p && !aligned16(p)) return fail(ctx, LUMO_ERR_ARG, "tensor pointers must be 16-byte aligned" + at);
+      bits |= reinterpret_cast<uintptr_t>(p);
+    if (bits & 15u) return bad(LUMO_ERR_ARG, "tensor pointers must be 16-byte aligned");
     LayerPtrs& p = lb->l[l];
     p.q = a.q; p.k = a.k; p.v = a.v; p.alpha = a.alpha; p.beta = a.beta;
     p.a_log = a.a_log; p.dt_bias = a.dt_bias;
@@ -93,6 +98,7 @@ int prepare(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_args* laye
     p.state = a.state; p.state_row = a.state_row; p.out = a.out;
     p.snap_nodes = a.snap_nodes; p.snap_out = a.snap_out; p.status = a.status;
   }
+  for (int l = n_layers; l < kFewLayers; ++l) lb->l[l] = LayerPtrs{};   // a launch of few layers hands over kFewLayers entries
   return LUMO_OK;
 }
 
@@ -482,7 +488,7 @@ int lumo_tree_accept(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_accep
   v.V = a->V; v.mode = a->mode; v.token = a->token; v.p_target = a->p_target; v.q_draft = a->q_draft;
   v.uniforms = a->uniforms; v.noise = a->noise; v.work = a->work;
   cudaError_t e = launch_accept(tree_view(desc, 0), desc->B, desc->N, desc->Ns, v, lmax, accepted_dev, len_dev,
-                                next_token_dev, final_node_dev, (cudaStream_t)stream);
+                                next_token_dev, final_node_dev, ctx->sm_count, (cudaStream_t)stream);
   ctx->last_call = lumo_ctx::kOther;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "accept launch");
 }
@@ -498,7 +504,8 @@ int lumo_select_spine_top3(lumo_ctx* ctx, const lumo_select_args* a, int32_t* sp
   if (sp != 0 && sp != 1 && sp != 2 && sp != 4 && sp != 8 && sp != 16)
     return fail(ctx, LUMO_ERR_ARG, "split must be 0, 1, 2, 4, 8 or 16");
   DeviceGuard g(ctx->device);
-  cudaError_t e = launch_select(a->logits, a->dtype, a->rows, a->V, sp, spine_dev, cand_dev, (cudaStream_t)stream);
+  cudaError_t e = launch_select(a->logits, a->dtype, a->rows, a->V, sp, spine_dev, cand_dev, ctx->sm_count,
+                                (cudaStream_t)stream);
   ctx->last_call = lumo_ctx::kOther;
   if (e == cudaErrorInvalidConfiguration) {
     (void)cudaGetLastError();
@@ -523,7 +530,6 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
                          void* stream) {
   Shape s;
   LayerBatch lb;
-  std::memset(&lb, 0, sizeof(lb));
   int rc = prepare(ctx, desc, layers, n_layers, true, &s, &lb);
   if (rc != LUMO_OK) return rc;
   DeviceGuard g(ctx->device);
@@ -540,7 +546,7 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
   if (gram_ok && ctx->scan_algo != 1) {
     cudaError_t e = cudaSuccess;
     if (layers[0].x) {
-      e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, use_overlap(ctx, s), st); });
+      e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, ctx->sm_count, use_overlap(ctx, s), st); });
       if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
     }
     const bool state_fresh = !layers[0].x && (prev_call == lumo_ctx::kCommit || prev_call == lumo_ctx::kCommitVerify);
@@ -569,7 +575,7 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
     ctx->scratch_bytes = stack_bytes;
   }
   if (layers[0].x) {
-    e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, use_overlap(ctx, s), st); });
+    e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, ctx->sm_count, use_overlap(ctx, s), st); });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
   }
   e = timed(ctx, LUMO_K_SCAN, st, [&] {
@@ -589,7 +595,6 @@ int lumo_gdn_tree_scan_static(lumo_ctx* ctx, const lumo_tree_desc* desc, const l
                               int n_layers, void* stream) {
   Shape s;
   LayerBatch lb;
-  std::memset(&lb, 0, sizeof(lb));
   int rc = prepare(ctx, desc, layers, n_layers, true, &s, &lb);
   if (rc != LUMO_OK) return rc;
   DeviceGuard g(ctx->device);
@@ -618,7 +623,6 @@ int lumo_gdn_commit(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_ar
     return fail(ctx, LUMO_ERR_ARG, "lmax must be in [1, " + std::to_string(kMaxNodes) + "] (a path holds each node at most once)");
   Shape s;
   LayerBatch lb;
-  std::memset(&lb, 0, sizeof(lb));
   int rc = prepare(ctx, desc, layers, n_layers, false, &s, &lb);
   if (rc != LUMO_OK) return rc;
   if (!accepted_dev || !len_dev) return fail(ctx, LUMO_ERR_ARG, "accepted_dev and len_dev are required");
@@ -643,8 +647,6 @@ int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const
   Shape ps, s;
   LayerBatch lb;
   FusedPrev fp;
-  std::memset(&lb, 0, sizeof(lb));
-  std::memset(&fp, 0, sizeof(fp));
   int rc = prepare(ctx, prev_desc, prev_layers, n_layers, false, &ps, &fp.lb);
   if (rc != LUMO_OK) return rc;
   rc = prepare(ctx, desc, layers, n_layers, true, &s, &lb);
@@ -696,7 +698,8 @@ int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const
   }
   if (layers[0].x) {
     e = timed(ctx, LUMO_K_CONV, st, [&] {
-      return fp.hist_in_kernels ? launch_conv_fused(s, t, lb, fp, pdl_conv, st) : launch_conv(s, t, lb, pdl_conv, st);
+      return fp.hist_in_kernels ? launch_conv_fused(s, t, lb, fp, ctx->sm_count, pdl_conv, st)
+                                : launch_conv(s, t, lb, ctx->sm_count, pdl_conv, st);
     });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
   }
@@ -735,14 +738,14 @@ int prepare_attn(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_attn_args
   if (a0.n_splits < 0 || a0.n_splits > 32) return fail(ctx, LUMO_ERR_ARG, "n_splits must be 0 (automatic) or in [1, 32]");
   for (int l = 0; l < n_layers; ++l) {
     const lumo_attn_args& a = layers[l];
-    const std::string at = " (layer " + std::to_string(l) + ")";
+    auto bad = [&](const char* msg) { return fail(ctx, LUMO_ERR_ARG, msg + (" (layer " + std::to_string(l) + ")")); };
     if (a.Hq != a0.Hq || a.Hkv != a0.Hkv || a.dh != a0.dh || a.scale != a0.scale || a.n_cache_rows != a0.n_cache_rows ||
         a.max_positions != a0.max_positions || a.ctx_len != a0.ctx_len || a.cache_row != a0.cache_row ||
         a.n_splits != a0.n_splits || a.kv_layout != a0.kv_layout)
-      return fail(ctx, LUMO_ERR_ARG, "all layers must share shapes, options, ctx_len and cache_row" + at);
-    if (!a.k_cache || !a.v_cache) return fail(ctx, LUMO_ERR_ARG, "k_cache and v_cache are required" + at);
+      return bad("all layers must share shapes, options, ctx_len and cache_row");
+    if (!a.k_cache || !a.v_cache) return bad("k_cache and v_cache are required");
     for (const void* p : {(const void*)a.k_cache, (const void*)a.v_cache, a.q, a.k_new, a.v_new, (const void*)a.out})
-      if (p && !aligned16(p)) return fail(ctx, LUMO_ERR_ARG, "tensor pointers must be 16-byte aligned" + at);
+      if (p && !aligned16(p)) return bad("tensor pointers must be 16-byte aligned");
   }
   s->B = desc->B; s->N = desc->N; s->Ns = desc->Ns; s->Hq = a0.Hq; s->Hkv = a0.Hkv;
   s->n_rows = a0.n_cache_rows; s->max_pos = a0.max_positions; s->scale = a0.scale;
@@ -776,10 +779,7 @@ int lumo_kv_write_tree(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_att
   KvLayers L;
   KvShape k;
   kv_views(desc, layers, n_layers, s, &L, &k);
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l < n_layers && e == cudaSuccess; ++l)
-    if (layers[l].status) e = cudaMemsetAsync(layers[l].status, 0, (size_t)s.B * sizeof(int32_t), st);
-  if (e == cudaSuccess) e = timed(ctx, LUMO_K_KV_WRITE, st, [&] { return launch_kv_write(L, k, n_layers, st); });
+  cudaError_t e = timed(ctx, LUMO_K_KV_WRITE, st, [&] { return launch_kv_write(L, k, n_layers, st); });
   ctx->last_call = lumo_ctx::kOther;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "kv write launch");
 }

@@ -343,6 +343,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     sm.timed_out = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
+  // The set-up above touches nothing of earlier kernels; the caches, queries, lengths and scratch below may.
+  pdl_wait();
+  pdl_trigger();
   if (tid < kSeqCache && tid < a.B) {          // the work iterator of every role reads these instead of global memory
     const int cx = a.ctx_len[tid], cr = a.cache_row[tid];
     sm.seq_ctx[tid] = cx; sm.seq_row[tid] = cr;
@@ -670,6 +673,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 template <int kBatch>
 __global__ void __launch_bounds__(256) attn_merge_kernel(const AttnArgs a) {
   pdl_wait();          // launched as a programmatic dependent of the attention kernel: its slots are complete from here on
+  pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int GN = a.G * a.N;
   const int upb = a.Hkv * a.RT;
@@ -825,8 +829,7 @@ cudaError_t attn_plan(const AttnShape& s, const AttnLayerPtrs& p, const uint32_t
 }
 
 cudaError_t launch_attn(const AttnPlan& plan, cudaStream_t st) {
-  tree_attn_kernel<<<plan.grid, kThreads, kSmemBytes, st>>>(plan.tk, plan.tv, plan.a);
-  return cudaGetLastError();
+  return launch_kernel(tree_attn_kernel, plan.grid, dim3(kThreads), kSmemBytes, st, true, plan.tk, plan.tv, plan.a);
 }
 
 cudaError_t launch_attn_merge(const AttnPlan& plan, cudaStream_t st) {

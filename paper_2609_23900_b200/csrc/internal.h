@@ -121,9 +121,24 @@ struct LayerPtrs {
   int32_t* status;
 };
 
-struct LayerBatch {
-  LayerPtrs l[kMaxLayers];
+// The layers of one call, passed by value as a kernel parameter.  A launch copies its parameters twice (host to
+// driver, driver to GPU): 64 layers are 8.7 KB and cost 0.6 us more per launch than 0.6 KB (measured with empty
+// kernels: 2.2 against 1.6 us of host time), so calls of up to kFewLayers layers, the bulk of the latency-bound
+// ones, take a kernel instance with a short array.
+constexpr int kFewLayers = 4;
+template <int CAP>
+struct LayersT {
+  static constexpr int kCap = CAP;
+  LayerPtrs l[CAP];
 };
+using LayerBatch = LayersT<kMaxLayers>;
+using FewLayers = LayersT<kFewLayers>;
+// the first kFewLayers entries of a batch of at most that many (prepare() clears the unused ones)
+inline FewLayers few_layers(const LayerBatch& lb) {
+  FewLayers f;
+  for (int i = 0; i < kFewLayers; ++i) f.l[i] = lb.l[i];
+  return f;
+}
 
 struct Shape {
   int B, N, Ns, Hk, Hv, d, C;
@@ -139,12 +154,22 @@ struct Shape {
 // What the fused commit + verify scan needs of the previous cycle: its layers (recorded k, v, gates,
 // status), its tree (parent, slot) and the device-resident accepted path.
 constexpr int kFusedMaxPath = 16;
-struct FusedPrev {
-  LayerBatch lb;
+template <class LB>
+struct FusedPrevT {
+  LB lb;
   const int32_t* parent; const int32_t* slot; int N, Ns;
   const int32_t* accepted; const int32_t* len; int lmax;
   int hist_in_kernels;   // 1: the conv reads the committed history through the path and the scan writes it back
 };
+using FusedPrev = FusedPrevT<LayerBatch>;
+inline FusedPrevT<FewLayers> few_layers(const FusedPrev& fp) {
+  FusedPrevT<FewLayers> f;
+  f.lb = few_layers(fp.lb);
+  f.parent = fp.parent; f.slot = fp.slot; f.N = fp.N; f.Ns = fp.Ns;
+  f.accepted = fp.accepted; f.len = fp.len; f.lmax = fp.lmax;
+  f.hist_in_kernels = fp.hist_in_kernels;
+  return f;
+}
 
 struct TreeDev {
   const int32_t* parent; const int32_t* depth; const int32_t* slot; const int32_t* slot_inv;
@@ -241,22 +266,32 @@ int max_cluster_ctas(K kern, int threads, int (&cache)[64]) {
   return cache[dev];
 }
 
-// launch of a kernel whose CTAs form clusters of `cluster` along x
+// The arguments are handed over by address: a batch of layers is not copied again on its way to the driver.
+template <typename... KArgs>
+cudaError_t launch_by_address(const cudaLaunchConfig_t& cfg, void (*kern)(KArgs...), const KArgs&... args) {
+  void* p[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), p);
+}
+
+// Launch of a kernel whose CTAs form clusters of `cluster` along x, as a programmatic dependent of the kernel before
+// it: its CTAs are placed while that one drains and pass pdl_wait() before they touch global memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, Args... args) {
+cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  cfg.numAttrs = 2;
+  return launch_by_address<KArgs...>(cfg, kern, args...);
 }
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
-                          Args... args) {
+                          const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -264,17 +299,17 @@ cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+  return launch_by_address<KArgs...>(cfg, kern, args...);
 }
 #endif
 
 // launchers (kernels.cu); all return cudaError_t and only enqueue
-cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, bool pdl, cudaStream_t st);
+cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, cudaStream_t st);
 // entries of the visiting order one CTA of the convolution takes (16, 8 or 4: fewer when the grid would not cover the GPU)
 int conv_rows_per_cta(int C, int Ns, int seqs, int sms);
 // same convolution reading the history the previous cycle's accepted path would commit (not yet in memory)
-cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, bool pdl,
-                              cudaStream_t st);
+cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, int sm_count,
+                              bool pdl, cudaStream_t st);
 cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, float* stack,
                         int grid, cudaStream_t st);
 // persistent grid size (CTAs resident at once) and the stack scratch it needs
@@ -286,10 +321,10 @@ struct AcceptView {
   float* work;
 };
 cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptView& a, int lmax, int32_t* accepted,
-                          int32_t* len, int32_t* next_token, int32_t* final_node, cudaStream_t st);
+                          int32_t* len, int32_t* next_token, int32_t* final_node, int sm_count, cudaStream_t st);
 // fused draft selection (select.cu)
 cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int split, int32_t* spine, int32_t* cand,
-                          cudaStream_t st);
+                          int sm_count, cudaStream_t st);
 // Gram-form scan on tcgen05 (scan_gram.cu)
 bool gram_supported(const Shape& s, int max_depth);
 // tail: 0 level-by-level substitution, 1 closed form (per-node back substitution, one output pass over the path),
@@ -342,11 +377,19 @@ struct AttnPlan {
   AttnArgs a;
   dim3 grid;
 };
-struct KvLayers {
-  void* k[kMaxAttnLayers]; void* v[kMaxAttnLayers];
-  const void* kn[kMaxAttnLayers]; const void* vn[kMaxAttnLayers];
-  int32_t* status[kMaxAttnLayers];
+template <int CAP>
+struct KvLayersT {
+  void* k[CAP]; void* v[CAP];
+  const void* kn[CAP]; const void* vn[CAP];
+  int32_t* status[CAP];
 };
+using KvLayers = KvLayersT<kMaxAttnLayers>;
+using FewKvLayers = KvLayersT<kFewLayers>;
+inline FewKvLayers few_layers(const KvLayers& L) {
+  FewKvLayers f;
+  for (int i = 0; i < kFewLayers; ++i) { f.k[i] = L.k[i]; f.v[i] = L.v[i]; f.kn[i] = L.kn[i]; f.vn[i] = L.vn[i]; f.status[i] = L.status[i]; }
+  return f;
+}
 struct KvShape {
   int B, N, Ns, Hkv, n_rows, max_pos, layout;
   const int32_t* ctx_len; const int32_t* cache_row;

@@ -9,6 +9,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <climits>
 #include <mutex>
 #include <type_traits>
@@ -89,8 +90,8 @@ template <> struct Packed4<__nv_bfloat16> {
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
 // scan that follows writes them to the history buffer once every CTA of this kernel has finished).
-template <typename T, int kConvRows, bool kFused>
-__device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp) {
+template <typename T, int kConvRows, bool kFused, class LB>
+__device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, const LB& lb, const FusedPrevT<LB>* fp) {
   __shared__ int s_win[kConvRows][4];
   __shared__ int s_prog[kConvRows];
   __shared__ int f_acc[kFusedMaxPath], f_par[kFusedMaxPath], f_phys[kFusedMaxPath];
@@ -231,13 +232,13 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   }
 }
 
-template <typename T, int kConvRows>
-__global__ void __launch_bounds__(256, 3) conv_kernel(Shape s, TreeDev t, LayerBatch lb) {
-  conv_body<T, kConvRows, false>(s, t, lb, nullptr);
+template <typename T, int kConvRows, class LB>
+__global__ void __launch_bounds__(256, 3) conv_kernel(Shape s, TreeDev t, LB lb) {
+  conv_body<T, kConvRows, false, LB>(s, t, lb, nullptr);
 }
-template <typename T, int kConvRows>
-__global__ void __launch_bounds__(256, 3) conv_fused_kernel(Shape s, TreeDev t, LayerBatch lb, FusedPrev fp) {
-  conv_body<T, kConvRows, true>(s, t, lb, &fp);
+template <typename T, int kConvRows, class LB>
+__global__ void __launch_bounds__(256, 3) conv_fused_kernel(Shape s, TreeDev t, LB lb, FusedPrevT<LB> fp) {
+  conv_body<T, kConvRows, true, LB>(s, t, lb, &fp);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -269,9 +270,9 @@ __host__ __device__ inline ScanSmem scan_smem(int N, int max_ops, int n_snap_lis
   return m;
 }
 
-template <int D, typename T>
+template <int D, typename T, class LB>
 __global__ void __launch_bounds__(kScanThreads)
-scan_kernel(Shape s, TreeDev t, LayerBatch lb, float* __restrict__ stack, int n_items) {
+scan_kernel(Shape s, TreeDev t, LB lb, float* __restrict__ stack, int n_items) {
   using Cfg = ScanCfg<D, T>;
   constexpr int NCH = Cfg::kChunks;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -499,9 +500,9 @@ scan_kernel(Shape s, TreeDev t, LayerBatch lb, float* __restrict__ stack, int n_
 // [old history ; x of the accepted nodes] (Algorithm 1).  The state tile is requested from memory
 // before the path is validated, so the two dependent chains (tile; length -> path -> operands) overlap;
 // nothing is written unless the path is valid.
-template <int D, typename T>
+template <int D, typename T, class LB>
 __global__ void __launch_bounds__(kScanThreads, (D == 128 && sizeof(T) == 2) ? 8 : 4)
-commit_kernel(Shape s, TreeDev t, LayerBatch lb, const int32_t* __restrict__ accepted,
+commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
               const int32_t* __restrict__ len_arr, int lmax, int n_state_ctas) {
   constexpr int NCH = D / 16;
   constexpr int kTiles = D / kRows;
@@ -617,6 +618,8 @@ __global__ void path_from_node_kernel(TreeDev t, int B, int N, const int32_t* __
                                       int lmax, int32_t* __restrict__ accepted,
                                       int32_t* __restrict__ len, int32_t* __restrict__ status) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
   if (b >= B) return;
   int32_t* acc = accepted + (size_t)b * lmax;
   for (int e = 0; e < lmax; ++e) acc[e] = -1;
@@ -659,33 +662,35 @@ int conv_rows_per_cta(int C, int Ns, int seqs, int sms) {
 }
 
 template <typename T>
-static cudaError_t launch_conv_t(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, bool pdl,
-                                 cudaStream_t st) {
+static cudaError_t launch_conv_t(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sms,
+                                 bool pdl, cudaStream_t st) {
   const int slabs = (s.C / 4 + 255) / 256, seqs = s.B * s.n_layers;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int rows = conv_rows_per_cta(s.C, s.Ns, seqs, sms);
+  const bool few = s.n_layers <= kFewLayers;
   auto go = [&](auto rows_c) {
-    constexpr int kRowsPerCta = decltype(rows_c)::value;
-    const dim3 grid(slabs, (s.Ns + kRowsPerCta - 1) / kRowsPerCta, seqs);
-    if (fp) return launch_kernel(conv_fused_kernel<T, kRowsPerCta>, grid, dim3(256), 0, st, pdl, s, t, lb, *fp);
-    return launch_kernel(conv_kernel<T, kRowsPerCta>, grid, dim3(256), 0, st, pdl, s, t, lb);
+    constexpr int R = decltype(rows_c)::value;
+    const dim3 grid(slabs, (s.Ns + R - 1) / R, seqs), block(256);
+    if constexpr (sizeof(T) == 2) {                               // the fused path serves bf16 operands only
+      if (fp && few) return launch_kernel(conv_fused_kernel<T, R, FewLayers>, grid, block, 0, st, pdl, s, t, few_layers(lb), few_layers(*fp));
+      if (fp) return launch_kernel(conv_fused_kernel<T, R, LayerBatch>, grid, block, 0, st, pdl, s, t, lb, *fp);
+    }
+    if (few) return launch_kernel(conv_kernel<T, R, FewLayers>, grid, block, 0, st, pdl, s, t, few_layers(lb));
+    return launch_kernel(conv_kernel<T, R, LayerBatch>, grid, block, 0, st, pdl, s, t, lb);
   };
   if (rows == 16) return go(std::integral_constant<int, 16>{});
   if (rows == 8) return go(std::integral_constant<int, 8>{});
   return go(std::integral_constant<int, 4>{});
 }
 
-cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, bool pdl, cudaStream_t st) {
-  if (s.in_dtype == LUMO_BF16) return launch_conv_t<__nv_bfloat16>(s, t, lb, nullptr, pdl, st);
-  return launch_conv_t<float>(s, t, lb, nullptr, pdl, st);
+cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, cudaStream_t st) {
+  if (s.in_dtype == LUMO_BF16) return launch_conv_t<__nv_bfloat16>(s, t, lb, nullptr, sm_count, pdl, st);
+  return launch_conv_t<float>(s, t, lb, nullptr, sm_count, pdl, st);
 }
 
-cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, bool pdl,
-                              cudaStream_t st) {
-  if (s.in_dtype != LUMO_BF16) return cudaErrorInvalidValue;      // the fused path serves bf16 operands only
-  return launch_conv_t<__nv_bfloat16>(s, t, lb, &fp, pdl, st);
+cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, int sm_count,
+                              bool pdl, cudaStream_t st) {
+  if (s.in_dtype != LUMO_BF16) return cudaErrorInvalidValue;
+  return launch_conv_t<__nv_bfloat16>(s, t, lb, &fp, sm_count, pdl, st);
 }
 
 cudaError_t scan_plan(const Shape& s, const TreeDev& t, int sm_count, int* grid, size_t* stack_bytes) {
@@ -695,13 +700,34 @@ cudaError_t scan_plan(const Shape& s, const TreeDev& t, int sm_count, int* grid,
     using T = decltype(tc);
     const int n_snap_list = s.snapshot_mode == 1 ? s.n_snap : 0;
     const ScanSmem lay = scan_smem(s.N, t.max_ops, n_snap_list, ScanCfg<D, T>::kStageBytes);
-    auto kern = scan_kernel<D, T>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
+    // occupancy of each instance at the shared-memory size it was last asked for: the two calls below cost more
+    // host time than the launch itself
+    static std::atomic<uint64_t> known[kMaxDevices][2] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kScanThreads, lay.total);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    const bool few = s.n_layers <= kFewLayers;
+    const uint64_t seen = known[dev][few].load(std::memory_order_relaxed);
+    int per_sm = (int)(seen & 0xFF);
+    if (seen >> 8 != (uint64_t)lay.total || per_sm == 0) {
+      auto kern = few ? (const void*)scan_kernel<D, T, FewLayers> : (const void*)scan_kernel<D, T, LayerBatch>;
+      // the limit only grows, so that a launch prepared for another size on another thread still fits
+      static std::mutex mu;
+      static int limit[kMaxDevices][2] = {};
+      {
+        std::lock_guard<std::mutex> lock(mu);
+        if (lay.total > limit[dev][few]) {
+          e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
+          if (e != cudaSuccess) return e;
+          limit[dev][few] = lay.total;
+        }
+      }
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kScanThreads, lay.total);
+      if (e != cudaSuccess) return e;
+      if (per_sm < 1) per_sm = 1;
+      known[dev][few].store((uint64_t)lay.total << 8 | (uint64_t)per_sm, std::memory_order_relaxed);
+    }
     const int resident = sm_count * per_sm;
     *grid = items < resident ? items : resident;
     *stack_bytes = (size_t)*grid * t.max_levels * kRows * D * sizeof(float);
@@ -745,8 +771,9 @@ cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, 
     using T = decltype(tc);
     const int n_snap_list = s.snapshot_mode == 1 ? s.n_snap : 0;
     const ScanSmem lay = scan_smem(s.N, t.max_ops, n_snap_list, ScanCfg<D, T>::kStageBytes);
-    scan_kernel<D, T><<<grid, kScanThreads, lay.total, st>>>(s, t, lb, stack, items);
-    return cudaGetLastError();
+    if (s.n_layers <= kFewLayers)
+      return launch_kernel(scan_kernel<D, T, FewLayers>, dim3(grid), dim3(kScanThreads), lay.total, st, false, s, t, few_layers(lb), stack, items);
+    return launch_kernel(scan_kernel<D, T, LayerBatch>, dim3(grid), dim3(kScanThreads), lay.total, st, false, s, t, lb, stack, items);
   });
 }
 
@@ -760,14 +787,15 @@ cudaError_t launch_commit(const Shape& s, const TreeDev& t, const LayerBatch& lb
     const int per_thread = 16 / (int)sizeof(T);
     const int n_hist = with_hist ? (s.C / per_thread + kScanThreads - 1) / kScanThreads : 0;
     dim3 grid(n_state + n_hist, s.B, s.n_layers);
-    return launch_kernel(commit_kernel<D, T>, grid, dim3(kScanThreads), 0, st, pdl, s, t, lb, accepted, len, lmax, n_state);
+    if (s.n_layers <= kFewLayers)
+      return launch_kernel(commit_kernel<D, T, FewLayers>, grid, dim3(kScanThreads), 0, st, pdl, s, t, few_layers(lb), accepted, len, lmax, n_state);
+    return launch_kernel(commit_kernel<D, T, LayerBatch>, grid, dim3(kScanThreads), 0, st, pdl, s, t, lb, accepted, len, lmax, n_state);
   });
 }
 
 cudaError_t launch_path_from_node(const TreeDev& t, int B, int N, const int32_t* node, int lmax,
                                   int32_t* accepted, int32_t* len, int32_t* status, cudaStream_t st) {
-  path_from_node_kernel<<<(B + 63) / 64, 64, 0, st>>>(t, B, N, node, lmax, accepted, len, status);
-  return cudaGetLastError();
+  return launch_kernel(path_from_node_kernel, dim3((B + 63) / 64), dim3(64), 0, st, true, t, B, N, node, lmax, accepted, len, status);
 }
 
 }  // namespace lumo

@@ -13,14 +13,15 @@ constexpr int kDh = 128;
 
 // Scatter of the tree's entries: grid (node, sequence, layer); a CTA copies the Hkv x 128 keys and
 // values of one node to position ctx + slot[node].
-__global__ void __launch_bounds__(128) kv_write_kernel(const KvLayers L, const KvShape s) {
+template <class KL>
+__global__ void __launch_bounds__(128) kv_write_kernel(const KL L, const KvShape s) {
   const int i = blockIdx.x, b = blockIdx.y, l = blockIdx.z;
+  pdl_wait();          // everything below may belong to earlier kernels
+  pdl_trigger();
   const int ctx = s.ctx_len[b], crow = s.cache_row[b];
   const int bad = seq_check(ctx, crow, s.Ns, s.n_rows, s.max_pos);
-  if (bad != LUMO_SEQ_OK) {
-    if (L.status[l] && i == 0 && threadIdx.x == 0) L.status[l][b] = bad;
-    return;
-  }
+  if (L.status[l] && i == 0 && threadIdx.x == 0) L.status[l][b] = bad;
+  if (bad != LUMO_SEQ_OK) return;
   const int chunks = s.Hkv * kDh / 8;      // 16-byte chunks per entry (16 per head)
   const size_t src = ((size_t)b * s.N + i) * chunks;
   const uint4* kn = reinterpret_cast<const uint4*>(L.kn[l]) + src;
@@ -40,13 +41,16 @@ __global__ void __launch_bounds__(128) kv_write_kernel(const KvLayers L, const K
 // Publication: grid (KV head x {K, V}, sequence, layer).  A CTA stages the 256-byte pieces of all
 // accepted entries that have to move (source != destination) in shared memory, then writes them: all
 // reads come before any write, and pieces of different heads never overlap.
-__global__ void __launch_bounds__(256) kv_publish_kernel(const KvLayers L, const KvShape s, const int32_t* __restrict__ accepted,
+template <class KL>
+__global__ void __launch_bounds__(256) kv_publish_kernel(const KL L, const KvShape s, const int32_t* __restrict__ accepted,
                                                          const int32_t* __restrict__ len, int lmax, int32_t* ctx_len_out) {
   extern __shared__ __align__(16) unsigned char stage[];     // [lmax][256 B]
   __shared__ int acc_s[kMaxNodes], par_s[kMaxNodes], src_s[kMaxNodes];
   __shared__ int st_s;
   const int hkv = blockIdx.x >> 1, which = blockIdx.x & 1, b = blockIdx.y, l = blockIdx.z;
   const int tid = threadIdx.x;
+  pdl_wait();          // everything below may belong to earlier kernels
+  pdl_trigger();
   const int ctx = s.ctx_len[b], crow = s.cache_row[b];
   const int n = len[b];
   const int nn = n < 0 ? 0 : (n > lmax ? lmax : n);
@@ -89,23 +93,31 @@ __global__ void __launch_bounds__(256) kv_publish_kernel(const KvLayers L, const
 }  // namespace
 
 cudaError_t launch_kv_write(const KvLayers& L, const KvShape& s, int n_layers, cudaStream_t st) {
-  kv_write_kernel<<<dim3(s.N, s.B, n_layers), 128, 0, st>>>(L, s);
-  return cudaGetLastError();
+  const dim3 grid(s.N, s.B, n_layers);
+  if (n_layers <= kFewLayers) return launch_kernel(kv_write_kernel<FewKvLayers>, grid, dim3(128), 0, st, true, few_layers(L), s);
+  return launch_kernel(kv_write_kernel<KvLayers>, grid, dim3(128), 0, st, true, L, s);
 }
 
-cudaError_t launch_kv_publish(const KvLayers& L, const KvShape& s, int n_layers, const int32_t* accepted, const int32_t* len,
-                              int lmax, int32_t* ctx_len_out, cudaStream_t st) {
+template <class KL>
+static cudaError_t launch_kv_publish_t(const KL& L, const KvShape& s, int n_layers, const int32_t* accepted, const int32_t* len,
+                                       int lmax, int32_t* ctx_len_out, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev >= 0 && dev < kMaxDevices && !configured[dev]) {
-    e = cudaFuncSetAttribute(kv_publish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxNodes * 256);
+    e = cudaFuncSetAttribute(kv_publish_kernel<KL>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxNodes * 256);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  kv_publish_kernel<<<dim3(2 * s.Hkv, s.B, n_layers), 256, (size_t)lmax * 256, st>>>(L, s, accepted, len, lmax, ctx_len_out);
-  return cudaGetLastError();
+  return launch_kernel(kv_publish_kernel<KL>, dim3(2 * s.Hkv, s.B, n_layers), dim3(256), (size_t)lmax * 256, st, true, L, s,
+                       accepted, len, lmax, ctx_len_out);
+}
+
+cudaError_t launch_kv_publish(const KvLayers& L, const KvShape& s, int n_layers, const int32_t* accepted, const int32_t* len,
+                              int lmax, int32_t* ctx_len_out, cudaStream_t st) {
+  if (n_layers <= kFewLayers) return launch_kv_publish_t(few_layers(L), s, n_layers, accepted, len, lmax, ctx_len_out, st);
+  return launch_kv_publish_t(L, s, n_layers, accepted, len, lmax, ctx_len_out, st);
 }
 
 }  // namespace lumo

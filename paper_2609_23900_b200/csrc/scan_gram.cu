@@ -596,9 +596,9 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
 // kDirect: the triangular system is solved on scalars per node (M = W (I + A)^-1 along each ancestry, no
 // dependency between nodes) and every output is one pass over its path; no level-by-level substitution.
 // kTensor (with kDirect): the output sum of the closed form runs on the tensor core (direct_tail_tc).
-template <int NT, bool kFused, bool kCompact = false, bool kDirect = false, bool kTensor = false>
-__device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t, const LayerBatch& lb, int n_items,
-                                               const FusedPrev* fp) {
+template <int NT, bool kFused, bool kCompact, bool kDirect, bool kTensor, class LB>
+__device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t, const LB& lb, int n_items,
+                                               const FusedPrevT<LB>* fp) {
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment for the swizzled operand tiles; plain pointer arithmetic on the shared
   // array keeps the pointers in the shared address space
@@ -1156,23 +1156,23 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(LY::kTmem) : "memory");
 }
 
-template <int NT, bool kDirect, bool kTensor = false>
+template <int NT, bool kDirect, bool kTensor, class LB>
 __global__ void __launch_bounds__(kThreads, 2)
-scan_gram_kernel(Shape s, TreeDev t, LayerBatch lb, int n_items) {
-  scan_gram_body<NT, false, false, kDirect, kTensor>(s, t, lb, n_items, nullptr);
+scan_gram_kernel(Shape s, TreeDev t, LB lb, int n_items) {
+  scan_gram_body<NT, false, false, kDirect, kTensor, LB>(s, t, lb, n_items, nullptr);
 }
 
 // trees of at most 32 nodes, launches of several waves: three smaller CTAs per SM
-template <bool kDirect, bool kTensor = false>
+template <bool kDirect, bool kTensor, class LB>
 __global__ void __launch_bounds__(kThreads, 3)
-scan_gram_compact_kernel(Shape s, TreeDev t, LayerBatch lb, int n_items) {
-  scan_gram_body<32, false, true, kDirect, kTensor>(s, t, lb, n_items, nullptr);
+scan_gram_compact_kernel(Shape s, TreeDev t, LB lb, int n_items) {
+  scan_gram_body<32, false, true, kDirect, kTensor, LB>(s, t, lb, n_items, nullptr);
 }
 
-template <int NT, bool kDirect, bool kTensor = false>
+template <int NT, bool kDirect, bool kTensor, class LB>
 __global__ void __launch_bounds__(kThreads, 2)
-scan_gram_fused_kernel(Shape s, TreeDev t, LayerBatch lb, int n_items, FusedPrev fp) {
-  scan_gram_body<NT, true, false, kDirect, kTensor>(s, t, lb, n_items, &fp);
+scan_gram_fused_kernel(Shape s, TreeDev t, LB lb, int n_items, FusedPrevT<LB> fp) {
+  scan_gram_body<NT, true, false, kDirect, kTensor, LB>(s, t, lb, n_items, &fp);
 }
 
 template <class K>
@@ -1186,27 +1186,31 @@ bool gram_supported(const Shape& s, int max_depth) {
   return s.d == kD && s.in_dtype == LUMO_BF16 && s.snapshot_mode == 0 && max_depth <= 16;
 }
 
-cudaError_t launch_scan_gram(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, int tail,
-                             cudaStream_t st) {
+// The dynamic shared-memory size of a kernel is a per-device attribute: set once per device and instance.
+struct Configured { bool done[kMaxDevices] = {}; };
+
+template <class LB>
+static cudaError_t launch_scan_gram_t(const Shape& s, const TreeDev& t, const LB& lb, int sm_count, bool pdl, int tail,
+                                      cudaStream_t st) {
   const bool direct = tail != 0;
   const int items = s.n_layers * t.n_groups * s.Hv;
-  static bool configured[kMaxDevices] = {};      // the attribute is a per-device setting
+  static Configured cfg;
   int dev = 0;
-  cudaError_t e0 = cudaGetDevice(&dev);
-  if (e0 != cudaSuccess) return e0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  if (!configured[dev]) {
-    cudaError_t e = allow_smem(scan_gram_kernel<64, false>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, false>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<64, true>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, true>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<false>, GL<true>::kBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true>, GL<true>::kBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<64, true, true>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, true, true>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true, true>, GL<true>::kBytes);
+  if (!cfg.done[dev]) {
+    e = allow_smem(scan_gram_kernel<64, false, false, LB>, kSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, false, false, LB>, kSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<64, true, false, LB>, kSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, true, false, LB>, kSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<false, false, LB>, GL<true>::kBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true, false, LB>, GL<true>::kBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<64, true, true, LB>, kSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, true, true, LB>, kSmemBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true, true, LB>, GL<true>::kBytes);
     if (e != cudaSuccess) return e;
-    configured[dev] = true;
+    cfg.done[dev] = true;
   }
   // two CTAs per SM by construction: 102 KB of shared memory, 128 registers x 256 threads and 256
   // of the 512 tensor-memory columns each
@@ -1214,40 +1218,55 @@ cudaError_t launch_scan_gram(const Shape& s, const TreeDev& t, const LayerBatch&
   // round trip per item: they win when a launch has several waves of items (the 48-layer stack: 205 ->
   // 190 us) and lose on a single wave (batch 1: 9.3 -> 10.5 us).
   if (t.max_group_nodes <= 32 && items >= 4 * sm_count) {
-    auto k = tail == 2 ? scan_gram_compact_kernel<true, true> : direct ? scan_gram_compact_kernel<true> : scan_gram_compact_kernel<false>;
+    auto k = tail == 2 ? scan_gram_compact_kernel<true, true, LB>
+                       : direct ? scan_gram_compact_kernel<true, false, LB> : scan_gram_compact_kernel<false, false, LB>;
     return launch_kernel(k, dim3(3 * sm_count), dim3(kThreads), GL<true>::kBytes, st, pdl, s, t, lb, items);
   }
   const int grid = items < 2 * sm_count ? items : 2 * sm_count;
-  auto k = t.max_group_nodes <= 32 ? (direct ? scan_gram_kernel<32, true> : scan_gram_kernel<32, false>)
-                                   : (direct ? scan_gram_kernel<64, true> : scan_gram_kernel<64, false>);
-  if (tail == 2) k = t.max_group_nodes <= 32 ? scan_gram_kernel<32, true, true> : scan_gram_kernel<64, true, true>;
+  auto k = t.max_group_nodes <= 32 ? (direct ? scan_gram_kernel<32, true, false, LB> : scan_gram_kernel<32, false, false, LB>)
+                                   : (direct ? scan_gram_kernel<64, true, false, LB> : scan_gram_kernel<64, false, false, LB>);
+  if (tail == 2) k = t.max_group_nodes <= 32 ? scan_gram_kernel<32, true, true, LB> : scan_gram_kernel<64, true, true, LB>;
   return launch_kernel(k, dim3(grid), dim3(kThreads), kSmemBytes, st, pdl, s, t, lb, items);
+}
+
+cudaError_t launch_scan_gram(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, int tail,
+                             cudaStream_t st) {
+  if (s.n_layers <= kFewLayers) return launch_scan_gram_t(s, t, few_layers(lb), sm_count, pdl, tail, st);
+  return launch_scan_gram_t(s, t, lb, sm_count, pdl, tail, st);
+}
+
+template <class LB>
+static cudaError_t launch_scan_gram_fused_t(const Shape& s, const TreeDev& t, const LB& lb, const FusedPrevT<LB>& fp,
+                                            int sm_count, bool pdl, int tail, cudaStream_t st) {
+  const bool direct = tail != 0;
+  const int items = s.n_layers * t.n_groups * s.Hv;
+  static Configured cfg;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (!cfg.done[dev]) {
+    e = allow_smem(scan_gram_fused_kernel<64, false, false, LB>, kSmemBytesFused);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<32, false, false, LB>, kSmemBytesFused);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<64, true, false, LB>, kSmemBytesFused);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<32, true, false, LB>, kSmemBytesFused);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<64, true, true, LB>, kSmemBytesFused);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<32, true, true, LB>, kSmemBytesFused);
+    if (e != cudaSuccess) return e;
+    cfg.done[dev] = true;
+  }
+  const int grid = items < 2 * sm_count ? items : 2 * sm_count;
+  auto k = t.max_group_nodes <= 32 ? (direct ? scan_gram_fused_kernel<32, true, false, LB> : scan_gram_fused_kernel<32, false, false, LB>)
+                                   : (direct ? scan_gram_fused_kernel<64, true, false, LB> : scan_gram_fused_kernel<64, false, false, LB>);
+  if (tail == 2) k = t.max_group_nodes <= 32 ? scan_gram_fused_kernel<32, true, true, LB> : scan_gram_fused_kernel<64, true, true, LB>;
+  return launch_kernel(k, dim3(grid), dim3(kThreads), kSmemBytesFused, st, pdl, s, t, lb, items, fp);
 }
 
 cudaError_t launch_scan_gram_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp,
                                    int sm_count, bool pdl, int tail, cudaStream_t st) {
-  const bool direct = tail != 0;
-  const int items = s.n_layers * t.n_groups * s.Hv;
-  static bool configured[kMaxDevices] = {};      // the attribute is a per-device setting
-  int dev = 0;
-  cudaError_t e0 = cudaGetDevice(&dev);
-  if (e0 != cudaSuccess) return e0;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-  if (!configured[dev]) {
-    cudaError_t e = allow_smem(scan_gram_fused_kernel<64, false>, kSmemBytesFused);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<32, false>, kSmemBytesFused);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<64, true>, kSmemBytesFused);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<32, true>, kSmemBytesFused);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<64, true, true>, kSmemBytesFused);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_fused_kernel<32, true, true>, kSmemBytesFused);
-    if (e != cudaSuccess) return e;
-    configured[dev] = true;
-  }
-  const int grid = items < 2 * sm_count ? items : 2 * sm_count;
-  auto k = t.max_group_nodes <= 32 ? (direct ? scan_gram_fused_kernel<32, true> : scan_gram_fused_kernel<32, false>)
-                                   : (direct ? scan_gram_fused_kernel<64, true> : scan_gram_fused_kernel<64, false>);
-  if (tail == 2) k = t.max_group_nodes <= 32 ? scan_gram_fused_kernel<32, true, true> : scan_gram_fused_kernel<64, true, true>;
-  return launch_kernel(k, dim3(grid), dim3(kThreads), kSmemBytesFused, st, pdl, s, t, lb, items, fp);
+  if (s.n_layers <= kFewLayers)
+    return launch_scan_gram_fused_t(s, t, few_layers(lb), few_layers(fp), sm_count, pdl, tail, st);
+  return launch_scan_gram_fused_t(s, t, lb, fp, sm_count, pdl, tail, st);
 }
 
 }  // namespace lumo

@@ -109,6 +109,8 @@ select_kernel(const T* __restrict__ logits, int V, int32_t* __restrict__ spine, 
   const int u_lo = min(units, rank * per), u_hi = min(units, u_lo + per);
   if (tid == 0) cta_thr = ordered_bits(__int_as_float(0xff800000));
   __syncthreads();
+  pdl_wait();          // the logits (and the outputs) may belong to earlier kernels
+  pdl_trigger();
   Best b;
   b.init();
   float thr = __int_as_float(0xff800000);              // -inf: everything passes until three entries are held
@@ -221,10 +223,7 @@ select_kernel(const T* __restrict__ logits, int V, int32_t* __restrict__ spine, 
 }  // namespace
 
 cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int split, int32_t* spine, int32_t* cand,
-                          cudaStream_t st) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+                          int sms, cudaStream_t st) {
   static int cache_f[64] = {}, cache_h[64] = {};
   const int cap = dtype == LUMO_BF16 ? max_cluster_ctas(select_kernel<__nv_bfloat16>, kSelThreads, cache_h)
                                      : max_cluster_ctas(select_kernel<float>, kSelThreads, cache_f);
