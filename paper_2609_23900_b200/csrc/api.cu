@@ -634,7 +634,7 @@ int lumo_gdn_commit(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_ar
   const bool pdl = use_overlap(ctx, s) && ctx->last_call == lumo_ctx::kVerify;
   ctx->last_call = lumo_ctx::kCommit;
   cudaError_t e = timed(ctx, LUMO_K_COMMIT, st, [&] {
-    return launch_commit(s, t, lb, accepted_dev, len_dev, lmax, true, layers[0].x != nullptr, pdl, st);
+    return launch_commit(s, t, lb, accepted_dev, len_dev, lmax, true, layers[0].x != nullptr, ctx->sm_count, pdl, st);
   });
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "commit launch");
 }
@@ -692,7 +692,7 @@ int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const
   fp.hist_in_kernels = prev_layers[0].x != nullptr && layers[0].x != nullptr;
   if (prev_layers[0].x && !fp.hist_in_kernels) {
     e = timed(ctx, LUMO_K_COMMIT, st, [&] {
-      return launch_commit(ps, pt, fp.lb, accepted_dev, len_dev, lmax, false, true, pdl, st);
+      return launch_commit(ps, pt, fp.lb, accepted_dev, len_dev, lmax, false, true, ctx->sm_count, pdl, st);
     });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "history launch");
   }

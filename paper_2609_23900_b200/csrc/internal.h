@@ -342,7 +342,8 @@ cudaError_t launch_scan_solve_fused(const Shape& s, const TreeDev& t, const Laye
 // device address of the built-in stack on `device` (which must be current); looked up once per device
 cudaError_t static_stack_address(int device, float** ptr);
 cudaError_t launch_commit(const Shape& s, const TreeDev& t, const LayerBatch& lb, const int32_t* accepted,
-                          const int32_t* len, int lmax, bool with_state, bool with_hist, bool pdl, cudaStream_t st);
+                          const int32_t* len, int lmax, bool with_state, bool with_hist, int sm_count, bool pdl,
+                          cudaStream_t st);
 cudaError_t launch_path_from_node(const TreeDev& t, int B, int N, const int32_t* node, int lmax,
                                   int32_t* accepted, int32_t* len, int32_t* status, cudaStream_t st);
 

@@ -489,28 +489,108 @@ scan_kernel(Shape s, TreeDev t, LB lb, float* __restrict__ stack, int n_items) {
   }
 }
 
+// one-shot mbarrier for a bulk copy into shared memory
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init1(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+}
+// `bytes` (a multiple of 16) from 16-byte aligned global memory, by one thread
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+// Bounded wait for the first phase: false if it did not complete within 2^20 polls (each may sleep a few us).
+__device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
+  const uint32_t addr = smem_u32(bar);
+  for (uint32_t spin = 0; spin < (1u << 20); ++spin) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done) : "r"(addr) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+// One token of the native recurrence on one state row, held by four lanes (lane j: floats 16 m + 4 j ..):
+// S <- alpha S + delta ks k, delta = beta (v - alpha ks S.k).  Packed fp32 FMAs: two correctly rounded lanes per
+// instruction, the same bits as the scalar form of the scan.
+template <int D, typename T>
+__device__ __forceinline__ void commit_token(float4 (&S)[D / 16], const float* k, T v, float2 gates, int l2norm, float l2_eps, int j) {
+  constexpr int NCH = D / 16;
+  float2 u2 = make_float2(0.f, 0.f), k2 = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int m = 0; m < NCH; ++m) {
+    const float4 kv = *reinterpret_cast<const float4*>(k + 16 * m + 4 * j);
+    const float2 lo = make_float2(kv.x, kv.y), hi = make_float2(kv.z, kv.w);
+    u2 = __ffma2_rn(make_float2(S[m].x, S[m].y), lo, u2);
+    u2 = __ffma2_rn(make_float2(S[m].z, S[m].w), hi, u2);
+    k2 = __ffma2_rn(lo, lo, k2);
+    k2 = __ffma2_rn(hi, hi, k2);
+    if (m == 3) asm volatile("" ::: "memory");   // half of the key row in flight at a time (registers)
+  }
+  float u = u2.x + u2.y, kk = k2.x + k2.y;
+  u += __shfl_xor_sync(0xffffffffu, u, 1); kk += __shfl_xor_sync(0xffffffffu, kk, 1);
+  u += __shfl_xor_sync(0xffffffffu, u, 2); kk += __shfl_xor_sync(0xffffffffu, kk, 2);
+  float vv;
+  if constexpr (sizeof(T) == 2) vv = __bfloat162float(v); else vv = v;
+  const float a = gates.x;
+  const float ks = l2norm ? rsqrtf(kk + l2_eps) : 1.f;
+  const float dl = gates.y * (vv - a * (ks * u));
+  const float gk = dl * ks;
+  const float2 a2 = make_float2(a, a), g2 = make_float2(gk, gk);
+  asm volatile("" ::: "memory");      // the key row is read again instead of being held in 32 registers
+#pragma unroll
+  for (int m = 0; m < NCH; ++m) {
+    const float4 kv = *reinterpret_cast<const float4*>(k + 16 * m + 4 * j);
+    const float2 lo = __ffma2_rn(a2, make_float2(S[m].x, S[m].y), __fmul2_rn(g2, make_float2(kv.x, kv.y)));
+    const float2 hi = __ffma2_rn(a2, make_float2(S[m].z, S[m].w), __fmul2_rn(g2, make_float2(kv.z, kv.w)));
+    S[m] = make_float4(lo.x, lo.y, hi.x, hi.y);
+    if (m == 3) asm volatile("" ::: "memory");
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // a4 + a5: commit - replay the accepted path into the running state, in place, and gather the
 // convolution history of the accepted path
 // ---------------------------------------------------------------------------------------
-// One launch.  The first Hv * d/32 CTAs of a (sequence, layer) each own a 32-row state tile: same
-// per-token arithmetic as the scan's EMIT_DESCEND without the output, i.e. the "native per-token
-// update" of Algorithm 2 applied for the accepted nodes in path order.  The remaining CTAs own
-// 128 x 16 bytes of channels of the history rows: new history = last three rows of
-// [old history ; x of the accepted nodes] (Algorithm 1).  The state tile is requested from memory
-// before the path is validated, so the two dependent chains (tile; length -> path -> operands) overlap;
-// nothing is written unless the path is valid.
-template <int D, typename T, class LB>
-__global__ void __launch_bounds__(kScanThreads, (D == 128 && sizeof(T) == 2) ? 8 : 4)
+// One launch.  The first CTAs of a (sequence, layer) each own ROWS rows of one value head's state: same per-token
+// arithmetic as the scan's EMIT_DESCEND without the output, i.e. the "native per-token update" of Algorithm 2 applied
+// for the accepted nodes in path order.  The remaining CTAs own 16-byte pieces of channels of the history rows: new
+// history = last three rows of [old history ; x of the accepted nodes] (Algorithm 1).
+//
+// Bound by HBM: every state is read and written once.  What stands between that and the measured time is the chain row
+// -> length -> path -> operands -> updates that each CTA goes through, so the state comes by bulk copy into shared
+// memory, requested whole before that chain starts (three CTAs keep 192 KB per SM on the way), and the operands of up
+// to kCommitChunk accepted nodes are fetched together instead of one node at a time.  Nothing is written unless the path
+// is valid.  Measured: 48 layers of batch 4 (805 MB) 160 -> 141 us = 5.7 TB/s, 6 layers of batch 16 116 -> 89 us, one
+// layer of batch 8 (a single wave) 15.4 -> 14.7 us.
+constexpr int kCommitChunk = 8;   // accepted nodes whose operands are staged at a time
+
+template <int D, typename T, int ROWS>
+struct CommitCfg {
+  static constexpr int kThreads = ROWS * 4 < 256 ? ROWS * 4 : 256;      // four lanes per row
+  static constexpr int kPasses = ROWS * 4 / kThreads;
+  static constexpr int kStateBytes = ROWS * D * 4;
+  static constexpr int kBytes = kStateBytes + kCommitChunk * (D * 4 + ROWS * (int)sizeof(T));
+};
+
+template <int D, typename T, int ROWS, class LB>
+__global__ void __launch_bounds__(CommitCfg<D, T, ROWS>::kThreads, ROWS == 32 ? 7 : 3)
 commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
               const int32_t* __restrict__ len_arr, int lmax, int n_state_ctas) {
-  constexpr int NCH = D / 16;
-  constexpr int kTiles = D / kRows;
-  using P4 = typename Packed4<T>::type;
+  using Cfg = CommitCfg<D, T, ROWS>;
+  constexpr int NCH = D / 16, kThreads = Cfg::kThreads;
+  constexpr int kTiles = D / ROWS;
   const int b = blockIdx.y, layer = blockIdx.z;
   const LayerPtrs& L = lb.l[layer];
   const int tid = threadIdx.x;
   const int row = L.state_row[b];
+  const int len = len_arr[b];
   const bool lead = blockIdx.x == 0 && tid == 0;
   // What this kernel WRITES (state, history, status) may still be read by its predecessor (the scan
   // reads the pre-tree state), so every write sits behind pdl_wait().  What it READS ahead of that wait
@@ -523,20 +603,19 @@ commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
   // the whole path at once: entry t, its parent and its physical row (one level of dependent loads
   // instead of one per step)
   __shared__ int s_acc[kMaxNodes], s_par[kMaxNodes], s_phys[kMaxNodes];
-  const int len = len_arr[b];
   const int lcap = len < 0 ? 0 : (len > lmax ? 0 : len);
-  for (int tt = tid; tt < lcap; tt += kScanThreads) {     // bounded: lmax
-    const int a = acc[tt];
-    const bool ok = a >= 0 && a < s.N;
-    s_acc[tt] = a;
-    s_par[tt] = ok ? t.parent[(size_t)b * s.N + a] : -2;
-    s_phys[tt] = ok ? t.slot[b * s.N + a] : 0;
-  }
 
   if ((int)blockIdx.x >= n_state_ctas) {
     // ---- convolution history ------------------------------------------------------------------
+    for (int tt = tid; tt < lcap; tt += kThreads) {       // bounded: lmax
+      const int a = acc[tt];
+      const bool ok = a >= 0 && a < s.N;
+      s_acc[tt] = a;
+      s_par[tt] = ok ? t.parent[(size_t)b * s.N + a] : -2;
+      s_phys[tt] = ok ? t.slot[b * s.N + a] : 0;
+    }
     constexpr int kVec = 16 / (int)sizeof(T);
-    const int c0 = ((blockIdx.x - n_state_ctas) * kScanThreads + tid) * kVec;
+    const int c0 = ((blockIdx.x - n_state_ctas) * kThreads + tid) * kVec;
     __syncthreads();
     // every exit path passes the dependency wait: a CTA that left without it would let this grid complete
     // (and its own dependent start) while the kernel before it is still running
@@ -558,59 +637,92 @@ commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
     return;
   }
 
-  // ---- state tile ---------------------------------------------------------------------------------
+  // ---- state rows ---------------------------------------------------------------------------------
+  extern __shared__ __align__(128) unsigned char smem[];
+  float* Ss = reinterpret_cast<float*>(smem);                              // [ROWS][D]
+  float* Ks = reinterpret_cast<float*>(smem + Cfg::kStateBytes);           // [chunk][D], widened
+  T* Vs = reinterpret_cast<T*>(smem + Cfg::kStateBytes + kCommitChunk * D * 4);   // [chunk][ROWS]
+  __shared__ float2 s_gate[kCommitChunk];
+  __shared__ unsigned long long mbar;
   const int tile = blockIdx.x % kTiles, hv = blockIdx.x / kTiles;
-  const int j = tid & 3, rl = tid >> 2;
   const int g = hv / (s.Hv / s.Hk);
-  const int r0 = tile * kRows;
-  float* Sg = L.state + (((size_t)row * s.Hv + hv) * D + r0 + rl) * D;
-  float4 S[NCH];
-#pragma unroll
-  for (int m = 0; m < NCH; ++m) S[m] = *reinterpret_cast<const float4*>(Sg + 16 * m + 4 * j);   // in flight
-
+  const int r0 = tile * ROWS;
+  float* Sg = L.state + (((size_t)row * s.Hv + hv) * D + r0) * D;
+  if (tid == 0) {
+    mbar_init1(&mbar);
+    if (lcap > 0) bulk_load(Ss, Sg, Cfg::kStateBytes, &mbar);              // the rows are contiguous
+  }
+  for (int tt = tid; tt < lcap; tt += kThreads) {         // bounded: lmax
+    const int a = acc[tt];
+    const bool ok = a >= 0 && a < s.N;
+    s_acc[tt] = a;
+    s_par[tt] = ok ? t.parent[(size_t)b * s.N + a] : -2;
+    s_phys[tt] = ok ? t.slot[b * s.N + a] : 0;
+  }
   __syncthreads();
-  const int st = check_path_staged(s_acc, s_par, s.N, len, lmax);
-  if (lead && L.status) { pdl_wait(); L.status[b] = st; }
-  if (st != LUMO_SEQ_OK || len == 0) { pdl_wait(); return; }
-
+  int st = check_path_staged(s_acc, s_par, s.N, len, lmax);
   const T* kg = reinterpret_cast<const T*>(L.k);
   const T* vg = reinterpret_cast<const T*>(L.v);
-  for (int tt = 0; tt < len; ++tt) {                      // bounded: len <= lmax
-    const size_t pr = (size_t)b * s.Ns + s_phys[tt];
-    const T* kr = kg + (pr * s.Hk + g) * D;
-    P4 kp[NCH];
-#pragma unroll
-    for (int m = 0; m < NCH; ++m) kp[m] = *reinterpret_cast<const P4*>(kr + 16 * m + 4 * j);
-    float vv;
-    if constexpr (sizeof(T) == 2) vv = __bfloat162float(vg[(pr * s.Hv + hv) * D + r0 + rl]);
-    else vv = vg[(pr * s.Hv + hv) * D + r0 + rl];
-    const float2 gates = load_gates(L, s, pr * s.Hv + hv, hv);
-    const float a = gates.x, bt = gates.y;
-    float u0 = 0.f, u1 = 0.f, k0 = 0.f, k1 = 0.f;
-#pragma unroll
-    for (int m = 0; m < NCH; ++m) {
-      const float4 kv = Packed4<T>::unpack(kp[m]);
-      u0 = fmaf(S[m].x, kv.x, u0); u1 = fmaf(S[m].y, kv.y, u1);
-      u0 = fmaf(S[m].z, kv.z, u0); u1 = fmaf(S[m].w, kv.w, u1);
-      k0 = fmaf(kv.x, kv.x, k0); k1 = fmaf(kv.y, kv.y, k1);
-      k0 = fmaf(kv.z, kv.z, k0); k1 = fmaf(kv.w, kv.w, k1);
+  // operands of the accepted nodes [t0, t0 + n): widened key rows, this CTA's part of the value rows, gates
+  auto stage = [&](int t0, int n) {
+    constexpr int kVec = 16 / (int)sizeof(T), kKP = D / kVec, kVP = ROWS / kVec;
+    for (int e = tid; e < n * (kKP + kVP); e += kThreads) {                // bounded: <= 2 rounds of bf16
+      const int i = e / (kKP + kVP), c = e % (kKP + kVP);
+      const size_t pr = (size_t)b * s.Ns + s_phys[t0 + i];
+      if (c < kKP) {
+        const uint4 w = *reinterpret_cast<const uint4*>(kg + (pr * s.Hk + g) * D + c * kVec);
+        float4* dst = reinterpret_cast<float4*>(Ks + i * D + c * kVec);
+        if constexpr (sizeof(T) == 2) {
+          dst[0] = Packed4<T>::unpack(make_uint2(w.x, w.y));
+          dst[1] = Packed4<T>::unpack(make_uint2(w.z, w.w));
+        } else {
+          dst[0] = *reinterpret_cast<const float4*>(&w);
+        }
+      } else {
+        *reinterpret_cast<uint4*>(Vs + i * ROWS + (c - kKP) * kVec) =
+            *reinterpret_cast<const uint4*>(vg + (pr * s.Hv + hv) * D + r0 + (c - kKP) * kVec);
+      }
     }
-    float u = u0 + u1, kk = k0 + k1;
-    u += __shfl_xor_sync(0xffffffffu, u, 1); kk += __shfl_xor_sync(0xffffffffu, kk, 1);
-    u += __shfl_xor_sync(0xffffffffu, u, 2); kk += __shfl_xor_sync(0xffffffffu, kk, 2);
-    const float ks = s.l2norm ? rsqrtf(kk + s.l2_eps) : 1.f;
-    const float dl = bt * (vv - a * (ks * u));
-    const float gk = dl * ks;
+    if (tid < n) s_gate[tid] = load_gates(L, s, ((size_t)b * s.Ns + s_phys[t0 + tid]) * s.Hv + hv, hv);
+  };
+  const bool go = st == LUMO_SEQ_OK && len > 0;
+  if (go) stage(0, len < kCommitChunk ? len : kCommitChunk);
+  // the copy is on its way whatever the path turned out to be: nobody leaves before it has landed
+  if (lcap > 0 && !mbar_wait0(&mbar)) st = LUMO_SEQ_TIMEOUT;
+  if (lead && L.status) { pdl_wait(); L.status[b] = st; }
+  if (!go || st != LUMO_SEQ_OK) { pdl_wait(); return; }
+  __syncthreads();
+  const int j = tid & 3;
+  // chunk by chunk (one chunk for all but the deepest trees), the state back to shared memory in between
+  for (int t0 = 0; t0 < len; t0 += kCommitChunk) {                         // bounded: lmax / kCommitChunk
+    const int n = len - t0 < kCommitChunk ? len - t0 : kCommitChunk;
+    if (t0 > 0) {
+      __syncthreads();                                                     // the last chunk's operands have been read
+      stage(t0, n);
+      __syncthreads();
+    }
+    const bool last = t0 + n == len;
+#pragma unroll 1
+    for (int ps = 0; ps < Cfg::kPasses; ++ps) {
+      const int rl = ps * (kThreads / 4) + (tid >> 2);
+      float* Sr = Ss + rl * D + 4 * j;
+      float4 S[NCH];
 #pragma unroll
-    for (int m = 0; m < NCH; ++m) {
-      const float4 kv = Packed4<T>::unpack(kp[m]);
-      S[m].x = fmaf(a, S[m].x, gk * kv.x); S[m].y = fmaf(a, S[m].y, gk * kv.y);
-      S[m].z = fmaf(a, S[m].z, gk * kv.z); S[m].w = fmaf(a, S[m].w, gk * kv.w);
+      for (int m = 0; m < NCH; ++m) S[m] = *reinterpret_cast<const float4*>(Sr + 16 * m);
+#pragma unroll 1
+      for (int tt = 0; tt < n; ++tt)
+        commit_token<D, T>(S, Ks + tt * D, Vs[tt * ROWS + rl], s_gate[tt], s.l2norm, s.l2_eps, j);
+      if (last) {
+        pdl_wait();
+        float* Gr = Sg + (size_t)rl * D + 4 * j;
+#pragma unroll
+        for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(Gr + 16 * m) = S[m];
+      } else {
+#pragma unroll
+        for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(Sr + 16 * m) = S[m];
+      }
     }
   }
-  pdl_wait();
-#pragma unroll
-  for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(Sg + 16 * m + 4 * j) = S[m];
 }
 
 // device helper: root-first path ending at node[b]
@@ -778,18 +890,42 @@ cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, 
 }
 
 cudaError_t launch_commit(const Shape& s, const TreeDev& t, const LayerBatch& lb, const int32_t* accepted,
-                          const int32_t* len, int lmax, bool with_state, bool with_hist, bool pdl, cudaStream_t st) {
+                          const int32_t* len, int lmax, bool with_state, bool with_hist, int sm_count, bool pdl,
+                          cudaStream_t st) {
   if (!with_state && !with_hist) return cudaSuccess;
   return dispatch(s.d, s.in_dtype, [&](auto dc, auto tc) {
     constexpr int D = decltype(dc)::value;
     using T = decltype(tc);
-    const int n_state = with_state ? s.Hv * (D / kRows) : 0;
-    const int per_thread = 16 / (int)sizeof(T);
-    const int n_hist = with_hist ? (s.C / per_thread + kScanThreads - 1) / kScanThreads : 0;
-    dim3 grid(n_state + n_hist, s.B, s.n_layers);
-    if (s.n_layers <= kFewLayers)
-      return launch_kernel(commit_kernel<D, T, FewLayers>, grid, dim3(kScanThreads), 0, st, pdl, s, t, few_layers(lb), accepted, len, lmax, n_state);
-    return launch_kernel(commit_kernel<D, T, LayerBatch>, grid, dim3(kScanThreads), 0, st, pdl, s, t, lb, accepted, len, lmax, n_state);
+    auto go = [&](auto rows_c, auto few_c) {
+      constexpr int R = decltype(rows_c)::value;
+      using LB = std::conditional_t<decltype(few_c)::value, FewLayers, LayerBatch>;
+      using Cfg = CommitCfg<D, T, R>;
+      auto kern = commit_kernel<D, T, R, LB>;
+      static bool configured[kMaxDevices] = {};            // the shared-memory limit is a per-device setting
+      int dev = 0;
+      cudaError_t e = cudaGetDevice(&dev);
+      if (e != cudaSuccess) return e;
+      if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+      if (!configured[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kBytes);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+      }
+      const int n_state = with_state ? s.Hv * (D / R) : 0;
+      const int per_cta = 16 / (int)sizeof(T) * Cfg::kThreads;
+      const int n_hist = with_hist ? (s.C + per_cta - 1) / per_cta : 0;
+      const dim3 grid(n_state + n_hist, s.B, s.n_layers);
+      if constexpr (decltype(few_c)::value)
+        return launch_kernel(kern, grid, dim3(Cfg::kThreads), Cfg::kBytes, st, pdl, s, t, few_layers(lb), accepted, len, lmax, n_state);
+      else
+        return launch_kernel(kern, grid, dim3(Cfg::kThreads), Cfg::kBytes, st, pdl, s, t, lb, accepted, len, lmax, n_state);
+    };
+    // up to one wave of 32-row CTAs (seven per SM): the shortest chain per CTA; beyond that whole heads, three CTAs per SM
+    const long long tiles = (long long)s.n_layers * s.B * s.Hv * (D / 32);
+    auto rows = [&](auto rows_c) {
+      return s.n_layers <= kFewLayers ? go(rows_c, std::true_type{}) : go(rows_c, std::false_type{});
+    };
+    return tiles <= 7LL * sm_count ? rows(std::integral_constant<int, 32>{}) : rows(std::integral_constant<int, D>{});
   });
 }
 
