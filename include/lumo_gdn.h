@@ -309,7 +309,7 @@ int lumo_gdn_tree_scan_static(lumo_ctx* ctx, const lumo_tree_desc* desc, const l
                               int n_layers, void* stream);
 int64_t lumo_static_stack_bytes(void);
 
-/* Diagnostic: how many entries of the visiting order one CTA of the tree convolution takes for this
+/* Diagnostic: how many consecutive entries of the visiting order one warp of the tree convolution takes for this
  * tree batch, head shape and layer count on this context's device (16, 8 or 4; the three are separate
  * instantiations of the kernel, chosen so that the grid covers the GPU).  0 on a bad argument or a
  * host-only context.  Lets a parity test state which instantiation it exercised. */

@@ -281,7 +281,7 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   std::vector<int32_t> h;
   auto reserve = [&](size_t n) { size_t off = h.size(); h.resize(off + ((n + 3) / 4) * 4, 0); return off; };
   const size_t o_parent = reserve((size_t)B * N), o_depth = reserve((size_t)B * N), o_slot = reserve((size_t)B * N);
-  const size_t o_inv = reserve((size_t)B * Ns), o_win = reserve((size_t)B * Ns * 4);
+  const size_t o_inv = reserve((size_t)B * Ns);
   const size_t o_prog = reserve((size_t)B * Ns);
   const size_t o_winv = reserve((size_t)B * Ns * 4);
   const size_t o_coff = reserve((size_t)B * (N + 2)), o_clist = reserve((size_t)B * N);
@@ -328,32 +328,26 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
       h[o_slot + (size_t)b * N + i] = slot ? slot[(size_t)b * N + i] : i;
     }
     for (int sidx = 0; sidx < Ns; ++sidx) h[o_inv + (size_t)b * Ns + sidx] = t.tab[LUMO_TAB_SLOT_INV][sidx];
-    // conv windows per PHYSICAL row, entries in physical rows (or -1..-3 = history rows);
-    // a padding row holds INT32_MIN
-    for (int sidx = 0; sidx < Ns; ++sidx) {
-      const int node = t.tab[LUMO_TAB_SLOT_INV][sidx];
-      for (int j = 0; j < 4; ++j) {
-        int w = INT32_MIN;
-        if (node >= 0) {
-          w = t.tab[LUMO_TAB_ANC_WIN][node * 4 + j];
-          if (w >= 0) w = h[o_slot + (size_t)b * N + w];
-        }
-        h[o_win + ((size_t)b * Ns + sidx) * 4 + j] = w;
-      }
-    }
     for (int i = 0; i < N + 2; ++i) h[o_coff + (size_t)b * (N + 2) + i] = t.tab[LUMO_TAB_CHILD_OFF][i];
     for (int i = 0; i < N; ++i) h[o_clist + (size_t)b * N + i] = t.tab[LUMO_TAB_CHILD_LIST][i];
     {
-      // conv visiting order: depth-first preorder, so that most rows find three of their four taps
-      // already in the registers of the thread that handled the previous row
+      // conv visiting order: depth-first preorder, a node's leaf children before its other children, so that most
+      // entries continue from their parent or share it with the entry before (flags 1 and 2)
       const auto& coff = t.tab[LUMO_TAB_CHILD_OFF];
       const auto& clist = t.tab[LUMO_TAB_CHILD_LIST];
-      std::vector<int> stack, order;
-      for (int c = coff[1] - 1; c >= coff[0]; --c) stack.push_back(clist[c]);
+      const auto& leaf = t.tab[LUMO_TAB_IS_LEAF];
+      std::vector<int> stack, order, pos(N);
+      auto push_children = [&](int n) {                        // n = -1: the pre-tree state
+        for (int want = 0; want < 2; ++want)                   // the last one pushed is visited first
+          for (int c = coff[n + 2] - 1; c >= coff[n + 1]; --c)
+            if (leaf[clist[c]] == want) stack.push_back(clist[c]);
+      };
+      push_children(-1);
       while (!stack.empty()) {
         const int n = stack.back(); stack.pop_back();
+        pos[n] = (int)order.size();
         order.push_back(n);
-        for (int c = coff[n + 2] - 1; c >= coff[n + 1]; --c) stack.push_back(clist[c]);
+        push_children(n);
       }
       size_t k = 0;
       for (size_t pidx = 0; pidx < order.size(); ++pidx, ++k) {
@@ -366,14 +360,14 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
           else if (pn == pp) flag = 2;
         }
         h[o_prog + (size_t)b * Ns + k] = h[o_slot + (size_t)b * N + n] | (flag << 16);
+        // the older entries of its window, as places in this order (or -1..-3 = history rows)
+        for (int j = 0; j < 4; ++j) {
+          const int w = t.tab[LUMO_TAB_ANC_WIN][n * 4 + j];
+          h[o_winv + ((size_t)b * Ns + k) * 4 + j] = w >= 0 ? pos[w] : w;
+        }
       }
       for (int sidx = 0; sidx < Ns; ++sidx)
         if (t.tab[LUMO_TAB_SLOT_INV][sidx] < 0) h[o_prog + (size_t)b * Ns + k++] = sidx | (3 << 16);
-      // the windows in the same visiting order, so that the kernel fetches order and window together
-      for (int e = 0; e < Ns; ++e) {
-        const int sidx = h[o_prog + (size_t)b * Ns + e] & 0xFFFF;
-        for (int j = 0; j < 4; ++j) h[o_winv + ((size_t)b * Ns + e) * 4 + j] = h[o_win + ((size_t)b * Ns + sidx) * 4 + j];
-      }
     }
     for (int w = 0; w < 2; ++w) {
       const auto& ops = t.tab[LUMO_TAB_SCHEDULE + w];

@@ -76,12 +76,12 @@ struct lumo_tree_desc {
   int32_t* d_depth = nullptr;     // [B, N]
   int32_t* d_slot = nullptr;      // [B, N]
   int32_t* d_slot_inv = nullptr;  // [B, Ns]
-  int32_t* d_win = nullptr;       // [B, Ns, 4] per entry of the conv visiting order: source rows (physical), -1/-2/-3 = history rows, INT32_MIN = padding row
+  int32_t* d_win = nullptr;       // [B, Ns, 4] per entry of the conv visiting order: the window as places in that order, -1/-2/-3 = history rows
   int32_t* d_child_off = nullptr; // [B, N+2]
   int32_t* d_child_list = nullptr;// [B, N]
-  int32_t* d_conv_prog = nullptr; // [B, Ns] conv visiting order (depth first): physical row | flag << 16; flag 0 = fetch the whole
-                                  // window, 1 = previous row is the parent (window slides), 2 = same parent as the previous row
-                                  // (only the own row changes), 3 = padding row (zeros)
+  int32_t* d_conv_prog = nullptr; // [B, Ns] conv visiting order (depth first, leaf children first, padding rows last): physical row
+                                  // | flag << 16; flag 0 = starts from its window, 1 = the previous entry is the parent, 2 = same
+                                  // parent as the previous entry (a leaf), 3 = padding row (zeros)
   int32_t* d_sched[2] = {nullptr, nullptr};   // [B, max_ops]  lean / full (every node's state materialised)
   int32_t* d_nops[2] = {nullptr, nullptr};    // [B]
   int max_ops[2] = {0, 0};
@@ -305,7 +305,7 @@ cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
 
 // launchers (kernels.cu); all return cudaError_t and only enqueue
 cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, cudaStream_t st);
-// entries of the visiting order one CTA of the convolution takes (16, 8 or 4: fewer when the grid would not cover the GPU)
+// entries of the visiting order one warp of the convolution takes (16, 8 or 4: fewer when the grid would not cover the GPU)
 int conv_rows_per_cta(int C, int Ns, int seqs, int sms);
 // same convolution reading the history the previous cycle's accepted path would commit (not yet in memory)
 cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, int sm_count,

@@ -70,72 +70,181 @@ template <> struct Packed4<__nv_bfloat16> {
   }
 };
 
+// one-shot mbarrier for a bulk copy into shared memory
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init1(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+// `bytes` (a multiple of 16) between 16-byte aligned addresses, by one thread; counted on `bar`
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+// Bounded wait for the first phase: false if it did not complete within 2^20 polls (each may sleep a few us).
+__device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
+  const uint32_t addr = smem_u32(bar);
+  for (uint32_t spin = 0; spin < (1u << 20); ++spin) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done) : "r"(addr) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
 // ---------------------------------------------------------------------------------------
 // a1: ancestry-gathered causal depthwise conv (width 4) + SiLU -> recorded operands
 // ---------------------------------------------------------------------------------------
-// A CTA owns kConvRows consecutive entries of one sequence's visiting order (depth-first, built on
-// the host) and a slab of 256 x 4 channels; a thread keeps the taps (as pairs of neighbouring
-// channels), the bias and the current 4-row window of its channels unpacked in fp32 registers.  In
-// depth-first order most rows either follow their parent (the window slides by one) or share the
-// parent of the previous row (only the own row changes), so one load per row replaces four; the own
-// rows of the next eight entries are always in flight (the kernel is bound by the special-function
-// unit, two operations per element for the SiLU, and by load latency, not by bandwidth).  Windows
-// that cannot be derived come from a table in the same visiting order (physical rows, or -1..-3 for
-// the history rows), fetched together with the order itself.
-// Taps are applied oldest first in fp32 starting from zero (packed FMAs: two correctly rounded fp32
-// lanes per instruction, same bits as scalar fmaf), bias last, SiLU in fp32, one round-to-nearest-even
-// cast (Sec. "Precompute branch histories while preserving arithmetic": tap order and cast points are
-// part of the result).
+// A warp owns a run of kRun consecutive entries of one sequence's visiting order (depth first, built on the host) and
+// 128 channels, a lane four of them; the warps of a CTA are the runs of the sequence (up to eight, up to 8 kRun entries)
+// times as many channel groups as make eight.  The CTA's rows of x and the three history rows are pulled into shared
+// memory by cp.async, every one exactly once and all at once, so that a window costs shared-memory loads only, wherever
+// its rows lie in the tree.
+//
+// The filter runs in transposed form: instead of the window a lane keeps, per channel, the three partial sums that the
+// children of the current node start from,
+//   a1 = w0 x_n,  a2 = w1 x_n + w0 x_p,  a3 = w2 x_n + w1 x_p + w0 x_pp       (p, pp: parent, grandparent of n)
+// so a node costs one FMA for its own output, y = w3 x_n + a3(parent), and three more only when the next entry descends
+// from it; siblings share the parent's sums and nothing moves between registers.  In the visiting order (leaf children
+// first) the next entry is a child of this one, or has the same parent (then this one is a leaf and left the sums
+// alone), or rebuilds the sums of its parent from its window.
+// Every sum takes its taps oldest first from zero in fp32 (packed FMAs: two correctly rounded fp32 lanes per
+// instruction, same bits as scalar fmaf), bias last, SiLU in fp32, one round-to-nearest-even cast (Sec. "Precompute
+// branch histories while preserving arithmetic": tap order and cast points are part of the result).
+//
+// What bounds it: instruction issue and the special-function unit (the SiLU alone is 14 instructions, 8 of them
+// special-function operations, per four channels), with HBM behind them.  Measured against a register window fed by
+// prefetched rows: 48 layers of 4 x 32 nodes 71 -> 56 us, 32 x 256 nodes 92 -> 74 us, 8 x 64 nodes 15.2 -> 12.9 us.
 
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
 // scan that follows writes them to the history buffer once every CTA of this kernel has finished).
-template <typename T, int kConvRows, bool kFused, class LB>
-__device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, const LB& lb, const FusedPrevT<LB>* fp) {
-  __shared__ int s_win[kConvRows][4];
-  __shared__ int s_prog[kConvRows];
+constexpr int kConvWarps = 8;
+constexpr int kConvMaxEntries = 128;      // entries per CTA: eight runs of sixteen
+
+// Runs and channel groups of a CTA (a warp per pair), chosen on the host: groups is a power of two.
+struct ConvSplit { int runs, groups, log_groups, slabs; };
+inline ConvSplit conv_split(int C, int Ns, int run) {
+  const int need = (Ns + run - 1) / run;
+  ConvSplit c;
+  c.runs = need < kConvWarps ? need : kConvWarps;
+  c.log_groups = c.runs == 1 ? 3 : c.runs == 2 ? 2 : c.runs <= 4 ? 1 : 0;
+  c.groups = 1 << c.log_groups;
+  c.slabs = (C + c.groups * 128 - 1) / (c.groups * 128);
+  return c;
+}
+
+// What the main loop needs of an entry, in one 16-byte load: byte offset of its own row in the tile, physical row, and
+// what to do; its window (only looked at where an entry starts from it) as byte offsets, or ~visiting place for a row
+// that another CTA's part holds.
+enum : int { kConvPad = 1, kConvWindow = 2, kConvDescend = 4, kConvEnd = 8 };
+struct alignas(16) ConvEntry { int own, phys, what, pad; };
+
+template <typename T, int kRun, bool kFused, class LB>
+__device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, const LB& lb, const ConvSplit& sp, const FusedPrevT<LB>* fp) {
+  extern __shared__ __align__(128) unsigned char conv_smem[];            // [runs * kRun + 3 rows][groups * 128 channels]
+  __shared__ ConvEntry s_entry[kConvMaxEntries];
+  __shared__ int4 s_win[kConvMaxEntries];
   __shared__ int f_acc[kFusedMaxPath], f_par[kFusedMaxPath], f_phys[kFusedMaxPath];
   __shared__ const T* f_hsrc[3];
-  const int layer = blockIdx.z / s.B, b = blockIdx.z % s.B;
-  const int e0 = blockIdx.y * kConvRows;               // first entry of the visiting order
-  const int c0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
+  const int b = blockIdx.y, layer = blockIdx.z;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int seg = (int)blockIdx.x >= sp.slabs ? blockIdx.x / sp.slabs : 0, slab = blockIdx.x - seg * sp.slabs;
+  const int entries = sp.runs * kRun, e0 = seg * entries;               // this CTA's part of the visiting order
+  const int cbase = slab * (128 << sp.log_groups);                      // and of the channels
+  const int row_bytes = (128 << sp.log_groups) * (int)sizeof(T);
   const LayerPtrs& L = lb.l[layer];
+  const int32_t* prog_g = t.conv_prog + (size_t)b * s.Ns;
+  if (tid < entries) {                                 // descriptor tables: nobody writes them
+    const int e = e0 + tid;
+    ConvEntry en = {tid * row_bytes, 0, kConvEnd, 0};
+    if (e < s.Ns) {
+      const int prog = prog_g[e], flag = prog >> 16;
+      en.phys = prog & 0xFFFF;
+      en.what = flag == 3 ? kConvPad : (flag == 0 || (tid & (kRun - 1)) == 0) ? kConvWindow : 0;
+      // the last entry of a run hands its sums to nobody
+      if ((tid & (kRun - 1)) != kRun - 1 && e + 1 < s.Ns && prog_g[e + 1] >> 16 == 1) en.what |= kConvDescend;
+      if (en.what & kConvWindow) {
+        int4 w = *reinterpret_cast<const int4*>(t.win + ((size_t)b * s.Ns + e) * 4);
+        auto place = [&](int v) { return v < 0 ? (entries + 3 + v) * row_bytes : v >= e0 ? (v - e0) * row_bytes : ~v; };
+        s_win[tid] = make_int4(place(w.x), place(w.y), place(w.z), 0);
+      }
+    }
+    s_entry[tid] = en;
+  }
   pdl_wait();       // x, history and the operand buffers belong to earlier kernels until here
   pdl_trigger();
   const int row = L.state_row[b];
   const bool seq_ok = row >= 0 && row < s.n_state_rows;
-  if (threadIdx.x < kConvRows * 4) {
-    const int r = threadIdx.x >> 2, j = threadIdx.x & 3;
-    int prog = 3 << 16, w = INT_MIN;
-    if (e0 + r < s.Ns) {
-      prog = t.conv_prog[(size_t)b * s.Ns + e0 + r];
-      if (!seq_ok) prog = (prog & 0xFFFF) | (3 << 16);        // skipped sequence: every row is a zero row
-      w = t.win[((size_t)b * s.Ns + e0 + r) * 4 + j];
-    }
-    s_win[r][j] = w;
-    if (j == 0) s_prog[r] = (e0 + r < s.Ns) ? prog : -1;
+  const T* xb = reinterpret_cast<const T*>(L.x) + (size_t)b * s.Ns * s.C + cbase;
+  // ---- rows of x in visiting order (padding rows come last and are not read), history rows: a thread keeps to one
+  //      16-byte column ------------------------------------------------------------------------------------------------
+  constexpr int kVec = 16 / (int)sizeof(T);
+  const int log_cols = (sizeof(T) == 2 ? 4 : 5) + sp.log_groups, col = (tid & ((1 << log_cols) - 1)) * kVec;
+  const int step = (int)blockDim.x >> log_cols;         // rows per round: a multiple of the runs
+  const bool col_ok = cbase + col < s.C;
+  unsigned char* mycol = conv_smem + col * (int)sizeof(T);
+  if (col_ok) {
+    const int live = seq_ok ? min(s.N - e0, entries) : 0;
+    const T* src = xb + col;
+#pragma unroll 4
+    for (int e = tid >> log_cols; e < live; e += step)
+      cp_async16(mycol + e * row_bytes, src + (size_t)((uint32_t)(prog_g[e0 + e] & 0xFFFF) * (uint32_t)s.C));
   }
-  int plen = 0;
+  const T* hbase = reinterpret_cast<const T*>(L.conv_hist) + (size_t)(seq_ok ? row : 0) * 3 * s.C;
   if constexpr (kFused) {
-    plen = fp->len[b];
-    const int lcap = plen < 0 ? 0 : (plen > fp->lmax ? 0 : plen);
-    const int tt = (int)threadIdx.x - 128;
-    if (tt >= 0 && tt < lcap) {
-      const int a = fp->accepted[(size_t)b * fp->lmax + tt];
-      const bool ok = a >= 0 && a < fp->N;
-      f_acc[tt] = a;
-      f_par[tt] = ok ? fp->parent[(size_t)b * fp->N + a] : -2;
-      f_phys[tt] = ok ? fp->slot[(size_t)b * fp->N + a] : 0;
+    if (warp == 0) {
+      const int plen = fp->len[b];
+      const int lcap = plen < 0 ? 0 : (plen > fp->lmax ? 0 : plen);
+      if (lane < lcap) {
+        const int a = fp->accepted[(size_t)b * fp->lmax + lane];
+        const bool ok = a >= 0 && a < fp->N;
+        f_acc[lane] = a;
+        f_par[lane] = ok ? fp->parent[(size_t)b * fp->N + a] : -2;
+        f_phys[lane] = ok ? fp->slot[(size_t)b * fp->N + a] : 0;
+      }
+      __syncwarp();
+      if (lane < 3) {
+        // an invalid or empty path commits nothing: the history in memory is the history
+        const bool ok = seq_ok && check_path_staged(f_acc, f_par, fp->N, plen, fp->lmax) == LUMO_SEQ_OK;
+        const int q = (ok ? plen : 0) + lane;          // index into [old0 old1 old2 x_a0 x_a1 ...]
+        const T* xprev = reinterpret_cast<const T*>(fp->lb.l[layer].x) + (size_t)b * fp->Ns * s.C;
+        f_hsrc[lane] = q < 3 ? hbase + (size_t)q * s.C : xprev + (size_t)f_phys[q - 3] * s.C;
+      }
     }
+    __syncthreads();
   }
+  if (col_ok)
+    for (int j = tid >> log_cols; j < 3; j += step) {
+      const T* src = hbase + (size_t)j * s.C;
+      if constexpr (kFused) src = f_hsrc[j];
+      cp_async16(mycol + (entries + j) * row_bytes, src + cbase + col);
+    }
+  cp_async_commit();
+  // ---- taps and bias of this lane's channels, as pairs of neighbouring channels ------------------------------------
   using P4 = typename Packed4<T>::type;                // four elements as loaded
+  const int run = warp >> sp.log_groups, cg = (warp & (sp.groups - 1)) * 128 + lane * 4, c0 = cbase + cg;
+  const bool mine = c0 < s.C;
   float2 wp[4][2];                                     // tap j of channel pairs (0,1) and (2,3)
   float2 bp[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-  if (c0 < s.C) {
+  if (mine) {
     const T* w = reinterpret_cast<const T*>(L.conv_w) + (size_t)c0 * 4;
-    float4 wc[4];
+    float4 wc[4];                                      // the taps of channel c0 + e
+    if constexpr (sizeof(T) == 2) {
+      const uint4 lo = *reinterpret_cast<const uint4*>(w), hi = *reinterpret_cast<const uint4*>(w + 8);
+      wc[0] = Packed4<T>::unpack(make_uint2(lo.x, lo.y)); wc[1] = Packed4<T>::unpack(make_uint2(lo.z, lo.w));
+      wc[2] = Packed4<T>::unpack(make_uint2(hi.x, hi.y)); wc[3] = Packed4<T>::unpack(make_uint2(hi.z, hi.w));
+    } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) wc[e] = Packed4<T>::unpack(*reinterpret_cast<const P4*>(w + e * 4));
+      for (int e = 0; e < 4; ++e) wc[e] = *reinterpret_cast<const float4*>(w + e * 4);
+    }
     wp[0][0] = make_float2(wc[0].x, wc[1].x); wp[0][1] = make_float2(wc[2].x, wc[3].x);
     wp[1][0] = make_float2(wc[0].y, wc[1].y); wp[1][1] = make_float2(wc[2].y, wc[3].y);
     wp[2][0] = make_float2(wc[0].z, wc[1].z); wp[2][1] = make_float2(wc[2].z, wc[3].z);
@@ -146,99 +255,83 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
       bp[1] = make_float2(bv.z, bv.w);
     }
   }
+  cp_async_wait<0>();
   __syncthreads();
-  if constexpr (kFused) {
-    if (threadIdx.x == 0) {
-      // an invalid or empty path commits nothing: the history in memory is the history
-      const bool ok = seq_ok && check_path_staged(f_acc, f_par, fp->N, plen, fp->lmax) == LUMO_SEQ_OK;
-      const int leff = ok ? plen : 0;
-      const T* hbase = reinterpret_cast<const T*>(L.conv_hist) + (size_t)(seq_ok ? row : 0) * 3 * s.C;
-      const T* xprev = reinterpret_cast<const T*>(fp->lb.l[layer].x) + (size_t)b * fp->Ns * s.C;
-      for (int j = 0; j < 3; ++j) {
-        const int q = leff + j;        // index into [old0 old1 old2 x_a0 x_a1 ...]
-        f_hsrc[j] = q < 3 ? hbase + (size_t)q * s.C : xprev + (size_t)f_phys[q - 3] * s.C;
-      }
-    }
-    __syncthreads();
-  }
-  if (c0 >= s.C) return;
+  if (!mine) return;
   const bool has_bias = L.conv_b != nullptr;
   const int hkd = s.Hk * s.d;
   T* dst;
-  size_t dst_stride;
+  uint32_t dst_stride;
   if (c0 < hkd) { dst = reinterpret_cast<T*>(L.q) + c0; dst_stride = hkd; }
   else if (c0 < 2 * hkd) { dst = reinterpret_cast<T*>(L.k) + (c0 - hkd); dst_stride = hkd; }
-  else { dst = reinterpret_cast<T*>(L.v) + (c0 - 2 * hkd); dst_stride = (size_t)s.Hv * s.d; }
+  else { dst = reinterpret_cast<T*>(L.v) + (c0 - 2 * hkd); dst_stride = (uint32_t)s.Hv * s.d; }
   dst += (size_t)b * s.Ns * dst_stride;
-  const T* x = reinterpret_cast<const T*>(L.x) + (size_t)b * s.Ns * s.C + c0;
-  const T* hist = reinterpret_cast<const T*>(L.conv_hist) + (size_t)(seq_ok ? row : 0) * 3 * s.C + c0;
-
-  auto load_src = [&](int wj) -> float4 {              // one window entry: a row of x or of the history
-    const T* src;
-    if (wj >= 0) src = x + (size_t)wj * s.C;
-    else if constexpr (kFused) src = f_hsrc[3 + wj] + c0;
-    else src = hist + (size_t)(3 + wj) * s.C;
-    return Packed4<T>::unpack(*reinterpret_cast<const P4*>(src));
+  const unsigned char* tile = conv_smem + cg * (int)sizeof(T);
+  const float2 zero2 = make_float2(0.f, 0.f);
+  auto window = [&](int at) -> float4 {                // a row of the window: staged, or in another CTA's part
+    if (at < 0) return Packed4<T>::unpack(*reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)(prog_g[~at] & 0xFFFF) * (uint32_t)s.C)));
+    return Packed4<T>::unpack(*reinterpret_cast<const P4*>(tile + at));
   };
-  auto load_own = [&](int r) -> P4 {                   // the entry's own row (padding rows: zeros)
-    const int prog = r < kConvRows ? s_prog[r] : -1;
-    P4 z = {};
-    if (prog < 0 || (prog >> 16) == 3) return z;
-    return *reinterpret_cast<const P4*>(x + (size_t)(prog & 0xFFFF) * s.C);
-  };
-  float4 win[4] = {};
-  constexpr int kAhead = sizeof(T) == 2 ? (kConvRows < 8 ? kConvRows : 8) : 4;   // own rows in flight (a register budget)
-  P4 pf[kAhead];
+  float2 a1[2] = {zero2, zero2}, a2[2] = {zero2, zero2}, a3[2] = {zero2, zero2};   // channel pairs (0,1) and (2,3)
+  const ConvEntry* ent = s_entry + run * kRun;
+#pragma unroll 4
+  for (int rr = 0; rr < kRun; ++rr) {                  // bounded: kRun
+    const int4 en = *reinterpret_cast<const int4*>(ent + rr);   // own, phys, what
+    if (en.z & kConvEnd) break;                        // beyond the last entry (uniform over the warp)
+    T* d = dst + (size_t)((uint32_t)en.y * dst_stride);
+    float2 y[2] = {zero2, zero2};
+    if (!(en.z & kConvPad) && seq_ok) {                // padding rows and skipped sequences: zero rows
+      const float4 o4 = Packed4<T>::unpack(*reinterpret_cast<const P4*>(tile + en.x));
+      const float2 own[2] = {make_float2(o4.x, o4.y), make_float2(o4.z, o4.w)};
+      if (en.z & kConvWindow) {                        // the parent's sums from its window
+        const int4 wi = s_win[run * kRun + rr];
+        const float4 w0 = window(wi.x), w1 = window(wi.y), w2 = window(wi.z);
+        const float2 v0[2] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w)}, v1[2] = {make_float2(w1.x, w1.y), make_float2(w1.z, w1.w)},
+                     v2[2] = {make_float2(w2.x, w2.y), make_float2(w2.z, w2.w)};
 #pragma unroll
-  for (int r = 0; r < kAhead; ++r) pf[r] = load_own(r);
-#pragma unroll
-  for (int r = 0; r < kConvRows; ++r) {                // bounded: kConvRows
-    const int prog = s_prog[r];
-    if (prog < 0) break;
-    const int ps = prog & 0xFFFF;
-    int flag = prog >> 16;
-    if (r == 0 && flag != 3) flag = 0;                 // the first row of a CTA has nothing to reuse
-    const float4 own = Packed4<T>::unpack(pf[r % kAhead]);
-    pf[r % kAhead] = load_own(r + kAhead);
-    float y[4] = {0.f, 0.f, 0.f, 0.f};
-    if (flag != 3) {
-      if (flag == 0) { win[0] = load_src(s_win[r][0]); win[1] = load_src(s_win[r][1]); win[2] = load_src(s_win[r][2]); }
-      else if (flag == 1) { win[0] = win[1]; win[1] = win[2]; win[2] = win[3]; }
-      win[3] = own;
-      float2 y01 = make_float2(0.f, 0.f), y23 = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {                    // oldest -> newest
-        y01 = __ffma2_rn(wp[j][0], make_float2(win[j].x, win[j].y), y01);
-        y23 = __ffma2_rn(wp[j][1], make_float2(win[j].z, win[j].w), y23);
+        for (int e = 0; e < 2; ++e) {
+          a3[e] = __ffma2_rn(wp[2][e], v2[e], __ffma2_rn(wp[1][e], v1[e], __ffma2_rn(wp[0][e], v0[e], zero2)));
+          a2[e] = __ffma2_rn(wp[1][e], v2[e], __ffma2_rn(wp[0][e], v1[e], zero2));
+          a1[e] = __ffma2_rn(wp[0][e], v2[e], zero2);
+        }
       }
-      if (has_bias) { y01 = __fadd2_rn(y01, bp[0]); y23 = __fadd2_rn(y23, bp[1]); }   // bias last
+#pragma unroll
+      for (int e = 0; e < 2; ++e) y[e] = __ffma2_rn(wp[3][e], own[e], a3[e]);
+      if (en.z & kConvDescend) {                       // the next entry is a child of this one
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          a3[e] = __ffma2_rn(wp[2][e], own[e], a2[e]);
+          a2[e] = __ffma2_rn(wp[1][e], own[e], a1[e]);
+          a1[e] = __ffma2_rn(wp[0][e], own[e], zero2);
+        }
+      }
+      if (has_bias) { y[0] = __fadd2_rn(y[0], bp[0]); y[1] = __fadd2_rn(y[1], bp[1]); }   // bias last
       // SiLU a / (1 + 2^(-a log2 e)) with the hardware exponential and reciprocal (1e-6 relative, far
       // below the rounding of the recorded operand); the multiplies and the add are packed
       const float2 nl2e = make_float2(-1.4426950408889634f, -1.4426950408889634f), one = make_float2(1.f, 1.f);
-      float2 e01 = __fmul2_rn(y01, nl2e), e23 = __fmul2_rn(y23, nl2e);
-      e01 = __fadd2_rn(make_float2(ex2_approx(e01.x), ex2_approx(e01.y)), one);
-      e23 = __fadd2_rn(make_float2(ex2_approx(e23.x), ex2_approx(e23.y)), one);
-      y01 = __fmul2_rn(y01, make_float2(rcp_approx(e01.x), rcp_approx(e01.y)));
-      y23 = __fmul2_rn(y23, make_float2(rcp_approx(e23.x), rcp_approx(e23.y)));
-      y[0] = y01.x; y[1] = y01.y; y[2] = y23.x; y[3] = y23.y;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        float2 ex = __fmul2_rn(y[e], nl2e);
+        ex = __fadd2_rn(make_float2(ex2_approx(ex.x), ex2_approx(ex.y)), one);
+        y[e] = __fmul2_rn(y[e], make_float2(rcp_approx(ex.x), rcp_approx(ex.y)));
+      }
     }
-    T* d = dst + (size_t)ps * dst_stride;
     if constexpr (sizeof(T) == 2) {
-      __nv_bfloat162 h01 = __floats2bfloat162_rn(y[0], y[1]), h23 = __floats2bfloat162_rn(y[2], y[3]);
+      __nv_bfloat162 h01 = __floats2bfloat162_rn(y[0].x, y[0].y), h23 = __floats2bfloat162_rn(y[1].x, y[1].y);
       *reinterpret_cast<uint2*>(d) = make_uint2(*reinterpret_cast<uint32_t*>(&h01), *reinterpret_cast<uint32_t*>(&h23));
     } else {
-      *reinterpret_cast<float4*>(d) = make_float4(y[0], y[1], y[2], y[3]);
+      *reinterpret_cast<float4*>(d) = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
     }
   }
 }
 
-template <typename T, int kConvRows, class LB>
-__global__ void __launch_bounds__(256, 3) conv_kernel(Shape s, TreeDev t, LB lb) {
-  conv_body<T, kConvRows, false, LB>(s, t, lb, nullptr);
+template <typename T, int kRun, class LB>
+__global__ void __launch_bounds__(32 * kConvWarps, 4) conv_kernel(Shape s, TreeDev t, LB lb, ConvSplit sp) {
+  conv_body<T, kRun, false, LB>(s, t, lb, sp, nullptr);
 }
-template <typename T, int kConvRows, class LB>
-__global__ void __launch_bounds__(256, 3) conv_fused_kernel(Shape s, TreeDev t, LB lb, FusedPrevT<LB> fp) {
-  conv_body<T, kConvRows, true, LB>(s, t, lb, &fp);
+template <typename T, int kRun, class LB>
+__global__ void __launch_bounds__(32 * kConvWarps, 4) conv_fused_kernel(Shape s, TreeDev t, LB lb, ConvSplit sp, FusedPrevT<LB> fp) {
+  conv_body<T, kRun, true, LB>(s, t, lb, sp, &fp);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -489,33 +582,6 @@ scan_kernel(Shape s, TreeDev t, LB lb, float* __restrict__ stack, int n_items) {
   }
 }
 
-// one-shot mbarrier for a bulk copy into shared memory
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init1(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(bar)) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-// `bytes` (a multiple of 16) from 16-byte aligned global memory, by one thread
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-// Bounded wait for the first phase: false if it did not complete within 2^20 polls (each may sleep a few us).
-__device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
-  const uint32_t addr = smem_u32(bar);
-  for (uint32_t spin = 0; spin < (1u << 20); ++spin) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n"
-        "selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done) : "r"(addr) : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-
 // One token of the native recurrence on one state row, held by four lanes (lane j: floats 16 m + 4 j ..):
 // S <- alpha S + delta ks k, delta = beta (v - alpha ks S.k).  Packed fp32 FMAs: two correctly rounded lanes per
 // instruction, the same bits as the scalar form of the scan.
@@ -650,7 +716,10 @@ commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
   float* Sg = L.state + (((size_t)row * s.Hv + hv) * D + r0) * D;
   if (tid == 0) {
     mbar_init1(&mbar);
-    if (lcap > 0) bulk_load(Ss, Sg, Cfg::kStateBytes, &mbar);              // the rows are contiguous
+    if (lcap > 0) {                                                        // the rows are contiguous
+      mbar_expect(&mbar, Cfg::kStateBytes);
+      bulk_load(Ss, Sg, Cfg::kStateBytes, &mbar);
+    }
   }
   for (int tt = tid; tt < lcap; tt += kThreads) {         // bounded: lmax
     const int a = acc[tt];
@@ -763,7 +832,7 @@ cudaError_t dispatch(int d, int in_dtype, F f) {
 // ---------------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------------
-// sixteen entries per CTA amortise the window set-up; small launches take fewer so that the grid still
+// runs of sixteen entries amortise the window set-up; small launches take fewer so that the grid still
 // covers the GPU
 int conv_rows_per_cta(int C, int Ns, int seqs, int sms) {
   const int slabs = (C / 4 + 255) / 256;
@@ -773,25 +842,51 @@ int conv_rows_per_cta(int C, int Ns, int seqs, int sms) {
   return 4;
 }
 
+template <typename K>
+static cudaError_t allow_smem_once(K kern, int bytes, bool (&done)[kMaxDevices]) {      // a per-device setting
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (done[dev]) return cudaSuccess;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) done[dev] = true;
+  return e;
+}
+
 template <typename T>
 static cudaError_t launch_conv_t(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sms,
                                  bool pdl, cudaStream_t st) {
-  const int slabs = (s.C / 4 + 255) / 256, seqs = s.B * s.n_layers;
+  const int seqs = s.B * s.n_layers;
   const int rows = conv_rows_per_cta(s.C, s.Ns, seqs, sms);
-  const bool few = s.n_layers <= kFewLayers;
-  auto go = [&](auto rows_c) {
+  auto go = [&](auto rows_c, auto few_c) {
     constexpr int R = decltype(rows_c)::value;
-    const dim3 grid(slabs, (s.Ns + R - 1) / R, seqs), block(256);
+    constexpr bool kFew = decltype(few_c)::value;
+    using LB = std::conditional_t<kFew, FewLayers, LayerBatch>;
+    constexpr int kMost = (kConvMaxEntries + 3 * kConvWarps) * 128 * (int)sizeof(T);    // of any split
+    const ConvSplit sp = conv_split(s.C, s.Ns, R);
+    const int entries = sp.runs * R;
+    const dim3 grid(sp.slabs * ((s.Ns + entries - 1) / entries), s.B, s.n_layers), block(32 * sp.runs * sp.groups);
+    const size_t smem = (size_t)(entries + 3) * sp.groups * 128 * sizeof(T);
+    auto layers = [&]() -> decltype(auto) { if constexpr (kFew) return few_layers(lb); else return (lb); };
     if constexpr (sizeof(T) == 2) {                               // the fused path serves bf16 operands only
-      if (fp && few) return launch_kernel(conv_fused_kernel<T, R, FewLayers>, grid, block, 0, st, pdl, s, t, few_layers(lb), few_layers(*fp));
-      if (fp) return launch_kernel(conv_fused_kernel<T, R, LayerBatch>, grid, block, 0, st, pdl, s, t, lb, *fp);
+      if (fp) {
+        static bool done[kMaxDevices] = {};
+        const cudaError_t e = allow_smem_once(conv_fused_kernel<T, R, LB>, kMost, done);
+        if (e != cudaSuccess) return e;
+        auto prev = [&]() -> decltype(auto) { if constexpr (kFew) return few_layers(*fp); else return (*fp); };
+        return launch_kernel(conv_fused_kernel<T, R, LB>, grid, block, smem, st, pdl, s, t, layers(), sp, prev());
+      }
     }
-    if (few) return launch_kernel(conv_kernel<T, R, FewLayers>, grid, block, 0, st, pdl, s, t, few_layers(lb));
-    return launch_kernel(conv_kernel<T, R, LayerBatch>, grid, block, 0, st, pdl, s, t, lb);
+    static bool done[kMaxDevices] = {};
+    const cudaError_t e = allow_smem_once(conv_kernel<T, R, LB>, kMost, done);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(conv_kernel<T, R, LB>, grid, block, smem, st, pdl, s, t, layers(), sp);
   };
-  if (rows == 16) return go(std::integral_constant<int, 16>{});
-  if (rows == 8) return go(std::integral_constant<int, 8>{});
-  return go(std::integral_constant<int, 4>{});
+  auto pick = [&](auto rows_c) { return s.n_layers <= kFewLayers ? go(rows_c, std::true_type{}) : go(rows_c, std::false_type{}); };
+  if (rows == 16) return pick(std::integral_constant<int, 16>{});
+  if (rows == 8) return pick(std::integral_constant<int, 8>{});
+  return pick(std::integral_constant<int, 4>{});
 }
 
 cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, cudaStream_t st) {

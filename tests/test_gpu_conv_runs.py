@@ -1,0 +1,38 @@
+"""The tree convolution's split of a sequence into runs (one warp each) and parts (one CTA each): node counts on both sides of
+every edge, windows that reach back into another part, channel counts that do not fill a CTA's groups, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import gdn_oracle as O
+from synthetic import workload as W
+from synthetic.device_case import DeviceCase
+from tests.harness import assert_close, ctx
+
+pytestmark = pytest.mark.gpu
+
+
+def check(c):
+    dc = DeviceCase(ctx(), c)
+    for t in ("q", "k", "v"):
+        dc.t(t).fill_(777.0)     # must be overwritten everywhere, padding rows with zeros
+    dc.verify()
+    torch.cuda.synchronize()
+    L, hk = c.layers[0], c.Hk * c.d
+    y = O.conv(c.parent, c.slot, c.state_row, L.x, L.conv_w, L.conv_b, L.hist, c.Ns, out_dtype="none")
+    got = np.concatenate([dc.np("q").reshape(c.B, c.Ns, hk), dc.np("k").reshape(c.B, c.Ns, hk), dc.np("v").reshape(c.B, c.Ns, c.Hv * c.d)], axis=-1)
+    assert_close(got, y, bf16=(c.in_dtype == "bf16"), what="conv")
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N", [1, 4, 5, 8, 9, 17, 33, 65, 129, 256])
+def test_runs_and_parts(N, dtype):
+    depth = 3 if N < 5 else 12
+    rand = W.tree_random(W.IntStream(N), N, depth) if N > 1 else [-1]
+    chain = [i - 1 for i in range(N)]
+    check(W.make_case("runs", [rand, chain], seed=N, Hk=1, Hv=1, d=64, in_dtype=dtype, Ns=N + 3, permute_slots=True, with_bias=True))
+
+
+@pytest.mark.parametrize("B,N", [(8, 64), (24, 40), (32, 28), (12, 200)])
+def test_longer_runs_of_large_launches(B, N):
+    check(W.make_case("runs", [W.tree_random(W.IntStream(N + b), N, 9) for b in range(B)], seed=B, Hk=3, Hv=6, d=128, in_dtype="bf16"))
