@@ -528,7 +528,8 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
   if (rc != LUMO_OK) return rc;
   DeviceGuard g(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
-  const TreeDev t = tree_view(desc, s.snapshot_mode != 0 ? 1 : 0);
+  const TreeDev lean = tree_view(desc, 0);
+  const TreeDev t = s.snapshot_mode != 0 && !scan_staged(s, lean) ? tree_view(desc, 1) : lean;
   const bool gram_ok = desc->d_tc_meta != nullptr && gram_supported(s, desc->max_depth);
   if (ctx->scan_algo >= 2 && !gram_ok)
     return fail(ctx, LUMO_ERR_UNSUPPORTED, "the Gram-form scan needs d = 128, bf16 operands, depth <= 16, no snapshots");
@@ -573,7 +574,7 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
     if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
   }
   e = timed(ctx, LUMO_K_SCAN, st, [&] {
-    return launch_scan(s, t, lb, reinterpret_cast<float*>(ctx->scratch), grid, st);
+    return launch_scan(s, t, lb, reinterpret_cast<float*>(ctx->scratch), grid, use_overlap(ctx, s), st);
   });
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "scan launch");
 }
@@ -593,7 +594,8 @@ int lumo_gdn_tree_scan_static(lumo_ctx* ctx, const lumo_tree_desc* desc, const l
   if (rc != LUMO_OK) return rc;
   DeviceGuard g(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
-  const TreeDev t = tree_view(desc, s.snapshot_mode != 0 ? 1 : 0);
+  const TreeDev lean = tree_view(desc, 0);
+  const TreeDev t = s.snapshot_mode != 0 && !scan_staged(s, lean) ? tree_view(desc, 1) : lean;
   int grid = 0;
   size_t stack_bytes = 0;
   cudaError_t e = scan_plan(s, t, ctx->sm_count, &grid, &stack_bytes);
@@ -605,7 +607,7 @@ int lumo_gdn_tree_scan_static(lumo_ctx* ctx, const lumo_tree_desc* desc, const l
   float* stack = nullptr;
   e = static_stack_address(ctx->device, &stack);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGetSymbolAddress(built-in scan stack)");
-  e = timed(ctx, LUMO_K_SCAN, st, [&] { return launch_scan(s, t, lb, stack, grid, st); });
+  e = timed(ctx, LUMO_K_SCAN, st, [&] { return launch_scan(s, t, lb, stack, grid, false, st); });
   ctx->last_call = lumo_ctx::kVerify;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "scan launch");
 }

@@ -311,7 +311,10 @@ int conv_rows_per_cta(int C, int Ns, int seqs, int sms);
 cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, int sm_count,
                               bool pdl, cudaStream_t st);
 cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, float* stack,
-                        int grid, cudaStream_t st);
+                        int grid, bool pdl, cudaStream_t st);
+// Whether the rank-1 scan holds all of a tree's operands in shared memory (`t`: the lean schedule, which that kernel
+// interprets in every snapshot mode).
+bool scan_staged(const Shape& s, const TreeDev& t);
 // persistent grid size (CTAs resident at once) and the stack scratch it needs
 cudaError_t scan_plan(const Shape& s, const TreeDev& t, int sm_count, int* grid, size_t* stack_bytes);
 // acceptance walk (accept.cu)

@@ -582,6 +582,284 @@ scan_kernel(Shape s, TreeDev t, LB lb, float* __restrict__ stack, int n_items) {
   }
 }
 
+// ---- the same walk with every node's operands in shared memory ---------------------------------------
+// For trees whose widened keys and queries fit (kStagedSmem): they are staged once per CTA, so the operations need no
+// barrier and a warp (eight rows) walks the tree at its own pace.  64 rows per CTA share the staging and the per-node
+// scalars.  In the snapshot modes a leaf's state is formed on its way to memory (a S_p + gk k) without disturbing the
+// registers, and with every state exported a branching node's state is fetched back from the export instead of a stack.
+// Bound by the state writes in the snapshot modes, by instruction latency in small launches.  Measured against the operand
+// ring below: every state of 8 layers of 4 x 32 nodes (2.1 GB) 573 -> 415 us, 5 x 17 nodes of two layers 102 -> 86 us; a step
+// of a seven-node fp32 tree (d = 64) 11.0 -> 8.3 us on the device.
+constexpr int kStagedRows = 64;
+constexpr int kStagedThreads = kStagedRows * kLanesPerRow;
+constexpr int kStagedSmem = 112 * 1024;      // at least two CTAs per SM
+
+struct StagedSmem { int ops, slot, params, snap, levels, k, q, v, dcache, total; };
+__host__ __device__ inline StagedSmem staged_smem(int N, int D, int max_ops, int n_snap_list, int max_levels) {
+  StagedSmem m;
+  int off = 0;
+  auto take = [&](int bytes) { const int at = off; off += (bytes + 15) / 16 * 16; return at; };
+  m.k = take(N * D * 4);
+  m.q = take(N * D * 4);
+  m.v = take(N * kStagedRows * 4);           // values, then outputs
+  m.dcache = take(N * kStagedRows * 4);
+  m.params = take(5 * N * 4);
+  m.ops = take(max_ops * 4);
+  m.slot = take(N * 4);
+  m.snap = take(n_snap_list * 4);
+  m.levels = take(max_levels * (kStagedThreads / 32) * 4);
+  m.total = off;
+  return m;
+}
+
+template <int D, typename T, class LB>
+__global__ void __launch_bounds__(kStagedThreads, 3)
+scan_staged_kernel(Shape s, TreeDev t, LB lb, float* __restrict__ stack, int n_items) {
+  constexpr int NCH = D / 16, kVec = 16 / (int)sizeof(T);
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int n_snap_list = s.snapshot_mode == 1 ? s.n_snap : 0;
+  const StagedSmem lay = staged_smem(s.N, D, t.max_ops, n_snap_list, t.max_levels);
+  float* s_k = reinterpret_cast<float*>(smem + lay.k);
+  float* s_q = reinterpret_cast<float*>(smem + lay.q);
+  float* s_v = reinterpret_cast<float*>(smem + lay.v);
+  float* s_dc = reinterpret_cast<float*>(smem + lay.dcache);
+  float* p_a = reinterpret_cast<float*>(smem + lay.params);
+  float* p_b = p_a + s.N;
+  float* p_ks = p_b + s.N;      // multiplies the raw key (1 / norm when normalising)
+  float* p_qs = p_ks + s.N;     // multiplies the raw query (scale / norm)
+  float* p_kq = p_qs + s.N;     // k_n . q_n with both factors applied
+  int32_t* s_ops = reinterpret_cast<int32_t*>(smem + lay.ops);
+  int32_t* s_slot = reinterpret_cast<int32_t*>(smem + lay.slot);
+  int32_t* s_snap = reinterpret_cast<int32_t*>(smem + lay.snap);
+
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int j = tid & 3;               // lane within the row group
+  const int rl = tid >> 2;             // local row
+  int32_t* lvl_node = reinterpret_cast<int32_t*>(smem + lay.levels) + warp * t.max_levels;   // node pushed at each level
+  constexpr int kTiles = D / kStagedRows;
+  const int rep = s.Hv / s.Hk;
+  float* my_stack = stack + ((size_t)blockIdx.x * t.max_levels * kStagedRows + rl) * D + 4 * j;
+
+  bool waited = false;
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {   // bounded: n_items
+    const int tile = item % kTiles;
+    const int hv = (item / kTiles) % s.Hv;
+    const int b = (item / (kTiles * s.Hv)) % s.B;
+    const int layer = item / (kTiles * s.Hv * s.B);
+    const LayerPtrs& L = lb.l[layer];
+    const int g = hv / rep;
+    const int r0 = tile * kStagedRows;
+    const size_t out_row_stride = (size_t)s.Hv * D;
+    __syncthreads();   // previous item's shared memory is no longer in use
+    const int nops = t.nops[b];
+    for (int e = tid; e < nops; e += kStagedThreads) s_ops[e] = t.sched[(size_t)b * t.max_ops + e];
+    for (int e = tid; e < s.N; e += kStagedThreads) s_slot[e] = t.slot[b * s.N + e];
+    if (!waited) { pdl_wait(); pdl_trigger(); waited = true; }        // only descriptor tables were read so far
+    const int row = L.state_row[b];
+    const bool lead = L.status && hv == 0 && tile == 0 && tid == 0;
+    if (row < 0 || row >= s.n_state_rows) {
+      // skipped sequence: zero outputs; flag a row outside the pool
+      for (int e = tid; e < s.Ns * kStagedRows; e += kStagedThreads)
+        store_scalar(L.out, ((size_t)b * s.Ns + e / kStagedRows) * out_row_stride + hv * D + r0 + e % kStagedRows, s.out_dtype, 0.f);
+      if (lead) L.status[b] = row < 0 ? LUMO_SEQ_OK : LUMO_SEQ_BAD_ROW;
+      continue;
+    }
+    if (lead) L.status[b] = LUMO_SEQ_OK;
+
+    // pre-tree state rows -> registers (issued first so the loads overlap the staging)
+    const float* S0 = L.state + (((size_t)row * s.Hv + hv) * D + r0 + rl) * D + 4 * j;
+    float4 S[NCH];
+#pragma unroll
+    for (int m = 0; m < NCH; ++m) S[m] = *reinterpret_cast<const float4*>(S0 + 16 * m);
+    for (int e = tid; e < n_snap_list; e += kStagedThreads) s_snap[e] = L.snap_nodes[(size_t)b * s.n_snap + e];
+    // padding rows: zero outputs
+    if (s.Ns > s.N)
+      for (int e = tid; e < s.Ns * kStagedRows; e += kStagedThreads) {
+        const int ps = e / kStagedRows;
+        if (t.slot_inv[b * s.Ns + ps] < 0)
+          store_scalar(L.out, ((size_t)b * s.Ns + ps) * out_row_stride + hv * D + r0 + e % kStagedRows, s.out_dtype, 0.f);
+      }
+    // gates of this thread's node (a CTA has more threads than a staged tree has nodes)
+    if (tid < s.N) {
+      const float2 gates = load_gates(L, s, ((size_t)b * s.Ns + t.slot[b * s.N + tid]) * s.Hv + hv, hv);
+      p_a[tid] = gates.x;
+      p_b[tid] = gates.y;
+    }
+    __syncthreads();   // slots
+    {
+      const T* qg = reinterpret_cast<const T*>(L.q) + (size_t)b * s.Ns * s.Hk * D + g * D;
+      const T* kg = reinterpret_cast<const T*>(L.k) + (size_t)b * s.Ns * s.Hk * D + g * D;
+      const T* vg = reinterpret_cast<const T*>(L.v) + (size_t)b * s.Ns * s.Hv * D + hv * D + r0;
+      auto put = [&](float* dst, const T* src) {
+        const uint4 w = *reinterpret_cast<const uint4*>(src);
+        if constexpr (sizeof(T) == 2) {
+          reinterpret_cast<float4*>(dst)[0] = Packed4<T>::unpack(make_uint2(w.x, w.y));
+          reinterpret_cast<float4*>(dst)[1] = Packed4<T>::unpack(make_uint2(w.z, w.w));
+        } else {
+          *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(&w);
+        }
+      };
+      constexpr int kKP = D / kVec, kVP = kStagedRows / kVec;       // 16-byte pieces of a row
+#pragma unroll 4
+      for (int e = tid; e < s.N * kKP; e += kStagedThreads) {
+        const int n = e / kKP, c = (e % kKP) * kVec;
+        const size_t off = (size_t)((uint32_t)s_slot[n] * (uint32_t)(s.Hk * D)) + c;
+        put(s_k + n * D + c, kg + off);
+        put(s_q + n * D + c, qg + off);
+      }
+#pragma unroll 2
+      for (int e = tid; e < s.N * kVP; e += kStagedThreads) {
+        const int n = e / kVP, c = (e % kVP) * kVec;
+        put(s_v + n * kStagedRows + c, vg + (size_t)((uint32_t)s_slot[n] * (uint32_t)(s.Hv * D)) + c);
+      }
+    }
+    __syncthreads();
+    {
+      // per-node scalars: normalisation factors and k.q, eight lanes per node; the trip count is uniform over the CTA
+      // so that every lane takes part in the shuffles
+      const int grp = tid >> 3, gl = tid & 7;
+      for (int n0 = 0; n0 < s.N; n0 += kStagedThreads / 8) {
+        const int n = n0 + grp;
+        const bool live = n < s.N;
+        float kk = 0.f, qq = 0.f, kq = 0.f;
+        if (live) {
+#pragma unroll
+          for (int c = 0; c < D / 32; ++c) {
+            const float4 kv = *reinterpret_cast<const float4*>(s_k + n * D + gl * 4 + 32 * c), qv = *reinterpret_cast<const float4*>(s_q + n * D + gl * 4 + 32 * c);
+            kk += kv.x * kv.x + kv.y * kv.y + kv.z * kv.z + kv.w * kv.w;
+            qq += qv.x * qv.x + qv.y * qv.y + qv.z * qv.z + qv.w * qv.w;
+            kq += kv.x * qv.x + kv.y * qv.y + kv.z * qv.z + kv.w * qv.w;
+          }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+          kk += __shfl_xor_sync(0xffffffffu, kk, o);
+          qq += __shfl_xor_sync(0xffffffffu, qq, o);
+          kq += __shfl_xor_sync(0xffffffffu, kq, o);
+        }
+        if (live && gl == 0) {
+          float ks = 1.f, qs = s.scale;
+          if (s.l2norm) { ks = rsqrtf(kk + s.l2_eps); qs = s.scale * rsqrtf(qq + s.l2_eps); }
+          p_ks[n] = ks; p_qs[n] = qs; p_kq[n] = kq * ks * qs;
+        }
+      }
+    }
+    __syncthreads();
+
+    // where node n's state goes (nullptr: nowhere); mode 1 may name a node more than once
+    auto snap_at = [&](int e) { return L.snap_out + ((((size_t)b * s.n_snap + e) * s.Hv + hv) * D + r0 + rl) * D + 4 * j; };
+    auto export_state = [&](int n, const float4 (&X)[NCH]) {
+      if (s.snapshot_mode == 2) {
+        float* dst = snap_at(n);
+#pragma unroll
+        for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(dst + 16 * m) = X[m];
+      } else {
+        for (int e = 0; e < s.n_snap; ++e) {          // bounded: the list
+          if (s_snap[e] != n) continue;
+          float* dst = snap_at(e);
+#pragma unroll
+          for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(dst + 16 * m) = X[m];
+        }
+      }
+    };
+    int cur = -1;                                      // node whose state the registers hold (-1: the pre-tree state)
+#pragma unroll 1
+    for (int i = 0; i < nops; ++i) {                   // bounded: nops <= max_ops
+      const int op = s_ops[i];
+      const int kind = op >> 24;
+      const int arg = op & 0xFFFF;
+      if (kind <= OP_DESCEND) {
+        const int n = arg;
+        const float* kr = s_k + n * D + 4 * j;
+        const float a = p_a[n], ks = p_ks[n];
+        float dl;
+        if (kind == OP_DESCEND) {
+          dl = s_dc[n * kStagedRows + rl];
+        } else {
+          const float* qr = s_q + n * D + 4 * j;
+          float2 u2 = make_float2(0.f, 0.f), w2 = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int m = 0; m < NCH; ++m) {
+            const float4 kv = *reinterpret_cast<const float4*>(kr + 16 * m), qv = *reinterpret_cast<const float4*>(qr + 16 * m);
+            const float2 lo = make_float2(S[m].x, S[m].y), hi = make_float2(S[m].z, S[m].w);
+            u2 = __ffma2_rn(lo, make_float2(kv.x, kv.y), u2); u2 = __ffma2_rn(hi, make_float2(kv.z, kv.w), u2);
+            w2 = __ffma2_rn(lo, make_float2(qv.x, qv.y), w2); w2 = __ffma2_rn(hi, make_float2(qv.z, qv.w), w2);
+          }
+          float u = u2.x + u2.y, w = w2.x + w2.y;
+          u += __shfl_xor_sync(0xffffffffu, u, 1); w += __shfl_xor_sync(0xffffffffu, w, 1);
+          u += __shfl_xor_sync(0xffffffffu, u, 2); w += __shfl_xor_sync(0xffffffffu, w, 2);
+          float* vo = s_v + n * kStagedRows + rl;
+          dl = p_b[n] * (*vo - a * (ks * u));                   // delta = beta (v - R' k)
+          const float o = a * (p_qs[n] * w) + dl * p_kq[n];     // o = R q = a R_p q + delta (k.q)
+          __syncwarp();                                         // the row's four lanes have read v
+          if (j == 0) *vo = o;
+          if ((op >> 20) & 1) {
+            if (j == 0) s_dc[n * kStagedRows + rl] = dl;
+            __syncwarp();
+          }
+        }
+        // the node's state: in place of its parent's, or (a leaf, snapshots) formed on its way out
+        const bool descend = kind != OP_EMIT;
+        if (descend || (s.snapshot_mode != 0 && !((op >> 20) & 1))) {
+          const float gk = dl * ks;
+          const float2 a2 = make_float2(a, a), g2 = make_float2(gk, gk);
+          auto child = [&](int m) {
+            const float4 kv = *reinterpret_cast<const float4*>(kr + 16 * m);
+            const float2 lo = __ffma2_rn(a2, make_float2(S[m].x, S[m].y), __fmul2_rn(g2, make_float2(kv.x, kv.y)));
+            const float2 hi = __ffma2_rn(a2, make_float2(S[m].z, S[m].w), __fmul2_rn(g2, make_float2(kv.z, kv.w)));
+            return make_float4(lo.x, lo.y, hi.x, hi.y);
+          };
+          asm volatile("" ::: "memory");                        // the key row is read again instead of being held in registers
+          if (descend) {
+#pragma unroll
+            for (int m = 0; m < NCH; ++m) S[m] = child(m);
+            cur = n;
+            if (s.snapshot_mode != 0) export_state(n, S);
+          } else if (s.snapshot_mode == 2) {
+            float* dst = snap_at(n);
+#pragma unroll
+            for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(dst + 16 * m) = child(m);
+          } else {
+            for (int e = 0; e < s.n_snap; ++e) {                // bounded: the list
+              if (s_snap[e] != n) continue;
+              float* dst = snap_at(e);
+#pragma unroll
+              for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(dst + 16 * m) = child(m);
+            }
+          }
+        }
+      } else if (kind == OP_PUSH) {
+        if (s.snapshot_mode == 2) {
+          if ((tid & 31) == 0) lvl_node[arg] = cur;             // its state has just been exported
+          __syncwarp();
+        } else {
+          float* dst = my_stack + (size_t)arg * kStagedRows * D;
+#pragma unroll
+          for (int m = 0; m < NCH; ++m) *reinterpret_cast<float4*>(dst + 16 * m) = S[m];
+        }
+      } else {  // OP_POP
+        const float* src = S0;
+        if (arg == kPopRoot) cur = -1;
+        else if (s.snapshot_mode == 2) { cur = lvl_node[arg]; src = snap_at(cur); }
+        else src = my_stack + (size_t)arg * kStagedRows * D;
+#pragma unroll
+        for (int m = 0; m < NCH; ++m) S[m] = *reinterpret_cast<const float4*>(src + 16 * m);
+      }
+    }
+    __syncthreads();
+    // outputs, two rows per thread
+#pragma unroll 2
+    for (int e = tid; e < s.N * (kStagedRows / 2); e += kStagedThreads) {
+      const int n = e / (kStagedRows / 2), c = (e % (kStagedRows / 2)) * 2;
+      const float2 o = *reinterpret_cast<const float2*>(s_v + n * kStagedRows + c);
+      const size_t i = ((size_t)b * s.Ns + s_slot[n]) * out_row_stride + hv * D + r0 + c;
+      if (s.out_dtype == LUMO_BF16) *reinterpret_cast<__nv_bfloat162*>(reinterpret_cast<__nv_bfloat16*>(L.out) + i) = __floats2bfloat162_rn(o.x, o.y);
+      else *reinterpret_cast<float2*>(reinterpret_cast<float*>(L.out) + i) = o;
+    }
+  }
+  if (!waited) pdl_wait();
+}
+
 // One token of the native recurrence on one state row, held by four lanes (lane j: floats 16 m + 4 j ..):
 // S <- alpha S + delta ks k, delta = beta (v - alpha ks S.k).  Packed fp32 FMAs: two correctly rounded lanes per
 // instruction, the same bits as the scalar form of the scan.
@@ -900,44 +1178,67 @@ cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch
   return launch_conv_t<__nv_bfloat16>(s, t, lb, &fp, sm_count, pdl, st);
 }
 
-cudaError_t scan_plan(const Shape& s, const TreeDev& t, int sm_count, int* grid, size_t* stack_bytes) {
-  const int items = s.n_layers * s.B * s.Hv * (s.d / kRows);
-  return dispatch(s.d, s.in_dtype, [&](auto dc, auto tc) {
-    constexpr int D = decltype(dc)::value;
-    using T = decltype(tc);
-    const int n_snap_list = s.snapshot_mode == 1 ? s.n_snap : 0;
-    const ScanSmem lay = scan_smem(s.N, t.max_ops, n_snap_list, ScanCfg<D, T>::kStageBytes);
-    // occupancy of each instance at the shared-memory size it was last asked for: the two calls below cost more
-    // host time than the launch itself
-    static std::atomic<uint64_t> known[kMaxDevices][2] = {};
+// Trees whose operands fit in shared memory take the staged kernel.
+bool scan_staged(const Shape& s, const TreeDev& t) {
+  return s.N <= kStagedThreads &&
+         staged_smem(s.N, s.d, t.max_ops, s.snapshot_mode == 1 ? s.n_snap : 0, t.max_levels).total <= kStagedSmem;
+}
+
+// CTAs of `kern` that an SM holds at `smem` bytes; raises the kernel's shared-memory limit when it has to.  The answer for
+// the size last asked for is kept per kernel instance and device: the two calls cost more host time than the launch itself.
+struct Occupancy {
+  std::atomic<uint64_t> known[kMaxDevices] = {};      // smem << 8 | CTAs
+  std::mutex mu;
+  int limit[kMaxDevices] = {};                        // only grows, so that a launch prepared for another size still fits
+  cudaError_t per_sm(const void* kern, int threads, int smem, int* ctas) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    const bool few = s.n_layers <= kFewLayers;
-    const uint64_t seen = known[dev][few].load(std::memory_order_relaxed);
-    int per_sm = (int)(seen & 0xFF);
-    if (seen >> 8 != (uint64_t)lay.total || per_sm == 0) {
-      auto kern = few ? (const void*)scan_kernel<D, T, FewLayers> : (const void*)scan_kernel<D, T, LayerBatch>;
-      // the limit only grows, so that a launch prepared for another size on another thread still fits
-      static std::mutex mu;
-      static int limit[kMaxDevices][2] = {};
-      {
-        std::lock_guard<std::mutex> lock(mu);
-        if (lay.total > limit[dev][few]) {
-          e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.total);
-          if (e != cudaSuccess) return e;
-          limit[dev][few] = lay.total;
-        }
+    const uint64_t seen = known[dev].load(std::memory_order_relaxed);
+    *ctas = (int)(seen & 0xFF);
+    if (seen >> 8 == (uint64_t)smem && *ctas > 0) return cudaSuccess;
+    {
+      std::lock_guard<std::mutex> lock(mu);
+      if (smem > limit[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        limit[dev] = smem;
       }
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kScanThreads, lay.total);
-      if (e != cudaSuccess) return e;
-      if (per_sm < 1) per_sm = 1;
-      known[dev][few].store((uint64_t)lay.total << 8 | (uint64_t)per_sm, std::memory_order_relaxed);
     }
-    const int resident = sm_count * per_sm;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, kern, threads, smem);
+    if (e != cudaSuccess) return e;
+    if (*ctas < 1) *ctas = 1;
+    known[dev].store((uint64_t)smem << 8 | (uint64_t)*ctas, std::memory_order_relaxed);
+    return cudaSuccess;
+  }
+};
+
+cudaError_t scan_plan(const Shape& s, const TreeDev& t, int sm_count, int* grid, size_t* stack_bytes) {
+  return dispatch(s.d, s.in_dtype, [&](auto dc, auto tc) {
+    constexpr int D = decltype(dc)::value;
+    using T = decltype(tc);
+    const int n_snap_list = s.snapshot_mode == 1 ? s.n_snap : 0;
+    const bool few = s.n_layers <= kFewLayers, staged = scan_staged(s, t);
+    static Occupancy occ[2][2];
+    int per_sm = 0, smem, rows;
+    cudaError_t e;
+    if (staged) {
+      rows = kStagedRows;
+      smem = staged_smem(s.N, D, t.max_ops, n_snap_list, t.max_levels).total;
+      e = occ[1][few].per_sm(few ? (const void*)scan_staged_kernel<D, T, FewLayers> : (const void*)scan_staged_kernel<D, T, LayerBatch>,
+                             kStagedThreads, smem, &per_sm);
+    } else {
+      rows = kRows;
+      smem = scan_smem(s.N, t.max_ops, n_snap_list, ScanCfg<D, T>::kStageBytes).total;
+      e = occ[0][few].per_sm(few ? (const void*)scan_kernel<D, T, FewLayers> : (const void*)scan_kernel<D, T, LayerBatch>, kScanThreads,
+                             smem, &per_sm);
+    }
+    if (e != cudaSuccess) return e;
+    const int items = s.n_layers * s.B * s.Hv * (D / rows), resident = sm_count * per_sm;
     *grid = items < resident ? items : resident;
-    *stack_bytes = (size_t)*grid * t.max_levels * kRows * D * sizeof(float);
+    // with every state exported the staged kernel needs no stack
+    *stack_bytes = staged && s.snapshot_mode == 2 ? 0 : (size_t)*grid * t.max_levels * rows * D * sizeof(float);
     return cudaSuccess;
   });
 }
@@ -971,14 +1272,22 @@ cudaError_t static_stack_address(int device, float** ptr) {
 }
 
 cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, float* stack,
-                        int grid, cudaStream_t st) {
-  const int items = s.n_layers * s.B * s.Hv * (s.d / kRows);
+                        int grid, bool pdl, cudaStream_t st) {
   return dispatch(s.d, s.in_dtype, [&](auto dc, auto tc) {
     constexpr int D = decltype(dc)::value;
     using T = decltype(tc);
     const int n_snap_list = s.snapshot_mode == 1 ? s.n_snap : 0;
+    const bool few = s.n_layers <= kFewLayers;
+    if (scan_staged(s, t)) {
+      const int items = s.n_layers * s.B * s.Hv * (D / kStagedRows);
+      const StagedSmem lay = staged_smem(s.N, D, t.max_ops, n_snap_list, t.max_levels);
+      if (few)
+        return launch_kernel(scan_staged_kernel<D, T, FewLayers>, dim3(grid), dim3(kStagedThreads), lay.total, st, pdl, s, t, few_layers(lb), stack, items);
+      return launch_kernel(scan_staged_kernel<D, T, LayerBatch>, dim3(grid), dim3(kStagedThreads), lay.total, st, pdl, s, t, lb, stack, items);
+    }
+    const int items = s.n_layers * s.B * s.Hv * (D / kRows);
     const ScanSmem lay = scan_smem(s.N, t.max_ops, n_snap_list, ScanCfg<D, T>::kStageBytes);
-    if (s.n_layers <= kFewLayers)
+    if (few)
       return launch_kernel(scan_kernel<D, T, FewLayers>, dim3(grid), dim3(kScanThreads), lay.total, st, false, s, t, few_layers(lb), stack, items);
     return launch_kernel(scan_kernel<D, T, LayerBatch>, dim3(grid), dim3(kScanThreads), lay.total, st, false, s, t, lb, stack, items);
   });
