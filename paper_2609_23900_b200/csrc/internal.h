@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lumo_gdn.h"
@@ -276,9 +277,10 @@ cudaError_t launch_by_address(const cudaLaunchConfig_t& cfg, void (*kern)(KArgs.
 // Launch of a kernel whose CTAs form clusters of `cluster` along x, as a programmatic dependent of the kernel before
 // it: its CTAs are placed while that one drains and pass pdl_wait() before they touch global memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, const Args&... args) {
+cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st,
+                                  const Args&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = st;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;

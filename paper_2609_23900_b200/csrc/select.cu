@@ -333,9 +333,9 @@ cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int sp
   }
   if (cluster > cap) return cudaErrorInvalidConfiguration;
   if (dtype == LUMO_BF16)
-    return launch_cluster_kernel(select_kernel<__nv_bfloat16>, dim3(cluster, rows), dim3(kSelThreads), cluster, st,
+    return launch_cluster_kernel(select_kernel<__nv_bfloat16>, dim3(cluster, rows), dim3(kSelThreads), cluster, 0, st,
                                  reinterpret_cast<const __nv_bfloat16*>(logits), V, spine, cand);
-  return launch_cluster_kernel(select_kernel<float>, dim3(cluster, rows), dim3(kSelThreads), cluster, st,
+  return launch_cluster_kernel(select_kernel<float>, dim3(cluster, rows), dim3(kSelThreads), cluster, 0, st,
                                reinterpret_cast<const float*>(logits), V, spine, cand);
 }
 
