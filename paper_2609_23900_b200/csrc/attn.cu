@@ -62,6 +62,7 @@ constexpr int kColP = 448;
 constexpr int kSeqCache = 64;         // sequences whose context length, cache row and tile count are kept in shared memory
 constexpr int kUnitCost = 5;          // what starting a unit costs a CTA (read-out of the one before, new queries, refill of
                                       // the pipeline: ~8 us measured), in tiles: the shares are evened out in these terms
+constexpr int kWholeSlack = 4;        // automatic mode: units stay whole when none exceeds an even share by more than this many tiles
 constexpr int kMinTilesPerCta = 4;    // automatic mode: do not cut the work finer than this
 constexpr float kRescaleStep = 16.f;  // the reference maximum moves when exceeded by more than this (log2 units)
 constexpr uint32_t kSpinLimit = 1u << 24;
@@ -210,6 +211,21 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
+// Visibility of 64 consecutive keys from suffix slot s0 on (negative: keys of the committed context, always visible), from a
+// node's 256-bit row over the suffix.
+__device__ __forceinline__ unsigned long long visible64(const uint32_t* row, int s0) {
+  if (s0 >= kMaxAttnSlots) return 0ull;
+  const int w = s0 > 0 ? s0 >> 5 : 0, off = s0 > 0 ? s0 & 31 : 0;
+  unsigned long long v = __ldg(row + w);
+  if (w + 1 < 8) v |= (unsigned long long)__ldg(row + w + 1) << 32;
+  if (off) {
+    v >>= off;
+    if (w + 2 < 8) v |= (unsigned long long)__ldg(row + w + 2) << (64 - off);
+  }
+  if (s0 < 0) v = s0 <= -64 ? ~0ull : v << -s0 | ((1ull << -s0) - 1ull);
+  return v;
+}
+
 // ---- work decomposition ----------------------------------------------------------------
 // Units are numbered u = (b * Hkv + hkv) * RT + rt; unit u owns nt(b) tiles (0 for a sequence that fails
 // its check).  Automatic mode: the units are laid end to end on a line, each preceded by kUnitCost idle
@@ -232,6 +248,7 @@ struct Work {
   int g_unit;         // position at which the current unit's stretch (idle prefix, then its tiles) starts
   int nt;             // tiles per unit of the current sequence
   int per;            // automatic mode: positions per CTA
+  int parts;          // partitions per unit when CTA c owns partition c mod parts of unit c / parts; 0: shares of the line
   bool fixed_done;
 
   __device__ __forceinline__ int tiles_of(const AttnArgs& a, int bb, int* ctx, int* crow) const {
@@ -244,15 +261,20 @@ struct Work {
 
   __device__ __forceinline__ void init() {
     b = 0; q = 0; g = 0; g_end = 0; g_unit = 0; nt = 0; per = 1; fixed_done = false;
-    if (a.S > 0) return;
+    parts = a.S;
+    if (parts > 0) return;
     const int upb = a.Hkv * a.RT;       // units per sequence
     int total = 0;
-    int cx, cr;
+    int cx, cr, most = 0;
     for (int bb = 0; bb < a.B; ++bb) {
       const int n = tiles_of(a, bb, &cx, &cr);
       if (n > 0) total += (n + kUnitCost) * upb;
+      most = max(most, n);
     }
     per = (total + (int)gridDim.x - 1) / (int)gridDim.x;
+    // Short contexts: when there is a CTA for every unit and no unit is much longer than an even share, units stay whole:
+    // nothing is cut, and with one segment per unit the outputs are final when they leave this kernel.
+    if (a.B * upb <= (int)gridDim.x && most <= per + kWholeSlack) { parts = 1; return; }
     if (per < kMinTilesPerCta) per = kMinTilesPerCta;
     g = (int)blockIdx.x * per;
     g_end = g + per < total ? g + per : total;
@@ -271,18 +293,19 @@ struct Work {
   // next segment of this CTA; false when the share is exhausted
   __device__ __forceinline__ bool next(Segment* s) {
     const int upb = a.Hkv * a.RT;
-    if (a.S > 0) {
+    if (parts > 0) {
       if (fixed_done) return false;
       fixed_done = true;
-      const int u = blockIdx.x / a.S, part = blockIdx.x - u * a.S;
+      const int u = blockIdx.x / parts, part = blockIdx.x - u * parts;
       s->b = u / upb;
+      if (s->b >= a.B) return false;
       const int r = u - s->b * upb;
       s->hkv = r / a.RT; s->rt = r - s->hkv * a.RT;
       const int n_all = tiles_of(a, s->b, &s->ctx, &s->crow);
-      s->t0 = (int)(((long long)part * n_all) / a.S);
-      s->n = (int)(((long long)(part + 1) * n_all) / a.S) - s->t0;
+      s->t0 = (int)(((long long)part * n_all) / parts);
+      s->n = (int)(((long long)(part + 1) * n_all) / parts) - s->t0;
       s->slot = blockIdx.x;
-      s->unit = u; s->slot0 = u * a.S; s->nslots = a.S;
+      s->unit = u; s->slot0 = u * parts; s->nslots = parts;
       return n_all > 0;
     }
     while (g < g_end && b < a.B) {
@@ -515,18 +538,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         const int kpos0 = (sg.t0 + j) * kKeys + half * 64;   // first key of this thread's 64
         const bool tail = (sg.t0 + j + 1) * kKeys > sg.ctx;  // uniform: the tile reaches past the committed context
         unsigned long long vm = ~0ull;
-        if (tail) {
-          vm = 0ull;
-          for (int c = 0; c < 64; ++c) {
-            const int p = kpos0 + c;
-            bool v = p < sg.ctx;
-            if (!v) {
-              const int s = p - sg.ctx;
-              if (s < a.Ns) v = (__ldg(visw + (s >> 5)) >> (s & 31)) & 1u;
-            }
-            vm |= (unsigned long long)v << c;
-          }
-        }
+        if (tail) vm = visible64(visw, kpos0 - sg.ctx);
         if (ok) ok = mbar_wait_relaxed(&sm.s_full[buf], (it >> 1) & 1u);
         tc_fence_after();
         __syncwarp();
@@ -637,12 +649,24 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
       asm volatile("bar.sync %0, 64;\n" ::"r"(pair_bar) : "memory");
       const float lt = sm.xchg[0][0][row] + sm.xchg[0][1][row];
       const float inv = lt > 0.f ? 1.f / lt : 0.f;
+      const bool whole = sg.nslots == 1;         // the only segment of its unit: these are the final outputs
+      const size_t out_row = (((size_t)sg.b * a.N + node) * a.Hq + (size_t)sg.hkv * a.G + hl);
 #pragma unroll 1
       for (int c = 0; c < 64; c += 32) {
         uint32_t orr[32];
         tmem_ld32(tmem_lane + kColO + half * 64 + c, orr);
         tmem_ld_wait();
-        if (row_ok) {
+        if (row_ok && whole) {
+          float* o = a.out + out_row * kDh + half * 64 + c;
+#pragma unroll
+          for (int e = 0; e < 32; e += 8) {      // a lane's 32 bytes: whole sectors
+            const float f[8] = {__uint_as_float(orr[e]) * inv,     __uint_as_float(orr[e + 1]) * inv, __uint_as_float(orr[e + 2]) * inv,
+                                __uint_as_float(orr[e + 3]) * inv, __uint_as_float(orr[e + 4]) * inv, __uint_as_float(orr[e + 5]) * inv,
+                                __uint_as_float(orr[e + 6]) * inv, __uint_as_float(orr[e + 7]) * inv};
+            *reinterpret_cast<float4*>(o + e) = make_float4(f[0], f[1], f[2], f[3]);
+            *reinterpret_cast<float4*>(o + e + 4) = make_float4(f[4], f[5], f[6], f[7]);
+          }
+        } else if (row_ok) {
 #pragma unroll
           for (int e = 0; e < 32; e += 4)
             slot_o[(size_t)((c + e) >> 2) * kRows] =
@@ -650,7 +674,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                             __uint_as_float(orr[e + 2]) * inv, __uint_as_float(orr[e + 3]) * inv);
         }
       }
-      if (row_ok && half == 0) *slot_l = lt > 0.f ? m + log2f(lt) : -INFINITY;
+      if (row_ok && half == 0) {
+        const float l2 = lt > 0.f ? m + log2f(lt) : -INFINITY;
+        if (!whole) *slot_l = l2;
+        else if (a.lse) a.lse[out_row] = lt > 0.f ? l2 * kLn2 : -INFINITY;
+      }
       tc_fence_before();
       asm volatile("bar.sync %0, 64;\n" ::"r"(pair_bar) : "memory");   // the partner has read xchg[0] before the next segment writes it
       if (lane == 0) mbar_arrive(&sm.o_free);
@@ -705,6 +733,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const AttnArgs a) {
     return;
   }
   const int slot0 = t.x, nslot = t.y;
+  if (nslot == 1) return;                    // a single segment: the attention kernel has written the outputs
   const float* lse_p = a.part_lse + (size_t)slot0 * kRows + r;                          // + slot * kRows
   const float4* row_p = reinterpret_cast<const float4*>(a.part_o) + ((size_t)slot0 * 32 + cg) * kRows + r;   // + slot * 32 * kRows
   // Second round trip: the rows of the first kBatch slots together with all log-sum-exps; further slots follow

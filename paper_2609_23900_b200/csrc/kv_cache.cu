@@ -18,23 +18,27 @@ __global__ void __launch_bounds__(128) kv_write_kernel(const KL L, const KvShape
   const int i = blockIdx.x, b = blockIdx.y, l = blockIdx.z;
   pdl_wait();          // everything below may belong to earlier kernels
   pdl_trigger();
-  const int ctx = s.ctx_len[b], crow = s.cache_row[b];
-  const int bad = seq_check(ctx, crow, s.Ns, s.n_rows, s.max_pos);
-  if (L.status[l] && i == 0 && threadIdx.x == 0) L.status[l][b] = bad;
-  if (bad != LUMO_SEQ_OK) return;
   const int chunks = s.Hkv * kDh / 8;      // 16-byte chunks per entry (16 per head)
   const size_t src = ((size_t)b * s.N + i) * chunks;
   const uint4* kn = reinterpret_cast<const uint4*>(L.kn[l]) + src;
   const uint4* vn = reinterpret_cast<const uint4*>(L.vn[l]) + src;
+  // the first pieces are requested together with the numbers that say where they go
+  const int c0 = threadIdx.x;
+  uint4 k0 = make_uint4(0, 0, 0, 0), v0 = k0;
+  if (c0 < chunks) { k0 = __ldg(kn + c0); v0 = __ldg(vn + c0); }
+  const int ctx = s.ctx_len[b], crow = s.cache_row[b], slot = s.slot[(size_t)b * s.N + i];
+  const int bad = seq_check(ctx, crow, s.Ns, s.n_rows, s.max_pos);
+  if (L.status[l] && i == 0 && threadIdx.x == 0) L.status[l][b] = bad;
+  if (bad != LUMO_SEQ_OK) return;
   // chunk strides of the cache: position and head
   const size_t pos_st = s.layout ? 16 : (size_t)s.Hkv * 16, head_st = s.layout ? (size_t)s.max_pos * 16 : 16;
-  const size_t dst = (size_t)crow * s.max_pos * chunks + (size_t)(ctx + s.slot[(size_t)b * s.N + i]) * pos_st;
+  const size_t dst = (size_t)crow * s.max_pos * chunks + (size_t)(ctx + slot) * pos_st;
   uint4* kc = reinterpret_cast<uint4*>(L.k[l]) + dst;
   uint4* vc = reinterpret_cast<uint4*>(L.v[l]) + dst;
-  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
+  for (int c = c0; c < chunks; c += blockDim.x) {
     const size_t o = (size_t)(c >> 4) * head_st + (c & 15);
-    kc[o] = __ldg(kn + c);
-    vc[o] = __ldg(vn + c);
+    kc[o] = c == c0 ? k0 : __ldg(kn + c);
+    vc[o] = c == c0 ? v0 : __ldg(vn + c);
   }
 }
 
@@ -54,7 +58,7 @@ __global__ void __launch_bounds__(256) kv_publish_kernel(const KL L, const KvSha
   const int ctx = s.ctx_len[b], crow = s.cache_row[b];
   const int n = len[b];
   const int nn = n < 0 ? 0 : (n > lmax ? lmax : n);
-  for (int t = tid; t < nn; t += blockDim.x) {
+  for (int t = tid; t < lmax; t += blockDim.x) {             // (all places: the length is still on its way)
     const int a = accepted[(size_t)b * lmax + t];
     acc_s[t] = a;
     const bool in = a >= 0 && a < s.N;
