@@ -103,25 +103,31 @@ constexpr int kSmemBytesFused = kOffPrev + (int)sizeof(PrevStage) + 1024;
 
 // Layout of one CTA.  Compact (trees of at most 32 nodes, not fused): the state crosses shared memory
 // one 64-column half at a time (hi + lo of one k-block, 32 KB), the aliased areas shrink with the node
-// count, and a CTA needs 68 KB of shared memory and 128 tensor-memory columns: three CTAs per SM
-// instead of two (and 80 registers per thread instead of 128).
+// count, and a CTA needs 52 KB of shared memory and 128 tensor-memory columns: four CTAs per SM instead of
+// two (64 registers per thread instead of 128).  The tails without the tensor-core product spill at 64 and keep three CTAs.
 template <bool C>
 struct GL {
   static constexpr int kNodes = C ? 32 : kNT;
-  static constexpr int kAhi = 0, kAlo = C ? 16384 : 32768;
-  static constexpr int kKQ = C ? 32768 : kOffKQ;
-  static constexpr int kSmall = C ? 65536 : kOffSmall;
+  static constexpr int kKQ = C ? 0 : kOffKQ;
+  static constexpr int kKBlock = C ? 8192 : 16384;             // bytes of one 64-column block of the K and Q rows
+  static constexpr int kAhi = C ? 16384 : 0, kAlo = 32768;
+  static constexpr int kSmall = C ? 49152 : kOffSmall;
+  static constexpr int kDump = C ? kAhi : kOffDump;            // the aliased areas start over the state tiles
   static constexpr int kStride = C ? 33 : kDumpStride;         // floats per dumped Gram row
-  static constexpr int kRec = C ? 128 * 33 * 4 : kOffRec;      // records behind the Gram dump / the deltas
+  static constexpr int kRec = kDump + (C ? 128 * 33 * 4 : kOffRec);      // records behind the Gram dump / the deltas
+  static constexpr int kMt = C ? kDump + 9216 : kOffKQ;        // M tiles of the closed form: behind the Gram rows in use, or over K and Q
   static constexpr int kV = kRec + kNodes * (int)sizeof(NodeRec);
   static constexpr int kZero = kNodes * kD;                    // element offset of the all-zero delta row
   static constexpr int kTmem = C ? 128 : kTmemCols;
   static constexpr int kGramCol = C ? 64 : 128;                // first tensor-memory column of the Gram block
   static constexpr int kBytes = kSmall + (int)sizeof(Small) + 1024;
 };
-static_assert((GL<true>::kNodes + 1) * kD * 4 <= GL<true>::kRec, "delta array overflows the dump area");
-static_assert(GL<true>::kV + GL<true>::kNodes * kD * 2 <= GL<true>::kKQ, "aliased region overflows the state tiles");
-static_assert(3 * (GL<true>::kBytes + 1024) <= 228 * 1024, "three compact CTAs must share an SM");
+static_assert(GL<true>::kDump + (GL<true>::kNodes + 1) * kD * 4 <= GL<true>::kRec, "delta array overflows the dump area");
+static_assert(GL<true>::kV + GL<true>::kNodes * kD * 2 <= GL<true>::kSmall, "aliased region overflows the state tiles");
+// the Gram product takes 128 rows from each K/Q block: the 64 rows behind the last one must lie inside the CTA's memory
+static_assert(GL<true>::kKQ + 2 * GL<true>::kKBlock + 8192 <= GL<true>::kSmall, "the Gram operand reaches past the state tiles");
+static_assert(GL<true>::kDump + 64 * GL<true>::kStride * 4 <= GL<true>::kMt && GL<true>::kMt + 4096 <= GL<true>::kRec, "M tiles overlap the Gram rows in use");
+static_assert(4 * (GL<true>::kBytes + 1024) <= 228 * 1024, "four compact CTAs must share an SM");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -155,6 +161,20 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t pari
   return false;
 }
 
+// The whole CTA waits for the products committed to sm.mbar: one warp polls, the others sit in the barrier behind it
+// (with every warp polling, several hundred of an item's 15,000 instructions were polls).  Returns the same answer in
+// every thread: false when the bounded wait ran out.
+__device__ __forceinline__ bool wait_products(Small& sm, uint32_t& phase, int tid) {
+  if (tid < 32) {
+    if (!mbar_wait(&sm.mbar, phase)) sm.timed_out = 1;
+    __syncwarp();
+  }
+  phase ^= 1;
+  __syncthreads();
+  tc_fence_after();
+  return sm.timed_out == 0;
+}
+
 // K-major, 128-byte swizzle: rows of 128 B, 8-row groups 1024 B apart; version 1 (sm_100).
 __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
   uint64_t d = 0;
@@ -175,6 +195,13 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, ui
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
       ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
 }
+// the same with A in tensor memory: lane = row, a 32-bit column holds two consecutive elements of the contraction
+__device__ __forceinline__ void umma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void umma_commit(unsigned long long* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -185,6 +212,11 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_st8_issue(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
 // 32 consecutive columns of this thread's TMEM lane -> shared memory dst[col * stride]
 __device__ __forceinline__ void tmem_cols32_to_smem(uint32_t taddr, float* dst, int stride) {
@@ -247,7 +279,7 @@ __device__ __forceinline__ void direct_tail(const Shape& s, const LayerPtrs& L, 
   float* Wm = Am + NT * 16;
   float* Mm = Wm + NT * 16;
   static_assert(LY::kRec + NT * 16 * 4 * 3 <= LY::kV, "coefficient tables overflow the record area");
-  float* Pq = reinterpret_cast<float*>(smem);                   // S0 q products [node][row], in the place of the dump
+  float* Pq = reinterpret_cast<float*>(smem + LY::kDump);       // S0 q products [node][row], in the place of the dump
   float* Rh = reinterpret_cast<float*>(smem + LY::kKQ);         // right-hand sides [node][row], in the place of K and Q
   // ---- A and W along each node's ancestry: sixteen lanes per node (lane j = path entry j); G(t, a_j)
   //      is a suffix product of the alphas over the lanes ----------------------------------------------
@@ -364,8 +396,9 @@ __device__ __forceinline__ void direct_tail(const Shape& s, const LayerPtrs& L, 
 // M = W (I + A)^-1 per node along its own root path); the sum o_t = g_t |q scale| S0 q_t + sum_s M[t][s] rhs_s
 // is then ONE product over all nodes of the group, O[row][t] = sum_s RHS[row][s] M[t][s] (M is zero off the
 // path), with both operands split into bf16 hi + lo (three products: hi.hi + hi.lo + lo.hi, relative error
-// 2^-16).  RHS [128 rows x NT nodes] and M [NT x NT] are K-major tiles with the 128-byte swizzle (a row of 64
-// nodes is one swizzle row; with NT = 32 the hi and lo halves share a row).  The result lands in the tensor-
+// 2^-16).  RHS [128 rows x NT nodes] goes from registers to tensor memory (a thread has a value row's nodes side by
+// side: no shared-memory store, no operand read there); M [NT x NT] is a K-major tile with the 128-byte swizzle (a row
+// of 64 nodes is one swizzle row; with NT = 32 the hi and lo halves share a row).  The result lands in the tensor-
 // memory columns of the Gram block and leaves lane = value row together with the query products.
 // A dense product would let a non-finite right-hand side of ANY node reach every output of the group (0 x NaN),
 // where the recurrence confines it to the node's subtree.  So a right-hand side that is not finite (or overflows
@@ -381,12 +414,12 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
   float* Am = reinterpret_cast<float*>(smem + LY::kRec);        // [node][16], in the place of the records
   float* Wm = Am + NT * 16;
   static_assert(LY::kRec + NT * 16 * 4 * 2 <= LY::kV, "coefficient tables overflow the record area");
-  constexpr int kRt = kCompact ? LY::kKQ : 0;                   // RHS tiles: over the dead Gram dump, or (compact) over K and Q
-  constexpr int kMt = kCompact ? LY::kKQ + 16384 : LY::kKQ;     // M tiles: over the dead K and Q rows
-  constexpr int kRtTerm = NT == 64 ? 16384 : 64;                // byte distance from the hi to the lo operand
-  constexpr int kMtTerm = NT == 64 ? 8192 : 64;
+  constexpr int kStage = kCompact ? LY::kKQ : 0;                // staged outputs: over the dead Gram dump, or (compact) over K and Q
+  constexpr int kRhsCol = LY::kGramCol + NT;                    // right-hand sides in tensor memory: NT / 2 columns hi, NT / 2 lo
+  static_assert(kRhsCol + NT <= LY::kTmem, "right-hand sides overflow the tensor-memory columns");
+  constexpr int kMt = LY::kMt;                                  // M tiles
+  constexpr int kMtTerm = NT == 64 ? 8192 : 64;                 // byte distance from the hi to the lo operand
   constexpr int kMtBytes = NT == 64 ? 16384 : 4096;
-  static_assert(kCompact || (NT == 64 ? 32768 : 16384) <= LY::kRec, "right-hand-side tiles overflow the dump area");
   // byte offset of element (row, col) of operand term 0 (hi) or 1 (lo): with NT = 64 the lo operand is a tile of
   // its own `term_bytes` on, with NT = 32 it is the upper half (k bytes 64..127) of the same swizzled rows
   auto tile_off = [](int row, int col, int term, int term_bytes) {
@@ -464,8 +497,8 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
       }
     }
   }
-  // ---- right-hand sides: lane = value row, each half of the CTA half of the nodes, eight nodes per 16-byte
-  //      store; padding nodes are written as zeros (their V bytes are stale) ----------------------------------
+  // ---- right-hand sides: lane = value row, each half of the CTA half of the nodes; they stay in
+  //      tensor memory as the A operand of the product; padding nodes are zeros (their V bytes are stale) ----------------------------------
   {
     constexpr int kPer = NT / 2;                                    // nodes per thread
     const int n0 = grp * kPer;
@@ -473,15 +506,17 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
     tmem_ld16_issue(tmem_lane + n0, pk);
     if constexpr (kPer == 32) tmem_ld16_issue(tmem_lane + n0 + 16, pk + 16);
     tmem_ld_wait();
+    uint32_t hi8[8], lo8[8];                                        // sixteen nodes = one contraction step
 #pragma unroll
     for (int c = 0; c < kPer / 8; ++c) {
       const int s0 = n0 + 8 * c;
+      uint32_t* hi = hi8 + 4 * (c & 1);
+      uint32_t* lo = lo8 + 4 * (c & 1);
       const float4 b0 = *reinterpret_cast<const float4*>(&sm.beta[s0]), b1 = *reinterpret_cast<const float4*>(&sm.beta[s0 + 4]);
       const float4 c0 = *reinterpret_cast<const float4*>(&sm.ks[s0]), c1 = *reinterpret_cast<const float4*>(&sm.ks[s0 + 4]);
       const float bt[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
       const float ck[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
       float r8[8];
-      uint32_t hi[4], lo[4];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int sn = s0 + e;
@@ -512,34 +547,36 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
         __nv_bfloat162 l = __floats2bfloat162_rn(r8[2 * e] - hf.x, r8[2 * e + 1] - hf.y);
         lo[e] = *reinterpret_cast<uint32_t*>(&l);
       }
-      *reinterpret_cast<uint4*>(smem + kRt + tile_off(vrow, s0, 0, kRtTerm)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-      *reinterpret_cast<uint4*>(smem + kRt + tile_off(vrow, s0, 1, kRtTerm)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      if (c & 1) {
+        __syncwarp();                                               // behind the rare branch above
+        tmem_st8_issue(tmem_lane + kRhsCol + (s0 - 8) / 2, hi8);
+        tmem_st8_issue(tmem_lane + kRhsCol + NT / 2 + (s0 - 8) / 2, lo8);
+      }
     }
+    tmem_st_wait();
   }
+  tc_fence_before();
   fence_async_proxy();          // generic-proxy writes -> visible to the tensor core's async proxy
   __syncthreads();
   // ---- O = RHS M^T: hi.hi + hi.lo + lo.hi, NT / 16 contraction steps each ----------------------------------
   if (tid == 0) {
     tc_fence_after();
     constexpr uint32_t idesc = umma_idesc(128, NT);
-    const uint64_t d_r = umma_desc(sbase + kRt), d_m = umma_desc(sbase + kMt);
-    constexpr uint64_t r_lo = (uint64_t)(kRtTerm >> 4), m_lo = (uint64_t)(kMtTerm >> 4);
+    const uint64_t d_m = umma_desc(sbase + kMt);
+    constexpr uint64_t m_lo = (uint64_t)(kMtTerm >> 4);
 #pragma unroll
     for (int ks = 0; ks < NT / 16; ++ks) {
       const uint64_t koff = (uint64_t)((ks * 32) >> 4);
-      umma(tmem + LY::kGramCol, d_r + koff, d_m + koff, idesc, ks ? 1u : 0u);
-      umma(tmem + LY::kGramCol, d_r + koff, d_m + m_lo + koff, idesc, 1u);
-      umma(tmem + LY::kGramCol, d_r + r_lo + koff, d_m + koff, idesc, 1u);
+      umma_ta(tmem + LY::kGramCol, tmem + kRhsCol + 8 * ks, d_m + koff, idesc, ks ? 1u : 0u);
+      umma_ta(tmem + LY::kGramCol, tmem + kRhsCol + 8 * ks, d_m + m_lo + koff, idesc, 1u);
+      umma_ta(tmem + LY::kGramCol, tmem + kRhsCol + NT / 2 + 8 * ks, d_m + koff, idesc, 1u);
     }
     umma_commit(&sm.mbar);
   }
-  const bool done = mbar_wait(&sm.mbar, phase);
-  phase ^= 1;
-  tc_fence_after();
-  if (!done) return false;
+  if (!wait_products(sm, phase, tid)) return false;
   // ---- outputs: they leave tensor memory lane = value row, cross shared memory [node][row] (over the dead
   //      right-hand-side tiles) and are written one node per warp, 256 or 512 contiguous bytes at a time -----------
-  float* stage = reinterpret_cast<float*>(smem + kRt);
+  float* stage = reinterpret_cast<float*>(smem + kStage);
   static_assert(kCompact || NT * kD * 4 <= LY::kRec, "output staging overflows the dump area");
   {
     constexpr int kPer = NT / 2;
@@ -607,8 +644,8 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
   static_assert(!kCompact || (NT == 32 && !kFused), "the compact layout serves the 32-node tile of the plain scan");
   using LY = GL<kCompact>;
   Small& sm = *reinterpret_cast<Small*>(smem + LY::kSmall);
-  float* dump = reinterpret_cast<float*>(smem + kOffDump);
-  float* dls = reinterpret_cast<float*>(smem + kOffDump);     // [nodes + 1][128]; the last row stays zero
+  float* dump = reinterpret_cast<float*>(smem + LY::kDump);
+  float* dls = reinterpret_cast<float*>(smem + LY::kDump);     // [nodes + 1][128]; the last row stays zero
   float* Pq = reinterpret_cast<float*>(smem + LY::kKQ);
   NodeRec* recs = reinterpret_cast<NodeRec*>(smem + LY::kRec);
   const __nv_bfloat16* Vs = reinterpret_cast<const __nv_bfloat16*>(smem + LY::kV);
@@ -616,7 +653,17 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = tid >> 7;            // half of the CTA: 0 or 1
   const int vrow = tid & 127;          // value row = TMEM lane
+  // Item -> (value head, node group, layer): divided out once, then stepped by the grid's own (head, group, layer);
+  // the divisions of every item and warp were a tenth of the kernel's instructions.
   const int rep = s.Hv / s.Hk;
+  const uint32_t rep_mul = 0xFFFFFFFFu / (uint32_t)rep + 1u;       // hv / rep = high word of hv * rep_mul (0 for rep = 1)
+  int hv = (int)blockIdx.x % s.Hv, gi = (int)blockIdx.x / s.Hv % t.n_groups, layer = (int)blockIdx.x / s.Hv / t.n_groups;
+  int n_hv = 0, n_gi = 0, n_layer = 0, step_hv = 0, step_gi = 0, step_layer = 0;
+  if (n_items > (int)gridDim.x) {
+    step_hv = (int)gridDim.x % s.Hv;
+    step_gi = (int)gridDim.x / s.Hv % t.n_groups;
+    step_layer = (int)gridDim.x / s.Hv / t.n_groups;
+  }
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&sm.tmem_base)), "r"(LY::kTmem) : "memory");
@@ -634,10 +681,12 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
   const int srow0 = 2 * warp + (lane >> 4), c4 = lane & 15;
   const uint32_t s0_off0 = sw128_offset(srow0, c4 >> 1) + (c4 & 1) * 8;   // rows 16 u on: + 2048 u
 
-  for (int item = blockIdx.x; item < n_items; item += gridDim.x) {   // bounded: n_items
-    const int hv = item % s.Hv;
-    const int gi = (item / s.Hv) % t.n_groups;                     // node group
-    const int layer = item / (s.Hv * t.n_groups);
+  for (int item = blockIdx.x; item < n_items; item += gridDim.x, hv = n_hv, gi = n_gi, layer = n_layer) {   // bounded: n_items
+    n_hv = hv + step_hv;
+    n_gi = gi + step_gi;
+    n_layer = layer + step_layer;
+    if (n_hv >= s.Hv) { n_hv -= s.Hv; ++n_gi; }
+    if (n_gi >= t.n_groups) { n_gi -= t.n_groups; ++n_layer; }
     // A tree of one group (every tree when there are as many groups as sequences) needs no look-up: group =
     // sequence, all nodes, first group.  That takes one dependent load off the head of the item's chain
     // (group -> state row -> state).
@@ -647,7 +696,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
     const int b = ginfo.x, N = ginfo.y;                            // sequence, nodes in this group
     const bool first_group = ginfo.z != 0;                         // writes the per-sequence zero rows
     const LayerPtrs& L = lb.l[layer];
-    const int g = hv / rep;
+    const int g = rep == 1 ? hv : (int)__umulhi((uint32_t)hv, rep_mul);
     const int row = L.state_row[b];
     const size_t out_row_stride = (size_t)s.Hv * kD;
     // The item this CTA takes next: its state and operand rows are pulled into L2 while this item
@@ -655,11 +704,8 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
     const int nxt = item + (int)gridDim.x;
     // (trees cut into several groups re-read one state per group from L2 anyway: there it measured slower)
     const bool has_next = !kFused && nxt < n_items && t.n_groups == s.B;
-    int n_hv = 0, n_layer = 0, n_b = 0, n_meta = -1, n_row = -1;
+    int n_b = 0, n_meta = -1, n_row = -1;
     if (has_next) {
-      n_hv = nxt % s.Hv;
-      const int n_gi = (nxt / s.Hv) % t.n_groups;
-      n_layer = nxt / (s.Hv * t.n_groups);
       const int4 gi4 = one_group ? make_int4(n_gi, s.N, 1, 0) : *reinterpret_cast<const int4*>(t.tc_group + n_gi * 4);
       n_b = gi4.x;
       if (tid < gi4.y) n_meta = t.tc_meta[n_gi * kNT + tid];
@@ -764,7 +810,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       if (n_meta >= 0) {      // a node's key, query and value rows (256 bytes = two lines each) and its gates
         const LayerPtrs& NL = lb.l[n_layer];
         const size_t pr = (size_t)n_b * s.Ns + (n_meta & 0xFFFF);
-        const int n_g = n_hv / rep;
+        const int n_g = rep == 1 ? n_hv : (int)__umulhi((uint32_t)n_hv, rep_mul);
         const __nv_bfloat16* pk = reinterpret_cast<const __nv_bfloat16*>(NL.k) + (pr * s.Hk + n_g) * kD;
         const __nv_bfloat16* pq = reinterpret_cast<const __nv_bfloat16*>(NL.q) + (pr * s.Hk + n_g) * kD;
         const __nv_bfloat16* pv = reinterpret_cast<const __nv_bfloat16*>(NL.v) + (pr * s.Hv + n_hv) * kD;
@@ -829,7 +875,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       for (int i = 0; i < kCopies; ++i) {
         const int idx = i * kThreads + tid;
         const int R = idx >> 4, c = idx & 15;
-        const uint32_t dst = sbase + LY::kKQ + (c >> 3) * 16384 + sw128_offset(R, c & 7);
+        const uint32_t dst = sbase + LY::kKQ + (c >> 3) * LY::kKBlock + sw128_offset(R, c & 7);
         if (src[i]) cp_async16(dst, src[i]);
         else asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};\n" ::"r"(dst), "r"(0u) : "memory");
       }
@@ -923,7 +969,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       const uint64_t d_kq = umma_desc(sbase + LY::kKQ), d_hi = umma_desc(sbase + LY::kAhi), d_lo = umma_desc(sbase + LY::kAlo);
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
-        const uint64_t koff = (uint64_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4);
+        const uint64_t koff = (uint64_t)(((ks >> 2) * LY::kKBlock + (ks & 3) * 32) >> 4);
         umma(tmem + LY::kGramCol, d_kq + koff, d_kq + koff, idesc_g, ks ? 1u : 0u);
       }
       if constexpr (kCompact) {
@@ -952,7 +998,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       float qq = 0.f;
 #pragma unroll
       for (int c = 0; c < 16; ++c) {
-        const uint4 w = *reinterpret_cast<const uint4*>(smem + LY::kKQ + (c >> 3) * 16384 + sw128_offset(R, c & 7));
+        const uint4 w = *reinterpret_cast<const uint4*>(smem + LY::kKQ + (c >> 3) * LY::kKBlock + sw128_offset(R, c & 7));
         const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -963,11 +1009,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       sm.qq[vrow] = qq;
     }
     // ---- f. wait for the tensor core (bounded) ---------------------------------------------------
-    if (!mbar_wait(&sm.mbar, phase)) sm.timed_out = 1;
-    phase ^= 1;
-    tc_fence_after();
-    __syncthreads();
-    if (sm.timed_out) {    // give up on this and all further items; report, free TMEM, leave
+    if (!wait_products(sm, phase, tid)) {    // give up on this and all further items; report, free TMEM, leave
       if (L.status && tid == 0) L.status[b] = LUMO_SEQ_TIMEOUT;
       break;
     }
@@ -980,7 +1022,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       if (tid == 0) {
         tc_fence_after();
         constexpr uint32_t idesc_p = umma_idesc(128, 2 * NT);
-        const uint64_t d_kq = umma_desc(sbase + LY::kKQ + 16384), d_hi = umma_desc(sbase + LY::kAhi), d_lo = umma_desc(sbase + LY::kAlo);
+        const uint64_t d_kq = umma_desc(sbase + LY::kKQ + LY::kKBlock), d_hi = umma_desc(sbase + LY::kAhi), d_lo = umma_desc(sbase + LY::kAlo);
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
           const uint64_t koff = (uint64_t)((ks * 32) >> 4);
@@ -989,11 +1031,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
         }
         umma_commit(&sm.mbar);
       }
-      if (!mbar_wait(&sm.mbar, phase)) sm.timed_out = 1;
-      phase ^= 1;
-      tc_fence_after();
-      __syncthreads();
-      if (sm.timed_out) {
+      if (!wait_products(sm, phase, tid)) {
         if (L.status && tid == 0) L.status[b] = LUMO_SEQ_TIMEOUT;
         break;
       }
@@ -1179,9 +1217,9 @@ scan_gram_kernel(Shape s, TreeDev t, LB lb, int n_items) {
   scan_gram_body<NT, false, false, kDirect, kTensor, LB>(s, t, lb, n_items, nullptr);
 }
 
-// trees of at most 32 nodes, launches of several waves: three smaller CTAs per SM
+// trees of at most 32 nodes, launches of several waves: four (three) smaller CTAs per SM
 template <bool kDirect, bool kTensor, class LB>
-__global__ void __launch_bounds__(kThreads, 3)
+__global__ void __launch_bounds__(kThreads, kTensor ? 4 : 3)
 scan_gram_compact_kernel(Shape s, TreeDev t, LB lb, int n_items) {
   scan_gram_body<32, false, true, kDirect, kTensor, LB>(s, t, lb, n_items, nullptr);
 }
@@ -1231,13 +1269,14 @@ static cudaError_t launch_scan_gram_t(const Shape& s, const TreeDev& t, const LB
   }
   // two CTAs per SM by construction: 102 KB of shared memory, 128 registers x 256 threads and 256
   // of the 512 tensor-memory columns each
-  // Compact CTAs (68 KB, 80 registers, 128 tensor-memory columns: three per SM) pay one more tensor-core
+  // Compact CTAs (52 KB, 64 registers, 128 tensor-memory columns: four per SM) pay one more tensor-core
   // round trip per item: they win when a launch has several waves of items (the 48-layer stack: 205 ->
-  // 190 us) and lose on a single wave (batch 1: 9.3 -> 10.5 us).
+  // 182 us; 3072 items of 7-node trees with raw gates: 89.8 us with three per SM, 86.5 with four) and lose
+  // on a single wave (batch 1: 9.3 -> 10.5 us).
   if (t.max_group_nodes <= 32 && items >= 4 * sm_count) {
     auto k = tail == 2 ? scan_gram_compact_kernel<true, true, LB>
                        : direct ? scan_gram_compact_kernel<true, false, LB> : scan_gram_compact_kernel<false, false, LB>;
-    return launch_kernel(k, dim3(3 * sm_count), dim3(kThreads), GL<true>::kBytes, st, pdl, s, t, lb, items);
+    return launch_kernel(k, dim3((tail == 2 ? 4 : 3) * sm_count), dim3(kThreads), GL<true>::kBytes, st, pdl, s, t, lb, items);
   }
   const int grid = items < 2 * sm_count ? items : 2 * sm_count;
   auto k = t.max_group_nodes <= 32 ? (direct ? scan_gram_kernel<32, true, false, LB> : scan_gram_kernel<32, false, false, LB>)
