@@ -982,10 +982,10 @@ commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
   }
 
   // ---- state rows ---------------------------------------------------------------------------------
-  extern __shared__ __align__(128) unsigned char smem[];
-  float* Ss = reinterpret_cast<float*>(smem);                              // [ROWS][D]
-  float* Ks = reinterpret_cast<float*>(smem + Cfg::kStateBytes);           // [chunk][D], widened
-  T* Vs = reinterpret_cast<T*>(smem + Cfg::kStateBytes + kCommitChunk * D * 4);   // [chunk][ROWS]
+  extern __shared__ __align__(128) unsigned char commit_smem[];
+  float* Ss = reinterpret_cast<float*>(commit_smem);                              // [ROWS][D]
+  float* Ks = reinterpret_cast<float*>(commit_smem + Cfg::kStateBytes);           // [chunk][D], widened
+  T* Vs = reinterpret_cast<T*>(commit_smem + Cfg::kStateBytes + kCommitChunk * D * 4);   // [chunk][ROWS]
   __shared__ float2 s_gate[kCommitChunk];
   __shared__ unsigned long long mbar;
   const int tile = blockIdx.x % kTiles, hv = blockIdx.x / kTiles;

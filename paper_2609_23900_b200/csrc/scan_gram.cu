@@ -71,8 +71,6 @@ constexpr int kOffDump = 0;                         // Gram [128][65] fp32; late
 constexpr int kOffRec = 34816;                      // NodeRec[64]
 static_assert(128 * kDumpStride * 4 <= kOffRec, "Gram dump overflows its area");
 constexpr int kOffV = kOffRec + kNT * (int)sizeof(NodeRec);   // 49152: V [64][128] bf16
-constexpr int kOffPq = kOffKQ;                      // S0 q^ products [64][128] fp32
-constexpr int kZeroRow = kNT * kD;                  // element offset of the all-zero delta row
 static_assert((kNT + 1) * kD * 4 <= kOffRec, "delta array overflows the dump area");
 static_assert(kOffV + kNT * kD * 2 <= kOffKQ, "aliased region overflows the S0 tiles");
 
@@ -228,6 +226,14 @@ __device__ __forceinline__ void tmem_cols32_to_smem(uint32_t taddr, float* dst, 
   for (int e = 0; e < 16; ++e) dst[e * stride] = __uint_as_float(r0[e]);
 #pragma unroll
   for (int e = 0; e < 16; ++e) dst[(16 + e) * stride] = __uint_as_float(r1[e]);
+}
+
+__device__ __forceinline__ void tmem_cols16_to_smem(uint32_t taddr, float* dst, int stride) {
+  uint32_t r[16];
+  tmem_ld16_issue(taddr, r);
+  tmem_ld_wait();
+#pragma unroll
+  for (int e = 0; e < 16; ++e) dst[e * stride] = __uint_as_float(r[e]);
 }
 
 __device__ __forceinline__ uint32_t sw128_offset(int row, int chunk16) {   // within one [rows x 128 B] k-block
@@ -1050,8 +1056,10 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
       }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
-    // both halves of the CTA read the Gram rows: 32 of the NT columns each (one half is enough for NT = 32)
-    if (grp * 32 < NT) tmem_cols32_to_smem(tmem_lane + LY::kGramCol + grp * 32, dump + vrow * LY::kStride + grp * 32, 1);
+    // both halves of the CTA read the Gram rows: 32 of the 64 columns each
+    // with NT = 32 only the first 64 of the product's 128 rows are in use: sixteen columns for each half's two warps
+    if constexpr (NT == 64) tmem_cols32_to_smem(tmem_lane + LY::kGramCol + grp * 32, dump + vrow * LY::kStride + grp * 32, 1);
+    else if (vrow < 64) tmem_cols16_to_smem(tmem_lane + LY::kGramCol + grp * 16, dump + vrow * LY::kStride + grp * 16, 1);
     __syncthreads();
     if constexpr (kDirect && kTensor) {
       if (!direct_tail_tc<NT, LY, kCompact>(s, L, sm, smem, sbase, dump, Vs, tmem, tmem_lane, N, b, hv, tid, phase)) sm.timed_out = 1;
