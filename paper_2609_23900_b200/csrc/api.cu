@@ -121,11 +121,16 @@ cudaError_t timed(lumo_ctx* ctx, int kind, cudaStream_t st, F launch) {
   return e;
 }
 
-// Overlapping a kernel with its predecessor pays when both are a single wave of CTAs (the set-up and
-// dependent-load chains hide under the predecessor's tail); with many waves it measured slower (the
-// early CTAs only take slots from the predecessor), so it is limited to small launches.
-bool use_overlap(const lumo_ctx* ctx, const Shape& s) {
-  return ctx->overlap && (long long)s.n_layers * s.B * s.Hv <= 4LL * ctx->sm_count;
+// Overlapping a kernel with its predecessor hides the set-up and the dependent-load chains under the predecessor's tail: a
+// kernel lets the next one in when all its CTAs have started, so the early CTAs take only slots that have become free.
+// `any_size`: a convolution before a tensor-core scan, which waits before it reads anything, and that scan behind it, whose
+// early reads (state, tables, path) were complete before the convolution passed its own wait; a commit that waits first.
+// Those pay at every size (48 layers of 28 nodes, fused: 115.1 -> 112.5 us; 4 x 5 layers of 40 nodes: 67.6 -> 64.4; the others
+// of 40 drawn sizes 0 to 3 %).  Limited to small launches: a commit and a scan without a convolution that read the caller's
+// data ahead of their wait, and the rank-1 scan, which deals its work out to the CTAs that fit at launch: entering one by one
+// they end up unevenly spread (8 layers with cached states: 435 -> 567 us).
+bool use_overlap(const lumo_ctx* ctx, const Shape& s, bool any_size = false) {
+  return ctx->overlap && (any_size || (long long)s.n_layers * s.B * s.Hv <= 4LL * ctx->sm_count);
 }
 
 TreeDev tree_view(const lumo_tree_desc* d, int which) {
@@ -541,12 +546,12 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
   if (gram_ok && ctx->scan_algo != 1) {
     cudaError_t e = cudaSuccess;
     if (layers[0].x) {
-      e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, ctx->sm_count, use_overlap(ctx, s), st); });
+      e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, ctx->sm_count, use_overlap(ctx, s, true), st); });
       if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
     }
     const bool state_fresh = !layers[0].x && (prev_call == lumo_ctx::kCommit || prev_call == lumo_ctx::kCommitVerify);
     e = timed(ctx, LUMO_K_SCAN, st, [&] {
-      const bool pdl = use_overlap(ctx, s) && !state_fresh;
+      const bool pdl = use_overlap(ctx, s, layers[0].x != nullptr) && !state_fresh;
       return ctx->scan_algo == 3 ? launch_scan_solve(s, t, lb, ctx->sm_count, pdl, st)
                                  : launch_scan_gram(s, t, lb, ctx->sm_count, pdl, scan_tail(ctx, desc, s), st);
     });
@@ -625,9 +630,10 @@ int lumo_gdn_commit(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_ar
   DeviceGuard g(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
   const TreeDev t = tree_view(desc, 0);
-  // the commit reads the path, the operands and the state ahead of its dependency wait: overlap only
-  // right behind a verify call (see commit_kernel)
-  const bool pdl = use_overlap(ctx, s) && ctx->last_call == lumo_ctx::kVerify;
+  // in a small launch right behind a verify call the commit reads the path, the operands and the state ahead of its
+  // dependency wait (see commit_kernel)
+  s.wait_first = !(use_overlap(ctx, s) && ctx->last_call == lumo_ctx::kVerify);
+  const bool pdl = use_overlap(ctx, s, true);
   ctx->last_call = lumo_ctx::kCommit;
   cudaError_t e = timed(ctx, LUMO_K_COMMIT, st, [&] {
     return launch_commit(s, t, lb, accepted_dev, len_dev, lmax, true, layers[0].x != nullptr, ctx->sm_count, pdl, st);
@@ -673,9 +679,9 @@ int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const
   // The convolution waits on its predecessor before it reads anything, so it may always overlap, and
   // so may a scan launched behind it.  A fused scan (or the history launch) directly behind another
   // call reads the path and the state ahead of its dependency wait: overlap then only behind a verify.
-  const bool pdl_conv = use_overlap(ctx, s);
-  const bool pdl = pdl_conv && ctx->last_call == lumo_ctx::kVerify;
-  const bool pdl_scan = pdl_conv && (layers[0].x != nullptr || ctx->last_call == lumo_ctx::kVerify);
+  const bool pdl_conv = use_overlap(ctx, s, true);
+  const bool pdl = use_overlap(ctx, s) && ctx->last_call == lumo_ctx::kVerify;
+  const bool pdl_scan = layers[0].x != nullptr ? pdl_conv : pdl;
   ctx->last_call = lumo_ctx::kCommitVerify;
   const TreeDev pt = tree_view(prev_desc, 0);
   const TreeDev t = tree_view(desc, 0);

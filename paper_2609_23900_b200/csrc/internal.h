@@ -150,6 +150,7 @@ struct Shape {
   int n_layers;
   int gate_mode;
   int debug_skip_mma;   // test aid of the tensor-core scan: issue no tensor-core work, let the bounded wait run out
+  int wait_first;         // commit: read nothing ahead of the dependency wait
 };
 
 // What the fused commit + verify scan needs of the previous cycle: its layers (recorded k, v, gates,

@@ -933,14 +933,15 @@ commit_kernel(Shape s, TreeDev t, LB lb, const int32_t* __restrict__ accepted,
   const int b = blockIdx.y, layer = blockIdx.z;
   const LayerPtrs& L = lb.l[layer];
   const int tid = threadIdx.x;
+  if (s.wait_first) pdl_wait();
   const int row = L.state_row[b];
   const int len = len_arr[b];
   const bool lead = blockIdx.x == 0 && tid == 0;
   // What this kernel WRITES (state, history, status) may still be read by its predecessor (the scan
   // reads the pre-tree state), so every write sits behind pdl_wait().  What it READS ahead of that wait
-  // (state tile, path, operands) must be older than its predecessor: the host launches it with the
-  // overlap attribute only right after a verify call, whose own dependency wait orders everything
-  // before it; after any other call of the library it is launched in plain stream order.
+  // (state tile, path, operands) must be older than its predecessor: that is so for a small launch right after a
+  // verify call, whose own dependency wait orders everything before it.  Otherwise (wait_first) it reads nothing
+  // ahead either, and the overlap hides its launch alone.
   if (row < 0) { pdl_wait(); if (lead && L.status) L.status[b] = LUMO_SEQ_OK; return; }
   if (row >= s.n_state_rows) { pdl_wait(); if (lead && L.status) L.status[b] = LUMO_SEQ_BAD_ROW; return; }
   const int32_t* acc = accepted + (size_t)b * lmax;
