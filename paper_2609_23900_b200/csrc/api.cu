@@ -128,7 +128,7 @@ cudaError_t timed(lumo_ctx* ctx, int kind, cudaStream_t st, F launch) {
 // Those pay at every size (48 layers of 28 nodes, fused: 115.1 -> 112.5 us; 4 x 5 layers of 40 nodes: 67.6 -> 64.4; the others
 // of 40 drawn sizes 0 to 3 %).  Limited to small launches: a commit and a scan without a convolution that read the caller's
 // data ahead of their wait, and the rank-1 scan, which deals its work out to the CTAs that fit at launch: entering one by one
-// they end up unevenly spread (8 layers with cached states: 435 -> 567 us).
+// they end up unevenly spread (8 layers with cached states: 435 -> 567 us; see launch_scan).
 bool use_overlap(const lumo_ctx* ctx, const Shape& s, bool any_size = false) {
   return ctx->overlap && (any_size || (long long)s.n_layers * s.B * s.Hv <= 4LL * ctx->sm_count);
 }
@@ -579,7 +579,7 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
     if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
   }
   e = timed(ctx, LUMO_K_SCAN, st, [&] {
-    return launch_scan(s, t, lb, reinterpret_cast<float*>(ctx->scratch), grid, use_overlap(ctx, s), st);
+    return launch_scan(s, t, lb, reinterpret_cast<float*>(ctx->scratch), grid, ctx->sm_count, use_overlap(ctx, s), st);
   });
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "scan launch");
 }
@@ -612,7 +612,7 @@ int lumo_gdn_tree_scan_static(lumo_ctx* ctx, const lumo_tree_desc* desc, const l
   float* stack = nullptr;
   e = static_stack_address(ctx->device, &stack);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGetSymbolAddress(built-in scan stack)");
-  e = timed(ctx, LUMO_K_SCAN, st, [&] { return launch_scan(s, t, lb, stack, grid, false, st); });
+  e = timed(ctx, LUMO_K_SCAN, st, [&] { return launch_scan(s, t, lb, stack, grid, ctx->sm_count, false, st); });
   ctx->last_call = lumo_ctx::kVerify;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "scan launch");
 }

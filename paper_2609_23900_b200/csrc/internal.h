@@ -314,7 +314,7 @@ int conv_rows_per_cta(int C, int Ns, int seqs, int sms);
 cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, int sm_count,
                               bool pdl, cudaStream_t st);
 cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, float* stack,
-                        int grid, bool pdl, cudaStream_t st);
+                        int grid, int sm_count, bool pdl, cudaStream_t st);
 // Whether the rank-1 scan holds all of a tree's operands in shared memory (`t`: the lean schedule, which that kernel
 // interprets in every snapshot mode).
 bool scan_staged(const Shape& s, const TreeDev& t);

@@ -1273,7 +1273,7 @@ cudaError_t static_stack_address(int device, float** ptr) {
 }
 
 cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, float* stack,
-                        int grid, bool pdl, cudaStream_t st) {
+                        int grid, int sm_count, bool pdl, cudaStream_t st) {
   return dispatch(s.d, s.in_dtype, [&](auto dc, auto tc) {
     constexpr int D = decltype(dc)::value;
     using T = decltype(tc);
@@ -1281,6 +1281,10 @@ cudaError_t launch_scan(const Shape& s, const TreeDev& t, const LayerBatch& lb, 
     const bool few = s.n_layers <= kFewLayers;
     if (scan_staged(s, t)) {
       const int items = s.n_layers * s.B * s.Hv * (D / kStagedRows);
+      // Entering early, the CTAs crowd onto the SMs that the convolution leaves first.  That costs nothing while there is one
+      // for each SM at most (seven-node step: 11.0 -> 8.3 us), and more than the launch it hides beyond (2 x 2 layers of
+      // 27 nodes with cached states, 256 CTAs: convolution 9 us and scan 52 us alone, 72 us together).
+      pdl = pdl && items <= sm_count;
       const StagedSmem lay = staged_smem(s.N, D, t.max_ops, n_snap_list, t.max_levels);
       if (few)
         return launch_kernel(scan_staged_kernel<D, T, FewLayers>, dim3(grid), dim3(kStagedThreads), lay.total, st, pdl, s, t, few_layers(lb), stack, items);
