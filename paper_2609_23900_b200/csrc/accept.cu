@@ -221,8 +221,9 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int p
     if constexpr (kMode == 0) {
       float bv = -1.f;
       int bi = 0x7fffffff;
-      // the rows the walk may go on with
-      if (prefetch)
+      // The rows the walk may go on with, while they are few: one of many is mostly fetched for nothing, and asking for all
+      // of them delays the row at hand (26 children, V = 22,988: 11.0 us against 7.1).
+      if (prefetch && c_hi - c_lo <= 3)
         for (int ci = c_lo; ci < c_hi; ++ci) prefetch_row(target(slot_map[child_list[ci]]), n);
       auto look = [&](float v, int e) { if (v > bv) { bv = v; bi = v_lo + e; } };
       float4 w[kFlight];
