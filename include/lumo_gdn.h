@@ -140,12 +140,12 @@ int lumo_ctx_set_scan_algo(lumo_ctx* ctx, int algo);
  * undefined.  Default off. */
 int lumo_ctx_set_timeout_drill(lumo_ctx* ctx, int on);
 
-/* Kernel overlap (default on): conv, scan and commit are launched with programmatic dependent launch,
+/* Kernel overlap (default on): the kernels of every call are launched with programmatic dependent launch,
  * so each kernel's set-up (and, for commit, its whole read phase) runs under the tail of the kernel
  * before it; each waits on the device before touching data its predecessor produces or still reads.
  * A scan without convolution and the rank-1 scan are overlapped only in small launches (n_layers *
  * B * Hv <= 4 x SM count), and only there the commit reads ahead of its wait.
- * Results are identical either way; 0 restores plain stream order.
+ * Results are identical either way; 0 restores plain stream order for every kernel launched through this context.
  * The commit (and a scan without convolution) reads part of its input ahead of that wait: the
  * accepted path, the recorded operands, the state.  The library therefore does that only when the
  * previous call on this context was a verify; behind any other library call the commit waits first

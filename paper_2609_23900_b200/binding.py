@@ -191,7 +191,7 @@ class Context:
         self._check(_lib.lumo_ctx_set_timeout_drill(self._h, int(on)))
 
     def set_overlap(self, on: bool = True):
-        """Programmatic dependent launch between conv, scan and commit (default on)."""
+        """Programmatic dependent launch of the library's kernels (default on); off: plain stream order."""
         self._check(_lib.lumo_ctx_set_overlap(self._h, int(on)))
 
     def timing_enable(self, on: bool = True):

@@ -336,7 +336,7 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int p
 }  // namespace
 
 cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptView& a, int lmax, int32_t* accepted,
-                          int32_t* len, int32_t* next_token, int32_t* final_node, int sms, cudaStream_t st) {
+                          int32_t* len, int32_t* next_token, int32_t* final_node, int sms, bool pdl, cudaStream_t st) {
   static int cache[64] = {};
   int cluster = max_cluster_ctas(accept_kernel<1, true, double>, kAcceptThreads, cache);
   if (cluster > kAcceptCluster && B * cluster > sms) cluster = kAcceptCluster;   // many sequences: smaller clusters
@@ -368,7 +368,7 @@ cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptVi
     }
     size_t smem = 0;
     if constexpr (kMode == 1 && !std::is_void_v<RT>) smem = held * (sizeof(RT) + 4);
-    return launch_cluster_kernel(kern, dim3(cluster, B), dim3(kAcceptThreads), cluster, smem, st, t, N, Ns, a, lmax, chunk, prefetch, accepted,
+    return launch_cluster_kernel(kern, dim3(cluster, B), dim3(kAcceptThreads), cluster, smem, st, pdl, t, N, Ns, a, lmax, chunk, prefetch, accepted,
                                  len, next_token, final_node);
   };
   auto pick = [&](auto vec_c) {

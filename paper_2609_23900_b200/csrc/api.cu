@@ -463,7 +463,7 @@ int lumo_tree_path_from_node(lumo_ctx* ctx, const lumo_tree_desc* desc, const in
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = timed(ctx, LUMO_K_PATH, st, [&] {
     return launch_path_from_node(tree_view(desc, 0), desc->B, desc->N, node_dev, lmax, accepted_dev, len_dev,
-                                 status_dev, st);
+                                 status_dev, ctx->overlap, st);
   });
   ctx->last_call = lumo_ctx::kOther;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "path_from_node launch");
@@ -487,7 +487,7 @@ int lumo_tree_accept(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_accep
   v.V = a->V; v.mode = a->mode; v.token = a->token; v.p_target = a->p_target; v.q_draft = a->q_draft;
   v.uniforms = a->uniforms; v.noise = a->noise; v.work = a->work;
   cudaError_t e = launch_accept(tree_view(desc, 0), desc->B, desc->N, desc->Ns, v, lmax, accepted_dev, len_dev,
-                                next_token_dev, final_node_dev, ctx->sm_count, (cudaStream_t)stream);
+                                next_token_dev, final_node_dev, ctx->sm_count, ctx->overlap, (cudaStream_t)stream);
   ctx->last_call = lumo_ctx::kOther;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "accept launch");
 }
@@ -504,7 +504,7 @@ int lumo_select_spine_top3(lumo_ctx* ctx, const lumo_select_args* a, int32_t* sp
     return fail(ctx, LUMO_ERR_ARG, "split must be 0, 1, 2, 4, 8 or 16");
   DeviceGuard g(ctx->device);
   cudaError_t e = launch_select(a->logits, a->dtype, a->rows, a->V, sp, spine_dev, cand_dev, ctx->sm_count,
-                                (cudaStream_t)stream);
+                                ctx->overlap, (cudaStream_t)stream);
   ctx->last_call = lumo_ctx::kOther;
   if (e == cudaErrorInvalidConfiguration) {
     (void)cudaGetLastError();
@@ -781,7 +781,7 @@ int lumo_kv_write_tree(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_att
   KvLayers L;
   KvShape k;
   kv_views(desc, layers, n_layers, s, &L, &k);
-  cudaError_t e = timed(ctx, LUMO_K_KV_WRITE, st, [&] { return launch_kv_write(L, k, n_layers, st); });
+  cudaError_t e = timed(ctx, LUMO_K_KV_WRITE, st, [&] { return launch_kv_write(L, k, n_layers, ctx->overlap, st); });
   ctx->last_call = lumo_ctx::kOther;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "kv write launch");
 }
@@ -825,9 +825,9 @@ int lumo_tree_attention(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_at
     cudaError_t e = attn_plan(s, p, desc->d_vis, desc->d_slot_used, reinterpret_cast<float*>(ctx->attn_scratch),
                               ctx->sm_count, launch_id, &plan, &err);
     if (e != cudaSuccess) return err.empty() ? cuda_fail(ctx, e, "attention set-up") : fail(ctx, LUMO_ERR_CUDA, err);
-    e = timed(ctx, LUMO_K_ATTN, st, [&] { return launch_attn(plan, st); });
+    e = timed(ctx, LUMO_K_ATTN, st, [&] { return launch_attn(plan, ctx->overlap, st); });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention launch");
-    e = timed(ctx, LUMO_K_ATTN_MERGE, st, [&] { return launch_attn_merge(plan, st); });
+    e = timed(ctx, LUMO_K_ATTN_MERGE, st, [&] { return launch_attn_merge(plan, ctx->overlap, st); });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention merge launch");
   }
   return LUMO_OK;
@@ -848,7 +848,7 @@ int lumo_kv_publish(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_attn_a
   KvShape k;
   kv_views(desc, layers, n_layers, s, &L, &k);
   cudaError_t e = timed(ctx, LUMO_K_KV_PUBLISH, st, [&] {
-    return launch_kv_publish(L, k, n_layers, accepted_dev, len_dev, lmax, ctx_len_out, st);
+    return launch_kv_publish(L, k, n_layers, accepted_dev, len_dev, lmax, ctx_len_out, ctx->overlap, st);
   });
   ctx->last_call = lumo_ctx::kOther;
   return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "kv publish launch");

@@ -857,19 +857,19 @@ cudaError_t attn_plan(const AttnShape& s, const AttnLayerPtrs& p, const uint32_t
   return cudaSuccess;
 }
 
-cudaError_t launch_attn(const AttnPlan& plan, cudaStream_t st) {
-  return launch_kernel(tree_attn_kernel, plan.grid, dim3(kThreads), kSmemBytes, st, true, plan.tk, plan.tv, plan.a);
+cudaError_t launch_attn(const AttnPlan& plan, bool pdl, cudaStream_t st) {
+  return launch_kernel(tree_attn_kernel, plan.grid, dim3(kThreads), kSmemBytes, st, pdl, plan.tk, plan.tv, plan.a);
 }
 
-cudaError_t launch_attn_merge(const AttnPlan& plan, cudaStream_t st) {
+cudaError_t launch_attn_merge(const AttnPlan& plan, bool pdl, cudaStream_t st) {
   // one warp per (unit, 32 rows, group of four columns): 128 warps per unit, 16 CTAs
   const long long ctas = (long long)plan.a.B * plan.a.Hkv * plan.a.RT * 16;
   // dependent launch: the CTAs are staged while the attention kernel drains and wait on the device for its end
   const long long units = (long long)plan.a.B * plan.a.Hkv * plan.a.RT;
   const long long slots_per_unit = plan.a.S > 0 ? plan.a.S : ((long long)plan.grid.x + units - 1) / units + 1;
   if (slots_per_unit > 12)
-    return launch_kernel(attn_merge_kernel<24>, dim3((unsigned)ctas), dim3(256), 0, st, true, plan.a);
-  return launch_kernel(attn_merge_kernel<8>, dim3((unsigned)ctas), dim3(256), 0, st, true, plan.a);
+    return launch_kernel(attn_merge_kernel<24>, dim3((unsigned)ctas), dim3(256), 0, st, pdl, plan.a);
+  return launch_kernel(attn_merge_kernel<8>, dim3((unsigned)ctas), dim3(256), 0, st, pdl, plan.a);
 }
 
 }  // namespace lumo

@@ -56,7 +56,7 @@ struct lumo_ctx {
   // optional per-launch timing (lumo_ctx_timing_*): a fixed pool of event pairs
   int scan_algo = 0;            // 0 auto, 1 rank-1, 2 Gram form with forward substitution, 3 solved Gram form, 4 Gram form with closed-form tail, 5 the same with the output sum on the tensor core
   bool timeout_drill = false;   // test aid: the tensor-core scan skips its tensor-core work (lumo_ctx_set_timeout_drill)
-  bool overlap = true;          // programmatic dependent launch between conv -> scan -> commit
+  bool overlap = true;          // kernels are launched as programmatic dependents of the kernel before them
   // Kind of the previous call that launched on this context.  Kernels that read some of their inputs
   // ahead of their dependency wait (commit: path and state; scan without convolution: state) get the
   // overlap attribute only when the call before them cannot have written those inputs.
@@ -275,10 +275,10 @@ cudaError_t launch_by_address(const cudaLaunchConfig_t& cfg, void (*kern)(KArgs.
   return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(kern), p);
 }
 
-// Launch of a kernel whose CTAs form clusters of `cluster` along x, as a programmatic dependent of the kernel before
-// it: its CTAs are placed while that one drains and pass pdl_wait() before they touch global memory.
+// Launch of a kernel whose CTAs form clusters of `cluster` along x; with `pdl` as a programmatic dependent of the kernel
+// before it: its CTAs are placed while that one drains and pass pdl_wait() before they touch global memory.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st,
+cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st, bool pdl,
                                   const Args&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
@@ -288,7 +288,7 @@ cudaError_t launch_cluster_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block,
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = pdl ? 2 : 1;
   return launch_by_address<KArgs...>(cfg, kern, args...);
 }
 
@@ -327,10 +327,10 @@ struct AcceptView {
   float* work;
 };
 cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptView& a, int lmax, int32_t* accepted,
-                          int32_t* len, int32_t* next_token, int32_t* final_node, int sm_count, cudaStream_t st);
+                          int32_t* len, int32_t* next_token, int32_t* final_node, int sm_count, bool pdl, cudaStream_t st);
 // fused draft selection (select.cu)
 cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int split, int32_t* spine, int32_t* cand,
-                          int sm_count, cudaStream_t st);
+                          int sm_count, bool pdl, cudaStream_t st);
 // Gram-form scan on tcgen05 (scan_gram.cu)
 bool gram_supported(const Shape& s, int max_depth);
 // tail: 0 level-by-level substitution, 1 closed form (per-node back substitution, one output pass over the path),
@@ -351,7 +351,7 @@ cudaError_t launch_commit(const Shape& s, const TreeDev& t, const LayerBatch& lb
                           const int32_t* len, int lmax, bool with_state, bool with_hist, int sm_count, bool pdl,
                           cudaStream_t st);
 cudaError_t launch_path_from_node(const TreeDev& t, int B, int N, const int32_t* node, int lmax,
-                                  int32_t* accepted, int32_t* len, int32_t* status, cudaStream_t st);
+                                  int32_t* accepted, int32_t* len, int32_t* status, bool pdl, cudaStream_t st);
 
 // ---- attention half (attn.cu) ------------------------------------------------------------
 struct AttnShape {
@@ -408,10 +408,10 @@ int attn_row_tiles(int G, int N);
 size_t attn_scratch_bytes(const AttnShape& s, int sm_count);
 cudaError_t attn_plan(const AttnShape& s, const AttnLayerPtrs& p, const uint32_t* vis, const uint32_t* used, float* scratch,
                       int sm_count, uint32_t launch_id, AttnPlan* plan, std::string* err);
-cudaError_t launch_attn(const AttnPlan& plan, cudaStream_t st);
-cudaError_t launch_attn_merge(const AttnPlan& plan, cudaStream_t st);
-cudaError_t launch_kv_write(const KvLayers& L, const KvShape& s, int n_layers, cudaStream_t st);
+cudaError_t launch_attn(const AttnPlan& plan, bool pdl, cudaStream_t st);
+cudaError_t launch_attn_merge(const AttnPlan& plan, bool pdl, cudaStream_t st);
+cudaError_t launch_kv_write(const KvLayers& L, const KvShape& s, int n_layers, bool pdl, cudaStream_t st);
 cudaError_t launch_kv_publish(const KvLayers& L, const KvShape& s, int n_layers, const int32_t* accepted, const int32_t* len,
-                              int lmax, int32_t* ctx_len_out, cudaStream_t st);
+                              int lmax, int32_t* ctx_len_out, bool pdl, cudaStream_t st);
 
 }  // namespace lumo

@@ -1339,8 +1339,8 @@ cudaError_t launch_commit(const Shape& s, const TreeDev& t, const LayerBatch& lb
 }
 
 cudaError_t launch_path_from_node(const TreeDev& t, int B, int N, const int32_t* node, int lmax,
-                                  int32_t* accepted, int32_t* len, int32_t* status, cudaStream_t st) {
-  return launch_kernel(path_from_node_kernel, dim3((B + 63) / 64), dim3(64), 0, st, true, t, B, N, node, lmax, accepted, len, status);
+                                  int32_t* accepted, int32_t* len, int32_t* status, bool pdl, cudaStream_t st) {
+  return launch_kernel(path_from_node_kernel, dim3((B + 63) / 64), dim3(64), 0, st, pdl, t, B, N, node, lmax, accepted, len, status);
 }
 
 }  // namespace lumo

@@ -96,15 +96,15 @@ __global__ void __launch_bounds__(256) kv_publish_kernel(const KL L, const KvSha
 
 }  // namespace
 
-cudaError_t launch_kv_write(const KvLayers& L, const KvShape& s, int n_layers, cudaStream_t st) {
+cudaError_t launch_kv_write(const KvLayers& L, const KvShape& s, int n_layers, bool pdl, cudaStream_t st) {
   const dim3 grid(s.N, s.B, n_layers);
-  if (n_layers <= kFewLayers) return launch_kernel(kv_write_kernel<FewKvLayers>, grid, dim3(128), 0, st, true, few_layers(L), s);
-  return launch_kernel(kv_write_kernel<KvLayers>, grid, dim3(128), 0, st, true, L, s);
+  if (n_layers <= kFewLayers) return launch_kernel(kv_write_kernel<FewKvLayers>, grid, dim3(128), 0, st, pdl, few_layers(L), s);
+  return launch_kernel(kv_write_kernel<KvLayers>, grid, dim3(128), 0, st, pdl, L, s);
 }
 
 template <class KL>
 static cudaError_t launch_kv_publish_t(const KL& L, const KvShape& s, int n_layers, const int32_t* accepted, const int32_t* len,
-                                       int lmax, int32_t* ctx_len_out, cudaStream_t st) {
+                                       int lmax, int32_t* ctx_len_out, bool pdl, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -114,14 +114,14 @@ static cudaError_t launch_kv_publish_t(const KL& L, const KvShape& s, int n_laye
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  return launch_kernel(kv_publish_kernel<KL>, dim3(2 * s.Hkv, s.B, n_layers), dim3(256), (size_t)lmax * 256, st, true, L, s,
+  return launch_kernel(kv_publish_kernel<KL>, dim3(2 * s.Hkv, s.B, n_layers), dim3(256), (size_t)lmax * 256, st, pdl, L, s,
                        accepted, len, lmax, ctx_len_out);
 }
 
 cudaError_t launch_kv_publish(const KvLayers& L, const KvShape& s, int n_layers, const int32_t* accepted, const int32_t* len,
-                              int lmax, int32_t* ctx_len_out, cudaStream_t st) {
-  if (n_layers <= kFewLayers) return launch_kv_publish_t(few_layers(L), s, n_layers, accepted, len, lmax, ctx_len_out, st);
-  return launch_kv_publish_t(L, s, n_layers, accepted, len, lmax, ctx_len_out, st);
+                              int lmax, int32_t* ctx_len_out, bool pdl, cudaStream_t st) {
+  if (n_layers <= kFewLayers) return launch_kv_publish_t(few_layers(L), s, n_layers, accepted, len, lmax, ctx_len_out, pdl, st);
+  return launch_kv_publish_t(L, s, n_layers, accepted, len, lmax, ctx_len_out, pdl, st);
 }
 
 }  // namespace lumo

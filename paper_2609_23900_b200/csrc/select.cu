@@ -318,7 +318,7 @@ select_kernel(const T* __restrict__ logits, int V, int32_t* __restrict__ spine, 
 }  // namespace
 
 cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int split, int32_t* spine, int32_t* cand,
-                          int sms, cudaStream_t st) {
+                          int sms, bool pdl, cudaStream_t st) {
   static int cache_f[64] = {}, cache_h[64] = {};
   const int cap = dtype == LUMO_BF16 ? max_cluster_ctas(select_kernel<__nv_bfloat16>, kSelThreads, cache_h)
                                      : max_cluster_ctas(select_kernel<float>, kSelThreads, cache_f);
@@ -333,9 +333,9 @@ cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int sp
   }
   if (cluster > cap) return cudaErrorInvalidConfiguration;
   if (dtype == LUMO_BF16)
-    return launch_cluster_kernel(select_kernel<__nv_bfloat16>, dim3(cluster, rows), dim3(kSelThreads), cluster, 0, st,
+    return launch_cluster_kernel(select_kernel<__nv_bfloat16>, dim3(cluster, rows), dim3(kSelThreads), cluster, 0, st, pdl,
                                  reinterpret_cast<const __nv_bfloat16*>(logits), V, spine, cand);
-  return launch_cluster_kernel(select_kernel<float>, dim3(cluster, rows), dim3(kSelThreads), cluster, 0, st,
+  return launch_cluster_kernel(select_kernel<float>, dim3(cluster, rows), dim3(kSelThreads), cluster, 0, st, pdl,
                                reinterpret_cast<const float*>(logits), V, spine, cand);
 }
 
