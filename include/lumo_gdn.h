@@ -147,10 +147,12 @@ int lumo_ctx_set_timeout_drill(lumo_ctx* ctx, int on);
  * B * Hv <= 4 x SM count), and only there the commit reads ahead of its wait.
  * Results are identical either way; 0 restores plain stream order for every kernel launched through this context.
  * The commit (and a scan without convolution) reads part of its input ahead of that wait: the
- * accepted path, the recorded operands, the state.  The library therefore does that only when the
- * previous call on this context was a verify; behind any other library call the commit waits first
- * and the scan runs in plain stream order.  A caller that fills accepted_dev / len_dev with a kernel of its own between verify and
- * commit, on the same stream, switches overlap off. */
+ * accepted path, the recorded operands, the state.  The commit does that only when the last library
+ * call on the device, of any context, was a verify of this context on the same stream, and otherwise waits
+ * first; a scan without convolution runs in plain stream order unless that last call was one of this context
+ * on the same stream that leaves the states alone.  What a caller's own kernels write the library cannot see:
+ * a caller that fills accepted_dev / len_dev, recorded operands or states with a kernel of its own between two
+ * library calls on the stream switches overlap off. */
 int lumo_ctx_set_overlap(lumo_ctx* ctx, int on);
 
 /* Measurement aid.  While enabled, every kernel the library launches is bracketed by two CUDA

@@ -22,6 +22,13 @@ int cuda_fail(lumo_ctx* ctx, cudaError_t e, const char* what) {
   return fail(ctx, LUMO_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// End of a call: the status of its last launch, and what stands in front of the next call from now on.
+int launched(lumo_ctx* ctx, cudaError_t e, CallOrder::Kind kind, const char* what) {
+  if (e != cudaSuccess) return cuda_fail(ctx, e, what);
+  ctx->order.done(kind);
+  return LUMO_OK;
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 struct DeviceGuard {
@@ -461,12 +468,12 @@ int lumo_tree_path_from_node(lumo_ctx* ctx, const lumo_tree_desc* desc, const in
   if (ctx->device < 0) return fail(ctx, LUMO_ERR_UNSUPPORTED, "host-only context cannot launch");
   DeviceGuard g(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
+  ctx->order.begin(ctx->device, st);
   cudaError_t e = timed(ctx, LUMO_K_PATH, st, [&] {
     return launch_path_from_node(tree_view(desc, 0), desc->B, desc->N, node_dev, lmax, accepted_dev, len_dev,
                                  status_dev, ctx->overlap, st);
   });
-  ctx->last_call = lumo_ctx::kOther;
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "path_from_node launch");
+  return launched(ctx, e, CallOrder::kOther, "path_from_node launch");
 }
 
 int lumo_tree_accept(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_accept_args* a, int lmax,
@@ -486,10 +493,10 @@ int lumo_tree_accept(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_accep
   AcceptView v;
   v.V = a->V; v.mode = a->mode; v.token = a->token; v.p_target = a->p_target; v.q_draft = a->q_draft;
   v.uniforms = a->uniforms; v.noise = a->noise; v.work = a->work;
+  ctx->order.begin(ctx->device, stream);
   cudaError_t e = launch_accept(tree_view(desc, 0), desc->B, desc->N, desc->Ns, v, lmax, accepted_dev, len_dev,
                                 next_token_dev, final_node_dev, ctx->sm_count, ctx->overlap, (cudaStream_t)stream);
-  ctx->last_call = lumo_ctx::kOther;
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "accept launch");
+  return launched(ctx, e, CallOrder::kOther, "accept launch");
 }
 
 int lumo_select_spine_top3(lumo_ctx* ctx, const lumo_select_args* a, int32_t* spine_dev, int32_t* cand_dev,
@@ -503,14 +510,14 @@ int lumo_select_spine_top3(lumo_ctx* ctx, const lumo_select_args* a, int32_t* sp
   if (sp != 0 && sp != 1 && sp != 2 && sp != 4 && sp != 8 && sp != 16)
     return fail(ctx, LUMO_ERR_ARG, "split must be 0, 1, 2, 4, 8 or 16");
   DeviceGuard g(ctx->device);
+  ctx->order.begin(ctx->device, stream);
   cudaError_t e = launch_select(a->logits, a->dtype, a->rows, a->V, sp, spine_dev, cand_dev, ctx->sm_count,
                                 ctx->overlap, (cudaStream_t)stream);
-  ctx->last_call = lumo_ctx::kOther;
   if (e == cudaErrorInvalidConfiguration) {
     (void)cudaGetLastError();
     return fail(ctx, LUMO_ERR_UNSUPPORTED, "this device does not schedule clusters of that size");
   }
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "select launch");
+  return launched(ctx, e, CallOrder::kOther, "select launch");
 }
 
 // Which tail the Gram-form scan takes: 0 level-by-level substitution, 1 closed form, 2 closed form with the output
@@ -538,24 +545,23 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
   const bool gram_ok = desc->d_tc_meta != nullptr && gram_supported(s, desc->max_depth);
   if (ctx->scan_algo >= 2 && !gram_ok)
     return fail(ctx, LUMO_ERR_UNSUPPORTED, "the Gram-form scan needs d = 128, bf16 operands, depth <= 16, no snapshots");
-  // The Gram-form scan requests the pre-tree state ahead of its dependency wait.  Behind a convolution
-  // that is safe (the convolution waits first, so whatever wrote the state has completed); launched
-  // directly behind a call that rewrote the state it takes plain stream order instead.
-  const int prev_call = ctx->last_call;
-  ctx->last_call = lumo_ctx::kVerify;
+  const CallOrder::Kind before = ctx->order.begin(ctx->device, stream);
   if (gram_ok && ctx->scan_algo != 1) {
     cudaError_t e = cudaSuccess;
     if (layers[0].x) {
       e = timed(ctx, LUMO_K_CONV, st, [&] { return launch_conv(s, t, lb, ctx->sm_count, use_overlap(ctx, s, true), st); });
       if (e != cudaSuccess) return cuda_fail(ctx, e, "conv launch");
     }
-    const bool state_fresh = !layers[0].x && (prev_call == lumo_ctx::kCommit || prev_call == lumo_ctx::kCommitVerify);
+    // The Gram-form scan requests the pre-tree state ahead of its dependency wait.  Behind a convolution that is safe (the
+    // convolution waits first, so whatever wrote the state has completed), and so it is behind a call that is known and
+    // leaves the state alone; behind anything else it takes plain stream order.
+    const bool state_settled = layers[0].x || before == CallOrder::kVerify || before == CallOrder::kOther;
     e = timed(ctx, LUMO_K_SCAN, st, [&] {
-      const bool pdl = use_overlap(ctx, s, layers[0].x != nullptr) && !state_fresh;
+      const bool pdl = use_overlap(ctx, s, layers[0].x != nullptr) && state_settled;
       return ctx->scan_algo == 3 ? launch_scan_solve(s, t, lb, ctx->sm_count, pdl, st)
                                  : launch_scan_gram(s, t, lb, ctx->sm_count, pdl, scan_tail(ctx, desc, s), st);
     });
-    return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "Gram-form scan launch");
+    return launched(ctx, e, CallOrder::kVerify, "Gram-form scan launch");
   }
   int grid = 0;
   size_t stack_bytes = 0;
@@ -581,7 +587,7 @@ int lumo_gdn_tree_verify(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_g
   e = timed(ctx, LUMO_K_SCAN, st, [&] {
     return launch_scan(s, t, lb, reinterpret_cast<float*>(ctx->scratch), grid, ctx->sm_count, use_overlap(ctx, s), st);
   });
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "scan launch");
+  return launched(ctx, e, CallOrder::kVerify, "scan launch");
 }
 
 int64_t lumo_static_stack_bytes(void) { return (int64_t)kStaticStackBytes; }
@@ -612,9 +618,9 @@ int lumo_gdn_tree_scan_static(lumo_ctx* ctx, const lumo_tree_desc* desc, const l
   float* stack = nullptr;
   e = static_stack_address(ctx->device, &stack);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGetSymbolAddress(built-in scan stack)");
+  ctx->order.begin(ctx->device, stream);
   e = timed(ctx, LUMO_K_SCAN, st, [&] { return launch_scan(s, t, lb, stack, grid, ctx->sm_count, false, st); });
-  ctx->last_call = lumo_ctx::kVerify;
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "scan launch");
+  return launched(ctx, e, CallOrder::kVerify, "scan launch");
 }
 
 int lumo_gdn_commit(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_args* layers, int n_layers,
@@ -632,13 +638,13 @@ int lumo_gdn_commit(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_ar
   const TreeDev t = tree_view(desc, 0);
   // in a small launch right behind a verify call the commit reads the path, the operands and the state ahead of its
   // dependency wait (see commit_kernel)
-  s.wait_first = !(use_overlap(ctx, s) && ctx->last_call == lumo_ctx::kVerify);
+  const CallOrder::Kind before = ctx->order.begin(ctx->device, stream);
+  s.wait_first = !(use_overlap(ctx, s) && before == CallOrder::kVerify);
   const bool pdl = use_overlap(ctx, s, true);
-  ctx->last_call = lumo_ctx::kCommit;
   cudaError_t e = timed(ctx, LUMO_K_COMMIT, st, [&] {
     return launch_commit(s, t, lb, accepted_dev, len_dev, lmax, true, layers[0].x != nullptr, ctx->sm_count, pdl, st);
   });
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "commit launch");
+  return launched(ctx, e, CallOrder::kCommit, "commit launch");
 }
 
 int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const lumo_gdn_args* prev_layers,
@@ -680,9 +686,9 @@ int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const
   // so may a scan launched behind it.  A fused scan (or the history launch) directly behind another
   // call reads the path and the state ahead of its dependency wait: overlap then only behind a verify.
   const bool pdl_conv = use_overlap(ctx, s, true);
-  const bool pdl = use_overlap(ctx, s) && ctx->last_call == lumo_ctx::kVerify;
+  const CallOrder::Kind before = ctx->order.begin(ctx->device, stream);
+  const bool pdl = use_overlap(ctx, s) && before == CallOrder::kVerify;
   const bool pdl_scan = layers[0].x != nullptr ? pdl_conv : pdl;
-  ctx->last_call = lumo_ctx::kCommitVerify;
   const TreeDev pt = tree_view(prev_desc, 0);
   const TreeDev t = tree_view(desc, 0);
   fp.parent = pt.parent; fp.slot = pt.slot; fp.N = prev_desc->N; fp.Ns = prev_desc->Ns;
@@ -709,7 +715,7 @@ int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const
     return ctx->scan_algo == 3 ? launch_scan_solve_fused(s, t, lb, fp, ctx->sm_count, pdl_scan, st)
                                : launch_scan_gram_fused(s, t, lb, fp, ctx->sm_count, pdl_scan, scan_tail(ctx, desc, s), st);
   });
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "fused scan launch");
+  return launched(ctx, e, CallOrder::kCommitVerify, "fused scan launch");
 }
 
 // ---- attention half ---------------------------------------------------------------------
@@ -781,9 +787,9 @@ int lumo_kv_write_tree(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_att
   KvLayers L;
   KvShape k;
   kv_views(desc, layers, n_layers, s, &L, &k);
+  ctx->order.begin(ctx->device, stream);
   cudaError_t e = timed(ctx, LUMO_K_KV_WRITE, st, [&] { return launch_kv_write(L, k, n_layers, ctx->overlap, st); });
-  ctx->last_call = lumo_ctx::kOther;
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "kv write launch");
+  return launched(ctx, e, CallOrder::kOther, "kv write launch");
 }
 
 int lumo_tree_attention(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_attn_args* layers, int n_layers, void* stream) {
@@ -811,7 +817,7 @@ int lumo_tree_attention(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_at
     e = cudaMemset(ctx->attn_scratch, 0, 256);   // the failure flag in the first bytes: launch numbers are never 0
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemset(attention scratch)");
   }
-  ctx->last_call = lumo_ctx::kOther;
+  ctx->order.begin(ctx->device, stream);
   // the layers of a model are not adjacent in time: one launch (and one pair of tensor maps) per layer;
   // they share the scratch, which stream order makes safe
   for (int l = 0; l < n_layers; ++l) {
@@ -830,6 +836,7 @@ int lumo_tree_attention(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_at
     e = timed(ctx, LUMO_K_ATTN_MERGE, st, [&] { return launch_attn_merge(plan, ctx->overlap, st); });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention merge launch");
   }
+  ctx->order.done(CallOrder::kOther);
   return LUMO_OK;
 }
 
@@ -847,11 +854,11 @@ int lumo_kv_publish(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_attn_a
   KvLayers L;
   KvShape k;
   kv_views(desc, layers, n_layers, s, &L, &k);
+  ctx->order.begin(ctx->device, stream);
   cudaError_t e = timed(ctx, LUMO_K_KV_PUBLISH, st, [&] {
     return launch_kv_publish(L, k, n_layers, accepted_dev, len_dev, lmax, ctx_len_out, ctx->overlap, st);
   });
-  ctx->last_call = lumo_ctx::kOther;
-  return e == cudaSuccess ? LUMO_OK : cuda_fail(ctx, e, "kv publish launch");
+  return launched(ctx, e, CallOrder::kOther, "kv publish launch");
 }
 
 }  // extern "C"

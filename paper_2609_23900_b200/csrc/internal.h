@@ -7,6 +7,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "call_order.h"
 #include "lumo_gdn.h"
 
 namespace lumo {
@@ -57,11 +58,7 @@ struct lumo_ctx {
   int scan_algo = 0;            // 0 auto, 1 rank-1, 2 Gram form with forward substitution, 3 solved Gram form, 4 Gram form with closed-form tail, 5 the same with the output sum on the tensor core
   bool timeout_drill = false;   // test aid: the tensor-core scan skips its tensor-core work (lumo_ctx_set_timeout_drill)
   bool overlap = true;          // kernels are launched as programmatic dependents of the kernel before them
-  // Kind of the previous call that launched on this context.  Kernels that read some of their inputs
-  // ahead of their dependency wait (commit: path and state; scan without convolution: state) get the
-  // overlap attribute only when the call before them cannot have written those inputs.
-  enum Call { kNone = 0, kVerify, kCommit, kCommitVerify, kOther };
-  int last_call = kNone;
+  lumo::CallOrder order;        // what is in front of a call in its stream: decides what may be read ahead of a dependency wait
   bool timing = false;
   std::vector<cudaEvent_t> ev_start, ev_stop;
   std::vector<int> ev_kind;
