@@ -105,7 +105,8 @@ int prepare(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_args* laye
     p.state = a.state; p.state_row = a.state_row; p.out = a.out;
     p.snap_nodes = a.snap_nodes; p.snap_out = a.snap_out; p.status = a.status;
   }
-  for (int l = n_layers; l < kFewLayers; ++l) lb->l[l] = LayerPtrs{};   // a launch of few layers hands over kFewLayers entries
+  // a launch hands over kFewLayers or all kMaxLayers entries: none of them holds what was on the stack
+  for (int l = n_layers; l < (n_layers <= kFewLayers ? kFewLayers : kMaxLayers); ++l) lb->l[l] = LayerPtrs{};
   return LUMO_OK;
 }
 
