@@ -149,7 +149,7 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 _cuda_ready = torch.cuda.is_initialized
-_cuda_device = getattr(torch._C, "_cuda_getDevice", None)              # absent in builds without CUDA, which are never ready
+_cuda_device = getattr(torch._C, "_cuda_getDevice", None)              # private: another build of torch may lack either
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
@@ -157,7 +157,7 @@ def _stream(stream) -> int:
     if stream is not None:
         return stream.cuda_stream
     # the current stream's handle without building a Stream object (0.1 against 3.2 us per call, measured)
-    if _cuda_ready():
+    if _raw_stream and _cuda_device and _cuda_ready():
         return _raw_stream(_cuda_device())
     return torch.cuda.current_stream().cuda_stream
 

@@ -209,3 +209,19 @@ def test_attention_calls_refuse_to_launch_on_a_host_only_context():
         assert fn(ctx._h, desc._h, arr, 1, None) == 4            # LUMO_ERR_UNSUPPORTED: there is no CPU path
     assert binding._lib.lumo_kv_publish(ctx._h, desc._h, arr, 1, None, None, 4, None, None) == 4
     assert b"host-only" in binding._lib.lumo_last_error(ctx._h)
+
+
+@pytest.mark.parametrize("missing", ["_raw_stream", "_cuda_device"])
+def test_current_stream_without_torchs_private_functions(monkeypatch, missing):
+    """A torch build with CUDA up and without one of the two private functions takes the public route."""
+    import types
+
+    import torch
+    monkeypatch.setattr(binding, "_cuda_ready", lambda: True)
+    monkeypatch.setattr(binding, "_raw_stream", lambda device: 77)
+    monkeypatch.setattr(binding, "_cuda_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=1234))
+    assert binding._stream(None) == 77
+    monkeypatch.setattr(binding, missing, None)
+    assert binding._stream(None) == 1234
+    assert binding._stream(types.SimpleNamespace(cuda_stream=5)) == 5
