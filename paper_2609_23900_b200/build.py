@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblumo_gdn.so")
 SOURCES = ["api.cu", "kernels.cu", "scan_gram.cu", "scan_solve.cu", "attn.cu", "kv_cache.cu", "accept.cu", "select.cu", "tree_desc.cpp"]
-HEADERS = [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "call_order.h"), os.path.join(ROOT, "include", "lumo_gdn.h")]
+HEADERS = [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "call_order.h"), os.path.join(CSRC, "conv_split.h"), os.path.join(ROOT, "include", "lumo_gdn.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

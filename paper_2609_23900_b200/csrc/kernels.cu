@@ -14,6 +14,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "conv_split.h"
 #include "internal.h"
 
 namespace lumo {
@@ -126,21 +127,6 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
 // scan that follows writes them to the history buffer once every CTA of this kernel has finished).
-constexpr int kConvWarps = 8;
-constexpr int kConvMaxEntries = 128;      // entries per CTA: eight runs of sixteen
-
-// Runs and channel groups of a CTA (a warp per pair), chosen on the host: groups is a power of two.
-struct ConvSplit { int runs, groups, log_groups, slabs; };
-inline ConvSplit conv_split(int C, int Ns, int run) {
-  const int need = (Ns + run - 1) / run;
-  ConvSplit c;
-  c.runs = need < kConvWarps ? need : kConvWarps;
-  c.log_groups = c.runs == 1 ? 3 : c.runs == 2 ? 2 : c.runs <= 4 ? 1 : 0;
-  c.groups = 1 << c.log_groups;
-  c.slabs = (C + c.groups * 128 - 1) / (c.groups * 128);
-  return c;
-}
-
 // What the main loop needs of an entry, in one 16-byte load: byte offset of its own row in the tile, physical row, and
 // what to do; its window (only looked at where an entry starts from it) as byte offsets, or ~visiting place for a row
 // that another CTA's part holds.
@@ -1143,7 +1129,7 @@ static cudaError_t launch_conv_t(const Shape& s, const TreeDev& t, const LayerBa
     constexpr bool kFew = decltype(few_c)::value;
     using LB = std::conditional_t<kFew, FewLayers, LayerBatch>;
     constexpr int kMost = (kConvMaxEntries + 3 * kConvWarps) * 128 * (int)sizeof(T);    // of any split
-    const ConvSplit sp = conv_split(s.C, s.Ns, R);
+    const ConvSplit sp = conv_split(s.C, s.Ns, R, seqs, sms);
     const int entries = sp.runs * R;
     const dim3 grid(sp.slabs * ((s.Ns + entries - 1) / entries), s.B, s.n_layers), block(32 * sp.runs * sp.groups);
     const size_t smem = (size_t)(entries + 3) * sp.groups * 128 * sizeof(T);

@@ -36,3 +36,11 @@ def test_runs_and_parts(N, dtype):
 @pytest.mark.parametrize("B,N", [(8, 64), (24, 40), (32, 28), (12, 200)])
 def test_longer_runs_of_large_launches(B, N):
     check(W.make_case("runs", [W.tree_random(W.IntStream(N + b), N, 9) for b in range(B)], seed=B, Hk=3, Hv=6, d=128, in_dtype="bf16"))
+
+
+@pytest.mark.parametrize("B,N", [(12, 41), (14, 33)])
+def test_runs_shared_out_evenly(B, N):
+    """More CTAs than run at once: eleven runs as six and five, nine as five and four."""
+    assert ctx().conv_rows_per_cta(ctx().tree_desc(np.array([[i - 1 for i in range(N)]] * B, dtype=np.int32)), 8, 16, 128) == 4
+    check(W.make_case("runs", [W.tree_random(W.IntStream(N + b), N, 9) for b in range(B)], seed=B, Hk=8, Hv=16, d=128, in_dtype="bf16",
+                      Ns=N, permute_slots=True))
