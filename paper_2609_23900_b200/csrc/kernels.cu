@@ -188,8 +188,7 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   if constexpr (kFused) {
     if (warp == 0) {
       const int plen = fp->len[b];
-      const int lcap = plen < 0 ? 0 : (plen > fp->lmax ? 0 : plen);
-      if (lane < lcap) {
+      if (lane < fp->lmax) {                             // every place: the length is still on its way
         const int a = fp->accepted[(size_t)b * fp->lmax + lane];
         const bool ok = a >= 0 && a < fp->N;
         f_acc[lane] = a;
