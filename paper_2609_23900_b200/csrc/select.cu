@@ -9,12 +9,16 @@
 // maximum per thread and nothing else (a packed maximum per two bf16 entries), so it runs at the rate of the loads; the
 // third largest of the threads' maxima is reached by three distinct entries and therefore bounds the third-best entry from
 // below, and only the few threads whose maximum reaches that bound have their entries looked at again (out of L2, a warp per
-// thread).  What they yield goes to a short list, from which four warp-wide selections take the result.  Many equal entries
-// can overflow the list (a constant row): then every thread ranks its own entries and the ranks are merged.  Both orders are
+// thread).  What they yield goes to a short list, from which four warp-wide selections take the result.  Where many threads
+// reach the bound (a constant, masked or coarsely quantised row) the visits would take longer than a second pass, in which
+// every thread notes the first and the last place of its maximum: the third largest of the (value, last place) keys is then a
+// bound that three threads reach.  If even those hold more than the list takes, every thread ranks its own entries and the
+// ranks are merged.  Both orders are
 // total, so the result depends neither on the way taken nor on how the row was split (any cluster size gives the same bytes).
 // Bound by HBM for large calls, by launch, one round trip and the selection for small ones.  Measured against ranking every
 // entry on the way (151,936 entries a row): 1024 rows bf16 76 -> 52 us = 6.0 TB/s, f32 107 -> 97 us = 6.4 TB/s; 40 rows bf16
-// 11.0 -> 5.4 us; 600 rows of 20,000 bf16 18.3 -> 8.1 us.
+// 11.0 -> 5.4 us; 600 rows of 20,000 bf16 18.3 -> 8.1 us.  Rows with ties, bf16, 1024 and 8 rows: constant 107 and 9.0 us (one
+// thread after the other: 568 and 43.5; ranking everything: 346 and 11.8), 1 % of the entries equal 103 and 7.9 us (272 and 21.4).
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -90,6 +94,10 @@ __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 
 constexpr int kListCap = 256;                            // entries the short list holds
+// Threads of a CTA whose entries are looked at again one thread at a time.  Visits and the second pass cost the same at about
+// 130 to 160 threads (1024 rows: 0.1 % equal entries, 130 threads, 92 against 102 us; 0.15 %, 180 threads, 119 against 102; 40
+// rows in quarters: 0.25 %, 87 threads, 12.4 against 14 us, 0.5 %, 159 threads, 16.0 against 15.3).
+constexpr int kVisitMost = 144;
 
 // Ordered maximum of a thread's entries.
 template <typename T> struct RunningMax;
@@ -158,7 +166,7 @@ select_kernel(const T* __restrict__ logits, int V, int32_t* __restrict__ spine, 
   constexpr int kWarps = kSelThreads / 32;
   __shared__ uint32_t top3[3 * kWarps];
   __shared__ Key list[kListCap];
-  __shared__ int n_list;
+  __shared__ int n_list, n_tied;
   __shared__ Best warp_best[kWarps];
   __shared__ Best cta_best;                            // its spine key holds the plain index in the low word
   cg::cluster_group cl = cg::this_cluster();
@@ -175,7 +183,7 @@ select_kernel(const T* __restrict__ logits, int V, int32_t* __restrict__ spine, 
   const int tail0 = head + units * n;
   const int per = (units + nblk - 1) / nblk;
   const int u_lo = min(units, rank * per), u_hi = min(units, u_lo + per);
-  if (tid == 0) n_list = 0;
+  if (tid == 0) n_list = n_tied = 0;
   pdl_wait();          // the logits (and the outputs) may belong to earlier kernels
   pdl_trigger();
   // ---- one pass: the thread's maximum ---------------------------------------------------------------------
@@ -230,44 +238,93 @@ select_kernel(const T* __restrict__ logits, int V, int32_t* __restrict__ spine, 
     thr = unordered_bits(top);
   }
   // ---- entries that reach it: those of the threads whose maximum does, looked at again by their whole warp ------
-  auto push = [&](float v, int i) {
-    if (v >= thr) {
-      const int at = atomicAdd(&n_list, 1);
-      if (at < kListCap) list[at] = (Key)ordered_bits(v) << 32 | (uint32_t)i;
+  auto visit = [&](uint32_t who, auto push) {
+    for (; who; who &= who - 1) {                                                         // bounded: 32 lanes
+      const int t = (warp << 5) + __ffs(who) - 1;
+      for (int w = u_lo + t + lane * kSelThreads; w < u_hi; w += 32 * kSelThreads) {      // bounded: units of one thread
+        const uint4 raw = unit(w);
+        const T* e = reinterpret_cast<const T*>(&raw);
+#pragma unroll
+        for (int k = 0; k < n; ++k) push(to_f32(e[k]), head + w * n + k);
+      }
+      if (rank == 0 && lane == 0) {
+        if (t < head) push(to_f32(row[t]), t);
+        if (t < V - tail0) push(to_f32(row[tail0 + t]), tail0 + t);
+      }
     }
   };
-  for (uint32_t who = __ballot_sync(0xffffffffu, mx >= thr); who; who &= who - 1) {      // bounded: 32 lanes
-    const int t = (warp << 5) + __ffs(who) - 1;
-    for (int w = u_lo + t + lane * kSelThreads; w < u_hi; w += 32 * kSelThreads) {        // bounded: units of one thread
+  auto key_of = [](float v, int i) { return (Key)ordered_bits(v) << 32 | (uint32_t)i; };
+  auto enter = [&](int* count, Key key) {
+    const int at = atomicAdd(count, 1);
+    if (at < kListCap) list[at] = key;
+  };
+  auto best_of_list = [&](int listed) {                // by one warp
+    constexpr int kPer = kListCap / 32;
+    if (listed <= 32) {
+      Key k[1] = {lane < listed ? list[lane] : 0};
+      return pick_best<1>(k, false, nullptr);
+    }
+    Key k[kPer];
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) k[e] = lane + 32 * e < listed ? list[lane + 32 * e] : 0;
+    return pick_best<kPer>(k, false, nullptr);
+  };
+  bool ranked = false;                                 // (uniform) warp 0 has the CTA's result
+  if (__syncthreads_count(mx >= thr) <= kVisitMost) {
+    visit(__ballot_sync(0xffffffffu, mx >= thr), [&](float v, int i) { if (v >= thr) enter(&n_list, key_of(v, i)); });
+    __syncthreads();
+    ranked = n_list <= kListCap;
+    if (ranked && warp == 0) {
+      const Best b = best_of_list(n_list);
+      if (lane == 0) cta_best = b;
+    }
+  }
+  if (!ranked) {
+    // Many equal entries (a constant, fully masked or coarsely quantised row): the value alone bounds too little.  Every
+    // thread looks for its largest value again and notes where it stands first and last; the third largest of the threads'
+    // (value, last place) keys bounds the candidates, and at most three threads reach it.
+    float tv = -INFINITY;
+    int first = -1, last = -1;
+    auto note = [&](float v, int i) {                  // ascending places
+      if (v > tv || first < 0) first = i;
+      if (v >= tv) { tv = v; last = i; }
+    };
+    if (rank == 0 && tid < head) note(to_f32(row[tid]), tid);
+    for (int w = u_lo + tid; w < u_hi; w += kSelThreads) {                               // bounded: units of this CTA
       const uint4 raw = unit(w);
       const T* e = reinterpret_cast<const T*>(&raw);
 #pragma unroll
-      for (int k = 0; k < n; ++k) push(to_f32(e[k]), head + w * n + k);
+      for (int k = 0; k < n; ++k) note(to_f32(e[k]), head + w * n + k);
     }
-    if (rank == 0 && lane == 0) {
-      if (t < head) push(to_f32(row[t]), t);
-      if (t < V - tail0) push(to_f32(row[tail0 + t]), tail0 + t);
+    if (rank == 0 && tid < V - tail0) note(to_f32(row[tail0 + tid]), tail0 + tid);
+    const Key mine = first < 0 ? 0 : key_of(tv, last);
+    {
+      Key k[1] = {mine};
+      const Key sk[1] = {first < 0 ? 0 : key_of(tv, first)};
+      const Best b = pick_best<1>(k, true, sk);
+      if (lane == 0) warp_best[warp] = b;
     }
-  }
-  __syncthreads();
-  const int listed = n_list;
-  if (listed <= kListCap) {
-    if (warp == 0) {
-      constexpr int kPer = kListCap / 32;
-      Best b;
-      if (listed <= 32) {
-        Key k[1] = {lane < listed ? list[lane] : 0};
-        b = pick_best<1>(k, false, nullptr);
-      } else {
-        Key k[kPer];
-#pragma unroll
-        for (int e = 0; e < kPer; ++e) k[e] = lane + 32 * e < listed ? list[lane + 32 * e] : 0;
-        b = pick_best<kPer>(k, false, nullptr);
-      }
+    __syncthreads();
+    Key k[3] = {0, 0, 0}, sk[3] = {0, 0, 0};
+    if (lane < kWarps) {
+      const Best& o = warp_best[lane];
+      k[0] = o.t0; k[1] = o.t1; k[2] = o.t2; sk[0] = o.s;
+    }
+    const Best bound = pick_best<3>(k, true, sk);
+    visit(__ballot_sync(0xffffffffu, mine != 0 && mine >= bound.t2), [&](float v, int i) {
+      const Key key = key_of(v, i);
+      if (key >= bound.t2) enter(&n_tied, key);
+    });
+    __syncthreads();
+    ranked = n_tied <= kListCap;
+    if (ranked && warp == 0) {
+      Best b = best_of_list(n_tied);
+      b.s = bound.s;
       if (lane == 0) cta_best = b;
     }
-  } else {
-    // many equal entries: every thread ranks its own
+  }
+  if (!ranked) {
+    // hundreds of the largest entries in the hands of three threads: every thread ranks its own
     Best b;
     b.init();
     for (int w = u_lo + tid; w < u_hi; w += kSelThreads) {                               // bounded: units of this CTA
