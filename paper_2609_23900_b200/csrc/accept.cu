@@ -341,9 +341,14 @@ cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptVi
   int cluster = max_cluster_ctas(accept_kernel<1, true, double>, kAcceptThreads, cache);
   if (cluster > kAcceptCluster && B * cluster > sms) cluster = kAcceptCluster;   // many sequences: smaller clusters
   while (cluster > 1 && a.V < cluster * kAcceptThreads) cluster >>= 1;           // small vocabularies
-  // many short rejection walks: a reduction costs more the more CTAs meet in it, and clusters that need nearly every SM wait
-  // for each other's place (16 sequences over 11,325 entries: 21.6 us in eights, 18.8 us in fours)
-  if (a.mode == 1 && cluster > 4 && 4LL * B * cluster > 3LL * sms && a.V <= cluster / 2 * 4096) cluster >>= 1;
+  // Many short rejection walks: a reduction costs more the more CTAs meet in it, and clusters that need nearly every SM wait
+  // for each other's place; against that stands the longer slice of a CTA.  The line lies where the clusters fill 5/6 of the
+  // SMs, or 9/10 where halving eights gives a thread a second pack.  us, whole clusters against halves:
+  //   16s  V = 22,988: 7 sequences 17.2 / 19.9, 8 22.4 / 21.9, 9 24.8 / 20.6; V = 11,325: 8 20.0 / 18.3, 9 21.4 / 17.9
+  //   8s   V = 8000 (one pack): 15 sequences 19.1 / 19.7, 16 22.1 / 19.0, 20 26.5 / 19.9
+  //        V = 13,000: 15 18.2 / 20.9, 16 19.9 / 22.2, 17 23.1 / 24.0, 18 22.3 / 20.9, 24 31.7 / 25.6
+  const bool second_pack = cluster <= kAcceptCluster && a.V > cluster / 2 * kPack;
+  if (a.mode == 1 && cluster > 4 && B * cluster > (second_pack ? 9 * sms / 10 : 5 * sms / 6) && a.V <= cluster / 2 * 4096) cluster >>= 1;
   const bool vec = (a.V & 3) == 0 && (reinterpret_cast<uintptr_t>(a.p_target) & 15) == 0 &&
                    (a.mode == 0 || ((reinterpret_cast<uintptr_t>(a.q_draft) | reinterpret_cast<uintptr_t>(a.noise)) & 15) == 0);
   const int chunk = ((a.V + cluster - 1) / cluster + 3) & ~3;

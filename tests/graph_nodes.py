@@ -45,7 +45,8 @@ class Captured:
         m = C.c_size_t()
         _cu("cuGraphGetEdges_v2", h, None, None, None, C.byref(m))
         src, dst, data = (C.c_void_p * m.value)(), (C.c_void_p * m.value)(), (_Edge * m.value)()
-        _cu("cuGraphGetEdges_v2", h, src, dst, data, C.byref(m))
+        if m.value:
+            _cu("cuGraphGetEdges_v2", h, src, dst, data, C.byref(m))
         self.edge_types = [e.type for e in data]
 
     def programmatic(self):

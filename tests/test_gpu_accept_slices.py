@@ -6,6 +6,7 @@ import torch
 
 from oracle import accept_oracle as A
 from synthetic import workload as W
+from tests.graph_nodes import Captured
 from tests.harness import ctx
 from tests.test_gpu_accept import make_inputs, run_device
 
@@ -26,3 +27,20 @@ def test_slices_match_the_oracle(B, V, mode):
     ref = A.accept(parents, slot, 4, token, p, q, u, noise, mode=A.GREEDY if mode == "greedy" else A.REJECTION, lmax=lmax)
     for g, r in zip(got, ref):
         assert g.cpu().numpy().tolist() == np.asarray(r).tolist()
+
+
+@pytest.mark.parametrize("B,V,halved", [(14, 11325, False), (16, 16384, False), (18, 11325, True), (15, 8000, False), (16, 8000, True)])
+def test_clusters_are_halved_only_where_they_crowd_the_gpu(B, V, halved):
+    """Eight CTAs a sequence or four, as measured: the walk's grid, read from a capture."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the lines are fractions of 148 SMs")
+    parents = np.tile(np.array([-1, -1], dtype=np.int32), (B, 1))
+    desc = ctx().tree_desc(parents)
+    z = lambda *s: torch.zeros(*s, device="cuda")
+    i = lambda *s: torch.zeros(*s, dtype=torch.int32, device="cuda")
+    args = dict(token=i(B, 2), p_target=z(B, 3, V), q_draft=z(B, 2, V), uniforms=z(B, 2), noise=z(B, V) + 1, work=z(B, V),
+                accepted=i(B, 1), length=i(B), next_token=i(B), final_node=i(B), mode="rejection")
+    ctx().accept(desc, **args)                    # kernel attributes are set on the first call
+    torch.cuda.synchronize()
+    (_, params), = Captured(lambda: ctx().accept(desc, **args)).kernels
+    assert tuple(params.grid) == (4 if halved else 8, B, 1)
