@@ -19,8 +19,7 @@
 // What bounds it: the chain of passes over a vocabulary row, each one memory round trip, the float64 conversions and one
 // cluster-wide reduction.  Hence: a thread keeps to the same entries in every pass, the residual stays in the CTA's shared
 // memory (as the float64 it is used as), the next candidate's proposal row is requested before the reduction that decides
-// whether it is needed, the target row of the candidate under test is pulled into L2 meanwhile, and a reduction is one
-// exchange: every CTA stores its partial into all CTAs of the cluster, one cluster barrier, and every warp adds up the
+// whether it is needed, and a reduction is one exchange: every CTA stores its partial into all CTAs of the cluster, one cluster barrier, and every warp adds up the
 // same values in the same order; the residual at the next candidate's token travels with it.  Measured on 151,936 entries against passes through global
 // memory and two barriers per candidate: rejection sampling 1 sequence 26.9 -> 23.4 us, 8 sequences 47.9 -> 36.8 us, 16
 // sequences 68 -> 52 us; greedy 16 sequences 18.0 -> 15.5 us.
@@ -106,11 +105,6 @@ __device__ __forceinline__ void stage_row(float* dst, const float* row, int n) {
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-__device__ __forceinline__ void prefetch_row(const float* row, int n) {
-  for (int e = (int)threadIdx.x * 32; e < n; e += kAcceptThreads * 32)            // one request per 128-byte line
-    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(row + e) : "memory");
-}
-
 struct Cluster {
   cg::cluster_group cl;
   int rank, nblk, lane, warp;
@@ -177,7 +171,7 @@ struct Cluster {
 // residual lives in the caller's float32 scratch and the proposal rows are read in place.
 template <int kMode, bool kVec, class RT>
 __global__ void __launch_bounds__(kAcceptThreads)
-accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int prefetch, int32_t* __restrict__ accepted,
+accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int32_t* __restrict__ accepted,
               int32_t* __restrict__ len_out, int32_t* __restrict__ next_token, int32_t* __restrict__ final_node) {
   constexpr bool kShared = !std::is_void_v<RT>;
   using R = std::conditional_t<kShared, RT, float>;
@@ -221,10 +215,9 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int p
     if constexpr (kMode == 0) {
       float bv = -1.f;
       int bi = 0x7fffffff;
-      // The rows the walk may go on with, while they are few: one of many is mostly fetched for nothing, and asking for all
-      // of them delays the row at hand (26 children, V = 22,988: 11.0 us against 7.1).
-      if (prefetch && c_hi - c_lo <= 3)
-        for (int ci = c_lo; ci < c_hi; ++ci) prefetch_row(target(slot_map[child_list[ci]]), n);
+      // (The rows the walk may go on with are not asked for ahead.  Eight steps, V = 151,936, one sequence: 22.5 us, with the
+      // rows of one, two or three children ahead 24.5, 26.5 and 26.6 where the rows lie in L2, as a softmax leaves them; 28.7
+      // against 26.7, 28.7 and 30.7 where they do not.  The same at 8000 to 151,936 entries and 1 to 13 sequences.)
       auto look = [&](float v, int e) { if (v > bv) { bv = v; bi = v_lo + e; } };
       float4 w[kFlight];
       for_packs(packs, [&](int k, int i) { w[i] = load_pack<kVec>(p, n, k, -2.f); },
@@ -241,9 +234,7 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int p
       auto proposal = [&](int ch) { return a.q_draft + ((size_t)b * Ns + slot_map[ch]) * V + v_lo; };
       auto request = [&](int ci) {                            // the proposal row of the candidate after next
         if (ci >= c_hi) return;
-        const int ch = child_list[ci];
-        if constexpr (kShared) stage_row<kVec>(q_staged, proposal(ch), n);
-        if (prefetch) prefetch_row(target(slot_map[ch]), n);
+        if constexpr (kShared) stage_row<kVec>(q_staged, proposal(child_list[ci]), n);
       };
       auto holds = [&](int x) { return x >= v_lo && x < v_lo + n && tid == holder_of<kVec>(x - v_lo); };
       auto token_of = [&](int ci) { return ci < c_hi ? tok_of_node[child_list[ci]] : -1; };
@@ -352,8 +343,6 @@ cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptVi
   const bool vec = (a.V & 3) == 0 && (reinterpret_cast<uintptr_t>(a.p_target) & 15) == 0 &&
                    (a.mode == 0 || ((reinterpret_cast<uintptr_t>(a.q_draft) | reinterpret_cast<uintptr_t>(a.noise)) & 15) == 0);
   const int chunk = ((a.V + cluster - 1) / cluster + 3) & ~3;
-  // rows that may not be needed are pulled into L2 only where that traffic is small beside what the walk reads anyway
-  const int prefetch = (long long)B * a.V * 4 <= 8LL << 20;
   constexpr size_t kSharedMost = 216 * 1024;
   const size_t held = (size_t)((chunk + kPack - 1) / kPack) * kPack;
   auto go = [&](auto mode_c, auto vec_c, auto* r_type) {
@@ -373,7 +362,7 @@ cudaError_t launch_accept(const TreeDev& t, int B, int N, int Ns, const AcceptVi
     }
     size_t smem = 0;
     if constexpr (kMode == 1 && !std::is_void_v<RT>) smem = held * (sizeof(RT) + 4);
-    return launch_cluster_kernel(kern, dim3(cluster, B), dim3(kAcceptThreads), cluster, smem, st, pdl, t, N, Ns, a, lmax, chunk, prefetch, accepted,
+    return launch_cluster_kernel(kern, dim3(cluster, B), dim3(kAcceptThreads), cluster, smem, st, pdl, t, N, Ns, a, lmax, chunk, accepted,
                                  len, next_token, final_node);
   };
   auto pick = [&](auto vec_c) {
