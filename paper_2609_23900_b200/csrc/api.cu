@@ -425,6 +425,9 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   cudaError_t e = cudaMalloc(&d->dev, h.size() * sizeof(int32_t));
   if (e != cudaSuccess) { delete d; return cuda_fail(ctx, e, "cudaMalloc(tree tables)"); }
   e = cudaMemcpy(d->dev, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+  // from pageable memory the copy may return before the bytes have arrived, and a call on a stream that does not wait for the
+  // default stream would read the tables too early
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) { cudaFree(d->dev); delete d; return cuda_fail(ctx, e, "cudaMemcpy(tree tables)"); }
   d->d_parent = d->dev + o_parent; d->d_depth = d->dev + o_depth; d->d_slot = d->dev + o_slot;
   d->d_slot_inv = d->dev + o_inv; d->d_win = d->dev + o_winv; d->d_conv_prog = d->dev + o_prog;
@@ -816,6 +819,7 @@ int lumo_tree_attention(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_at
     if (e != cudaSuccess) return fail(ctx, LUMO_ERR_NOMEM, std::string("scratch allocation failed: ") + cudaGetErrorString(e));
     ctx->attn_scratch_bytes = need;
     e = cudaMemset(ctx->attn_scratch, 0, 256);   // the failure flag in the first bytes: launch numbers are never 0
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // (asynchronous, on another stream than the call's)
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemset(attention scratch)");
   }
   ctx->order.begin(ctx->device, stream);
