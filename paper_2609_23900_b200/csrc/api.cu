@@ -110,6 +110,18 @@ int prepare(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_args* laye
   return LUMO_OK;
 }
 
+// Fills device memory that calls on any stream read from then on.  On the default stream (cudaMemcpy, cudaMemset) the fill may
+// still be queued when the function returns, behind whatever that stream has to do, and a call on a stream that does not wait
+// for it would read too early.  Hence a stream of its own, waited for: done on return, and behind nobody's work.
+template <typename F>
+cudaError_t set_up(lumo_ctx* ctx, F fill) {
+  cudaError_t e = cudaSuccess;
+  if (!ctx->setup) e = cudaStreamCreateWithFlags(&ctx->setup, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = fill(ctx->setup);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->setup);
+  return e;
+}
+
 constexpr size_t kTimingPool = 16384;
 
 // Brackets one launch with events when timing is on.
@@ -191,6 +203,7 @@ void lumo_ctx_destroy(lumo_ctx* ctx) {
     DeviceGuard g(ctx->device);
     if (ctx->scratch) cudaFree(ctx->scratch);
     if (ctx->attn_scratch) cudaFree(ctx->attn_scratch);
+    if (ctx->setup) cudaStreamDestroy(ctx->setup);
     for (cudaEvent_t e : ctx->ev_start) cudaEventDestroy(e);
     for (cudaEvent_t e : ctx->ev_stop) cudaEventDestroy(e);
   }
@@ -424,10 +437,7 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   DeviceGuard g(ctx->device);
   cudaError_t e = cudaMalloc(&d->dev, h.size() * sizeof(int32_t));
   if (e != cudaSuccess) { delete d; return cuda_fail(ctx, e, "cudaMalloc(tree tables)"); }
-  e = cudaMemcpy(d->dev, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-  // from pageable memory the copy may return before the bytes have arrived, and a call on a stream that does not wait for the
-  // default stream would read the tables too early
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+  e = set_up(ctx, [&](cudaStream_t st) { return cudaMemcpyAsync(d->dev, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st); });
   if (e != cudaSuccess) { cudaFree(d->dev); delete d; return cuda_fail(ctx, e, "cudaMemcpy(tree tables)"); }
   d->d_parent = d->dev + o_parent; d->d_depth = d->dev + o_depth; d->d_slot = d->dev + o_slot;
   d->d_slot_inv = d->dev + o_inv; d->d_win = d->dev + o_winv; d->d_conv_prog = d->dev + o_prog;
@@ -818,8 +828,8 @@ int lumo_tree_attention(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_at
     e = cudaMalloc(&ctx->attn_scratch, need);
     if (e != cudaSuccess) return fail(ctx, LUMO_ERR_NOMEM, std::string("scratch allocation failed: ") + cudaGetErrorString(e));
     ctx->attn_scratch_bytes = need;
-    e = cudaMemset(ctx->attn_scratch, 0, 256);   // the failure flag in the first bytes: launch numbers are never 0
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // (asynchronous, on another stream than the call's)
+    // the failure flag in the first bytes: launch numbers are never 0
+    e = set_up(ctx, [&](cudaStream_t st) { return cudaMemsetAsync(ctx->attn_scratch, 0, 256, st); });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemset(attention scratch)");
   }
   ctx->order.begin(ctx->device, stream);

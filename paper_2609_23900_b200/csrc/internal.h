@@ -54,6 +54,7 @@ struct lumo_ctx {
   void* attn_scratch = nullptr; // partial results of the attention partitions
   size_t attn_scratch_bytes = 0;
   uint32_t attn_launch_id = 0;
+  cudaStream_t setup = nullptr; // set-up copies, waited for by the call that makes them (created by the first)
   // optional per-launch timing (lumo_ctx_timing_*): a fixed pool of event pairs
   int scan_algo = 0;            // 0 auto, 1 rank-1, 2 Gram form with forward substitution, 3 solved Gram form, 4 Gram form with closed-form tail, 5 the same with the output sum on the tensor core
   bool timeout_drill = false;   // test aid: the tensor-core scan skips its tensor-core work (lumo_ctx_set_timeout_drill)
@@ -305,7 +306,8 @@ cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t 
 
 // launchers (kernels.cu); all return cudaError_t and only enqueue
 cudaError_t launch_conv(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, cudaStream_t st);
-// entries of the visiting order one warp of the convolution takes (16, 8 or 4: fewer when the grid would not cover the GPU)
+// entries of the visiting order one warp of the convolution takes (16, 8 or 4: fewer when the grid would not cover the GPU;
+// named after the ABI entry)
 int conv_rows_per_cta(int C, int Ns, int seqs, int sms);
 // same convolution reading the history the previous cycle's accepted path would commit (not yet in memory)
 cudaError_t launch_conv_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp, int sm_count,
