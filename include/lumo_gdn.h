@@ -314,8 +314,8 @@ int64_t lumo_static_stack_bytes(void);
 
 /* Diagnostic: how many consecutive entries of the visiting order one warp of the tree convolution takes for this
  * tree batch, head shape and layer count on this context's device (16, 8 or 4; the three are separate
- * instantiations of the kernel, chosen so that the grid covers the GPU).  0 on a bad argument or a
- * host-only context.  Lets a parity test state which instantiation it exercised. */
+ * instantiations of the kernel, chosen so that the grid covers the GPU).  (The name is from a kernel that gave a CTA
+ * one such run; it stays for the sake of the ABI.)  0 on a bad argument or a host-only context.  Lets a parity test state which instantiation it exercised. */
 int lumo_conv_rows_per_cta(const lumo_ctx* ctx, const lumo_tree_desc* desc, int Hk, int Hv, int d, int n_layers);
 
 /* Replays accepted_dev [B, lmax] (logical ids, root first; entries at or beyond len_dev[b] are

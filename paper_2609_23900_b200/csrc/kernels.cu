@@ -1096,13 +1096,16 @@ cudaError_t dispatch(int d, int in_dtype, F f) {
 // ---------------------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------------------
-// runs of sixteen entries amortise the window set-up; small launches take fewer so that the grid still
-// covers the GPU
+// Entries per run: sixteen amortise the window set-up, fewer let a small launch reach more SMs.  Counted are groups of eight
+// warps (a warp is one run of 128 channels), however conv_split deals them out to CTAs: a run length is taken when it gives
+// every SM sixteen warps.  Convolution and scan together, us, at four / eight / sixteen entries (4096 channels): 4 sequences of
+// 60 entries (32 groups of sixteen) 20.5 / 22.2 / 22.1, 12 of 60 30.0 / 28.7 / 30.2, 24 of 28 37.4 / 36.9 / 37.5, 48 of 28
+// 59.4 / 60.1 / 57.5.
 int conv_rows_per_cta(int C, int Ns, int seqs, int sms) {
   const int slabs = (C / 4 + 255) / 256;
-  auto ctas = [&](int rows) { return (long long)slabs * ((Ns + rows - 1) / rows) * seqs; };
-  if (ctas(16) >= 2LL * sms) return 16;
-  if (ctas(8) >= 2LL * sms) return 8;
+  auto groups = [&](int run) { return (long long)slabs * ((Ns + run - 1) / run) * seqs; };
+  if (groups(16) >= 2LL * sms) return 16;
+  if (groups(8) >= 2LL * sms) return 8;
   return 4;
 }
 

@@ -708,7 +708,9 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
     // The item this CTA takes next: its state and operand rows are pulled into L2 while this item
     // computes (requests issued behind the dependency wait below), so that its own loads find them there.
     const int nxt = item + (int)gridDim.x;
-    // (trees cut into several groups re-read one state per group from L2 anyway: there it measured slower)
+    // (trees cut into several groups re-read one state per group from L2 anyway: there it measured slower; a fused launch, which
+    // would have to name the recorded rows of the next item's accepted path too, does not ask ahead, and what it would gain has
+    // not been measured)
     const bool has_next = !kFused && nxt < n_items && t.n_groups == s.B;
     int n_b = 0, n_meta = -1, n_row = -1;
     if (has_next) {

@@ -381,8 +381,10 @@ cudaError_t launch_select(const void* logits, int dtype, int rows, int V, int sp
                                      : max_cluster_ctas(select_kernel<float>, kSelThreads, cache_f);
   int cluster = split;
   if (cluster == 0) {
-    // few rows: each over more SMs, as long as a CTA keeps 64 KB to read (the two cluster barriers cost as much as a CTA
-    // takes for about that: 40 rows of 64 KB take 3.5 us whole and 5.1 us in quarters, 40 rows of 304 KB 6.0 and 5.4 us)
+    // Few rows: each over more SMs, as long as a CTA keeps 64 KB to read (the two cluster barriers cost as much as a CTA
+    // takes for about that).  Of 168 sizes (1 to 400 rows, 16 to 594 KB a row) 117 are within 4 % of the best split and all
+    // within 15 %; us, whole / halves / quarters / eighths / sixteenths: 40 rows of 128 KB 4.9 / 5.1 / 5.0 / 8.0 / 12, 16 of 297
+    // KB 6.8 / 6.0 / 5.3 / 4.9 / 8.0, 1 of 297 KB 4.4 / 4.4 / 4.0 / 3.6 / 3.5, 100 of 128 KB 5.8 / 6.4 / 9.0 / 15 / -.
     cluster = cap;
     while (cluster > 1 && (long long)rows * cluster > 2LL * sms) cluster >>= 1;
     const long long row_bytes = (long long)V * (dtype == LUMO_BF16 ? 2 : 4);
