@@ -162,6 +162,7 @@ TreeDev tree_view(const lumo_tree_desc* d, int which) {
   t.tc_group = d->d_tc_group; t.tc_meta = d->d_tc_meta; t.tc_anc = d->d_tc_anc; t.tc_lvl = d->d_tc_lvl;
   t.n_groups = d->n_groups;
   t.max_group_nodes = d->max_group_nodes;
+  t.st_off = d->d_st_off; t.st_meta = d->d_st_meta; t.st_anc = d->d_st_anc; t.st_groups = d->st_groups;
   return t;
 }
 
@@ -316,10 +317,13 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   for (int b = 0; b < B; ++b)
     for (int i = 0; i < N; ++i) d->max_depth = std::max(d->max_depth, (int)d->trees[b].tab[LUMO_TAB_DEPTH][i]);
   const bool tc = d->max_depth <= 16;
-  std::vector<std::vector<GramGroup>> groups(B);
+  std::vector<std::vector<GramGroup>> groups(B), small_groups(B);
   if (tc)
     for (int b = 0; b < B; ++b) {
-      build_gram_groups(parent + (size_t)b * N, N, d->trees[b], &groups[b]);
+      build_gram_groups(parent + (size_t)b * N, N, d->trees[b], 64, &groups[b]);
+      if (N > 32) build_gram_groups(parent + (size_t)b * N, N, d->trees[b], 32, &small_groups[b]);
+      else small_groups[b] = groups[b];
+      d->st_groups += (int)small_groups[b].size();
       d->n_groups += (int)groups[b].size();
       auto& tab = d->trees[b].tab[LUMO_TAB_GRAM_GROUPS];
       tab.push_back((int32_t)groups[b].size());
@@ -333,10 +337,26 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   const size_t G = (size_t)d->n_groups;
   const size_t o_tc_group = tc ? reserve(G * 4) : 0, o_tc_meta = tc ? reserve(G * 64) : 0;
   const size_t o_tc_anc = tc ? reserve(G * 64 * 4) : 0, o_tc_lvl = tc ? reserve(G * 5) : 0;
+  const size_t g32 = (size_t)d->st_groups;
+  const size_t o_st_off = tc ? reserve(B + 1) : 0, o_st_meta = tc ? reserve(g32 * 32) : 0, o_st_anc = tc ? reserve(g32 * 32 * 4) : 0;
   const bool attn = Ns <= kMaxAttnSlots;
   const size_t o_vis = attn ? reserve((size_t)B * N * 8) : 0, o_used = attn ? reserve((size_t)B * 8) : 0;
-  size_t gi = 0;
+  size_t gi = 0, sgi = 0;
   long long subst_rounds = 0, group_nodes = 0;     // over all groups: rounds of the substitution, nodes
+  // a group's members: physical row | depth << 16 | emit << 24, and the positions of their ancestors, root first, then their own
+  auto group_tables = [&](int b, const GramGroup& gr, int32_t* meta, uint8_t* anc) {
+    const int n = (int)gr.nodes.size();
+    std::vector<int> pos(N, -1);
+    for (int pi = 0; pi < n; ++pi) pos[gr.nodes[pi]] = pi;
+    for (int pi = 0; pi < n; ++pi) {
+      const int node = gr.nodes[pi];
+      const int dep = d->trees[b].tab[LUMO_TAB_DEPTH][node];
+      meta[pi] = h[o_slot + (size_t)b * N + node] | (dep << 16) | ((int)gr.emit[pi] << 24);
+      int cur = parent[(size_t)b * N + node];
+      anc[pi * 16 + dep - 1] = (uint8_t)pi;
+      for (int j = dep - 2; j >= 0; --j) { anc[pi * 16 + j] = (uint8_t)pos[cur]; cur = parent[(size_t)b * N + cur]; }
+    }
+  };
   for (int b = 0; b < B; ++b) {
     const HostTree& t = d->trees[b];
     if (attn) {
@@ -407,22 +427,19 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
         h[o_tc_group + gi * 4 + 0] = b;
         h[o_tc_group + gi * 4 + 1] = n;
         h[o_tc_group + gi * 4 + 2] = k == 0;
-        std::vector<int> pos(N, -1);
-        for (int pi = 0; pi < n; ++pi) pos[gr.nodes[pi]] = pi;
         uint8_t* lvl = reinterpret_cast<uint8_t*>(h.data() + o_tc_lvl) + gi * 20;
-        uint8_t* anc = reinterpret_cast<uint8_t*>(h.data() + o_tc_anc) + gi * 64 * 16;
-        for (int pi = 0; pi < n; ++pi) {
-          const int node = gr.nodes[pi];
-          const int dep = t.tab[LUMO_TAB_DEPTH][node];
-          h[o_tc_meta + gi * 64 + pi] = h[o_slot + (size_t)b * N + node] | (dep << 16) | ((int)gr.emit[pi] << 24);
-          int cur = parent[(size_t)b * N + node];
-          anc[pi * 16 + dep - 1] = (uint8_t)pi;
-          for (int j = dep - 2; j >= 0; --j) { anc[pi * 16 + j] = (uint8_t)pos[cur]; cur = parent[(size_t)b * N + cur]; }
-          for (int dd = dep; dd < 20; ++dd) lvl[dd] += 1;      // lvl[d] = members of depth <= d
-        }
+        group_tables(b, gr, h.data() + o_tc_meta + gi * 64, reinterpret_cast<uint8_t*>(h.data() + o_tc_anc) + gi * 64 * 16);
+        for (int node : gr.nodes)
+          for (int dd = t.tab[LUMO_TAB_DEPTH][node]; dd < 20; ++dd) lvl[dd] += 1;      // lvl[d] = members of depth <= d
         for (int dd = 1; dd < 20; ++dd) subst_rounds += (lvl[dd] - lvl[dd - 1] + 7) / 8;
         group_nodes += n;
       }
+      h[o_st_off + b] = (int32_t)sgi;
+      for (const GramGroup& gr : small_groups[b]) {
+        group_tables(b, gr, h.data() + o_st_meta + sgi * 32, reinterpret_cast<uint8_t*>(h.data() + o_st_anc) + sgi * 32 * 16);
+        ++sgi;
+      }
+      h[o_st_off + B] = (int32_t)sgi;
     }
   }
   // measured on B200 (us per item): substitution 0.45 per round, closed form 1.7 + 0.08 per node; the
@@ -448,6 +465,9 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
     d->d_tc_meta = d->dev + o_tc_meta;
     d->d_tc_anc = reinterpret_cast<uint8_t*>(d->dev + o_tc_anc);
     d->d_tc_lvl = reinterpret_cast<uint8_t*>(d->dev + o_tc_lvl);
+    d->d_st_off = d->dev + o_st_off;
+    d->d_st_meta = d->dev + o_st_meta;
+    d->d_st_anc = reinterpret_cast<uint8_t*>(d->dev + o_st_anc);
   }
   if (attn) {
     d->d_vis = reinterpret_cast<uint32_t*>(d->dev + o_vis);

@@ -94,6 +94,11 @@ struct lumo_tree_desc {
   int32_t* d_tc_meta = nullptr;   // [G, 64] physical row | depth << 16 | emit << 24 of the node at position pi
   uint8_t* d_tc_anc = nullptr;    // [G, 64, 16] positions of the ancestors, root first, then the node's own position
   uint8_t* d_tc_lvl = nullptr;    // [G, 20] lvl[d] = number of group nodes of depth <= d (lvl[0] = 0)
+  // the same for the streamed scan, whose groups hold at most 32 nodes: g = number of its groups over the batch
+  int st_groups = 0;
+  int32_t* d_st_off = nullptr;    // [B + 1] first group of each sequence
+  int32_t* d_st_meta = nullptr;   // [g, 32] as d_tc_meta; 0 beyond the group's nodes
+  uint8_t* d_st_anc = nullptr;    // [g, 32, 16] as d_tc_anc
   // Which tail the Gram-form scan takes by default.  The level-by-level substitution costs one round per
   // eight nodes of a level, the closed-form tail a fixed part plus a part per node: thin, deep trees (a
   // spine with small side branches) are cheaper in closed form, wide ones by levels.
@@ -176,9 +181,10 @@ struct TreeDev {
   const int32_t* win; const int32_t* conv_prog; const int32_t* sched; const int32_t* nops; int max_ops; int max_levels;
   const int32_t* child_off; const int32_t* child_list;   // [B, N+2] CSR (entry 0 = pre-tree state), [B, N]
   const int32_t* tc_group; const int32_t* tc_meta; const uint8_t* tc_anc; const uint8_t* tc_lvl; int n_groups; int max_group_nodes;
+  const int32_t* st_off; const int32_t* st_meta; const uint8_t* st_anc; int st_groups;
 };
 
-void build_gram_groups(const int32_t* parent, int N, const HostTree& t, std::vector<GramGroup>* out);
+void build_gram_groups(const int32_t* parent, int N, const HostTree& t, int cap, std::vector<GramGroup>* out);
 // host-side tree tables (tree_desc.cpp)
 bool build_tree(const int32_t* parent, const int32_t* slot, int N, int Ns, HostTree* t,
                 int* levels_lean, int* levels_full, std::string* err);
@@ -192,22 +198,25 @@ bool build_tree(const int32_t* parent, const int32_t* slot, int N, int Ns, HostT
 // Gates of one (physical row, value head) as the recurrence consumes them: the stored values, or in
 // raw-gate mode alpha = exp(-exp(a_log) softplus(g + dt_bias)), beta = sigmoid(b), in fp32.  Every
 // kernel goes through this one function, so verify and commit see bit-identical gates.
-__device__ __forceinline__ float2 load_gates(const LayerPtrs& L, const Shape& s, size_t i, int hv) {
-  float a, b;
-  if (s.gate_dtype == LUMO_BF16) {
-    a = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short*>(L.alpha)[i] << 16);
-    b = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short*>(L.beta)[i] << 16);
-  } else {
-    a = reinterpret_cast<const float*>(L.alpha)[i];
-    b = reinterpret_cast<const float*>(L.beta)[i];
-  }
+__device__ __forceinline__ uint2 load_gate_words(const LayerPtrs& L, const Shape& s, size_t i) {      // as stored
+  if (s.gate_dtype == LUMO_BF16) return make_uint2(reinterpret_cast<const unsigned short*>(L.alpha)[i], reinterpret_cast<const unsigned short*>(L.beta)[i]);
+  return make_uint2(reinterpret_cast<const uint32_t*>(L.alpha)[i], reinterpret_cast<const uint32_t*>(L.beta)[i]);
+}
+// a_log, dt_bias: the head's parameters (raw-gate mode only)
+__device__ __forceinline__ float2 finish_gates(uint2 stored, const Shape& s, float a_log, float dt_bias) {
+  const int up = s.gate_dtype == LUMO_BF16 ? 16 : 0;
+  float a = __uint_as_float(stored.x << up), b = __uint_as_float(stored.y << up);
   if (s.gate_mode == 1) {
-    const float x = a + L.dt_bias[hv];
+    const float x = a + dt_bias;
     const float sp = x > 20.f ? x : log1pf(expf(x));
-    a = expf(-expf(L.a_log[hv]) * sp);
+    a = expf(-expf(a_log) * sp);
     b = 1.f / (1.f + expf(-b));
   }
   return make_float2(a, b);
+}
+__device__ __forceinline__ float2 load_gates(const LayerPtrs& L, const Shape& s, size_t i, int hv) {
+  const bool raw = s.gate_mode == 1;
+  return finish_gates(load_gate_words(L, s, i), s, raw ? L.a_log[hv] : 0.f, raw ? L.dt_bias[hv] : 0.f);
 }
 
 // Accepted-path check; every CTA of a sequence reaches the same answer.  Order of checks: length,
@@ -339,6 +348,11 @@ cudaError_t launch_scan_gram(const Shape& s, const TreeDev& t, const LayerBatch&
 // same scan, first replaying the previous cycle's accepted path into the state it has just loaded
 cudaError_t launch_scan_gram_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp,
                                    int sm_count, bool pdl, int tail, cudaStream_t st);
+// solved Gram form with the state streamed through shared memory, for launches of several waves (scan_stream.cu);
+// fp: replay the previous cycle's accepted path first (null: plain scan)
+bool scan_stream_pays(const Shape& s, const TreeDev& t, bool fused, int sm_count);
+cudaError_t launch_scan_stream(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sm_count, bool pdl,
+                               cudaStream_t st);
 // solved Gram form on tcgen05 (scan_solve.cu): the triangular system solved on scalars, one state product
 cudaError_t launch_scan_solve(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl,
                               cudaStream_t st);

@@ -22,7 +22,8 @@
 // previous level, so that only the ancestors' deltas are fetched after it.
 //
 // A second tail (kDirect, below) replaces the level-by-level walk by a closed form: M = W (I + A)^-1 per
-// node along its own root path, then one pass over right-hand sides; the host picks per descriptor.
+// node along its own root path, then one pass over right-hand sides.  Where the host picks the closed form (per descriptor and
+// launch size), the streamed scan of scan_stream.cu takes its place at nearly all sizes.
 //
 // One CTA (256 threads) handles one (layer, sequence, value head) at a time; two CTAs per SM
 // overlap one item's loads with the other's arithmetic.  Limits of this
@@ -101,8 +102,8 @@ constexpr int kSmemBytesFused = kOffPrev + (int)sizeof(PrevStage) + 1024;
 
 // Layout of one CTA.  Compact (trees of at most 32 nodes, not fused): the state crosses shared memory
 // one 64-column half at a time (hi + lo of one k-block, 32 KB), the aliased areas shrink with the node
-// count, and a CTA needs 52 KB of shared memory and 128 tensor-memory columns: four CTAs per SM instead of
-// two (64 registers per thread instead of 128).  The tails without the tensor-core product spill at 64 and keep three CTAs.
+// count, and a CTA needs 52 KB of shared memory, 80 registers per thread and 128 tensor-memory columns: three CTAs per SM
+// instead of two.
 template <bool C>
 struct GL {
   static constexpr int kNodes = C ? 32 : kNT;
@@ -113,7 +114,6 @@ struct GL {
   static constexpr int kDump = C ? kAhi : kOffDump;            // the aliased areas start over the state tiles
   static constexpr int kStride = C ? 33 : kDumpStride;         // floats per dumped Gram row
   static constexpr int kRec = kDump + (C ? 128 * 33 * 4 : kOffRec);      // records behind the Gram dump / the deltas
-  static constexpr int kMt = C ? kDump + 9216 : kOffKQ;        // M tiles of the closed form: behind the Gram rows in use, or over K and Q
   static constexpr int kV = kRec + kNodes * (int)sizeof(NodeRec);
   static constexpr int kZero = kNodes * kD;                    // element offset of the all-zero delta row
   static constexpr int kTmem = C ? 128 : kTmemCols;
@@ -124,8 +124,7 @@ static_assert(GL<true>::kDump + (GL<true>::kNodes + 1) * kD * 4 <= GL<true>::kRe
 static_assert(GL<true>::kV + GL<true>::kNodes * kD * 2 <= GL<true>::kSmall, "aliased region overflows the state tiles");
 // the Gram product takes 128 rows from each K/Q block: the 64 rows behind the last one must lie inside the CTA's memory
 static_assert(GL<true>::kKQ + 2 * GL<true>::kKBlock + 8192 <= GL<true>::kSmall, "the Gram operand reaches past the state tiles");
-static_assert(GL<true>::kDump + 64 * GL<true>::kStride * 4 <= GL<true>::kMt && GL<true>::kMt + 4096 <= GL<true>::kRec, "M tiles overlap the Gram rows in use");
-static_assert(4 * (GL<true>::kBytes + 1024) <= 228 * 1024, "four compact CTAs must share an SM");
+static_assert(3 * (GL<true>::kBytes + 1024) <= 228 * 1024, "three compact CTAs must share an SM");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -398,7 +397,8 @@ __device__ __forceinline__ void direct_tail(const Shape& s, const LayerPtrs& L, 
   }
 }
 
-// Closed-form tail with the output sum on the tensor core.  Same scalar part as direct_tail (A, W, then
+// Closed-form tail with the output sum on the tensor core; it serves the sizes at which the streamed scan (scan_stream.cu) does
+// not pay.  Same scalar part as direct_tail (A, W, then
 // M = W (I + A)^-1 per node along its own root path); the sum o_t = g_t |q scale| S0 q_t + sum_s M[t][s] rhs_s
 // is then ONE product over all nodes of the group, O[row][t] = sum_s RHS[row][s] M[t][s] (M is zero off the
 // path), with both operands split into bf16 hi + lo (three products: hi.hi + hi.lo + lo.hi, relative error
@@ -412,7 +412,7 @@ __device__ __forceinline__ void direct_tail(const Shape& s, const LayerPtrs& L, 
 // nodes with a marked node on their path are written as NaN.  Non-finite keys, queries and gates need no such
 // care: they reach M only in the rows of the node's descendants, and the query products only the node itself.
 // Returns false when the bounded wait for the product ran out.
-template <int NT, class LY, bool kCompact>
+template <int NT, class LY>
 __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& L, Small& sm, unsigned char* smem, uint32_t sbase,
                                                const float* dump, const __nv_bfloat16* Vs, uint32_t tmem, uint32_t tmem_lane,
                                                int N, int b, int hv, int tid, uint32_t& phase) {
@@ -420,10 +420,10 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
   float* Am = reinterpret_cast<float*>(smem + LY::kRec);        // [node][16], in the place of the records
   float* Wm = Am + NT * 16;
   static_assert(LY::kRec + NT * 16 * 4 * 2 <= LY::kV, "coefficient tables overflow the record area");
-  constexpr int kStage = kCompact ? LY::kKQ : 0;                // staged outputs: over the dead Gram dump, or (compact) over K and Q
+  constexpr int kStage = 0;                                     // staged outputs: over the dead Gram dump
   constexpr int kRhsCol = LY::kGramCol + NT;                    // right-hand sides in tensor memory: NT / 2 columns hi, NT / 2 lo
   static_assert(kRhsCol + NT <= LY::kTmem, "right-hand sides overflow the tensor-memory columns");
-  constexpr int kMt = LY::kMt;                                  // M tiles
+  constexpr int kMt = kOffKQ;                                   // M tiles: over K and Q
   constexpr int kMtTerm = NT == 64 ? 8192 : 64;                 // byte distance from the hi to the lo operand
   constexpr int kMtBytes = NT == 64 ? 16384 : 4096;
   // byte offset of element (row, col) of operand term 0 (hi) or 1 (lo): with NT = 64 the lo operand is a tile of
@@ -583,7 +583,7 @@ __device__ __forceinline__ bool direct_tail_tc(const Shape& s, const LayerPtrs& 
   // ---- outputs: they leave tensor memory lane = value row, cross shared memory [node][row] (over the dead
   //      right-hand-side tiles) and are written one node per warp, 256 or 512 contiguous bytes at a time -----------
   float* stage = reinterpret_cast<float*>(smem + kStage);
-  static_assert(kCompact || NT * kD * 4 <= LY::kRec, "output staging overflows the dump area");
+  static_assert(NT * kD * 4 <= LY::kRec, "output staging overflows the dump area");
   {
     constexpr int kPer = NT / 2;
     const int n0 = grp * kPer;
@@ -647,7 +647,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
   // array keeps the pointers in the shared address space
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
-  static_assert(!kCompact || (NT == 32 && !kFused), "the compact layout serves the 32-node tile of the plain scan");
+  static_assert(!kCompact || (NT == 32 && !kFused && !kTensor), "the compact layout serves the 32-node tile of the plain scan");
   using LY = GL<kCompact>;
   Small& sm = *reinterpret_cast<Small*>(smem + LY::kSmall);
   float* dump = reinterpret_cast<float*>(smem + LY::kDump);
@@ -1064,7 +1064,7 @@ __device__ __forceinline__ void scan_gram_body(const Shape& s, const TreeDev& t,
     else if (vrow < 64) tmem_cols16_to_smem(tmem_lane + LY::kGramCol + grp * 16, dump + vrow * LY::kStride + grp * 16, 1);
     __syncthreads();
     if constexpr (kDirect && kTensor) {
-      if (!direct_tail_tc<NT, LY, kCompact>(s, L, sm, smem, sbase, dump, Vs, tmem, tmem_lane, N, b, hv, tid, phase)) sm.timed_out = 1;
+      if (!direct_tail_tc<NT, LY>(s, L, sm, smem, sbase, dump, Vs, tmem, tmem_lane, N, b, hv, tid, phase)) sm.timed_out = 1;
       tc_fence_before();
       __syncthreads();      // tensor memory and the aliased shared memory are free for the next item
       if (sm.timed_out) {
@@ -1227,11 +1227,11 @@ scan_gram_kernel(Shape s, TreeDev t, LB lb, int n_items) {
   scan_gram_body<NT, false, false, kDirect, kTensor, LB>(s, t, lb, n_items, nullptr);
 }
 
-// trees of at most 32 nodes, launches of several waves: four (three) smaller CTAs per SM
-template <bool kDirect, bool kTensor, class LB>
-__global__ void __launch_bounds__(kThreads, kTensor ? 4 : 3)
+// trees of at most 32 nodes, launches of several waves: three smaller CTAs per SM
+template <bool kDirect, class LB>
+__global__ void __launch_bounds__(kThreads, 3)
 scan_gram_compact_kernel(Shape s, TreeDev t, LB lb, int n_items) {
-  scan_gram_body<32, false, true, kDirect, kTensor, LB>(s, t, lb, n_items, nullptr);
+  scan_gram_body<32, false, true, kDirect, false, LB>(s, t, lb, n_items, nullptr);
 }
 
 template <int NT, bool kDirect, bool kTensor, class LB>
@@ -1269,34 +1269,31 @@ static cudaError_t launch_scan_gram_t(const Shape& s, const TreeDev& t, const LB
     if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, false, false, LB>, kSmemBytes);
     if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<64, true, false, LB>, kSmemBytes);
     if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, true, false, LB>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<false, false, LB>, GL<true>::kBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true, false, LB>, GL<true>::kBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<false, LB>, GL<true>::kBytes);
+    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true, LB>, GL<true>::kBytes);
     if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<64, true, true, LB>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_kernel<32, true, true, LB>, kSmemBytes);
-    if (e == cudaSuccess) e = allow_smem(scan_gram_compact_kernel<true, true, LB>, GL<true>::kBytes);
     if (e != cudaSuccess) return e;
     cfg.done[dev] = true;
   }
   // two CTAs per SM by construction: 102 KB of shared memory, 128 registers x 256 threads and 256
   // of the 512 tensor-memory columns each
-  // Compact CTAs (52 KB, 64 registers, 128 tensor-memory columns: four per SM) pay one more tensor-core
+  // Compact CTAs (52 KB, 80 registers, 128 tensor-memory columns: three per SM) pay one more tensor-core
   // round trip per item: they win when a launch has several waves of items (the 48-layer stack: 205 ->
-  // 182 us; 3072 items of 7-node trees with raw gates: 89.8 us with three per SM, 86.5 with four) and lose
-  // on a single wave (batch 1: 9.3 -> 10.5 us).
-  if (t.max_group_nodes <= 32 && items >= 4 * sm_count) {
-    auto k = tail == 2 ? scan_gram_compact_kernel<true, true, LB>
-                       : direct ? scan_gram_compact_kernel<true, false, LB> : scan_gram_compact_kernel<false, false, LB>;
-    return launch_kernel(k, dim3((tail == 2 ? 4 : 3) * sm_count), dim3(kThreads), GL<true>::kBytes, st, pdl, s, t, lb, items);
+  // 190 us) and lose on a single wave (batch 1: 9.3 -> 10.5 us).
+  if (tail != 2 && t.max_group_nodes <= 32 && items >= 4 * sm_count) {
+    auto k = direct ? scan_gram_compact_kernel<true, LB> : scan_gram_compact_kernel<false, LB>;
+    return launch_kernel(k, dim3(3 * sm_count), dim3(kThreads), GL<true>::kBytes, st, pdl, s, t, lb, items);
   }
   const int grid = items < 2 * sm_count ? items : 2 * sm_count;
   auto k = t.max_group_nodes <= 32 ? (direct ? scan_gram_kernel<32, true, false, LB> : scan_gram_kernel<32, false, false, LB>)
                                    : (direct ? scan_gram_kernel<64, true, false, LB> : scan_gram_kernel<64, false, false, LB>);
-  if (tail == 2) k = t.max_group_nodes <= 32 ? scan_gram_kernel<32, true, true, LB> : scan_gram_kernel<64, true, true, LB>;
+  if (tail == 2) k = scan_gram_kernel<64, true, true, LB>;       // (trees of at most 32 nodes are streamed)
   return launch_kernel(k, dim3(grid), dim3(kThreads), kSmemBytes, st, pdl, s, t, lb, items);
 }
 
 cudaError_t launch_scan_gram(const Shape& s, const TreeDev& t, const LayerBatch& lb, int sm_count, bool pdl, int tail,
                              cudaStream_t st) {
+  if (tail == 2 && scan_stream_pays(s, t, false, sm_count)) return launch_scan_stream(s, t, lb, nullptr, sm_count, pdl, st);
   if (s.n_layers <= kFewLayers) return launch_scan_gram_t(s, t, few_layers(lb), sm_count, pdl, tail, st);
   return launch_scan_gram_t(s, t, lb, sm_count, pdl, tail, st);
 }
@@ -1330,6 +1327,7 @@ static cudaError_t launch_scan_gram_fused_t(const Shape& s, const TreeDev& t, co
 
 cudaError_t launch_scan_gram_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp,
                                    int sm_count, bool pdl, int tail, cudaStream_t st) {
+  if (tail == 2 && scan_stream_pays(s, t, true, sm_count)) return launch_scan_stream(s, t, lb, &fp, sm_count, pdl, st);
   if (s.n_layers <= kFewLayers)
     return launch_scan_gram_fused_t(s, t, few_layers(lb), few_layers(fp), sm_count, pdl, tail, st);
   return launch_scan_gram_fused_t(s, t, lb, fp, sm_count, pdl, tail, st);

@@ -5,7 +5,6 @@
 // (dependent path groups, cut states; Sec. "Path-parallel verification and state
 // lifetime").  The depth-first op list is this library's own schedule.
 #include <algorithm>
-#include <bitset>
 #include <functional>
 
 #include "internal.h"
@@ -27,27 +26,27 @@ int build_schedule(const Kids& kids, int N, const std::function<bool(int)>& need
   // recursion depth is bounded by the tree depth (<= 256)
   std::function<void(int, int)> visit = [&](int p, int lvl) {
     const std::vector<int>& ch = p < 0 ? kids.root : kids.of[p];
-    std::vector<int> inner;
+    int last = -1, n_inner = 0;
     for (int c : ch)
-      if (need_state(c)) inner.push_back(c);
-    if (inner.empty()) {
+      if (need_state(c)) { last = c; ++n_inner; }
+    if (n_inner == 0) {
       for (int c : ch) ops->push_back(make_op(OP_EMIT, 0, c));
       return;
     }
-    const int last = inner.back();
     for (int c : ch) {
       if (c == last) continue;
       ops->push_back(make_op(OP_EMIT, need_state(c) ? 1 : 0, c));
     }
-    if (inner.size() > 1) {
+    if (n_inner > 1) {
       const bool at_root = p < 0;
       if (!at_root) {
         ops->push_back(make_op(OP_PUSH, 0, lvl));
         max_levels = std::max(max_levels, lvl + 1);
       }
-      for (size_t j = 0; j + 1 < inner.size(); ++j) {
-        ops->push_back(make_op(OP_DESCEND, 0, inner[j]));
-        visit(inner[j], at_root ? lvl : lvl + 1);
+      for (int c : ch) {
+        if (c == last || !need_state(c)) continue;
+        ops->push_back(make_op(OP_DESCEND, 0, c));
+        visit(c, at_root ? lvl : lvl + 1);
         ops->push_back(make_op(OP_POP, 0, at_root ? kPopRoot : lvl));
       }
     }
@@ -175,56 +174,81 @@ bool build_tree(const int32_t* parent, const int32_t* slot, int N, int Ns, HostT
   return true;
 }
 
-// Node groups of the tensor-core scan.  A group is a set of at most 64 nodes closed under "parent
+// Node groups of the tensor-core scans.  A group is a set of at most `cap` nodes closed under "parent
 // of", so that it can be solved from the pre-tree state alone; every node is emitted (written) by
 // exactly one group and may be recomputed, unwritten, in others.  Fewer groups mean fewer passes
 // over the state, so the tree is first cut into atoms (a complete subtree if it fits together with
 // its ancestors, else the node alone and its children in turn) and the atoms are packed, largest
 // closure first, each into the group whose node set grows least (groups that already hold the
 // atom's ancestors take it for little), or into a new group.  Members are ordered by (depth, index).
-void build_gram_groups(const int32_t* parent, int N, const HostTree& t, std::vector<GramGroup>* out) {
+void build_gram_groups(const int32_t* parent, int N, const HostTree& t, int cap, std::vector<GramGroup>* out) {
   const auto& depth = t.tab[LUMO_TAB_DEPTH];
   const auto& coff = t.tab[LUMO_TAB_CHILD_OFF];
   const auto& clist = t.tab[LUMO_TAB_CHILD_LIST];
-  constexpr int kCap = 64;
-  using Mask = std::bitset<kMaxNodes>;
-  std::vector<int> size(N, 1);
-  for (int i = N - 1; i >= 0; --i)
-    if (parent[i] >= 0) size[parent[i]] += size[i];
+  // a set of nodes; counted in registers (the generic count is a call for each word)
+  struct Mask {
+    uint64_t w[kMaxNodes / 64] = {};
+    void set(int n) { w[n >> 6] |= 1ull << (n & 63); }
+    bool test(int n) const { return w[n >> 6] >> (n & 63) & 1; }
+    void operator|=(const Mask& o) { for (int i = 0; i < kMaxNodes / 64; ++i) w[i] |= o.w[i]; }
+    int count_without(const Mask& o) const {
+      uint64_t bytes = 0;                            // per byte: at most 8 in each of four words
+      for (int i = 0; i < kMaxNodes / 64; ++i) {
+        uint64_t x = w[i] & ~o.w[i];
+        x -= x >> 1 & 0x5555555555555555ull;
+        x = (x & 0x3333333333333333ull) + (x >> 2 & 0x3333333333333333ull);
+        bytes += (x + (x >> 4)) & 0x0F0F0F0F0F0F0F0Full;
+      }
+      return (int)((((bytes & 0x00FF00FF00FF00FFull) + (bytes >> 8 & 0x00FF00FF00FF00FFull)) * 0x0001000100010001ull) >> 48);
+    }
+  };
+  const Mask none;
+  // subtree and strict ancestors of every node (parents precede children), and the nodes by (depth, index)
+  std::vector<Mask> below(N), above(N);
+  std::vector<int> order(N), at_depth(N + 2, 0);
+  for (int i = 0; i < N; ++i) {
+    if (parent[i] >= 0) { above[i] = above[parent[i]]; above[i].set(parent[i]); }
+    ++at_depth[depth[i] + 1];
+  }
+  for (int i = N - 1; i >= 0; --i) {
+    below[i].set(i);
+    if (parent[i] >= 0) below[parent[i]] |= below[i];
+  }
+  for (int d = 1; d < N + 2; ++d) at_depth[d] += at_depth[d - 1];
+  for (int i = 0; i < N; ++i) order[at_depth[depth[i]]++] = i;
   struct Atom { Mask emit, closure; int count; };
   std::vector<Atom> atoms;
-  // depth-first over the tree with an explicit stack (a = -1: children of the pre-tree state)
+  atoms.reserve(N);
+  // depth-first over the tree with an explicit stack
   std::vector<int> todo;
   for (int ci = coff[1] - 1; ci >= coff[0]; --ci) todo.push_back(clist[ci]);
   while (!todo.empty()) {
     const int c = todo.back();
     todo.pop_back();
     Atom at;
-    if (size[c] + depth[c] - 1 <= kCap) {            // the whole subtree and its ancestors fit
-      std::vector<int> st{c};
-      while (!st.empty()) {
-        const int n = st.back();
-        st.pop_back();
-        at.emit.set(n);
-        for (int k = coff[n + 1]; k < coff[n + 2]; ++k) st.push_back(clist[k]);
-      }
+    const int whole = below[c].count_without(none) + depth[c] - 1;
+    if (whole <= cap) {                              // the whole subtree and its ancestors fit
+      at.emit = below[c];
+      at.count = whole;
     } else {
       at.emit.set(c);
+      at.count = depth[c];
       for (int k = coff[c + 2] - 1; k >= coff[c + 1]; --k) todo.push_back(clist[k]);
     }
     at.closure = at.emit;
-    for (int a = parent[c]; a >= 0; a = parent[a]) at.closure.set(a);
-    at.count = (int)at.closure.count();
+    at.closure |= above[c];
     atoms.push_back(at);
   }
-  std::stable_sort(atoms.begin(), atoms.end(), [](const Atom& x, const Atom& y) { return x.count > y.count; });
+  std::vector<int> by_size(atoms.size());            // largest first, in order of discovery among equals
+  for (size_t a = 0; a < atoms.size(); ++a) by_size[a] = (int)a;
+  std::stable_sort(by_size.begin(), by_size.end(), [&](int x, int y) { return atoms[x].count > atoms[y].count; });
   std::vector<Atom> bins;
-  for (const Atom& at : atoms) {
+  for (int a : by_size) {
+    const Atom& at = atoms[a];
     int best = -1, best_growth = 0;
     for (int b = 0; b < (int)bins.size(); ++b) {
-      const int total = (int)(bins[b].closure | at.closure).count();
-      if (total > kCap) continue;
-      const int growth = total - bins[b].count;
+      const int growth = at.closure.count_without(bins[b].closure);
+      if (bins[b].count + growth > cap) continue;
       if (best < 0 || growth < best_growth) { best = b; best_growth = growth; }
     }
     if (best < 0) {
@@ -232,19 +256,18 @@ void build_gram_groups(const int32_t* parent, int N, const HostTree& t, std::vec
     } else {
       bins[best].emit |= at.emit;
       bins[best].closure |= at.closure;
-      bins[best].count = (int)bins[best].closure.count();
+      bins[best].count += best_growth;
     }
   }
   for (const Atom& bin : bins) {
     GramGroup g;
-    std::vector<int> all;
-    for (int n = 0; n < N; ++n)
-      if (bin.closure.test(n)) all.push_back(n);
-    std::sort(all.begin(), all.end(), [&](int x, int y) { return depth[x] != depth[y] ? depth[x] < depth[y] : x < y; });
-    for (int n : all) {
-      g.nodes.push_back(n);
-      g.emit.push_back(bin.emit.test(n) ? 1 : 0);
-    }
+    g.nodes.reserve(bin.count);
+    g.emit.reserve(bin.count);
+    for (int n : order)
+      if (bin.closure.test(n)) {
+        g.nodes.push_back(n);
+        g.emit.push_back(bin.emit.test(n) ? 1 : 0);
+      }
     out->push_back(std::move(g));
   }
 }

@@ -1,0 +1,67 @@
+"""The streamed scan (closed form, state in tensor memory) at its edges: groups of 32 nodes and what is left over, trees cut into
+groups that share one state or are dealt out to several CTAs, skipped and padded rows, both output types, and values that are
+not finite.  Bound: keys, values and queries enter exactly, the state, q~ and M diag(beta) as two bf16 terms each, which leaves
+2^-17 of every factor; products of at most 128 + 32 terms of the outputs' own size stay below 2^-17 * sqrt(160) = 1e-4."""
+import numpy as np
+import pytest
+import torch
+
+from synthetic import workload as W
+from synthetic.device_case import DeviceCase
+from tests.harness import assert_close, ctx, oracle_scan_from_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(N, B, Hk, Hv, L, depth, seed=0):
+    trees = [W.tree_random(W.IntStream(N + b + seed), N, depth) if N > 1 else [-1] for b in range(B)]
+    return W.make_case("stream", trees, seed=N + seed, Hk=Hk, Hv=Hv, d=128, in_dtype="bf16", n_layers=L, Ns=N + 3, permute_slots=True)
+
+
+@pytest.mark.parametrize("N,B,Hk,Hv,L,depth", [(1, 1, 2, 4, 1, 1), (2, 2, 1, 3, 1, 2), (15, 3, 4, 4, 2, 16), (16, 1, 2, 4, 3, 4), (17, 2, 2, 4, 1, 9),
+                                               (32, 1, 4, 8, 1, 16), (33, 1, 2, 4, 1, 6), (64, 1, 2, 4, 2, 5), (65, 2, 4, 8, 1, 16), (150, 1, 2, 6, 1, 12),
+                                               (256, 1, 4, 8, 1, 16), (256, 5, 16, 32, 2, 11), (100, 3, 8, 24, 5, 8)])
+@pytest.mark.parametrize("out_dtype", ["f32", "bf16"])
+def test_outputs_match_oracle(N, B, Hk, Hv, L, depth, out_dtype):
+    c = _case(N, B, Hk, Hv, L, depth)
+    if B > 1:
+        c.state_row[B - 1] = -1                       # a skipped sequence
+    dc = DeviceCase(ctx("tensor"), c, out_dtype=out_dtype)
+    for l in range(L):
+        dc.t("out", l).fill_(float("nan"))
+    dc.verify()
+    torch.cuda.synchronize()
+    ctx("auto")
+    for l in range(L):
+        ref, _, _ = oracle_scan_from_device(dc, layer=l)
+        worst = assert_close(dc.np("out", l), ref, bf16=out_dtype == "bf16", what=f"layer {l}")
+        assert out_dtype == "bf16" or worst < 1e-4
+        assert dc.np("status", l).tolist() == [0] * B
+        for b in range(B):
+            pad = sorted(set(range(c.Ns)) - set(c.slot[b].tolist()))
+            assert np.all(dc.np("out", l)[b, pad] == 0.0)
+
+
+@pytest.mark.parametrize("which", ["q", "k", "v"])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+@pytest.mark.parametrize("N,B,L", [(30, 3, 8), (150, 2, 3)])
+def test_values_that_are_not_finite_stay_on_their_paths(which, value, N, B, L):
+    """One element of one node: its descendants' outputs are gone (a query's: its own alone), every other output keeps its bits."""
+    c = _case(N, B, 16, 32, L, 9, seed=3)
+    dc = DeviceCase(ctx("tensor"), c, use_conv=False, qk_l2norm=True)
+    dc.verify()
+    torch.cuda.synchronize()
+    clean = dc.t("out", L - 1).clone()
+    node, b = N // 3, B - 1
+    dc.t(which, L - 1)[b, int(c.slot[b, node]), :, 77] = value
+    dc.verify()
+    torch.cuda.synchronize()
+    ctx("auto")
+    got = dc.t("out", L - 1)
+    below = np.zeros(N, dtype=bool)
+    for i in range(N):
+        below[i] = i == node or (which != "q" and c.parent[b, i] >= 0 and below[c.parent[b, i]])
+    gone = [int(c.slot[b, i]) for i in range(N) if below[i]]
+    kept = [int(c.slot[b, i]) for i in range(N) if not below[i]]
+    assert not torch.isfinite(got[b, gone]).all(dim=-1).any()
+    assert torch.equal(got[b, kept], clean[b, kept]) and torch.equal(got[:b], clean[:b])
