@@ -305,8 +305,8 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
     }
   }
   // one device allocation holding every table
-  std::vector<int32_t> h;
-  auto reserve = [&](size_t n) { size_t off = h.size(); h.resize(off + ((n + 3) / 4) * 4, 0); return off; };
+  size_t total = 0;
+  auto reserve = [&](size_t n) { const size_t off = total; total += (n + 3) / 4 * 4; return off; };
   const size_t o_parent = reserve((size_t)B * N), o_depth = reserve((size_t)B * N), o_slot = reserve((size_t)B * N);
   const size_t o_inv = reserve((size_t)B * Ns);
   const size_t o_prog = reserve((size_t)B * Ns);
@@ -341,6 +341,7 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   const size_t o_st_off = tc ? reserve(B + 1) : 0, o_st_meta = tc ? reserve(g32 * 32) : 0, o_st_anc = tc ? reserve(g32 * 32 * 4) : 0;
   const bool attn = Ns <= kMaxAttnSlots;
   const size_t o_vis = attn ? reserve((size_t)B * N * 8) : 0, o_used = attn ? reserve((size_t)B * 8) : 0;
+  std::vector<int32_t> h(total, 0);                  // sized once: growing table by table, it was copied and paged in several times over
   size_t gi = 0, sgi = 0;
   long long subst_rounds = 0, group_nodes = 0;     // over all groups: rounds of the substitution, nodes
   // a group's members: physical row | depth << 16 | emit << 24, and the positions of their ancestors, root first, then their own
