@@ -71,6 +71,22 @@ template <> struct Packed4<__nv_bfloat16> {
   }
 };
 
+// c + a[i] * b[j] of four-element packs.  bf16: products of two bf16 values and an fp32 sum in one instruction (sm_100), the same
+// bits as widening both first, which takes an instruction each.
+template <typename T>
+__device__ __forceinline__ float mul_add(const typename Packed4<T>::type& a, int i, const typename Packed4<T>::type& b, int j, float c) {
+  if constexpr (sizeof(T) == 2) {
+    const uint32_t aw = i & 2 ? a.y : a.x, bw = j & 2 ? b.y : b.x;
+    const unsigned short ah = i & 1 ? aw >> 16 : aw & 0xFFFF, bh = j & 1 ? bw >> 16 : bw & 0xFFFF;
+    float d;
+    asm("fma.rn.f32.bf16 %0, %1, %2, %3;" : "=f"(d) : "h"(ah), "h"(bh), "f"(c));
+    return d;
+  } else {
+    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+    return fmaf(av[i], bv[j], c);
+  }
+}
+
 // one-shot mbarrier for a bulk copy into shared memory
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init1(unsigned long long* bar) {
@@ -109,37 +125,30 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
 // memory by cp.async, every one exactly once and all at once, so that a window costs shared-memory loads only, wherever
 // its rows lie in the tree.
 //
-// The filter runs in transposed form: instead of the window a lane keeps, per channel, the three partial sums that the
-// children of the current node start from,
-//   a1 = w0 x_n,  a2 = w1 x_n + w0 x_p,  a3 = w2 x_n + w1 x_p + w0 x_pp       (p, pp: parent, grandparent of n)
-// so a node costs one FMA for its own output, y = w3 x_n + a3(parent), and three more only when the next entry descends
-// from it; siblings share the parent's sums and nothing moves between registers.  In the visiting order (leaf children
-// first) the next entry is a child of this one, or has the same parent (then this one is a leaf and left the sums
-// alone), or rebuilds the sums of its parent from its window.
+// An entry takes its four rows from there and is done: nothing is carried from one entry to the next.  (The transposed form,
+// which hands a parent's partial sums down, reads a row once instead of four times, but telling the cases apart, starting
+// sums over and pairing registers for them cost more: 105 against 70 warp instructions per entry and 128 channels.)
 // Every sum takes its taps oldest first from zero in fp32 (packed FMAs: two correctly rounded fp32 lanes per
 // instruction, same bits as scalar fmaf), bias last, SiLU in fp32, one round-to-nearest-even cast (Sec. "Precompute
 // branch histories while preserving arithmetic": tap order and cast points are part of the result).
 //
-// What bounds it: instruction issue and the special-function unit (the SiLU alone is 14 instructions, 8 of them
-// special-function operations, per four channels), with HBM behind them.  Measured against a register window fed by
-// prefetched rows: 48 layers of 4 x 32 nodes 71 -> 56 us, 32 x 256 nodes 92 -> 74 us, 8 x 64 nodes 15.2 -> 12.9 us.
+// What bounds it: HBM, with instruction issue (the SiLU alone is 14 instructions per four channels, 8 of them special-function
+// operations) close behind.
 
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
 // scan that follows writes them to the history buffer once every CTA of this kernel has finished).
-// What the main loop needs of an entry, in one 16-byte load: byte offset of its own row in the tile, physical row, and
-// what to do; its window (only looked at where an entry starts from it) as byte offsets, or ~visiting place for a row
-// that another CTA's part holds.
-enum : int { kConvPad = 1, kConvWindow = 2, kConvDescend = 4, kConvEnd = 8 };
-struct alignas(16) ConvEntry { int own, phys, what, pad; };
+// What the main loop needs of an entry, in one 16-byte load: its physical row, and its window as byte offsets in the tile,
+// oldest first, or ~visiting place for a row that another CTA's part holds.
+struct alignas(16) ConvEntry { int phys, w0, w1, w2; };
 
 template <typename T, int kRun, bool kFused, class LB>
 __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, const LB& lb, const ConvSplit& sp, const FusedPrevT<LB>* fp) {
   extern __shared__ __align__(128) unsigned char conv_smem[];            // [runs * kRun + 3 rows][groups * 128 channels]
   __shared__ ConvEntry s_entry[kConvMaxEntries];
-  __shared__ int4 s_win[kConvMaxEntries];
   __shared__ int f_acc[kFusedMaxPath], f_par[kFusedMaxPath], f_phys[kFusedMaxPath];
   __shared__ const T* f_hsrc[3];
+  using P4 = typename Packed4<T>::type;                // four elements as loaded
   const int b = blockIdx.y, layer = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int seg = (int)blockIdx.x >= sp.slabs ? blockIdx.x / sp.slabs : 0, slab = blockIdx.x - seg * sp.slabs;
@@ -150,20 +159,12 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   const int32_t* prog_g = t.conv_prog + (size_t)b * s.Ns;
   if (tid < entries) {                                 // descriptor tables: nobody writes them
     const int e = e0 + tid;
-    ConvEntry en = {tid * row_bytes, 0, kConvEnd, 0};
     if (e < s.Ns) {
-      const int prog = prog_g[e], flag = prog >> 16;
-      en.phys = prog & 0xFFFF;
-      en.what = flag == 3 ? kConvPad : (flag == 0 || (tid & (kRun - 1)) == 0) ? kConvWindow : 0;
-      // the last entry of a run hands its sums to nobody
-      if ((tid & (kRun - 1)) != kRun - 1 && e + 1 < s.Ns && prog_g[e + 1] >> 16 == 1) en.what |= kConvDescend;
-      if (en.what & kConvWindow) {
-        int4 w = *reinterpret_cast<const int4*>(t.win + ((size_t)b * s.Ns + e) * 4);
-        auto place = [&](int v) { return v < 0 ? (entries + 3 + v) * row_bytes : v >= e0 ? (v - e0) * row_bytes : ~v; };
-        s_win[tid] = make_int4(place(w.x), place(w.y), place(w.z), 0);
-      }
+      const int prog = prog_g[e];
+      const int4 w = *reinterpret_cast<const int4*>(t.win + ((size_t)b * s.Ns + e) * 4);
+      auto place = [&](int v) { return v < 0 ? (entries + 3 + v) * row_bytes : v >= e0 ? (v - e0) * row_bytes : ~v; };
+      s_entry[tid] = {prog & 0xFFFF, place(w.x), place(w.y), place(w.z)};
     }
-    s_entry[tid] = en;
   }
   pdl_wait();       // x, history and the operand buffers belong to earlier kernels until here
   pdl_trigger();
@@ -214,34 +215,32 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
     }
   cp_async_commit();
   // ---- taps and bias of this lane's channels, as pairs of neighbouring channels ------------------------------------
-  using P4 = typename Packed4<T>::type;                // four elements as loaded
   const int run = warp >> sp.log_groups, cg = (warp & (sp.groups - 1)) * 128 + lane * 4, c0 = cbase + cg;
   const bool mine = c0 < s.C;
-  float2 wp[4][2];                                     // tap j of channel pairs (0,1) and (2,3)
-  float2 bp[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  P4 taps[4];                                          // of channel c0 + e, oldest first
+  float bias[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) taps[e] = P4{};
   if (mine) {
     const T* w = reinterpret_cast<const T*>(L.conv_w) + (size_t)c0 * 4;
-    float4 wc[4];                                      // the taps of channel c0 + e
     if constexpr (sizeof(T) == 2) {
       const uint4 lo = *reinterpret_cast<const uint4*>(w), hi = *reinterpret_cast<const uint4*>(w + 8);
-      wc[0] = Packed4<T>::unpack(make_uint2(lo.x, lo.y)); wc[1] = Packed4<T>::unpack(make_uint2(lo.z, lo.w));
-      wc[2] = Packed4<T>::unpack(make_uint2(hi.x, hi.y)); wc[3] = Packed4<T>::unpack(make_uint2(hi.z, hi.w));
+      taps[0] = make_uint2(lo.x, lo.y); taps[1] = make_uint2(lo.z, lo.w);
+      taps[2] = make_uint2(hi.x, hi.y); taps[3] = make_uint2(hi.z, hi.w);
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) wc[e] = *reinterpret_cast<const float4*>(w + e * 4);
+      for (int e = 0; e < 4; ++e) taps[e] = *reinterpret_cast<const float4*>(w + e * 4);
     }
-    wp[0][0] = make_float2(wc[0].x, wc[1].x); wp[0][1] = make_float2(wc[2].x, wc[3].x);
-    wp[1][0] = make_float2(wc[0].y, wc[1].y); wp[1][1] = make_float2(wc[2].y, wc[3].y);
-    wp[2][0] = make_float2(wc[0].z, wc[1].z); wp[2][1] = make_float2(wc[2].z, wc[3].z);
-    wp[3][0] = make_float2(wc[0].w, wc[1].w); wp[3][1] = make_float2(wc[2].w, wc[3].w);
     if (L.conv_b) {
       const float4 bv = Packed4<T>::unpack(*reinterpret_cast<const P4*>(reinterpret_cast<const T*>(L.conv_b) + c0));
-      bp[0] = make_float2(bv.x, bv.y);
-      bp[1] = make_float2(bv.z, bv.w);
+      bias[0] = bv.x; bias[1] = bv.y; bias[2] = bv.z; bias[3] = bv.w;
     }
   }
   cp_async_wait<0>();
   __syncthreads();
+  const int first = e0 + run * kRun, live = seq_ok ? min(s.N - first, kRun) : 0;       // padding rows come last
+  const ConvEntry* ent = s_entry + run * kRun;
+  const bool elsewhere = __any_sync(0xffffffffu, lane < live && (ent[lane].w0 | ent[lane].w1 | ent[lane].w2) < 0);
   if (!mine) return;
   const bool has_bias = L.conv_b != nullptr;
   const int hkd = s.Hk * s.d;
@@ -253,44 +252,38 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   dst += (size_t)b * s.Ns * dst_stride;
   const unsigned char* tile = conv_smem + cg * (int)sizeof(T);
   const float2 zero2 = make_float2(0.f, 0.f);
-  auto window = [&](int at) -> float4 {                // a row of the window: staged, or in another CTA's part
-    if (at < 0) return Packed4<T>::unpack(*reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)(prog_g[~at] & 0xFFFF) * (uint32_t)s.C)));
-    return Packed4<T>::unpack(*reinterpret_cast<const P4*>(tile + at));
+  const unsigned char* own = tile + run * kRun * row_bytes;
+  auto put = [&](int phys, float2 y0, float2 y1) {
+    T* d = dst + (size_t)((uint32_t)phys * dst_stride);
+    if constexpr (sizeof(T) == 2) {
+      __nv_bfloat162 h01 = __floats2bfloat162_rn(y0.x, y0.y), h23 = __floats2bfloat162_rn(y1.x, y1.y);
+      *reinterpret_cast<uint2*>(d) = make_uint2(*reinterpret_cast<uint32_t*>(&h01), *reinterpret_cast<uint32_t*>(&h23));
+    } else {
+      *reinterpret_cast<float4*>(d) = make_float4(y0.x, y0.y, y1.x, y1.y);
+    }
   };
-  float2 a1[2] = {zero2, zero2}, a2[2] = {zero2, zero2}, a3[2] = {zero2, zero2};   // channel pairs (0,1) and (2,3)
-  const ConvEntry* ent = s_entry + run * kRun;
+  auto entries_of_run = [&](auto elsewhere_c) {        // elsewhere: a window reaches into another CTA's part
+    auto row = [&](int at) -> P4 { return *reinterpret_cast<const P4*>(tile + at); };
+    auto row_anywhere = [&](int at) -> P4 {
+      if (at >= 0) return row(at);
+      return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)(prog_g[~at] & 0xFFFF) * (uint32_t)s.C));
+    };
 #pragma unroll 4
-  for (int rr = 0; rr < kRun; ++rr) {                  // bounded: kRun
-    const int4 en = *reinterpret_cast<const int4*>(ent + rr);   // own, phys, what
-    if (en.z & kConvEnd) break;                        // beyond the last entry (uniform over the warp)
-    T* d = dst + (size_t)((uint32_t)en.y * dst_stride);
-    float2 y[2] = {zero2, zero2};
-    if (!(en.z & kConvPad) && seq_ok) {                // padding rows and skipped sequences: zero rows
-      const float4 o4 = Packed4<T>::unpack(*reinterpret_cast<const P4*>(tile + en.x));
-      const float2 own[2] = {make_float2(o4.x, o4.y), make_float2(o4.z, o4.w)};
-      if (en.z & kConvWindow) {                        // the parent's sums from its window
-        const int4 wi = s_win[run * kRun + rr];
-        const float4 w0 = window(wi.x), w1 = window(wi.y), w2 = window(wi.z);
-        const float2 v0[2] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w)}, v1[2] = {make_float2(w1.x, w1.y), make_float2(w1.z, w1.w)},
-                     v2[2] = {make_float2(w2.x, w2.y), make_float2(w2.z, w2.w)};
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          a3[e] = __ffma2_rn(wp[2][e], v2[e], __ffma2_rn(wp[1][e], v1[e], __ffma2_rn(wp[0][e], v0[e], zero2)));
-          a2[e] = __ffma2_rn(wp[1][e], v2[e], __ffma2_rn(wp[0][e], v1[e], zero2));
-          a1[e] = __ffma2_rn(wp[0][e], v2[e], zero2);
-        }
+    for (int rr = 0; rr < live; ++rr) {                // bounded: kRun
+      const ConvEntry en = ent[rr];
+      const P4 r3 = *reinterpret_cast<const P4*>(own + rr * row_bytes);
+      P4 r0, r1, r2;
+      if (decltype(elsewhere_c)::value && __builtin_expect((en.w0 | en.w1 | en.w2) < 0, 0)) {    // uniform
+        r0 = row_anywhere(en.w0); r1 = row_anywhere(en.w1); r2 = row_anywhere(en.w2);
+      } else {
+        r0 = row(en.w0); r1 = row(en.w1); r2 = row(en.w2);
       }
+      float a[4];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) y[e] = __ffma2_rn(wp[3][e], own[e], a3[e]);
-      if (en.z & kConvDescend) {                       // the next entry is a child of this one
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          a3[e] = __ffma2_rn(wp[2][e], own[e], a2[e]);
-          a2[e] = __ffma2_rn(wp[1][e], own[e], a1[e]);
-          a1[e] = __ffma2_rn(wp[0][e], own[e], zero2);
-        }
-      }
-      if (has_bias) { y[0] = __fadd2_rn(y[0], bp[0]); y[1] = __fadd2_rn(y[1], bp[1]); }   // bias last
+      for (int e = 0; e < 4; ++e)
+        a[e] = mul_add<T>(taps[e], 3, r3, e, mul_add<T>(taps[e], 2, r2, e, mul_add<T>(taps[e], 1, r1, e, mul_add<T>(taps[e], 0, r0, e, 0.f))));
+      if (has_bias) { a[0] += bias[0]; a[1] += bias[1]; a[2] += bias[2]; a[3] += bias[3]; }   // bias last
+      float2 y[2] = {make_float2(a[0], a[1]), make_float2(a[2], a[3])};
       // SiLU a / (1 + 2^(-a log2 e)) with the hardware exponential and reciprocal (1e-6 relative, far
       // below the rounding of the recorded operand); the multiplies and the add are packed
       const float2 nl2e = make_float2(-1.4426950408889634f, -1.4426950408889634f), one = make_float2(1.f, 1.f);
@@ -300,14 +293,12 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
         ex = __fadd2_rn(make_float2(ex2_approx(ex.x), ex2_approx(ex.y)), one);
         y[e] = __fmul2_rn(y[e], make_float2(rcp_approx(ex.x), rcp_approx(ex.y)));
       }
+      put(en.phys, y[0], y[1]);
     }
-    if constexpr (sizeof(T) == 2) {
-      __nv_bfloat162 h01 = __floats2bfloat162_rn(y[0].x, y[0].y), h23 = __floats2bfloat162_rn(y[1].x, y[1].y);
-      *reinterpret_cast<uint2*>(d) = make_uint2(*reinterpret_cast<uint32_t*>(&h01), *reinterpret_cast<uint32_t*>(&h23));
-    } else {
-      *reinterpret_cast<float4*>(d) = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
-    }
-  }
+  };
+  if (elsewhere) entries_of_run(std::true_type{});
+  else entries_of_run(std::false_type{});
+  for (int rr = max(live, 0); rr < min(s.Ns - first, kRun); ++rr) put(ent[rr].phys, zero2, zero2);   // padding rows, skipped sequences
 }
 
 template <typename T, int kRun, class LB>
