@@ -22,7 +22,12 @@
 // whether it is needed, and a reduction is one exchange: every CTA stores its partial into all CTAs of the cluster, one cluster barrier, and every warp adds up the
 // same values in the same order; the residual at the next candidate's token travels with it.  Measured on 151,936 entries against passes through global
 // memory and two barriers per candidate: rejection sampling 1 sequence 26.9 -> 23.4 us, 8 sequences 47.9 -> 36.8 us, 16
-// sequences 68 -> 52 us; greedy 16 sequences 18.0 -> 15.5 us.
+// sequences 68 -> 52 us; greedy 16 sequences 18.0 -> 15.5 us.  The race divides few entries, a candidate's uniform and probability
+// are asked for ahead of the reduction before its test, proposals are widened by integer instructions, and a pack's place in the
+// slice is looked up once: 8 sequences 42.4 -> 34.9 us, 1 sequence 17.2 -> 14.0, 2 of 131,071 entries 26.7 -> 22.6 (other inputs
+// than the figures before).
+// Staging the target row of the candidate under test too, so that an accepted one costs no wait, gained nothing (8 sequences 42.5 ->
+// 42.1, 1 sequence 17.2 -> 17.9): a level's time goes into its passes and reductions.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -52,6 +57,9 @@ __device__ __forceinline__ int entry_of(int k, int j) {
   return kVec ? 4 * (k * kAcceptThreads + (int)threadIdx.x) + j : (4 * k + j) * kAcceptThreads + (int)threadIdx.x;
 }
 constexpr int kPack = 4 * kAcceptThreads;          // entries of a pack over the CTA
+// whether a slice of n entries (a multiple of four where kVec) has that place
+template <bool kVec>
+__device__ __forceinline__ bool in_slice(int k, int j, int n) { return entry_of<kVec>(k, kVec ? 0 : j) < n; }
 constexpr int kFlight = 5;                         // packs requested together
 // where the residual of that entry is kept: neighbouring threads, neighbouring places (no bank conflicts either way)
 __device__ __forceinline__ int place_of(int k, int j) { return (4 * k + j) * kAcceptThreads + (int)threadIdx.x; }
@@ -104,6 +112,15 @@ __device__ __forceinline__ void stage_row(float* dst, const float* row, int n) {
   }
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// (double)f.  The conversion instruction takes 16 lanes a clock and SM, and an update needs three per entry; for a positive
+// normal number it is three integer instructions.
+__device__ __forceinline__ double widen(float f) {
+  const uint32_t u = __float_as_uint(f);
+  if (u - 0x00800000u >= 0x7F000000u) return (double)f;        // zero, denormal, negative, infinite, NaN
+  return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
+__device__ __forceinline__ float rcp_approx(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
 struct Cluster {
   cg::cluster_group cl;
@@ -239,6 +256,13 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int32
       auto holds = [&](int x) { return x >= v_lo && x < v_lo + n && tid == holder_of<kVec>(x - v_lo); };
       auto token_of = [&](int ci) { return ci < c_hi ? tok_of_node[child_list[ci]] : -1; };
       double at_x = 0.0;                                      // residual at the token under test
+      float u_x = 0.f, q_x = 0.f;                             // the candidate's uniform, its proposal's probability of the token
+      auto candidate = [&](int ci) {                          // requested ahead of the reduction that the test waits for
+        if (ci >= c_hi) return;
+        const int ch = child_list[ci];
+        u_x = __ldg(a.uniforms + (size_t)b * Ns + slot_map[ch]);
+        q_x = __ldg(proposal(ch) - v_lo + tok_of_node[ch]);
+      };
       auto finish = [&](const double (&z)[4], int x) {
         const bool here = holds(x);
         return c.sum((z[0] + z[1]) + (z[2] + z[3]), here, here ? (double)r[kShared ? place_of_entry<kVec>(x - v_lo) : x - v_lo] : 0.0, &at_x);
@@ -258,13 +282,14 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int32
                   });
         return finish(z, x);
       };
+      candidate(c_lo);
       request(c_lo);
       double Z = start(token_of(c_lo));
       for (int ci = c_lo; ci < c_hi; ++ci) {                  // bounded: children of one node
-        const int ch = child_list[ci], sc = slot_map[ch], x = tok_of_node[ch];
+        const int ch = child_list[ci];
         const float* q = proposal(ch);
         // every CTA evaluates the same test on the same values
-        const double lhs = __dmul_rn(__dmul_rn((double)a.uniforms[(size_t)b * Ns + sc], (double)__ldg(q - v_lo + x)), Z);
+        const double lhs = __dmul_rn(__dmul_rn((double)u_x, (double)q_x), Z);
         if (lhs < at_x) { took = ch; break; }
         if constexpr (kShared) stage_wait();
         double z[4] = {0.0, 0.0, 0.0, 0.0};
@@ -280,13 +305,14 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int32
                     const float qv[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                      if (entry_of<kVec>(k, j) < n) {
-                        const double d = __dsub_rn((double)get(k, j), __dmul_rn(Z, (double)qv[j]));
+                      if (in_slice<kVec>(k, j, n)) {
+                        const double d = __dsub_rn((double)get(k, j), __dmul_rn(Z, widen(qv[j])));
                         const double rd = (double)(float)(d > 0.0 ? d : 0.0);
                         put(k, j, (R)rd);
                         z[j] += rd;
                       }
                   });
+        candidate(ci + 1);
         request(ci + 1);
         const int nx = token_of(ci + 1);
         const double Zn = finish(z, nx);
@@ -297,19 +323,45 @@ accept_kernel(TreeDev t, int N, int Ns, AcceptView a, int lmax, int chunk, int32
         const float* noise = a.noise + (size_t)b * V + v_lo;
         float bv = -1.f;
         int bi = 0x7fffffff;
-        float4 w[kFlight];
-        for_packs(packs, [&](int k, int i) { w[i] = load_pack<kVec>(noise, n, k, 1.f); },
-                  [&](int k, int i) {
-                    const float nv[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+        // Correctly rounded quotients only for entries that may be the largest: what r times an approximate 1 / e (to 2^-21) puts
+        // below the warp's best by more than 2^-18 of it is not.  Outside 2^-100 .. 2^100 (denormals, zeros, infinities) all
+        // entries are divided.  (All of them always: 9 to 15 thousand cycles of a walk's 30 to 70.)
+        float top = 0.f;
+        for (int k0 = 0; k0 < packs; k0 += kFlight) {          // bounded: the slice
+          float4 w[kFlight];
+          float about[4 * kFlight];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                      const int e = entry_of<kVec>(k, j);
-                      if (e < n) {
-                        const float key = __fdiv_rn((float)get(k, j), nv[j]);
-                        if (key > bv) { bv = key; bi = v_lo + e; }
-                      }
-                    }
-                  });
+          for (int i = 0; i < kFlight; ++i)
+            if (k0 + i < packs) w[i] = load_pack<kVec>(noise, n, k0 + i, 1.f);
+          float best = 0.f;
+          uint32_t mine = 0;
+#pragma unroll
+          for (int i = 0; i < kFlight; ++i) {
+            const float nv[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              about[4 * i + j] = 0.f;
+              if (k0 + i < packs && in_slice<kVec>(k0 + i, j, n)) {
+                mine |= 1u << (4 * i + j);
+                about[4 * i + j] = (float)get(k0 + i, j) * rcp_approx(nv[j]);
+                best = fmaxf(best, about[4 * i + j]);
+              }
+            }
+          }
+          top = fmaxf(top, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(best))));
+          const bool plain = top >= 0x1p-100f && top <= 0x1p100f;
+          const float line = top * (1.f - 0x1p-18f);
+          uint32_t closer = mine;
+#pragma unroll
+          for (int i = 0; i < 4 * kFlight; ++i)
+            if (plain && about[i] < line) closer &= ~(1u << i);
+          while (closer) {                                      // bounded: 20; ascending entries
+            const int i = __ffs(closer) - 1, k = k0 + (i >> 2), j = i & 3, e = entry_of<kVec>(k, j);
+            closer &= closer - 1;
+            const float key = __fdiv_rn((float)get(k, j), __ldg(noise + e));
+            if (key > bv) { bv = key; bi = v_lo + e; }
+          }
+        }
         nxt = c.argmax(bv, bi);
       } else if constexpr (kShared) {
         stage_wait();                                          // the row that turned out not to be needed
