@@ -127,13 +127,15 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
 //
 // An entry takes its four rows from there and is done: nothing is carried from one entry to the next.  (The transposed form,
 // which hands a parent's partial sums down, reads a row once instead of four times, but telling the cases apart, starting
-// sums over and pairing registers for them cost more: 105 against 70 warp instructions per entry and 128 channels.)
+// sums over and pairing registers for them cost more: 101 against 76 warp instructions per entry and 128 channels, 48 layers.)
 // Every sum takes its taps oldest first from zero in fp32 (packed FMAs: two correctly rounded fp32 lanes per
 // instruction, same bits as scalar fmaf), bias last, SiLU in fp32, one round-to-nearest-even cast (Sec. "Precompute
 // branch histories while preserving arithmetic": tap order and cast points are part of the result).
 //
-// What bounds it: HBM, with instruction issue (the SiLU alone is 14 instructions per four channels, 8 of them special-function
-// operations) close behind.
+// What bounds it: instruction issue (70 % of the slots; the SiLU alone is 14 instructions per four channels, 8 of them special-
+// function operations, whose unit is half busy) with HBM close behind.  Measured against the transposed form: 48 layers of 4 x 32
+// nodes 51.4 -> 43.0 us, 32 x 256 nodes 70.0 -> 66.0, 8 x 64 nodes 11.9 -> 11.4.  Five or six CTAs per SM instead of four spill: 46.7
+// and 50.0 us against 44.5; two entries at a time instead of eight 44.5.
 
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
@@ -268,7 +270,7 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
       if (at >= 0) return row(at);
       return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)(prog_g[~at] & 0xFFFF) * (uint32_t)s.C));
     };
-#pragma unroll 4
+#pragma unroll 8
     for (int rr = 0; rr < live; ++rr) {                // bounded: kRun
       const ConvEntry en = ent[rr];
       const P4 r3 = *reinterpret_cast<const P4*>(own + rr * row_bytes);
