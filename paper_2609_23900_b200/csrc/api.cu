@@ -334,13 +334,14 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
         tab.insert(tab.end(), gr.emit.begin(), gr.emit.end());
       }
     }
+  const bool attn = Ns <= kMaxAttnSlots;
+  const size_t o_vis = attn ? reserve((size_t)B * N * 8) : 0, o_used = attn ? reserve((size_t)B * 8) : 0;
+  const size_t n_trees = total;                      // what follows lies in the second allocation
   const size_t G = (size_t)d->n_groups;
   const size_t o_tc_group = tc ? reserve(G * 4) : 0, o_tc_meta = tc ? reserve(G * 64) : 0;
   const size_t o_tc_anc = tc ? reserve(G * 64 * 4) : 0, o_tc_lvl = tc ? reserve(G * 5) : 0;
   const size_t g32 = (size_t)d->st_groups;
   const size_t o_st_off = tc ? reserve(B + 1) : 0, o_st_meta = tc ? reserve(g32 * 32) : 0, o_st_anc = tc ? reserve(g32 * 32 * 4) : 0;
-  const bool attn = Ns <= kMaxAttnSlots;
-  const size_t o_vis = attn ? reserve((size_t)B * N * 8) : 0, o_used = attn ? reserve((size_t)B * 8) : 0;
   std::vector<int32_t> h(total, 0);                  // sized once: growing table by table, it was copied and paged in several times over
   size_t gi = 0, sgi = 0;
   long long subst_rounds = 0, group_nodes = 0;     // over all groups: rounds of the substitution, nodes
@@ -453,22 +454,29 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
   d->tensor_tail_pays = tc && 450 * subst_rounds > 300 * (long long)G + 78 * group_nodes;
   if (ctx->device < 0) { *out = d; return LUMO_OK; }   // host-only: tables stay on the host
   DeviceGuard g(ctx->device);
-  cudaError_t e = cudaMalloc(&d->dev, h.size() * sizeof(int32_t));
-  if (e != cudaSuccess) { delete d; return cuda_fail(ctx, e, "cudaMalloc(tree tables)"); }
-  e = set_up(ctx, [&](cudaStream_t st) { return cudaMemcpyAsync(d->dev, h.data(), h.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st); });
-  if (e != cudaSuccess) { cudaFree(d->dev); delete d; return cuda_fail(ctx, e, "cudaMemcpy(tree tables)"); }
+  cudaError_t e = cudaMalloc(&d->dev, n_trees * sizeof(int32_t));
+  if (e == cudaSuccess && total > n_trees) e = cudaMalloc(&d->dev_groups, (total - n_trees) * sizeof(int32_t));
+  if (e != cudaSuccess) { lumo_tree_desc_destroy(d); return cuda_fail(ctx, e, "cudaMalloc(tree tables)"); }
+  e = set_up(ctx, [&](cudaStream_t st) {
+    cudaError_t c = cudaMemcpyAsync(d->dev, h.data(), n_trees * sizeof(int32_t), cudaMemcpyHostToDevice, st);
+    if (c == cudaSuccess && total > n_trees)
+      c = cudaMemcpyAsync(d->dev_groups, h.data() + n_trees, (total - n_trees) * sizeof(int32_t), cudaMemcpyHostToDevice, st);
+    return c;
+  });
+  if (e != cudaSuccess) { lumo_tree_desc_destroy(d); return cuda_fail(ctx, e, "cudaMemcpy(tree tables)"); }
   d->d_parent = d->dev + o_parent; d->d_depth = d->dev + o_depth; d->d_slot = d->dev + o_slot;
   d->d_slot_inv = d->dev + o_inv; d->d_win = d->dev + o_winv; d->d_conv_prog = d->dev + o_prog;
   d->d_child_off = d->dev + o_coff; d->d_child_list = d->dev + o_clist;
   for (int w = 0; w < 2; ++w) { d->d_sched[w] = d->dev + o_sched[w]; d->d_nops[w] = d->dev + o_nops[w]; }
   if (tc) {
-    d->d_tc_group = d->dev + o_tc_group;
-    d->d_tc_meta = d->dev + o_tc_meta;
-    d->d_tc_anc = reinterpret_cast<uint8_t*>(d->dev + o_tc_anc);
-    d->d_tc_lvl = reinterpret_cast<uint8_t*>(d->dev + o_tc_lvl);
-    d->d_st_off = d->dev + o_st_off;
-    d->d_st_meta = d->dev + o_st_meta;
-    d->d_st_anc = reinterpret_cast<uint8_t*>(d->dev + o_st_anc);
+    auto group_table = [&](size_t o) { return d->dev_groups + (o - n_trees); };
+    d->d_tc_group = group_table(o_tc_group);
+    d->d_tc_meta = group_table(o_tc_meta);
+    d->d_tc_anc = reinterpret_cast<uint8_t*>(group_table(o_tc_anc));
+    d->d_tc_lvl = reinterpret_cast<uint8_t*>(group_table(o_tc_lvl));
+    d->d_st_off = group_table(o_st_off);
+    d->d_st_meta = group_table(o_st_meta);
+    d->d_st_anc = reinterpret_cast<uint8_t*>(group_table(o_st_anc));
   }
   if (attn) {
     d->d_vis = reinterpret_cast<uint32_t*>(d->dev + o_vis);
@@ -483,6 +491,7 @@ void lumo_tree_desc_destroy(lumo_tree_desc* desc) {
   if (desc->dev) {
     DeviceGuard g(desc->ctx->device);
     cudaFree(desc->dev);
+    cudaFree(desc->dev_groups);
   }
   delete desc;
 }

@@ -69,8 +69,8 @@ struct lumo_tree_desc {
   lumo_ctx* ctx = nullptr;
   int B = 0, N = 0, Ns = 0;
   std::vector<lumo::HostTree> trees;     // per sequence
-  // device tables (one allocation), all int32
-  int32_t* dev = nullptr;
+  // device tables, all int32, in two allocations: above 1 MiB the driver maps memory for each instead of cutting it from a block
+  int32_t *dev = nullptr, *dev_groups = nullptr;     // the trees and attention masks; the scans' groups
   int32_t* d_parent = nullptr;    // [B, N]
   int32_t* d_depth = nullptr;     // [B, N]
   int32_t* d_slot = nullptr;      // [B, N]
