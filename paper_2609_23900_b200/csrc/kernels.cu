@@ -270,13 +270,19 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
       if (at >= 0) return row(at);
       return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)(prog_g[~at] & 0xFFFF) * (uint32_t)s.C));
     };
+    P4 far0 = {}, far1 = {}, far2 = {};                // the last window that reached elsewhere, and the parent it belongs to
+    int of = INT_MIN;
 #pragma unroll 8
     for (int rr = 0; rr < live; ++rr) {                // bounded: kRun
       const ConvEntry en = ent[rr];
       const P4 r3 = *reinterpret_cast<const P4*>(own + rr * row_bytes);
       P4 r0, r1, r2;
       if (decltype(elsewhere_c)::value && __builtin_expect((en.w0 | en.w1 | en.w2) < 0, 0)) {    // uniform
-        r0 = row_anywhere(en.w0); r1 = row_anywhere(en.w1); r2 = row_anywhere(en.w2);
+        if (en.w2 != of) {                             // siblings follow one another: a star's root is fetched once, not 255 times
+          far0 = row_anywhere(en.w0); far1 = row_anywhere(en.w1); far2 = row_anywhere(en.w2);
+          of = en.w2;
+        }
+        r0 = far0; r1 = far1; r2 = far2;
       } else {
         r0 = row(en.w0); r1 = row(en.w1); r2 = row(en.w2);
       }
