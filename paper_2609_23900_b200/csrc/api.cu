@@ -379,8 +379,8 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
     for (int i = 0; i < N + 2; ++i) h[o_coff + (size_t)b * (N + 2) + i] = t.tab[LUMO_TAB_CHILD_OFF][i];
     for (int i = 0; i < N; ++i) h[o_clist + (size_t)b * N + i] = t.tab[LUMO_TAB_CHILD_LIST][i];
     {
-      // conv visiting order: depth-first preorder, a node's leaf children before its other children, so that most
-      // entries continue from their parent or share it with the entry before (flags 1 and 2)
+      // conv visiting order: depth-first preorder, a node's leaf children before its other children: siblings that are leaves
+      // follow one another, and a part of the order reaches into few rows of another
       const auto& coff = t.tab[LUMO_TAB_CHILD_OFF];
       const auto& clist = t.tab[LUMO_TAB_CHILD_LIST];
       const auto& leaf = t.tab[LUMO_TAB_IS_LEAF];
@@ -400,14 +400,7 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
       size_t k = 0;
       for (size_t pidx = 0; pidx < order.size(); ++pidx, ++k) {
         const int n = order[pidx];
-        int flag = 0;
-        if (pidx > 0) {
-          const int prev = order[pidx - 1];
-          const int pn = parent[(size_t)b * N + n], pp = parent[(size_t)b * N + prev];
-          if (pn == prev) flag = 1;
-          else if (pn == pp) flag = 2;
-        }
-        h[o_prog + (size_t)b * Ns + k] = h[o_slot + (size_t)b * N + n] | (flag << 16);
+        h[o_prog + (size_t)b * Ns + k] = h[o_slot + (size_t)b * N + n];
         // the older entries of its window, as places in this order (or -1..-3 = history rows)
         for (int j = 0; j < 4; ++j) {
           const int w = t.tab[LUMO_TAB_ANC_WIN][n * 4 + j];
@@ -415,7 +408,7 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
         }
       }
       for (int sidx = 0; sidx < Ns; ++sidx)
-        if (t.tab[LUMO_TAB_SLOT_INV][sidx] < 0) h[o_prog + (size_t)b * Ns + k++] = sidx | (3 << 16);
+        if (t.tab[LUMO_TAB_SLOT_INV][sidx] < 0) h[o_prog + (size_t)b * Ns + k++] = sidx;
     }
     for (int w = 0; w < 2; ++w) {
       const auto& ops = t.tab[LUMO_TAB_SCHEDULE + w];

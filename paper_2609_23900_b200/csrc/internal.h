@@ -78,9 +78,7 @@ struct lumo_tree_desc {
   int32_t* d_win = nullptr;       // [B, Ns, 4] per entry of the conv visiting order: the window as places in that order, -1/-2/-3 = history rows
   int32_t* d_child_off = nullptr; // [B, N+2]
   int32_t* d_child_list = nullptr;// [B, N]
-  int32_t* d_conv_prog = nullptr; // [B, Ns] conv visiting order (depth first, leaf children first, padding rows last): physical row
-                                  // | flag << 16; flag 0 = starts from its window, 1 = the previous entry is the parent, 2 = same
-                                  // parent as the previous entry (a leaf), 3 = padding row (zeros)
+  int32_t* d_conv_prog = nullptr; // [B, Ns] conv visiting order (depth first, leaf children first, padding rows last): physical rows
   int32_t* d_sched[2] = {nullptr, nullptr};   // [B, max_ops]  lean / full (every node's state materialised)
   int32_t* d_nops[2] = {nullptr, nullptr};    // [B]
   int max_ops[2] = {0, 0};

@@ -162,10 +162,9 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   if (tid < entries) {                                 // descriptor tables: nobody writes them
     const int e = e0 + tid;
     if (e < s.Ns) {
-      const int prog = prog_g[e];
       const int4 w = *reinterpret_cast<const int4*>(t.win + ((size_t)b * s.Ns + e) * 4);
       auto place = [&](int v) { return v < 0 ? (entries + 3 + v) * row_bytes : v >= e0 ? (v - e0) * row_bytes : ~v; };
-      s_entry[tid] = {prog & 0xFFFF, place(w.x), place(w.y), place(w.z)};
+      s_entry[tid] = {prog_g[e], place(w.x), place(w.y), place(w.z)};
     }
   }
   pdl_wait();       // x, history and the operand buffers belong to earlier kernels until here
@@ -185,7 +184,7 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
     const T* src = xb + col;
 #pragma unroll 4
     for (int e = tid >> log_cols; e < live; e += step)
-      cp_async16(mycol + e * row_bytes, src + (size_t)((uint32_t)(prog_g[e0 + e] & 0xFFFF) * (uint32_t)s.C));
+      cp_async16(mycol + e * row_bytes, src + (size_t)((uint32_t)prog_g[e0 + e] * (uint32_t)s.C));
   }
   const T* hbase = reinterpret_cast<const T*>(L.conv_hist) + (size_t)(seq_ok ? row : 0) * 3 * s.C;
   if constexpr (kFused) {
@@ -268,7 +267,7 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
     auto row = [&](int at) -> P4 { return *reinterpret_cast<const P4*>(tile + at); };
     auto row_anywhere = [&](int at) -> P4 {
       if (at >= 0) return row(at);
-      return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)(prog_g[~at] & 0xFFFF) * (uint32_t)s.C));
+      return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)prog_g[~at] * (uint32_t)s.C));
     };
     P4 far0 = {}, far1 = {}, far2 = {};                // the last window that reached elsewhere, and the parent it belongs to
     int of = INT_MIN;

@@ -570,7 +570,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
     *reinterpret_cast<uint4*>(smem + kOffMb + tid * 16) = make_uint4(0, 0, 0, 0);
     if (rarely(cur.lead && s.Ns > s.N)) {
       for (int e = s.N + r16; e < s.Ns; e += 16) {              // padding rows, last in the convolution's visiting order
-        const uint32_t ps = (uint32_t)t.conv_prog[(size_t)cur.b * s.Ns + e] & 0xFFFFu;
+        const uint32_t ps = (uint32_t)t.conv_prog[(size_t)cur.b * s.Ns + e];
         for (int c = c16 * 16; c < kD * out_size; c += 256) *reinterpret_cast<uint4*>(const_cast<unsigned char*>(cur.out) + (size_t)ps * v_pitch * out_size + c) = make_uint4(0, 0, 0, 0);
       }
     }
