@@ -3,7 +3,8 @@
     python -m paper_2609_23900_b200.build [--force] [--verbose]
 
 nvcc cross-compiles without a GPU.  The shared object is placed next to this file so
-that it travels with the source tree.
+that it travels with the source tree; what ptxas says of each kernel (registers, spills)
+is kept beside the object files, in build/<source>.ptxas.
 """
 from __future__ import annotations
 
@@ -46,13 +47,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(os.path.join(HERE, "build"), exist_ok=True)
     for src in SOURCES:
         obj = os.path.join(HERE, "build", src + ".o")
-        cmd = [_nvcc(), *NVCC_FLAGS, "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-x", "cu",
+        cmd = [_nvcc(), *NVCC_FLAGS, "-Xptxas", "-v", "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-x", "cu",
                "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
-            cmd.insert(1, "-Xptxas")
-            cmd.insert(2, "-v")
             print(" ".join(cmd), flush=True)
-        subprocess.check_call(cmd)
+        done = subprocess.run(cmd, stderr=subprocess.PIPE, text=True)
+        if verbose or done.returncode:
+            print(done.stderr, file=sys.stderr, flush=True)
+        done.check_returncode()
+        with open(os.path.join(HERE, "build", src + ".ptxas"), "w") as f:
+            f.write(done.stderr)
         objs.append(obj)
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.check_call([_nvcc(), "-shared", "-gencode", "arch=compute_100a,code=sm_100a", *objs, "-o", tmp])

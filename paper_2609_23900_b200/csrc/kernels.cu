@@ -71,21 +71,55 @@ template <> struct Packed4<__nv_bfloat16> {
   }
 };
 
-// c + a[i] * b[j] of four-element packs.  bf16: products of two bf16 values and an fp32 sum in one instruction (sm_100), the same
-// bits as widening both first, which takes an instruction each.
-template <typename T>
-__device__ __forceinline__ float mul_add(const typename Packed4<T>::type& a, int i, const typename Packed4<T>::type& b, int j, float c) {
-  if constexpr (sizeof(T) == 2) {
-    const uint32_t aw = i & 2 ? a.y : a.x, bw = j & 2 ? b.y : b.x;
-    const unsigned short ah = i & 1 ? aw >> 16 : aw & 0xFFFF, bh = j & 1 ? bw >> 16 : bw & 0xFFFF;
-    float d;
-    asm("fma.rn.f32.bf16 %0, %1, %2, %3;" : "=f"(d) : "h"(ah), "h"(bh), "f"(c));
-    return d;
-  } else {
-    const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-    return fmaf(av[i], bv[j], c);
+// The convolution's taps of four neighbouring channels, and the sum over a window of four rows, r0 the oldest: oldest first from
+// zero in fp32, the same bits in either form.
+template <typename T> struct ConvTaps;
+template <> struct ConvTaps<float> {                   // tap j of the channel pairs (0, 1) and (2, 3): packed FMAs
+  float2 w[4][2] = {};
+  __device__ __forceinline__ void load(const float* p) {
+    float4 c[4];                                       // the taps of channel e
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] = *reinterpret_cast<const float4*>(p + e * 4);
+    w[0][0] = make_float2(c[0].x, c[1].x); w[0][1] = make_float2(c[2].x, c[3].x);
+    w[1][0] = make_float2(c[0].y, c[1].y); w[1][1] = make_float2(c[2].y, c[3].y);
+    w[2][0] = make_float2(c[0].z, c[1].z); w[2][1] = make_float2(c[2].z, c[3].z);
+    w[3][0] = make_float2(c[0].w, c[1].w); w[3][1] = make_float2(c[2].w, c[3].w);
   }
-}
+  __device__ __forceinline__ void sum(const float4& r0, const float4& r1, const float4& r2, const float4& r3, float2 (&y)[2]) const {
+    const float2 zero2 = make_float2(0.f, 0.f);
+    y[0] = __ffma2_rn(w[0][0], make_float2(r0.x, r0.y), zero2); y[1] = __ffma2_rn(w[0][1], make_float2(r0.z, r0.w), zero2);
+    y[0] = __ffma2_rn(w[1][0], make_float2(r1.x, r1.y), y[0]);  y[1] = __ffma2_rn(w[1][1], make_float2(r1.z, r1.w), y[1]);
+    y[0] = __ffma2_rn(w[2][0], make_float2(r2.x, r2.y), y[0]);  y[1] = __ffma2_rn(w[2][1], make_float2(r2.z, r2.w), y[1]);
+    y[0] = __ffma2_rn(w[3][0], make_float2(r3.x, r3.y), y[0]);  y[1] = __ffma2_rn(w[3][1], make_float2(r3.z, r3.w), y[1]);
+  }
+};
+template <> struct ConvTaps<__nv_bfloat16> {           // as loaded: a product of two bf16 values and an fp32 sum are one
+  uint2 w[4] = {};                                     // instruction (sm_100), where widening both first takes one each
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) {
+    const uint4 lo = *reinterpret_cast<const uint4*>(p), hi = *reinterpret_cast<const uint4*>(p + 8);
+    w[0] = make_uint2(lo.x, lo.y); w[1] = make_uint2(lo.z, lo.w);
+    w[2] = make_uint2(hi.x, hi.y); w[3] = make_uint2(hi.z, hi.w);
+  }
+  static __device__ __forceinline__ unsigned short element(const uint2& p, int i) {
+    const uint32_t word = i & 2 ? p.y : p.x;
+    return (unsigned short)(i & 1 ? word >> 16 : word & 0xFFFF);
+  }
+  __device__ __forceinline__ float channel(const uint2 (&r)[4], int e) const {
+    float c = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float d;
+      asm("fma.rn.f32.bf16 %0, %1, %2, %3;" : "=f"(d) : "h"(element(w[e], j)), "h"(element(r[j], e)), "f"(c));
+      c = d;
+    }
+    return c;
+  }
+  __device__ __forceinline__ void sum(const uint2& r0, const uint2& r1, const uint2& r2, const uint2& r3, float2 (&y)[2]) const {
+    const uint2 r[4] = {r0, r1, r2, r3};
+    y[0] = make_float2(channel(r, 0), channel(r, 1));
+    y[1] = make_float2(channel(r, 2), channel(r, 3));
+  }
+};
 
 // one-shot mbarrier for a bulk copy into shared memory
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -128,14 +162,20 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
 // An entry takes its four rows from there and is done: nothing is carried from one entry to the next.  (The transposed form,
 // which hands a parent's partial sums down, reads a row once instead of four times, but telling the cases apart, starting
 // sums over and pairing registers for them cost more: 101 against 76 warp instructions per entry and 128 channels, 48 layers.)
-// Every sum takes its taps oldest first from zero in fp32 (packed FMAs: two correctly rounded fp32 lanes per
-// instruction, same bits as scalar fmaf), bias last, SiLU in fp32, one round-to-nearest-even cast (Sec. "Precompute
+// Every sum takes its taps oldest first from zero in fp32 (bf16 by the mixed fma, fp32 by packed FMAs: two correctly rounded
+// lanes per instruction, the same bits as scalar fmaf), bias last, SiLU in fp32, one round-to-nearest-even cast (Sec. "Precompute
 // branch histories while preserving arithmetic": tap order and cast points are part of the result).
 //
 // What bounds it: instruction issue (70 % of the slots; the SiLU alone is 14 instructions per four channels, 8 of them special-
-// function operations, whose unit is half busy) with HBM close behind.  Measured against the transposed form: 48 layers of 4 x 32
-// nodes 51.4 -> 43.0 us, 32 x 256 nodes 70.0 -> 66.0, 8 x 64 nodes 11.9 -> 11.4.  Five or six CTAs per SM instead of four spill: 46.7
-// and 50.0 us against 44.5; two entries at a time instead of eight 44.5.
+// function operations, whose unit is half busy) with HBM behind it (0.5 to 0.6 of the copy rate by the bytes it cannot do without).
+// Kernel times against the transposed form, bf16: 48 layers of 4 x 32 nodes 51.6 -> 41.0 us, 32 x 256 nodes 69.6 -> 61.4, 8 x 64
+// nodes 7.8 -> 6.2.  Five or six CTAs per SM instead of four spill: 46.7 and 50.0 us against 44.5; two entries at a time instead
+// of eight 44.5.
+// fp32 rows take twice the registers: one entry at a time and no window kept is what fits 64 of them without spills (63).  As the
+// bf16 form has it, with scalar fmaf (84 bytes spilled), it lost to the transposed form: 8 x 64 nodes of 4096 channels 6.5 (transposed)
+// -> 6.9 -> 6.3 us (now), spines of 64 7.3 -> 8.1 -> 7.2, 32 x 256 of 8192 channels 105 -> 115 -> 105; three CTAs per SM with room for
+// everything 8.1 us (8 x 64: no longer one wave).  What is left behind is a star of 256 nodes, 99.9 -> 108.5, whose root row
+// every entry fetches from L1.
 
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
@@ -218,23 +258,14 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   // ---- taps and bias of this lane's channels, as pairs of neighbouring channels ------------------------------------
   const int run = warp >> sp.log_groups, cg = (warp & (sp.groups - 1)) * 128 + lane * 4, c0 = cbase + cg;
   const bool mine = c0 < s.C;
-  P4 taps[4];                                          // of channel c0 + e, oldest first
-  float bias[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int e = 0; e < 4; ++e) taps[e] = P4{};
+  ConvTaps<T> taps;
+  float2 bias[2] = {};
   if (mine) {
-    const T* w = reinterpret_cast<const T*>(L.conv_w) + (size_t)c0 * 4;
-    if constexpr (sizeof(T) == 2) {
-      const uint4 lo = *reinterpret_cast<const uint4*>(w), hi = *reinterpret_cast<const uint4*>(w + 8);
-      taps[0] = make_uint2(lo.x, lo.y); taps[1] = make_uint2(lo.z, lo.w);
-      taps[2] = make_uint2(hi.x, hi.y); taps[3] = make_uint2(hi.z, hi.w);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) taps[e] = *reinterpret_cast<const float4*>(w + e * 4);
-    }
+    taps.load(reinterpret_cast<const T*>(L.conv_w) + (size_t)c0 * 4);
     if (L.conv_b) {
       const float4 bv = Packed4<T>::unpack(*reinterpret_cast<const P4*>(reinterpret_cast<const T*>(L.conv_b) + c0));
-      bias[0] = bv.x; bias[1] = bv.y; bias[2] = bv.z; bias[3] = bv.w;
+      bias[0] = make_float2(bv.x, bv.y);
+      bias[1] = make_float2(bv.z, bv.w);
     }
   }
   cp_async_wait<0>();
@@ -269,28 +300,32 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
       if (at >= 0) return row(at);
       return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)prog_g[~at] * (uint32_t)s.C));
     };
-    P4 far0 = {}, far1 = {}, far2 = {};                // the last window that reached elsewhere, and the parent it belongs to
-    int of = INT_MIN;
-#pragma unroll 8
+    // bf16: eight entries at a time, and a window that reaches elsewhere kept for the siblings behind it, which follow one
+    // another (a star's root is fetched once, not 255 times).  fp32 has no registers for either: see above.
+    constexpr int kAtATime = sizeof(T) == 2 ? 8 : 1;
+    [[maybe_unused]] P4 far[3] = {};                   // the last window that reached elsewhere, and the parent it belongs to
+    [[maybe_unused]] int of = INT_MIN;
+#pragma unroll kAtATime
     for (int rr = 0; rr < live; ++rr) {                // bounded: kRun
       const ConvEntry en = ent[rr];
       const P4 r3 = *reinterpret_cast<const P4*>(own + rr * row_bytes);
       P4 r0, r1, r2;
       if (decltype(elsewhere_c)::value && __builtin_expect((en.w0 | en.w1 | en.w2) < 0, 0)) {    // uniform
-        if (en.w2 != of) {                             // siblings follow one another: a star's root is fetched once, not 255 times
-          far0 = row_anywhere(en.w0); far1 = row_anywhere(en.w1); far2 = row_anywhere(en.w2);
-          of = en.w2;
+        if constexpr (sizeof(T) == 2) {
+          if (en.w2 != of) {
+            far[0] = row_anywhere(en.w0); far[1] = row_anywhere(en.w1); far[2] = row_anywhere(en.w2);
+            of = en.w2;
+          }
+          r0 = far[0]; r1 = far[1]; r2 = far[2];
+        } else {
+          r0 = row_anywhere(en.w0); r1 = row_anywhere(en.w1); r2 = row_anywhere(en.w2);
         }
-        r0 = far0; r1 = far1; r2 = far2;
       } else {
         r0 = row(en.w0); r1 = row(en.w1); r2 = row(en.w2);
       }
-      float a[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        a[e] = mul_add<T>(taps[e], 3, r3, e, mul_add<T>(taps[e], 2, r2, e, mul_add<T>(taps[e], 1, r1, e, mul_add<T>(taps[e], 0, r0, e, 0.f))));
-      if (has_bias) { a[0] += bias[0]; a[1] += bias[1]; a[2] += bias[2]; a[3] += bias[3]; }   // bias last
-      float2 y[2] = {make_float2(a[0], a[1]), make_float2(a[2], a[3])};
+      float2 y[2];
+      taps.sum(r0, r1, r2, r3, y);
+      if (has_bias) { y[0] = __fadd2_rn(y[0], bias[0]); y[1] = __fadd2_rn(y[1], bias[1]); }   // bias last
       // SiLU a / (1 + 2^(-a log2 e)) with the hardware exponential and reciprocal (1e-6 relative, far
       // below the rounding of the recorded operand); the multiplies and the add are packed
       const float2 nl2e = make_float2(-1.4426950408889634f, -1.4426950408889634f), one = make_float2(1.f, 1.f);
