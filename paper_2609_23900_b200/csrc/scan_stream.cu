@@ -45,7 +45,7 @@ constexpr int kD = 128;
 constexpr int kNT = 32;               // nodes of a group at most
 constexpr int kWarps = 8;             // that compute, and one more that leads them (below)
 constexpr int kThreads = 32 * kWarps;
-constexpr uint32_t kSpinLimit = 1u << 24;
+constexpr uint32_t kSpinLimit = 1u << 24, kSpinLimitDrill = 1024;
 constexpr uint32_t kStateBytes = kD * kD * 4;
 
 // shared memory map (bytes from a 1024-aligned base)
@@ -124,9 +124,9 @@ __device__ __forceinline__ void mbar_init(unsigned long long* bar, uint32_t coun
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
 }
 // Bounded wait: false if the phase did not complete within the spin limit.
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, uint32_t limit) {
   const uint32_t addr = smem_u32(bar);
-  for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
+  for (uint32_t spin = 0; spin < limit; ++spin) {
     uint32_t done;
     asm volatile(
         "{\n.reg .pred p;\n"
@@ -261,6 +261,9 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
   const uint32_t rep_mul = 0xFFFFFFFFu / (uint32_t)rep + 1u;    // hv / rep = high word of hv * rep_mul (rep > 1)
   const int out_size = s.out_dtype == LUMO_BF16 ? 2 : 4;
   const uint32_t k_pitch = (uint32_t)s.Hk * kD, v_pitch = (uint32_t)s.Hv * kD;   // elements from one physical row to the next
+  // Test aid: nothing asynchronous is issued to the tensor core or the state's barrier, every wait runs out.
+  const bool drill = s.debug_skip_mma != 0;
+  const uint32_t spin_limit = drill ? kSpinLimitDrill : kSpinLimit;
   auto live = [](int meta) { return ((meta >> 16) & 0xFF) != 0; };               // a node, not the rest of the group's table
 
   // ---- the leading warp looks ahead ------------------------------------------------------------------------------------
@@ -437,7 +440,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       sm.unit = u;
       sm.unit_fresh = true;
       // the state is settled before this kernel may enter early; everything else may still be in the making
-      if (any) {
+      if (any && !drill) {
         request_state(sbase + kOffS, state_of(u.layer, u.row, u.hv), &sm.mb_state);
         ++requested;
       }
@@ -456,7 +459,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       store_gates(sm.node[0]);
       if constexpr (kFused) path_store(sm.step[0]);
     }
-    const uint32_t lead = elect_one();
+    const uint32_t lead = drill ? 0u : elect_one();
     uint32_t landed = 0;                                        // states that have been waited for by the others
     for (; sm.step[k & 3].have; ++k) {                          // bounded: the launch's work
       const Step &cur = sm.step[k & 3], &nxt = sm.step[(k + 1) & 3];
@@ -501,7 +504,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
           umma(lead, tmem + kColO, d_v + (uint64_t)(((i & 1) * 2048) >> 4), d_b + (uint64_t)((i * 32) >> 4), umma_idesc(32, 1, 0), i ? 1u : 0u);
       }
       if constexpr (kFused) if (nxt.have && nxt.fresh) path_nodes(nxt);
-      if (!mbar_wait(&sm.mb_mma, ph_mma)) sm.timed_out = 1;
+      if (!mbar_wait(&sm.mb_mma, ph_mma, spin_limit)) sm.timed_out = 1;
       ph_mma ^= 1;
       all();                                                    // q~ is in tensor memory
       all();                                                    // q~ and the state are operands
@@ -517,17 +520,30 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
         umma_commit(lead, &sm.mb_mma);
       }
       if (nxt.have) {
-        if (nxt.fresh && lane == 0) request_state(sbase + kOffS, state_of(nxt.layer, nxt.row, nxt.hv), &sm.mb_state);
-        if (nxt.fresh && lane == 0) ++requested;
+        if (nxt.fresh && lane == 0 && !drill) {
+          request_state(sbase + kOffS, state_of(nxt.layer, nxt.row, nxt.hv), &sm.mb_state);
+          ++requested;
+        }
         request_gates(nxt);
       }
-      if (!mbar_wait(&sm.mb_mma, ph_mma)) sm.timed_out = 1;
+      if (!mbar_wait(&sm.mb_mma, ph_mma, spin_limit)) sm.timed_out = 1;
       ph_mma ^= 1;
       __syncwarp();
       all();                                                    // the outputs are in tensor memory
-      if (sm.timed_out) {                                       // the same in every thread; report and leave
-        int32_t* status = lb.l[cur.layer].status;
-        if (lane == 0 && status) status[cur.b] = LUMO_SEQ_TIMEOUT;
+      if (sm.timed_out) {                                       // the same in every thread: report this unit and all that are left
+        auto give_up = [&](int layer, int b) {
+          int32_t* status = lb.l[layer].status;
+          if (lane == 0 && status) status[b] = LUMO_SEQ_TIMEOUT;
+        };
+        give_up(cur.layer, cur.b);
+        if (nxt.have) give_up(nxt.layer, nxt.b);
+        Unit u = sm.unit;                                       // of the step after that
+        __syncwarp();
+        while (u.layer < s.n_layers) {                          // bounded: the launch's units
+          give_up(u.layer, u.b);
+          advance(u);
+          open(u);
+        }
         break;
       }
       if (nxt.have) {
@@ -536,7 +552,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       }
     }
     // nobody leaves before its own copies have landed
-    if (lane == 0 && requested > landed) mbar_wait(&sm.mb_state, landed & 1);
+    if (lane == 0 && requested > landed) mbar_wait(&sm.mb_state, landed & 1, spin_limit);
   } else {
   __syncthreads();
   uint32_t ph_state = 0;
@@ -607,7 +623,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
     }
     // ---- Gram rows out of tensor memory; normalisation factors ---------------------------------------------------------
     if ((warp & 3) < 2) {                                       // lanes 0..31 the key rows, 32..63 the query rows
-      if (!mbar_wait(&sm.mb_mma, ph_mma)) sm.timed_out = 1;
+      if (!mbar_wait(&sm.mb_mma, ph_mma, spin_limit)) sm.timed_out = 1;
       tc_fence_after();
       const bool is_q = warp & 1;
       uint32_t r[16];
@@ -734,7 +750,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
           crew();
         }
       }
-      if (mbar_wait(&sm.mb_state, ph_state)) ph_state ^= 1;
+      if (mbar_wait(&sm.mb_state, ph_state, spin_limit)) ph_state ^= 1;
       else sm.timed_out = 1;
       const int r0 = 32 * (warp & 3) + 16 * (warp >> 2) + (lane >> 2);           // rows r0 and r0 + 8
       const float* base = reinterpret_cast<const float*>(smem + kOffS) + r0 * kD + (lane & 3) * 4;
