@@ -87,6 +87,7 @@ struct Small {
   uint32_t bad[2];                   // nodes whose key or value row is not finite; the steps take turns
   uint32_t look[2];                  // set when some |k|^2 is not finite: the key rows are to be looked over
   uint32_t timed_out;
+  uint32_t state_missing;            // the wait for a state ran out (kept by the computing warps): its copy may still be on its way
   uint32_t tmem_base;
   unsigned long long mb_state, mb_mma;
   // kept by the leading warp
@@ -413,7 +414,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
   if (tid == 0) {
     mbar_init(&sm.mb_state, 1);
     mbar_init(&sm.mb_mma, 1);
-    sm.timed_out = 0; sm.bad[0] = sm.bad[1] = sm.look[0] = sm.look[1] = 0; sm.plen = 0;
+    sm.timed_out = sm.state_missing = 0; sm.bad[0] = sm.bad[1] = sm.look[0] = sm.look[1] = 0; sm.plen = 0;
   }
   tc_fence_before();
   __syncthreads();
@@ -460,7 +461,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       if constexpr (kFused) path_store(sm.step[0]);
     }
     const uint32_t lead = drill ? 0u : elect_one();
-    uint32_t landed = 0;                                        // states that have been waited for by the others
+    uint32_t landed = 0;                                        // states that the others have seen arrive
     for (; sm.step[k & 3].have; ++k) {                          // bounded: the launch's work
       const Step &cur = sm.step[k & 3], &nxt = sm.step[(k + 1) & 3];
       all();                                                    // key and query rows are there
@@ -474,7 +475,6 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
         }
         umma_commit(lead, &sm.mb_mma);
       }
-      if (cur.fresh) ++landed;
       if (lane == 0) {
         sm.bad[(k & 1) ^ 1] = sm.look[(k & 1) ^ 1] = 0;
         int32_t* status = lb.l[cur.layer].status;
@@ -520,7 +520,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
         umma_commit(lead, &sm.mb_mma);
       }
       if (nxt.have) {
-        if (nxt.fresh && lane == 0 && !drill) {
+        if (nxt.fresh && lane == 0 && !drill && !sm.state_missing) {   // (one copy at a time on the barrier)
           request_state(sbase + kOffS, state_of(nxt.layer, nxt.row, nxt.hv), &sm.mb_state);
           ++requested;
         }
@@ -530,6 +530,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       ph_mma ^= 1;
       __syncwarp();
       all();                                                    // the outputs are in tensor memory
+      if (cur.fresh && !sm.state_missing) ++landed;
       if (sm.timed_out) {                                       // the same in every thread: report this unit and all that are left
         auto give_up = [&](int layer, int b) {
           int32_t* status = lb.l[layer].status;
@@ -747,17 +748,17 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
             for (int o = 16; o > 0; o >>= 1) kk += __shfl_xor_sync(0xffffffffu, kk, o);
             if (lane == 0) sm.prev_ks[tt] = s.l2norm ? rsqrtf(kk + s.l2_eps) : 1.f;
           }
-          crew();
         }
       }
       if (mbar_wait(&sm.mb_state, ph_state, spin_limit)) ph_state ^= 1;
-      else sm.timed_out = 1;
+      else sm.timed_out = sm.state_missing = 1;
       const int r0 = 32 * (warp & 3) + 16 * (warp >> 2) + (lane >> 2);           // rows r0 and r0 + 8
       const float* base = reinterpret_cast<const float*>(smem + kOffS) + r0 * kD + (lane & 3) * 4;
       const uint32_t to = tmem + ((uint32_t)(32 * (warp & 3) + 16 * (warp >> 2)) << 16) + kColS;
       if constexpr (kFused) {
         const int plen = sm.plen;
-        if (plen > 0) {
+        if (plen > 0) crew();
+        if (plen > 0 && !sm.state_missing) {                    // (the same in every warp: nothing but a state that is there goes back)
 #pragma unroll 1
           for (int r = 0; r < 2; ++r) {                         // eight rows at a time, a lane four columns of each; back to where
             const int first = 32 * (warp & 3) + 16 * (warp >> 2) + 8 * r;        // they were, and to memory

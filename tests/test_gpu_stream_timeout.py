@@ -73,3 +73,20 @@ def test_every_unit_of_a_fused_call_reports_the_timeout(drill):
     torch.cuda.synchronize()
     for layer in layers:
         assert layer.tensors["status"].tolist() == [binding.SEQ_TIMEOUT] * 3
+
+
+def test_a_state_that_does_not_arrive_is_not_written_back(drill):
+    """The accepted path is replayed into the state in shared memory and the rows go back to memory: never rows that did not come."""
+    dcP, dcC, layers, call = _cycle()
+    before = [dcP.t("state", l).clone() for l in range(len(layers))]
+    drill(True)
+    call()
+    torch.cuda.synchronize()
+    for l in range(len(layers)):
+        assert torch.equal(dcP.t("state", l), before[l])
+    drill(False)
+    call()
+    torch.cuda.synchronize()
+    for l, layer in enumerate(layers):
+        assert layer.tensors["status"].tolist() == [binding.SEQ_OK] * 3
+        assert not torch.equal(dcP.t("state", l), before[l])
