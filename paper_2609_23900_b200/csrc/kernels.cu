@@ -174,8 +174,9 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
 // fp32 rows take twice the registers: one entry at a time and no window kept is what fits 64 of them without spills (63).  As the
 // bf16 form has it, with scalar fmaf (84 bytes spilled), it lost to the transposed form: 8 x 64 nodes of 4096 channels 6.5 (transposed)
 // -> 6.9 -> 6.3 us (now), spines of 64 7.3 -> 8.1 -> 7.2, 32 x 256 of 8192 channels 105 -> 115 -> 105; three CTAs per SM with room for
-// everything 8.1 us (8 x 64: no longer one wave).  What is left behind is a star of 256 nodes, 99.9 -> 108.5, whose root row
-// every entry fetches from L1.
+// everything 8.1 us (8 x 64: no longer one wave).  Where a sequence falls into several parts, the window of a part's first entry is
+// staged with the part's own rows, so that whoever shares it (in a star everyone) does not go to L1 for it: 32 stars of 256 nodes, fp32,
+// 102.5 (transposed) -> 111.5 (fetched by every entry) -> 103.0 us (now), 12 x 140 nodes 22.9 -> 25.1 -> 22.4; bf16 as before.
 
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
@@ -186,7 +187,7 @@ struct alignas(16) ConvEntry { int phys, w0, w1, w2; };
 
 template <typename T, int kRun, bool kFused, class LB>
 __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, const LB& lb, const ConvSplit& sp, const FusedPrevT<LB>* fp) {
-  extern __shared__ __align__(128) unsigned char conv_smem[];            // [runs * kRun + 3 rows][groups * 128 channels]
+  extern __shared__ __align__(128) unsigned char conv_smem[];            // [runs * kRun + 3 (+ 3) rows][groups * 128 channels]
   __shared__ ConvEntry s_entry[kConvMaxEntries];
   __shared__ int f_acc[kFusedMaxPath], f_par[kFusedMaxPath], f_phys[kFusedMaxPath];
   __shared__ const T* f_hsrc[3];
@@ -199,11 +200,19 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
   const int row_bytes = (128 << sp.log_groups) * (int)sizeof(T);
   const LayerPtrs& L = lb.l[layer];
   const int32_t* prog_g = t.conv_prog + (size_t)b * s.Ns;
+  // The window of the part's first entry lies in other parts; its rows are staged behind the history, for all who share them
+  // (a part of a star: every entry).
+  int4 before = make_int4(-1, -1, -1, -1);
+  if (seg > 0) before = *reinterpret_cast<const int4*>(t.win + ((size_t)b * s.Ns + e0) * 4);
   if (tid < entries) {                                 // descriptor tables: nobody writes them
     const int e = e0 + tid;
     if (e < s.Ns) {
       const int4 w = *reinterpret_cast<const int4*>(t.win + ((size_t)b * s.Ns + e) * 4);
-      auto place = [&](int v) { return v < 0 ? (entries + 3 + v) * row_bytes : v >= e0 ? (v - e0) * row_bytes : ~v; };
+      auto place = [&](int v) {
+        if (v < 0) return (entries + 3 + v) * row_bytes;
+        if (v >= e0) return (v - e0) * row_bytes;
+        return v == before.z ? (entries + 5) * row_bytes : v == before.y ? (entries + 4) * row_bytes : v == before.x ? (entries + 3) * row_bytes : ~v;
+      };
       s_entry[tid] = {prog_g[e], place(w.x), place(w.y), place(w.z)};
     }
   }
@@ -225,6 +234,11 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
 #pragma unroll 4
     for (int e = tid >> log_cols; e < live; e += step)
       cp_async16(mycol + e * row_bytes, src + (size_t)((uint32_t)prog_g[e0 + e] * (uint32_t)s.C));
+    if (seg > 0 && live > 0)
+      for (int j = tid >> log_cols; j < 3; j += step) {
+        const int v = j == 0 ? before.x : j == 1 ? before.y : before.z;
+        if (v >= 0) cp_async16(mycol + (entries + 3 + j) * row_bytes, src + (size_t)((uint32_t)prog_g[v] * (uint32_t)s.C));
+      }
   }
   const T* hbase = reinterpret_cast<const T*>(L.conv_hist) + (size_t)(seq_ok ? row : 0) * 3 * s.C;
   if constexpr (kFused) {
@@ -255,7 +269,7 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
       cp_async16(mycol + (entries + j) * row_bytes, src + cbase + col);
     }
   cp_async_commit();
-  // ---- taps and bias of this lane's channels, as pairs of neighbouring channels ------------------------------------
+  // ---- taps and bias of this lane's four channels --------------------------------------------------------------------
   const int run = warp >> sp.log_groups, cg = (warp & (sp.groups - 1)) * 128 + lane * 4, c0 = cbase + cg;
   const bool mine = c0 < s.C;
   ConvTaps<T> taps;
@@ -300,8 +314,8 @@ __device__ __forceinline__ void conv_body(const Shape& s, const TreeDev& t, cons
       if (at >= 0) return row(at);
       return *reinterpret_cast<const P4*>(xb + cg + (size_t)((uint32_t)prog_g[~at] * (uint32_t)s.C));
     };
-    // bf16: eight entries at a time, and a window that reaches elsewhere kept for the siblings behind it, which follow one
-    // another (a star's root is fetched once, not 255 times).  fp32 has no registers for either: see above.
+    // bf16: eight entries at a time, and a window that reaches elsewhere kept for the siblings behind it in the run.  fp32 has no
+    // registers for either: see above.
     constexpr int kAtATime = sizeof(T) == 2 ? 8 : 1;
     [[maybe_unused]] P4 far[3] = {};                   // the last window that reached elsewhere, and the parent it belongs to
     [[maybe_unused]] int of = INT_MIN;
@@ -1166,8 +1180,9 @@ static cudaError_t launch_conv_t(const Shape& s, const TreeDev& t, const LayerBa
     constexpr int kMost = (kConvMaxEntries + 3 * kConvWarps) * 128 * (int)sizeof(T);    // of any split
     const ConvSplit sp = conv_split(s.C, s.Ns, R, seqs, sms);
     const int entries = sp.runs * R;
-    const dim3 grid(sp.slabs * ((s.Ns + entries - 1) / entries), s.B, s.n_layers), block(32 * sp.runs * sp.groups);
-    const size_t smem = (size_t)(entries + 3) * sp.groups * 128 * sizeof(T);
+    const int parts = (s.Ns + entries - 1) / entries;
+    const dim3 grid(sp.slabs * parts, s.B, s.n_layers), block(32 * sp.runs * sp.groups);
+    const size_t smem = (size_t)(entries + (parts > 1 ? 6 : 3)) * sp.groups * 128 * sizeof(T);   // (several parts: one group)
     auto layers = [&]() -> decltype(auto) { if constexpr (kFew) return few_layers(lb); else return (lb); };
     if constexpr (sizeof(T) == 2) {                               // the fused path serves bf16 operands only
       if (fp) {

@@ -44,3 +44,13 @@ def test_runs_shared_out_evenly(B, N):
     assert ctx().conv_rows_per_cta(ctx().tree_desc(np.array([[i - 1 for i in range(N)]] * B, dtype=np.int32)), 8, 16, 128) == 4
     check(W.make_case("runs", [W.tree_random(W.IntStream(N + b), N, 9) for b in range(B)], seed=B, Hk=8, Hv=16, d=128, in_dtype="bf16",
                       Ns=N, permute_slots=True))
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N", [130, 256])
+def test_windows_shared_across_parts(N, dtype):
+    """The second part's first entry hangs off a node of the first part: the root of a star (two history rows and one staged), a spine of
+    four whose last three nodes all have children there (windows that are the first entry's own, and others one and two rows older)."""
+    star = [-1] + [0] * (N - 1)
+    spine = [-1, 0, 1, 2] + [3] * (N - 24) + [2] * 10 + [1] * 10
+    check(W.make_case("shared", [star, spine], seed=N, Hk=1, Hv=2, d=64, in_dtype=dtype, Ns=N + 2, permute_slots=True, with_bias=True))
