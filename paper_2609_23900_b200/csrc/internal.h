@@ -346,7 +346,7 @@ cudaError_t launch_scan_gram(const Shape& s, const TreeDev& t, const LayerBatch&
 // same scan, first replaying the previous cycle's accepted path into the state it has just loaded
 cudaError_t launch_scan_gram_fused(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev& fp,
                                    int sm_count, bool pdl, int tail, cudaStream_t st);
-// solved Gram form with the state streamed through shared memory, for launches of several waves (scan_stream.cu);
+// solved Gram form with the state streamed through shared memory (scan_stream.cu); where it pays: the rule there;
 // fp: replay the previous cycle's accepted path first (null: plain scan)
 bool scan_stream_pays(const Shape& s, const TreeDev& t, bool fused, int sm_count);
 cudaError_t launch_scan_stream(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sm_count, bool pdl,

@@ -1,4 +1,4 @@
-// Tree scan for launches of several waves: solved Gram form on tcgen05, the state streamed through shared memory.
+// Tree scan in the solved Gram form on tcgen05, the state streamed through shared memory.
 //
 // The algebra is the solved Gram form (paper Eq. 2-3, exact; see scan_gram.cu for the symbols):
 //
@@ -958,18 +958,41 @@ cudaError_t launch_t(const Shape& s, const TreeDev& t, const LB& lb, const Fused
 
 }  // namespace
 
-// Where the streamed scan takes the place of the closed form with the tensor-core sum (scan_gram.cu).  It is faster nearly
-// everywhere (launches overlapped, us, before / now): trees of 28 nodes over 12 levels, 32 items 7.6 / 5.5, 256 9.7 / 8.0, 768
-// 29.4 / 24.4, 2048 64.3 / 47.4; 48 nodes, 32 10.2 / 5.6, 512 25.8 / 21.5; 256 random nodes, 1 sequence 12.4 / 10.9, 8 58 / 46,
-// 32 212 / 158.  The exception: a tree that one group of 64 holds and that falls into three or more groups of 32, at one
-// to four items per SM, where those groups neither find CTAs of their own nor fill waves: 64 nodes over 12 levels, 128 items
-// 10.5 / 11.0, 256 13.3 / 15.8, 384 26.1 / 27.9, 512 28.6 / 29.3, 640 43.4 / 42.9.
-// With the commit folded in (whole calls): 28 nodes, 32 items 13.3 / 13.6, 128 16.5 / 15.6, 512 38.7 / 35.6, 3072 184 / 165; but
-// trees that need a second group keep the 64-node tile: 34 nodes, 1536 items 118 / 122, 64 nodes 141 / 154.
+// Where the streamed scan takes the place of the closed form with the tensor-core sum (scan_gram.cu).  Measured at 380 points over
+// 4 to 256 nodes and 32 to 4096 items (a state each), launches overlapped, us, closed form / streamed:
+//   * groups of 32 alone: always.  16 nodes, 32 items 6.0 / 5.6, 304 14.8 / 11.2, 2048 54.9 / 48.4; 28 nodes 7.0 / 5.7, 16.6 / 11.9,
+//     61.5 / 49.7.
+//   * one group of 64 that falls into two or three of 32.  As long as the parts of a tree find SMs of their own, always (64 nodes,
+//     72 items 10.6 / 9.9; 56 nodes 10.6 / 6.8).  Then a second CTA on the SM, or two or three steps in a row, cost more than the
+//     one wave of larger tiles: 2.0 groups, 148 items 11.1 / 9.3 but 2.2 11.4 / 11.9 and 3 11.6 / 12.7; one wave of whole trees, 2.0
+//     groups 50 nodes, 224 items 13.2 / 12.7, 44 nodes, 292 13.6 / 14.5, 2.03 groups, 152 12.6 / 14.9, 3 14.8 / 18.4.  From the
+//     second wave on two groups win (50 nodes, 304 items 22.8 / 17.9, 800 44 / 40), three lose (64 nodes, 512 28.8 / 31.3, 2048
+//     98.8 / 107.3) and 2.2 lie between: 304 23.4 / 20.0, 440 26.8 / 29.4, 1000 55.7 / 49.0.
+//   * several groups of 64: nearly always (256 nodes, 1024 items 213 / 172; 70 nodes, 224 items 24.4 / 16.8).  Not where the larger
+//     tiles make one wave and the tree's halves, on shared SMs, three steps (128 nodes, 84 items 13.2 / 16.3; 96 nodes, two steps,
+//     148 items 14.2 / 13.7), nor where they make two and the whole trees a second CTA on a few SMs (160 nodes, 180 items 26.0 / 32.5).
+// With the commit folded in (whole calls) groups of 32 alone: from two full waves on at any size (8 nodes, 592 items 34.8 / 35.8, 1200
+// 67.4 / 65.5, 28 nodes, 1536 99.8 / 94.1), before that at 28 nodes and more where no SM holds a second CTA (28 nodes, 128 items 21.3
+// / 20.0) or one wave is not enough (320 33.9 / 32.8), but 200 23.5 / 24.4; 8 nodes, 96 items 14.6 / 17.5.  Trees that need a second
+// group keep the 64-node tile: 34 nodes, 1536 items 118 / 122, 64 nodes 141 / 154.
 bool scan_stream_pays(const Shape& s, const TreeDev& t, bool fused, int sm_count) {
-  const long long items = (long long)s.n_layers * s.B * s.Hv;
-  if (fused) return t.st_groups == s.B && 2 * items > sm_count;
-  return !(t.n_groups == s.B && t.st_groups >= 3 * s.B && items > sm_count && items < 4LL * sm_count);
+  const long long sms = sm_count, items = (long long)s.n_layers * s.B * s.Hv, B = s.B, g32 = t.st_groups;
+  const bool apart = 2 * items <= sms, one_each = items <= sms, one_wave = items <= 2 * sms;     // CTAs with an SM to themselves, a state each
+  if (fused) {
+    if (g32 != B) return false;
+    return items > 4 * sms || (s.N >= 28 && !apart && (one_each || !one_wave));
+  }
+  if (g32 == B || apart) return true;
+  const bool two = 16 * g32 <= 33 * B;                            // groups a tree: two, but for a few
+  if (t.n_groups == s.B) {
+    if (one_each) return two;
+    if (one_wave) return g32 == 2 * B && s.N >= 50;
+    if (5 * items > 13 * sms && items <= 4 * sms) return two;
+    return 3 * g32 <= 7 * B;
+  }
+  const long long tiles = (long long)s.n_layers * t.n_groups * s.Hv;
+  if (tiles <= 2 * sms) return g32 <= 4 * B;
+  return one_each || tiles > 4 * sms || 2 * g32 <= 9 * B;
 }
 
 cudaError_t launch_scan_stream(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sm_count, bool pdl,

@@ -8,6 +8,7 @@ import torch
 
 from synthetic import workload as W
 from synthetic.device_case import DeviceCase
+from tests.graph_nodes import Captured
 from tests.harness import assert_close, ctx, oracle_scan_from_device
 
 pytestmark = pytest.mark.gpu
@@ -65,3 +66,20 @@ def test_values_that_are_not_finite_stay_on_their_paths(which, value, N, B, L):
     kept = [int(c.slot[b, i]) for i in range(N) if not below[i]]
     assert not torch.isfinite(got[b, gone]).all(dim=-1).any()
     assert torch.equal(got[b, kept], clean[b, kept]) and torch.equal(got[:b], clean[:b])
+
+
+@pytest.mark.parametrize("N,depth,items,streamed", [(64, 12, 72, True), (64, 12, 80, False), (64, 12, 304, False), (64, 12, 640, False), (50, 12, 148, True),
+                                                    (50, 12, 304, True), (44, 12, 224, False), (44, 12, 304, True), (128, 9, 92, False), (128, 9, 100, True),
+                                                    (128, 9, 152, False), (128, 9, 224, True), (96, 12, 148, True), (28, 12, 224, True)])
+def test_the_form_that_measured_faster_is_taken(N, depth, items, streamed):
+    """Closed form over groups of 64 or streamed groups of 32, on a B200's 148 SMs; either way the oracle's outputs."""
+    c = _case(N, items // 4, 2, 4, 1, depth)
+    dc = DeviceCase(ctx("tensor"), c, use_conv=False, qk_l2norm=True)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        name, = [n for n, _ in Captured(dc.verify).kernels]
+        assert ("scan_stream_kernel" in name) == streamed and ("scan_gram_kernel" in name) == (not streamed)
+    dc.verify()
+    torch.cuda.synchronize()
+    ctx("auto")
+    ref, _, _ = oracle_scan_from_device(dc)
+    assert assert_close(dc.np("out"), ref) < 1e-4
