@@ -45,7 +45,6 @@ constexpr int kD = 128;
 constexpr int kNT = 32;               // nodes of a group at most
 constexpr int kWarps = 8;             // that compute, and one more that leads them (below)
 constexpr int kThreads = 32 * kWarps;
-constexpr uint32_t kSpinLimit = 1u << 24, kSpinLimitDrill = 1024;
 constexpr uint32_t kStateBytes = kD * kD * 4;
 
 // shared memory map (bytes from a 1024-aligned base)
@@ -242,7 +241,8 @@ __device__ __noinline__ bool drop_non_finite(uint4* piece) {
   return any;
 }
 
-template <bool kFused, class LB>
+// kDrill: a test aid; nothing asynchronous is issued to the tensor core or the state's barrier, and every wait runs out.
+template <bool kFused, bool kDrill, class LB>
 __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& t, const LB& lb, int log_parts, const FusedPrevT<LB>* fp) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -262,9 +262,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
   const uint32_t rep_mul = 0xFFFFFFFFu / (uint32_t)rep + 1u;    // hv / rep = high word of hv * rep_mul (rep > 1)
   const int out_size = s.out_dtype == LUMO_BF16 ? 2 : 4;
   const uint32_t k_pitch = (uint32_t)s.Hk * kD, v_pitch = (uint32_t)s.Hv * kD;   // elements from one physical row to the next
-  // Test aid: nothing asynchronous is issued to the tensor core or the state's barrier, every wait runs out.
-  const bool drill = s.debug_skip_mma != 0;
-  const uint32_t spin_limit = drill ? kSpinLimitDrill : kSpinLimit;
+  constexpr uint32_t spin_limit = kDrill ? 1024 : 1u << 24;
   auto live = [](int meta) { return ((meta >> 16) & 0xFF) != 0; };               // a node, not the rest of the group's table
 
   // ---- the leading warp looks ahead ------------------------------------------------------------------------------------
@@ -441,7 +439,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       sm.unit = u;
       sm.unit_fresh = true;
       // the state is settled before this kernel may enter early; everything else may still be in the making
-      if (any && !drill) {
+      if (any && !kDrill) {
         request_state(sbase + kOffS, state_of(u.layer, u.row, u.hv), &sm.mb_state);
         ++requested;
       }
@@ -460,7 +458,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       store_gates(sm.node[0]);
       if constexpr (kFused) path_store(sm.step[0]);
     }
-    const uint32_t lead = drill ? 0u : elect_one();
+    const uint32_t lead = kDrill ? 0u : elect_one();
     uint32_t landed = 0;                                        // states that the others have seen arrive
     for (; sm.step[k & 3].have; ++k) {                          // bounded: the launch's work
       const Step &cur = sm.step[k & 3], &nxt = sm.step[(k + 1) & 3];
@@ -520,7 +518,7 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
         umma_commit(lead, &sm.mb_mma);
       }
       if (nxt.have) {
-        if (nxt.fresh && lane == 0 && !drill && !sm.state_missing) {   // (one copy at a time on the barrier)
+        if (nxt.fresh && lane == 0 && !kDrill && !sm.state_missing) {   // (one copy at a time on the barrier)
           request_state(sbase + kOffS, state_of(nxt.layer, nxt.row, nxt.hv), &sm.mb_state);
           ++requested;
         }
@@ -532,18 +530,24 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
       all();                                                    // the outputs are in tensor memory
       if (cur.fresh && !sm.state_missing) ++landed;
       if (sm.timed_out) {                                       // the same in every thread: report this unit and all that are left
-        auto give_up = [&](int layer, int b) {
+        auto give_up = [&](int layer, int b, bool replayed) {
+          const int row = lb.l[layer].state_row[b];
+          const int32_t st = row < 0 ? LUMO_SEQ_OK : row >= s.n_state_rows ? LUMO_SEQ_BAD_ROW : LUMO_SEQ_TIMEOUT;
           int32_t* status = lb.l[layer].status;
-          if (lane == 0 && status) status[b] = LUMO_SEQ_TIMEOUT;
+          if (status) status[b] = st;
+          if constexpr (kFused) {
+            int32_t* pst = fp->lb.l[layer].status;
+            if (pst && !replayed) pst[b] = st;
+          }
         };
-        give_up(cur.layer, cur.b);
-        if (nxt.have) give_up(nxt.layer, nxt.b);
-        Unit u = sm.unit;                                       // of the step after that
-        __syncwarp();
-        while (u.layer < s.n_layers) {                          // bounded: the launch's units
-          give_up(u.layer, u.b);
-          advance(u);
-          open(u);
+        if (lane == 0) {
+          give_up(cur.layer, cur.b, !(cur.fresh && sm.state_missing));
+          if (nxt.have) give_up(nxt.layer, nxt.b, !nxt.fresh);
+          Unit u = sm.unit;                                     // of the step after that
+          while (u.layer < s.n_layers) {                        // bounded: the launch's units
+            give_up(u.layer, u.bp >> log_parts, false);
+            advance(u);
+          }
         }
         break;
       }
@@ -917,16 +921,16 @@ __device__ __forceinline__ void scan_stream_body(const Shape& s, const TreeDev& 
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
 
-template <class LB>
+template <bool kDrill, class LB>
 __global__ void __launch_bounds__(kThreads + 32, 2) scan_stream_kernel(Shape s, TreeDev t, LB lb, int log_parts) {
-  scan_stream_body<false, LB>(s, t, lb, log_parts, nullptr);
+  scan_stream_body<false, kDrill, LB>(s, t, lb, log_parts, nullptr);
 }
-template <class LB>
+template <bool kDrill, class LB>
 __global__ void __launch_bounds__(kThreads + 32, 2) scan_stream_fused_kernel(Shape s, TreeDev t, LB lb, FusedPrevT<LB> fp) {
-  scan_stream_body<true, LB>(s, t, lb, 0, &fp);
+  scan_stream_body<true, kDrill, LB>(s, t, lb, 0, &fp);
 }
 
-template <class LB>
+template <bool kDrill, class LB>
 cudaError_t launch_t(const Shape& s, const TreeDev& t, const LB& lb, const FusedPrevT<LB>* fp, int sm_count, bool pdl, cudaStream_t st) {
   static bool configured[kMaxDevices] = {};                     // the shared-memory limit is a per-device setting
   int dev = 0;
@@ -934,13 +938,13 @@ cudaError_t launch_t(const Shape& s, const TreeDev& t, const LB& lb, const Fused
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (!configured[dev]) {
-    e = cudaFuncSetAttribute(scan_stream_kernel<LB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(scan_stream_fused_kernel<LB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = cudaFuncSetAttribute(scan_stream_kernel<kDrill, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(scan_stream_fused_kernel<kDrill, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
   const int items = s.n_layers * s.B * s.Hv, resident = 2 * sm_count;
-  if (fp) return launch_kernel(scan_stream_fused_kernel<LB>, dim3(items < resident ? items : resident), dim3(kThreads + 32), kSmemBytes, st, pdl, s, t, lb, *fp);
+  if (fp) return launch_kernel(scan_stream_fused_kernel<kDrill, LB>, dim3(items < resident ? items : resident), dim3(kThreads + 32), kSmemBytes, st, pdl, s, t, lb, *fp);
   // A tree of several groups may be shared by CTAs that fetch the same state: what counts is the longest CTA, in steps
   // (a state's fetch and conversion cost about a third of a step)
   int log_parts = 0;
@@ -953,7 +957,7 @@ cudaError_t launch_t(const Shape& s, const TreeDev& t, const LB& lb, const Fused
     }
   }
   const int units = items << log_parts;
-  return launch_kernel(scan_stream_kernel<LB>, dim3(units < resident ? units : resident), dim3(kThreads + 32), kSmemBytes, st, pdl, s, t, lb, log_parts);
+  return launch_kernel(scan_stream_kernel<kDrill, LB>, dim3(units < resident ? units : resident), dim3(kThreads + 32), kSmemBytes, st, pdl, s, t, lb, log_parts);
 }
 
 }  // namespace
@@ -997,11 +1001,15 @@ bool scan_stream_pays(const Shape& s, const TreeDev& t, bool fused, int sm_count
 
 cudaError_t launch_scan_stream(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sm_count, bool pdl,
                                cudaStream_t st) {
-  if (s.n_layers > kFewLayers) return launch_t(s, t, lb, fp, sm_count, pdl, st);
-  const FewLayers few = few_layers(lb);
-  if (!fp) return launch_t<FewLayers>(s, t, few, nullptr, sm_count, pdl, st);
-  const FusedPrevT<FewLayers> prev = few_layers(*fp);
-  return launch_t<FewLayers>(s, t, few, &prev, sm_count, pdl, st);
+  auto launch = [&](auto drill) {                               // (the kernels in use do not carry the test aid)
+    constexpr bool kDrill = decltype(drill)::value;
+    if (s.n_layers > kFewLayers) return launch_t<kDrill>(s, t, lb, fp, sm_count, pdl, st);
+    const FewLayers few = few_layers(lb);
+    if (!fp) return launch_t<kDrill, FewLayers>(s, t, few, nullptr, sm_count, pdl, st);
+    const FusedPrevT<FewLayers> prev = few_layers(*fp);
+    return launch_t<kDrill, FewLayers>(s, t, few, &prev, sm_count, pdl, st);
+  };
+  return s.debug_skip_mma ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 }  // namespace lumo

@@ -1,7 +1,11 @@
 """The streamed scan (closed form, state in tensor memory) at its edges: groups of 32 nodes and what is left over, trees cut into
 groups that share one state or are dealt out to several CTAs, skipped and padded rows, both output types, and values that are
-not finite.  Bound: keys, values and queries enter exactly, the state, q~ and M diag(beta) as two bf16 terms each, which leaves
-2^-17 of every factor; products of at most 128 + 32 terms of the outputs' own size stay below 2^-17 * sqrt(160) = 1e-4."""
+not finite.
+
+Bound: keys, values and queries enter exactly, the state, q~, M diag(beta) and the coefficients of q~ as two bf16 terms each, which leaves
+2^-18 of a factor, and the product of two low terms is dropped, another 2^-18.  The same arithmetic in float64 on trees like these is off
+by 1.1e-6 to 3.3e-6 (1 + |ref|), and the tensor core's fp32 sums add as much again (measured 4.7e-6 at most).  With a low term left out
+it is off by 9e-6 to 3e-5 (coefficients of q~), 1e-4 (q~, the state) or 6e-4 to 2e-3 (M diag(beta))."""
 import numpy as np
 import pytest
 import torch
@@ -12,6 +16,7 @@ from tests.graph_nodes import Captured
 from tests.harness import assert_close, ctx, oracle_scan_from_device
 
 pytestmark = pytest.mark.gpu
+BOUND = 8e-6
 
 
 def _case(N, B, Hk, Hv, L, depth, seed=0):
@@ -36,7 +41,7 @@ def test_outputs_match_oracle(N, B, Hk, Hv, L, depth, out_dtype):
     for l in range(L):
         ref, _, _ = oracle_scan_from_device(dc, layer=l)
         worst = assert_close(dc.np("out", l), ref, bf16=out_dtype == "bf16", what=f"layer {l}")
-        assert out_dtype == "bf16" or worst < 1e-4
+        assert out_dtype == "bf16" or worst < BOUND
         assert dc.np("status", l).tolist() == [0] * B
         for b in range(B):
             pad = sorted(set(range(c.Ns)) - set(c.slot[b].tolist()))
@@ -45,11 +50,13 @@ def test_outputs_match_oracle(N, B, Hk, Hv, L, depth, out_dtype):
 
 @pytest.mark.parametrize("which", ["q", "k", "v"])
 @pytest.mark.parametrize("value", [float("nan"), float("inf")])
-@pytest.mark.parametrize("N,B,L", [(30, 3, 8), (150, 2, 3)])
-def test_values_that_are_not_finite_stay_on_their_paths(which, value, N, B, L):
-    """One element of one node: its descendants' outputs are gone (a query's: its own alone), every other output keeps its bits."""
+@pytest.mark.parametrize("N,B,L", [(30, 3, 8), (150, 2, 3), (150, 2, 4)])
+@pytest.mark.parametrize("out_dtype", ["f32", "bf16"])
+def test_values_that_are_not_finite_stay_on_their_paths(which, value, N, B, L, out_dtype):
+    """One element of one node: its descendants' outputs are gone (a key's or value's: NaN in whole rows; a query's: its own alone), every
+    other output keeps its bits."""
     c = _case(N, B, 16, 32, L, 9, seed=3)
-    dc = DeviceCase(ctx("tensor"), c, use_conv=False, qk_l2norm=True)
+    dc = DeviceCase(ctx("tensor"), c, out_dtype=out_dtype, use_conv=False, qk_l2norm=True)
     dc.verify()
     torch.cuda.synchronize()
     clean = dc.t("out", L - 1).clone()
@@ -65,6 +72,7 @@ def test_values_that_are_not_finite_stay_on_their_paths(which, value, N, B, L):
     gone = [int(c.slot[b, i]) for i in range(N) if below[i]]
     kept = [int(c.slot[b, i]) for i in range(N) if not below[i]]
     assert not torch.isfinite(got[b, gone]).all(dim=-1).any()
+    assert which == "q" or torch.isnan(got[b, gone]).all()
     assert torch.equal(got[b, kept], clean[b, kept]) and torch.equal(got[:b], clean[:b])
 
 
@@ -82,4 +90,4 @@ def test_the_form_that_measured_faster_is_taken(N, depth, items, streamed):
     torch.cuda.synchronize()
     ctx("auto")
     ref, _, _ = oracle_scan_from_device(dc)
-    assert assert_close(dc.np("out"), ref) < 1e-4
+    assert assert_close(dc.np("out"), ref) < (BOUND if streamed else 2 ** -15)     # (the closed form: pairs of 2^-16 on either side)

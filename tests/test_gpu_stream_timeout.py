@@ -71,8 +71,9 @@ def test_every_unit_of_a_fused_call_reports_the_timeout(drill):
     drill(True)
     call()
     torch.cuda.synchronize()
-    for layer in layers:
+    for l, layer in enumerate(layers):
         assert layer.tensors["status"].tolist() == [binding.SEQ_TIMEOUT] * 3
+        assert dcP.np("status", l).tolist() == [binding.SEQ_TIMEOUT] * 3         # nothing was committed
 
 
 def test_a_state_that_does_not_arrive_is_not_written_back(drill):
