@@ -964,39 +964,29 @@ cudaError_t launch_t(const Shape& s, const TreeDev& t, const LB& lb, const Fused
 
 // Where the streamed scan takes the place of the closed form with the tensor-core sum (scan_gram.cu).  Measured at 380 points over
 // 4 to 256 nodes and 32 to 4096 items (a state each), launches overlapped, us, closed form / streamed:
-//   * groups of 32 alone: always.  16 nodes, 32 items 6.0 / 5.6, 304 14.8 / 11.2, 2048 54.9 / 48.4; 28 nodes 7.0 / 5.7, 16.6 / 11.9,
-//     61.5 / 49.7.
-//   * one group of 64 that falls into two or three of 32.  As long as the parts of a tree find SMs of their own, always (64 nodes,
-//     72 items 10.6 / 9.9; 56 nodes 10.6 / 6.8).  Then a second CTA on the SM, or two or three steps in a row, cost more than the
-//     one wave of larger tiles: 2.0 groups, 148 items 11.1 / 9.3 but 2.2 11.4 / 11.9 and 3 11.6 / 12.7; one wave of whole trees, 2.0
-//     groups 50 nodes, 224 items 13.2 / 12.7, 44 nodes, 292 13.6 / 14.5, 2.03 groups, 152 12.6 / 14.9, 3 14.8 / 18.4.  From the
-//     second wave on two groups win (50 nodes, 304 items 22.8 / 17.9, 800 44 / 40), three lose (64 nodes, 512 28.8 / 31.3, 2048
-//     98.8 / 107.3) and 2.2 lie between: 304 23.4 / 20.0, 440 26.8 / 29.4, 1000 55.7 / 49.0.
-//   * several groups of 64: nearly always (256 nodes, 1024 items 213 / 172; 70 nodes, 224 items 24.4 / 16.8).  Not where the larger
-//     tiles make one wave and the tree's halves, on shared SMs, three steps (128 nodes, 84 items 13.2 / 16.3; 96 nodes, two steps,
-//     148 items 14.2 / 13.7), nor where they make two and the whole trees a second CTA on a few SMs (160 nodes, 180 items 26.0 / 32.5).
-// With the commit folded in (whole calls) groups of 32 alone: from two full waves on at any size (8 nodes, 592 items 34.8 / 35.8, 1200
-// 67.4 / 65.5, 28 nodes, 1536 99.8 / 94.1), before that at 28 nodes and more where no SM holds a second CTA (28 nodes, 128 items 21.3
-// / 20.0) or one wave is not enough (320 33.9 / 32.8), but 200 23.5 / 24.4; 8 nodes, 96 items 14.6 / 17.5.  Trees that need a second
-// group keep the 64-node tile: 34 nodes, 1536 items 118 / 122, 64 nodes 141 / 154.
+//   * groups of 32 alone: always.  16 nodes, 32 items 6.0 / 5.0, 304 14.8 / 10.4, 2048 54.9 / 45.1; 28 nodes 7.0 / 5.3, 16.6 / 11.0, 61.5 / 46.6.
+//   * one group of 64 that falls into two or three of 32: nearly always.  As long as the parts of a tree find SMs of their own (64
+//     nodes, 72 items 10.6 / 8.8); from the fifth wave on (56 nodes, 2048 items 95.8 / 76.3; 64 nodes 98.8 / 98.4); with fewer than three
+//     groups also between (58 nodes, 448 items 26.7 / 25.0; 62 nodes, 148 11.6 / 11.6), where three lose (64 nodes, 148 items 11.3 /
+//     12.0, 340 23.9 / 27.9).  One wave of whole trees waits for its longest: two groups each win (50 nodes, 224 items 13.2 / 11.9), a
+//     few trees of three turn it (57 nodes, 156 items 12.9 / 13.4), three lose most (64 nodes, 292 items 14.6 / 17.0).
+//   * several groups of 64: nearly always (256 nodes, 1024 items 213 / 157; 70 nodes, 224 items 24.4 / 15.5).  Not where the larger
+//     tiles make one wave and a tree's halves, on shared SMs, three steps (150 nodes, 84 items 13.4 / 16.7; 96 nodes, two steps, 148
+//     items 14.2 / 12.9), nor where they make two and whole trees of six steps put a second CTA on a few SMs (160 nodes, 180 items
+//     26.0 / 30.0; 128 nodes, five steps, 176 items 25.2 / 24.7).
+// With the commit folded in (whole calls) groups of 32 alone: from the second wave on (8 nodes, 448 items 32.3 / 31.7, 1200 67.4 / 62.6;
+// 20 nodes, 1200 75.2 / 69.6), before that from 20 nodes on (20 nodes, 76 items 19.2 / 17.9; 16 nodes 16.5 / 17.6; 8 nodes, 152 17.4 /
+// 19.4), never where every CTA has an SM to itself (28 nodes, 64 items 18.4 / 19.6).  Trees that need a second group keep the 64-node
+// tile: 34 nodes, 1536 items 118 / 122, 64 nodes 141 / 154.
 bool scan_stream_pays(const Shape& s, const TreeDev& t, bool fused, int sm_count) {
   const long long sms = sm_count, items = (long long)s.n_layers * s.B * s.Hv, B = s.B, g32 = t.st_groups;
-  const bool apart = 2 * items <= sms, one_each = items <= sms, one_wave = items <= 2 * sms;     // CTAs with an SM to themselves, a state each
-  if (fused) {
-    if (g32 != B) return false;
-    return items > 4 * sms || (s.N >= 28 && !apart && (one_each || !one_wave));
-  }
+  const bool apart = 2 * items <= sms, one_wave = items > sms && items <= 2 * sms;
+  if (fused) return g32 == B && !apart && (s.N >= 20 || items > 2 * sms);
   if (g32 == B || apart) return true;
-  const bool two = 16 * g32 <= 33 * B;                            // groups a tree: two, but for a few
-  if (t.n_groups == s.B) {
-    if (one_each) return two;
-    if (one_wave) return g32 == 2 * B && s.N >= 50;
-    if (5 * items > 13 * sms && items <= 4 * sms) return two;
-    return 3 * g32 <= 7 * B;
-  }
+  if (t.n_groups == s.B) return one_wave ? g32 == 2 * B : items > 4 * sms || 10 * g32 < 29 * B;
   const long long tiles = (long long)s.n_layers * t.n_groups * s.Hv;
-  if (tiles <= 2 * sms) return g32 <= 4 * B;
-  return one_each || tiles > 4 * sms || 2 * g32 <= 9 * B;
+  if (tiles <= 2 * sms) return 12 * g32 <= 49 * B;                // (four groups a tree, but for a few)
+  return items <= sms || tiles > 4 * sms || 10 * g32 <= 51 * B;
 }
 
 cudaError_t launch_scan_stream(const Shape& s, const TreeDev& t, const LayerBatch& lb, const FusedPrev* fp, int sm_count, bool pdl,
