@@ -127,17 +127,18 @@ int64_t lumo_ctx_scratch_bytes(const lumo_ctx* ctx);
  * waits for another node), 5 = the closed form of 4 with that sum as one more tensor-core product over all
  * nodes of a group (right-hand sides and coefficients as bf16 hi + lo: relative 2^-16 on the sum; a right-hand
  * side that is not finite is kept out of the product and turns the outputs of its own subtree into NaN, as the
- * recurrence would).  "Automatic" picks between 2 and 5 per descriptor and launch (thin deep trees, a spine with
+ * recurrence would), or, where that measured faster (nearly everywhere), the same closed form with the state streamed
+ * through tensor memory in groups of 32 nodes.  "Automatic" picks between 2 and 5 per descriptor and launch (thin deep trees, a spine with
  * small side branches, take 5; other trees take 5 in launches of several waves where it measured faster; the
  * rest take 2).  2 to 5 return LUMO_ERR_UNSUPPORTED on other shapes. */
 int lumo_ctx_set_scan_algo(lumo_ctx* ctx, int algo);
 
-/* Test aid for the failure path of the tensor-core scan.  That kernel waits for its tensor-core work
- * on an mbarrier with a bounded number of polls; when the bound runs out it writes LUMO_SEQ_TIMEOUT
- * into the status words, frees its tensor memory and returns.  With the drill on, the kernel issues
- * no tensor-core work at all (so nothing asynchronous is in flight) and polls only 1024 times: the
- * wait runs out by construction and the failure path executes, harmlessly.  Outputs of such a call are
- * undefined.  Default off. */
+/* Test aid for the failure path of the tensor-core scans.  They wait for their tensor-core work (the streamed scan also
+ * for the state's copy) on mbarriers with a bounded number of polls; when the bound runs out they write LUMO_SEQ_TIMEOUT
+ * into the status words, free their tensor memory and return.  With the drill on, the solved scan (algorithm 3) and the
+ * streamed scan (0 and 5, where they stream) issue no tensor-core work and no such copy (so nothing asynchronous is in
+ * flight) and poll only 1024 times: the waits run out by construction and the failure path executes, harmlessly.  The
+ * other forms run as ever.  Outputs of such a call are undefined (a streamed commit_verify changes no state).  Default off. */
 int lumo_ctx_set_timeout_drill(lumo_ctx* ctx, int on);
 
 /* Kernel overlap (default on): the kernels of every call are launched with programmatic dependent launch,
@@ -338,7 +339,8 @@ int lumo_gdn_commit(lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo_gdn_ar
  * Sec. "Temporary state versus recomputation").  prev_layers[l] and layers[l] must name the same
  * state, state_row and conv_hist and must share shapes, dtypes and options; the previous cycle's
  * q/k/v/x/gates must live in buffers of their own (they are read while the new ones are written).
- * prev_layers[l].status receives the commit's per-sequence status, layers[l].status the verify's.
+ * prev_layers[l].status receives the commit's per-sequence status, layers[l].status the verify's.  After LUMO_SEQ_TIMEOUT a
+ * sequence's history and the states of some of its heads may be the committed ones, the others as they were.
  * The fused kernel serves d = 128, bf16 operands, trees of at most 64 nodes and depth 16,
  * lmax <= 16; every other case runs the two calls above one after the other.  Enqueues only. */
 int lumo_gdn_commit_verify(lumo_ctx* ctx, const lumo_tree_desc* prev_desc, const lumo_gdn_args* prev_layers,

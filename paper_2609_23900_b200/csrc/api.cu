@@ -437,13 +437,14 @@ int lumo_tree_desc_create(lumo_ctx* ctx, int batch, int n_nodes, int n_slots, co
       h[o_st_off + B] = (int32_t)sgi;
     }
   }
-  // measured on B200 (us per item): substitution 0.45 per round, closed form 1.7 + 0.08 per node; the
-  // closed form is taken when it wins by a margin (28-node spine trees of depth 12: 18.5 -> 17.0 us per
-  // launch at batch 8; 64-node trees of depth 8 stay with the substitution: 19.1 against 20.5 us)
+  // Both lines are the substitution (0.45 us per round and item) against the closed forms of scan_gram.cu; the streamed scan, which now
+  // takes their place nearly everywhere, is faster than they are and could be taken on more trees (and loses accuracy: 2.6e-6 against 2
+  // to 5e-7).  Closed form 1.7 us + 0.08 per node, taken when it wins by a margin (28-node spine trees of depth 12: 18.5 -> 17.0 us
+  // per launch at batch 8; 64-node trees of depth 8 stay with the substitution: 19.1 against 20.5 us).
   d->closed_form_pays = tc && 100 * subst_rounds > 600 * (long long)G + 18 * group_nodes;
-  // measured with the tensor-core sum (launch times, us, substitution against it): 48 layers of 32-node trees
-  // 190 -> 175, 256-node chains 225 -> 190, random 256-node trees 236 -> 218; a 255-child star 177 -> 200 and
-  // single-wave launches (64-node trees at batch 8: equal within 1%, at four times the error) stay
+  // With the tensor-core sum 0.3 + 0.078 per node (launch times, us, substitution / it / streamed): 48 layers of 32-node trees 190 /
+  // 175 / 121, 256-node chains 225 / 190 / 138, random 256-node trees 236 / 218 / 157; a 255-child star (177 / 200, not measured
+  // streamed) and single-wave launches (64-node trees at batch 8, substitution 19.1) stay.
   d->tensor_tail_pays = tc && 450 * subst_rounds > 300 * (long long)G + 78 * group_nodes;
   if (ctx->device < 0) { *out = d; return LUMO_OK; }   // host-only: tables stay on the host
   DeviceGuard g(ctx->device);
@@ -558,7 +559,7 @@ int lumo_select_spine_top3(lumo_ctx* ctx, const lumo_select_args* a, int32_t* sp
 }
 
 // Which tail the Gram-form scan takes: 0 level-by-level substitution, 1 closed form, 2 closed form with the output
-// sum on the tensor core.  Automatic: thin deep trees take 2 (equal to 1 there, measured); other trees take 2 when
+// sum on the tensor core, streamed where that pays (scan_stream.cu).  Automatic: thin deep trees take 2 (equal to 1 there, measured); other trees take 2 when
 // the descriptor says it pays and the launch has several waves of items; everything else takes 0.
 static int scan_tail(const lumo_ctx* ctx, const lumo_tree_desc* desc, const lumo::Shape& s) {
   if (ctx->scan_algo == 5) return 2;

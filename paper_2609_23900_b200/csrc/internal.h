@@ -57,7 +57,7 @@ struct lumo_ctx {
   cudaStream_t setup = nullptr; // set-up copies, waited for by the call that makes them (created by the first)
   // optional per-launch timing (lumo_ctx_timing_*): a fixed pool of event pairs
   int scan_algo = 0;            // 0 auto, 1 rank-1, 2 Gram form with forward substitution, 3 solved Gram form, 4 Gram form with closed-form tail, 5 the same with the output sum on the tensor core
-  bool timeout_drill = false;   // test aid: the tensor-core scan skips its tensor-core work (lumo_ctx_set_timeout_drill)
+  bool timeout_drill = false;   // test aid: the solved and the streamed scan skip their tensor-core work (lumo_ctx_set_timeout_drill)
   bool overlap = true;          // kernels are launched as programmatic dependents of the kernel before them
   lumo::CallOrder order;        // what is in front of a call in its stream: decides what may be read ahead of a dependency wait
   bool timing = false;
@@ -101,7 +101,8 @@ struct lumo_tree_desc {
   // eight nodes of a level, the closed-form tail a fixed part plus a part per node: thin, deep trees (a
   // spine with small side branches) are cheaper in closed form, wide ones by levels.
   bool closed_form_pays = false;
-  // the same comparison for the closed form whose output sum is one tensor-core product (0.3 + 0.078 per node):
+  // the same comparison for the closed form whose output sum is one tensor-core product (0.3 + 0.078 per node; the streamed
+  // scan, which runs in its place nearly everywhere, is cheaper):
   // it pays on more trees, but only in launches of several waves, where an item's instruction count rather than
   // its latency sets the pace
   bool tensor_tail_pays = false;
@@ -150,7 +151,7 @@ struct Shape {
   int snapshot_mode, n_snap;
   int n_layers;
   int gate_mode;
-  int debug_skip_mma;   // test aid of the tensor-core scan: issue no tensor-core work, let the bounded wait run out
+  int debug_skip_mma;   // test aid of the solved and the streamed scan: issue no tensor-core work, let the bounded wait run out
   int wait_first;         // commit: read nothing ahead of the dependency wait
 };
 

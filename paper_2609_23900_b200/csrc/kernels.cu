@@ -176,7 +176,8 @@ __device__ __forceinline__ bool mbar_wait0(unsigned long long* bar) {
 // -> 6.9 -> 6.3 us (now), spines of 64 7.3 -> 8.1 -> 7.2, 32 x 256 of 8192 channels 105 -> 115 -> 105; three CTAs per SM with room for
 // everything 8.1 us (8 x 64: no longer one wave).  Where a sequence falls into several parts, the window of a part's first entry is
 // staged with the part's own rows, so that whoever shares it (in a star everyone) does not go to L1 for it: 32 stars of 256 nodes, fp32,
-// 102.5 (transposed) -> 111.5 (fetched by every entry) -> 103.0 us (now), 12 x 140 nodes 22.9 -> 25.1 -> 22.4; bf16 as before.
+// 102.5 (transposed) -> 111.5 (fetched by every entry) -> 103.0 us (now), 12 x 140 nodes 22.9 -> 25.1 -> 22.4;
+// bf16 stars 61.1 -> 58.4, other trees of several parts within 2 % of before.
 
 // kFused: the three history rows are the ones the previous cycle's accepted path will commit, i.e. the
 // last three of [old history ; raw inputs of the accepted nodes], read in place through the path (the
